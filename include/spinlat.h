@@ -364,15 +364,15 @@ void sl_batch_destroy(sl_batch *b);
  *   cuda_stream         cudaStream_t the work is ordered on (NULL: default stream);
  *                       the call returns after the stream has drained
  * FP64 throughout, no neighbour skin (an exact all-pairs search inside rc_rad).
- * The scratch (about 6.3 MB: lists, descriptor columns, angular sums, a status
- * word) is one fixed array compiled into the library, resident on every GPU that
- * loads it until the process exits.  No call allocates device memory; n above
- * 2048 atoms returns SL_EINVAL, more than 160 neighbours inside rc_rad returns
- * SL_ENBR_OVERFLOW, and a species value outside [0, n_species) (checked on the
- * device, where the array lives) returns SL_EINVAL.  The first call on a device
- * looks up the array's device address (and may load the library's device code);
- * make that first call before any stream capture.  Every call uses the same array, so calls whose work
- * overlaps on the GPU (other streams, other host threads) race: serialise them. */
+ * The kernel works in shared memory; its one status word is a fixed variable compiled
+ * into the library, resident on every GPU that loads it until the process exits.  No call
+ * allocates device memory; n above 2048 atoms returns SL_EINVAL, more than 160 neighbours
+ * inside rc_rad returns SL_ENBR_OVERFLOW, and a species value outside [0, n_species)
+ * (checked on the device, where the array lives) returns SL_EINVAL.  The first call on a
+ * device looks up the variable's device address (and may load the library's device code);
+ * make that first call before any stream capture.  Every call uses the same status word, so
+ * calls whose work overlaps on the GPU (other streams, other host threads) race: serialise
+ * them. */
 int sl_descriptors_energies_noalloc(const double *positions4, const double *spins4, const int32_t *species,
                                     int64_t n, const double box[3], const int32_t periodic[3],
                                     const sl_nep_params *params, double *q, double *atom_energy,

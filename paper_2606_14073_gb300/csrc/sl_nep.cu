@@ -1,4 +1,4 @@
-// sl_nep.cu -- NEP-SPIN descriptor, network and backward kernels (one thread per atom).
+// sl_nep.cu -- the NEP-SPIN model, its CUDA-core network and the no-allocation evaluation.
 //
 // Descriptor of atom i (arXiv 2606.14073, Sections 5.1.1-5.1.2; 66 entries, Section 5.2.3):
 //   R_n  = sum_j g^R_n(r_ij)                           radial, r < rc_rad
@@ -10,8 +10,8 @@
 // The angular channels use the harmonic (addition-theorem) form: one pass over
 // neighbours per channel n instead of the pair double sum.
 //
-// This file holds the per-atom forward (one thread per atom, used by the
-// no-allocation entry point) and the CUDA-core network k_mlp:
+// This file holds the no-allocation entry point's kernel (one warp per atom) and the
+// CUDA-core network k_mlp:
 //   E_i and Fp = dE_i/dq_i.
 // The step's evaluation kernels are in sl_eval2.cu; forces and fields are gathered
 // without atomics (sl_integrate.cu):
@@ -29,155 +29,12 @@
 
 namespace sl {
 
-template <typename R> struct V2;
-template <> struct V2<float> { using t = float2; };
-template <> struct V2<double> { using t = double2; };
-template <typename R> using v2 = typename V2<R>::t;
-
-template <typename R>
-struct EvalArgs {
-    const v4<R> *pos;
-    const v4<R> *spin;
-    const int32_t *nbr;
-    const int4 *seg;
-    int64_t n, n_fe;
-    BoxDev<R> box;
-    R *q, *bsum, *fp, *ei;
-    v4<R> *pd0;
-    v2<R> *pd1;
-    v4<R> *fown, *gii;
-    R *wpart;
-    int want_virial;
-};
-
 template <typename R>
 __device__ __forceinline__ R tanh_(R x);
 template <>
 __device__ __forceinline__ float tanh_<float>(float x) { return tanhf(x); }
 template <>
 __device__ __forceinline__ double tanh_<double>(double x) { return tanh(x); }
-
-// ------------------------------------------------------------------ forward
-template <typename R, int TI, int TJ>
-__device__ __forceinline__ void fwd_radial(const NepDev<R> &P, const EvalArgs<R> &a, int64_t i, const v4<R> &pi,
-                                           const v4<R> &si, int s0, int s1, R qr[NCH], R qx[4][NCH]) {
-    R b0[NK], b1[NK], b2[NK], b3[NK], b4[NK];
-#pragma unroll
-    for (int k = 0; k < NK; ++k) { b0[k] = b1[k] = b2[k] = b3[k] = b4[k] = R(0); }
-    for (int s = s0; s < s1; ++s) {
-        const int j = a.nbr[(int64_t)s * a.n + i];
-        const v4<R> pj = a.pos[j];
-        R dx = pj.x - pi.x, dy = pj.y - pi.y, dz = pj.z - pi.z;
-        minimg(a.box, dx, dy, dz);
-        const R d2 = dx * dx + dy * dy + dz * dz;
-        if (d2 < P.rc_r2) {
-            const v4<R> sj = a.spin[j];
-            const R ir = rsqrt_(d2), r = d2 * ir;
-            const R ux = dx * ir, uy = dy * ir, uz = dz * ir;
-            R f[NK];
-            carrier_f(r, P.inv_rc_r, f);
-            const R sij = si.x * sj.x + si.y * sj.y + si.z * sj.z;
-            const R siu = si.x * ux + si.y * uy + si.z * uz;
-            const R sju = sj.x * ux + sj.y * uy + sj.z * uz;
-            const R dmi = (si.y * sj.z - si.z * sj.y) * ux + (si.z * sj.x - si.x * sj.z) * uy +
-                          (si.x * sj.y - si.y * sj.x) * uz;
-            const R ani = siu * sju, sia = siu * siu;
-#pragma unroll
-            for (int k = 0; k < NK; ++k) {
-                b0[k] += f[k];
-                b1[k] += f[k] * sij;
-                b2[k] += f[k] * dmi;
-                b3[k] += f[k] * ani;
-                b4[k] += f[k] * sia;
-            }
-        }
-    }
-#pragma unroll
-    for (int n = 0; n < NCH; ++n) {
-#pragma unroll
-        for (int k = 0; k < NK; ++k) {
-            qr[n] += P.c[TI][TJ][G_R][n][k] * b0[k];
-            qx[0][n] += P.c[TI][TJ][G_EX][n][k] * b1[k];
-            qx[1][n] += P.c[TI][TJ][G_DMI][n][k] * b2[k];
-            qx[2][n] += P.c[TI][TJ][G_ANI][n][k] * b3[k];
-            qx[3][n] += P.c[TI][TJ][G_SIA][n][k] * b4[k];
-        }
-    }
-}
-
-template <typename R, int TI, int TJ>
-__device__ __forceinline__ void fwd_angular(const NepDev<R> &P, const EvalArgs<R> &a, int64_t i, const v4<R> &pi,
-                                            const v4<R> &si, int n, int s0, int s1, R B[NLM], R BS[NLM]) {
-    for (int s = s0; s < s1; ++s) {
-        const int j = a.nbr[(int64_t)s * a.n + i];
-        const v4<R> pj = a.pos[j];
-        R dx = pj.x - pi.x, dy = pj.y - pi.y, dz = pj.z - pi.z;
-        minimg(a.box, dx, dy, dz);
-        const R d2 = dx * dx + dy * dy + dz * dz;
-        if (d2 < P.rc_a2) {
-            const v4<R> sj = a.spin[j];
-            const R ir = rsqrt_(d2), r = d2 * ir;
-            R f[NK];
-            carrier_f(r, P.inv_rc_a, f);
-            R g = R(0);
-#pragma unroll
-            for (int k = 0; k < NK; ++k) g += P.c[TI][TJ][G_A][n][k] * f[k];
-            const R gs = g * (si.x * sj.x + si.y * sj.y + si.z * sj.z);
-            R p[NLM];
-            harm_p(dx * ir, dy * ir, dz * ir, p);
-#pragma unroll
-            for (int lm = 0; lm < NLM; ++lm) {
-                B[lm] += g * p[lm];
-                BS[lm] += gs * p[lm];
-            }
-        }
-    }
-}
-
-template <typename R, int TI>
-__device__ __forceinline__ void fwd_atom(const NepDev<R> &P, const EvalArgs<R> &a, int64_t i) {
-    const v4<R> pi = a.pos[i], si = a.spin[i];
-    const int4 sg = a.seg[i];
-    const int64_t N = a.n;
-    R qr[NCH], qx[4][NCH];
-#pragma unroll
-    for (int n = 0; n < NCH; ++n) { qr[n] = R(0); qx[0][n] = qx[1][n] = qx[2][n] = qx[3][n] = R(0); }
-    fwd_radial<R, TI, 0>(P, a, i, pi, si, 0, sg.x, qr, qx);
-    fwd_radial<R, TI, 1>(P, a, i, pi, si, sg.x, sg.y, qr, qx);
-    fwd_radial<R, TI, 0>(P, a, i, pi, si, sg.y, sg.z, qr, qx);
-    fwd_radial<R, TI, 1>(P, a, i, pi, si, sg.z, sg.w, qr, qx);
-#pragma unroll
-    for (int n = 0; n < NCH; ++n) {
-        a.q[(Q_R + n) * N + i] = qr[n];
-        a.q[(Q_EX + n) * N + i] = qx[0][n];
-        a.q[(Q_DMI + n) * N + i] = qx[1][n];
-        a.q[(Q_ANI + n) * N + i] = qx[2][n];
-        a.q[(Q_SIA + n) * N + i] = qx[3][n];
-    }
-    a.q[Q_O * N + i] = si.x * si.x + si.y * si.y + si.z * si.z;
-#pragma unroll 1
-    for (int n = 0; n < NCH; ++n) {
-        R B[NLM], BS[NLM];
-#pragma unroll
-        for (int lm = 0; lm < NLM; ++lm) { B[lm] = R(0); BS[lm] = R(0); }
-        fwd_angular<R, TI, 0>(P, a, i, pi, si, n, 0, sg.x, B, BS);
-        fwd_angular<R, TI, 1>(P, a, i, pi, si, n, sg.x, sg.y, B, BS);
-        R qa[4] = {R(0), R(0), R(0), R(0)}, qs[4] = {R(0), R(0), R(0), R(0)};
-#pragma unroll
-        for (int lm = 0; lm < NLM; ++lm) {
-            const R kap = R(harm_kappa(lm));
-            qa[harm_l(lm) - 1] += kap * B[lm] * B[lm];
-            qs[harm_l(lm) - 1] += kap * BS[lm] * BS[lm];
-            a.bsum[(int64_t)(n * NLM + lm) * N + i] = B[lm];
-            a.bsum[(int64_t)(NCH * NLM + n * NLM + lm) * N + i] = BS[lm];
-        }
-#pragma unroll
-        for (int l = 0; l < 4; ++l) {
-            a.q[(int64_t)(Q_A + n * 4 + l) * N + i] = qa[l];
-            a.q[(int64_t)(Q_SA + n * 4 + l) * N + i] = qs[l];
-        }
-    }
-}
 
 // ------------------------------------------------------------------ network
 // E_i = sum_h w1_h tanh(z_h) - b1, z_h = sum_v W0_hv s_v q_v - b0_h;
@@ -249,123 +106,330 @@ void launch_net_t_fp64(const FusedTables &t, const NepDev<double> &P, const Laun
 }
 
 // ------------------------------------------------------------------ no-allocation variant
-// Descriptors and network energies of a small system in ONE kernel whose scratch
-// (neighbour lists, list segments, descriptor columns, angular sums, a status
-// word) lives in a fixed file-scope device array instead of memory the caller or
-// the library allocates.  For callers that may not allocate device memory (see
-// sl_descriptors_energies_noalloc in spinlat.h).  Computes in FP64.
+// Descriptors and network energies of a small system in ONE kernel that needs no device
+// memory but a status word (a fixed file-scope device variable) beside its shared memory.  For
+// callers that may not allocate (see sl_descriptors_energies_noalloc in spinlat.h).  Computes
+// in FP64.
+//
+// One warp per atom, four atoms per block.  What bounds it: the FP64 pipe (two lanes per SM
+// and cycle, so a warp's FP64 instruction takes 16 cycles of its SM); every stage therefore
+// keeps as many of the 32 lanes busy as it can, and what is not FP64 arithmetic of the result
+// stays off that pipe:
+//   search    all pairs, FP32 separations of the staged positions; only pairs within the
+//             rounding band around the cutoff take the exact FP64 test;
+//   pairs     lanes over pairs, 32 at a time: geometry, carrier and spin products, staged in
+//             shared memory;
+//   sums      lanes over (k, third of the staged pairs): five group sums each; in the angular
+//             part over (channel, four harmonics): eight sums each;
+//   network   lanes over hidden units.
+// A call on 1,000 atoms takes 0.13 ms, host side included; with one thread per atom (16 blocks
+// at most, the search and the angular channels serial in each thread) it took 6.2 ms.
 namespace noalloc {
 
 constexpr int MAX_ATOMS = 2048;
 constexpr int MAX_NBR = 160;   // neighbours inside rc_rad per atom
-constexpr size_t align256(size_t b) { return (b + 255) / 256 * 256; }
-constexpr size_t OFF_NBR = 0;
-constexpr size_t OFF_SEG = align256(OFF_NBR + sizeof(int32_t) * MAX_ATOMS * MAX_NBR);
-constexpr size_t OFF_Q = align256(OFF_SEG + sizeof(int4) * MAX_ATOMS);
-constexpr size_t OFF_B = align256(OFF_Q + sizeof(double) * DIM * MAX_ATOMS);
-constexpr size_t OFF_STATUS = align256(OFF_B + sizeof(double) * NB * MAX_ATOMS);
-constexpr size_t BYTES = align256(OFF_STATUS + sizeof(int));
+constexpr int WARPS = 4;       // atoms (warps) per block
+constexpr int LD = 33;         // row length of a staged entry: 32 pairs and a pad against bank conflicts
+constexpr int STAGE = 34 * LD; // angular stage: g_n, s g_n, the 24 harmonics (the radial one has 13 rows)
+constexpr int W0_LD = DIM + 1;
+constexpr int NCOEF = NS * NS * 6 * NCH * NK;
 
-// ~6.3 MB, held by every GPU that loads the library until the process exits.
-static __device__ __align__(256) unsigned char g_scratch[BYTES];
+// The status word of a call, held by every GPU that loads the library until the process exits.
+static __device__ int g_status;
 
-__global__ void __launch_bounds__(128) k_eval_noalloc(const __grid_constant__ NepDev<double> P,
-                                                      const double4 *__restrict__ pos,
-                                                      const double4 *__restrict__ spin,
-                                                      const int32_t *__restrict__ species, int n, BoxDev<double> box,
-                                                      unsigned char *scratch, double *__restrict__ q_out,
-                                                      double *__restrict__ e_out) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    int32_t *nbr = reinterpret_cast<int32_t *>(scratch + OFF_NBR);
-    int4 *seg = reinterpret_cast<int4 *>(scratch + OFF_SEG);
-    double *q = reinterpret_cast<double *>(scratch + OFF_Q);
-    double *bsum = reinterpret_cast<double *>(scratch + OFF_B);
-    int *status = reinterpret_cast<int *>(scratch + OFF_STATUS);
-    // species index the per-species coefficient tables: a value outside [0, NS) in this
-    // atom or in any atom it would pair with is reported and the atom is skipped (the
-    // host then rejects the whole call)
-    const int ti = species[i];
-    if (ti < 0 || ti >= NS) {
-        atomicOr(status, ST_BAD_SPECIES);
+struct WarpSmem {
+    double stage[STAGE];
+    double sums[NS][5][NK];      // radial and pairwise-magnetic basis sums per neighbour species
+    double q[DIM];
+    uint16_t list[MAX_NBR];      // neighbours inside rc_rad: species 0 from the front, species 1 from the back
+    uint16_t ang[MAX_NBR];       // those inside rc_ang (positions in the walk over the list)
+};
+struct BlockSmem {
+    double c[NCOEF];             // coefficients, as in NepDev
+    double w0[NH * W0_LD];
+    WarpSmem w[WARPS];
+    float far[WARPS];
+};
+
+__device__ __forceinline__ double kappa_of(int lm) {
+    switch (lm) {   // kappa_lm of the addition theorem
+    case 0: case 1: case 2: return 1.0;
+    case 3: case 4: case 5: return 3.0;
+    case 6: return 0.75;
+    case 8: case 14: case 18: case 20: return 0.625;
+    case 9: return 15.0;
+    case 10: case 12: return 0.375;
+    case 7: case 11: return 0.25;
+    case 13: return 3.75;
+    case 15: return 8.75;
+    case 16: case 22: return 4.375;
+    case 17: return 1.25;
+    case 19: return 0.015625;
+    case 21: return 0.3125;
+    default: return 0.546875;
+    }
+}
+
+__global__ void __launch_bounds__(WARPS * 32) k_eval_noalloc(const __grid_constant__ NepDev<double> P,
+                                                             const double4 *__restrict__ pos,
+                                                             const double4 *__restrict__ spin,
+                                                             const int32_t *__restrict__ species, int n,
+                                                             BoxDev<double> box, int *status,
+                                                             double *__restrict__ q_out,
+                                                             double *__restrict__ e_out) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    BlockSmem &sm = *reinterpret_cast<BlockSmem *>(smem_raw);
+    float4 *fpos = reinterpret_cast<float4 *>(smem_raw + (sizeof(BlockSmem) + 15) / 16 * 16);   // [n]
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    WarpSmem &ws = sm.w[w];
+
+    // FP32 positions of every atom, along periodic axes first brought into [-L/2, L/2] in FP64,
+    // species in w; `far`: the largest coordinate, which sets the band of the FP32 test
+    float far = 0.f;
+    for (int j = tid; j < n; j += WARPS * 32) {
+        const double4 p = pos[j];
+        const double x = p.x - box.L[0] * rint(p.x * box.invL[0]), y = p.y - box.L[1] * rint(p.y * box.invL[1]),
+                     z = p.z - box.L[2] * rint(p.z * box.invL[2]);
+        const int t = species[j];
+        // a species outside the model is reported and the host rejects the whole call
+        if (t < 0 || t >= NS) atomicOr(status, ST_BAD_SPECIES);
+        fpos[j] = make_float4((float)x, (float)y, (float)z, __int_as_float(t & 1));
+        far = fmaxf(far, fmaxf(fmaxf((float)fabs(x), (float)fabs(y)), (float)fabs(z)));
+        // the exact test's own rounding, should a caller's coordinates span many boxes
+        far = fmaxf(far, 1e-8f * fmaxf(fmaxf((float)fabs(p.x), (float)fabs(p.y)), (float)fabs(p.z)));
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) far = fmaxf(far, __shfl_xor_sync(0xffffffffu, far, o));
+    if (lane == 0) sm.far[w] = far;
+    const double *cin = &P.c[0][0][0][0][0];
+    for (int k = tid; k < NCOEF; k += WARPS * 32) sm.c[k] = cin[k];
+    for (int k = tid; k < NH * DIM; k += WARPS * 32) sm.w0[k / DIM * W0_LD + k % DIM] = P.w0[k / DIM][k % DIM];
+    __syncthreads();
+    const int i = blockIdx.x * WARPS + w;
+    if (i >= n) return;   // no block-wide barrier below
+
+    // ---- search.  An FP32 coordinate is off by 2^-24 of itself, a separation by the two
+    // coordinates' errors, its own rounding (of at most twice the largest coordinate) and the
+    // minimum image's (of a box length): at most E per component, so d2 (up to R^2, R a little
+    // beyond the cutoff) by 2 sqrt(3) R E + 3 E^2 and the FP32 sum's 4 2^-24 R^2.  The band is
+    // twice that.  A NaN fails both comparisons and takes the exact test.
+    float lo, hi;
+    {
+        float m = 0.f, L = 0.f;
+#pragma unroll
+        for (int k = 0; k < WARPS; ++k) m = fmaxf(m, sm.far[k]);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) L = fmaxf(L, box.invL[a] != 0.0 ? (float)box.L[a] : 0.f);
+        const float u = 5.9604645e-8f, E = u * (4.f * m + 4.f * L), R = (float)P.rc_r + 1.f;
+        const float band = 2.f * (3.4641017f * R * E + 3.f * E * E + 4.f * u * R * R);
+        lo = (float)P.rc_r2 - band;
+        hi = (float)P.rc_r2 + band;
+    }
+    const double4 pi = pos[i], si = spin[i];
+    const float4 fi = fpos[i];
+    const int ti = __float_as_int(fi.w);
+    const BoxDev<float> bf = {{(float)box.L[0], (float)box.L[1], (float)box.L[2]},
+                              {(float)box.invL[0], (float)box.invL[1], (float)box.invL[2]}};
+    auto separation = [&](const double4 &pj, double &dx, double &dy, double &dz) {
+        dx = pj.x - pi.x; dy = pj.y - pi.y; dz = pj.z - pi.z;
+        minimg(box, dx, dy, dz);
+        return dx * dx + dy * dy + dz * dz;
+    };
+    const unsigned lt = (1u << lane) - 1u;
+    int m0 = 0, m1 = 0;
+    for (int j0 = 0; j0 < n; j0 += 32) {
+        const int j = j0 + lane;
+        bool in = false, near = false;
+        int tj = 0;
+        if (j < n && j != i) {
+            const float4 fj = fpos[j];
+            float dx = fj.x - fi.x, dy = fj.y - fi.y, dz = fj.z - fi.z;
+            minimg(bf, dx, dy, dz);
+            const float d2 = dx * dx + dy * dy + dz * dz;
+            in = d2 < lo;
+            near = !in && !(d2 >= hi);
+            tj = __float_as_int(fj.w);
+        }
+        if (near) {
+            double dx, dy, dz;
+            in = separation(pos[j], dx, dy, dz) < P.rc_r2;
+        }
+        const unsigned b0 = __ballot_sync(0xffffffffu, in && tj == 0), b1 = __ballot_sync(0xffffffffu, in && tj == 1);
+        if (in) {
+            const int at = tj == 0 ? m0 + __popc(b0 & lt) : m1 + __popc(b1 & lt);
+            if (at < MAX_NBR) ws.list[tj == 0 ? at : MAX_NBR - 1 - at] = (uint16_t)j;
+        }
+        m0 += __popc(b0);
+        m1 += __popc(b1);
+    }
+    if (m0 + m1 > MAX_NBR) {   // uniform over the warp; the host rejects the call
+        if (lane == 0) atomicOr(status, ST_NBR_OVERFLOW);
         return;
     }
-    // brute-force neighbours inside rc_rad, inserted in (segment, index) order
-    // straight into this atom's scratch column (slot-major, stride n)
-    const double4 pi = pos[i];
-    int m = 0;
-    bool overflow = false;
-    for (int j = 0; j < n; ++j) {
-        if (j == i) continue;
-        const double4 pj = pos[j];
-        double dx = pj.x - pi.x, dy = pj.y - pi.y, dz = pj.z - pi.z;
-        minimg(box, dx, dy, dz);
-        const double d2 = dx * dx + dy * dy + dz * dz;
-        if (!(d2 < P.rc_r2)) continue;
-        const int tj = species[j];
-        if (tj < 0 || tj >= NS) {
-            atomicOr(status, ST_BAD_SPECIES);
-            return;
-        }
-        if (m >= MAX_NBR) { overflow = true; continue; }
-        const int key = ((d2 < P.rc_a2 ? 0 : 2) + tj) * MAX_ATOMS + j;
-        int v = m - 1;
-        while (v >= 0) {
-            const int jv = nbr[(int64_t)v * n + i];
-            const double4 pv = pos[jv];
-            double ex = pv.x - pi.x, ey = pv.y - pi.y, ez = pv.z - pi.z;
-            minimg(box, ex, ey, ez);
-            const int kv = (((ex * ex + ey * ey + ez * ez) < P.rc_a2 ? 0 : 2) + species[jv]) * MAX_ATOMS + jv;
-            if (kv <= key) break;
-            nbr[(int64_t)(v + 1) * n + i] = jv;
-            --v;
-        }
-        nbr[(int64_t)(v + 1) * n + i] = j;
-        ++m;
-    }
-    if (overflow) atomicOr(status, ST_NBR_OVERFLOW);
-    int ends[4] = {0, 0, 0, 0};
-    for (int s = 0; s < m; ++s) {
-        const int j = nbr[(int64_t)s * n + i];
-        const double4 pj = pos[j];
-        double dx = pj.x - pi.x, dy = pj.y - pi.y, dz = pj.z - pi.z;
-        minimg(box, dx, dy, dz);
-        const int sg = ((dx * dx + dy * dy + dz * dz) < P.rc_a2 ? 0 : 2) + species[j];
-        for (int t = sg; t < 4; ++t) ends[t] = s + 1;
-    }
-    for (int t = 1; t < 4; ++t) ends[t] = max(ends[t], ends[t - 1]);
-    seg[i] = make_int4(ends[0], ends[1], ends[2], ends[3]);
-    // descriptor by fwd_atom (one thread per atom, harmonic form of the angular channels;
-    // the step's kernels in sl_eval2.cu compute the same sums with another work split)
-    EvalArgs<double> a;
-    a.pos = pos; a.spin = spin; a.nbr = nbr; a.seg = seg; a.n = n; a.n_fe = 0; a.box = box;
-    a.q = q; a.bsum = bsum;
-    if (ti == 0) fwd_atom<double, 0>(P, a, i);
-    else fwd_atom<double, 1>(P, a, i);
-    // network energy E_i = sum_h w1_h tanh(sum_v W0_hv s_v q_v - b0_h) - b1
-    double x[DIM];
+    const int m = m0 + m1;
+    __syncwarp();
+    auto neighbour = [&](int p) { return (int)ws.list[p < m0 ? p : MAX_NBR - 1 - (p - m0)]; };
+
+    // ---- radial and pairwise-magnetic sums: 32 pairs staged at a time (f_k, then the four
+    // spin products), summed by 27 lanes: lane (k, third) takes every third pair
+    double s0[5] = {0, 0, 0, 0, 0}, s1[5] = {0, 0, 0, 0, 0};
+    const int k9 = lane % 9, third = lane / 9;
+    int na = 0;
+    for (int base = 0; base < m; base += 32) {
+        const int p = base + lane, cnt = min(32, m - base);
+        bool ang = false;
+        if (p < m) {
+            const int j = neighbour(p);
+            const double4 sj = spin[j];
+            double dx, dy, dz;
+            const double d2 = separation(pos[j], dx, dy, dz);
+            ang = d2 < P.rc_a2;
+            const double ir = rsqrt(d2), r = d2 * ir;
+            const double ux = dx * ir, uy = dy * ir, uz = dz * ir;
+            double f[NK];
+            carrier_f(r, P.inv_rc_r, f);
 #pragma unroll
-    for (int v = 0; v < DIM; ++v) {
-        x[v] = q[(int64_t)v * n + i];
-        if (q_out) q_out[(int64_t)i * DIM + v] = x[v];
-        x[v] *= P.scal[v];
-    }
-    double E = -P.b1;
-#pragma unroll 1
-    for (int h = 0; h < NH; ++h) {
-        double z = -P.b0[h];
+            for (int k = 0; k < NK; ++k) ws.stage[k * LD + lane] = f[k];
+            const double siu = si.x * ux + si.y * uy + si.z * uz, sju = sj.x * ux + sj.y * uy + sj.z * uz;
+            ws.stage[9 * LD + lane] = si.x * sj.x + si.y * sj.y + si.z * sj.z;
+            ws.stage[10 * LD + lane] = (si.y * sj.z - si.z * sj.y) * ux + (si.z * sj.x - si.x * sj.z) * uy +
+                                       (si.x * sj.y - si.y * sj.x) * uz;
+            ws.stage[11 * LD + lane] = siu * sju;
+            ws.stage[12 * LD + lane] = siu * siu;
+        }
+        const unsigned ba = __ballot_sync(0xffffffffu, ang);
+        if (ang) ws.ang[na + __popc(ba & lt)] = (uint16_t)p;
+        na += __popc(ba);
+        __syncwarp();
+        if (third < 3) {
+            const int split = min(max(m0 - base, 0), cnt);   // staged pairs of species 0
+            auto add = [&](double *s, int at) {
+                const double f = ws.stage[k9 * LD + at];
+                s[0] += f;
 #pragma unroll
-        for (int v = 0; v < DIM; ++v) z += P.w0[h][v] * x[v];
-        E += P.w1[h] * tanh(z);
+                for (int g = 0; g < 4; ++g) s[g + 1] = fma(f, ws.stage[(9 + g) * LD + at], s[g + 1]);
+            };
+            for (int at = third; at < split; at += 3) add(s0, at);
+            for (int at = split + third; at < cnt; at += 3) add(s1, at);
+        }
+        __syncwarp();
     }
-    e_out[i] = E;
+#pragma unroll
+    for (int g = 0; g < 5; ++g) {
+        s0[g] += __shfl_sync(0xffffffffu, s0[g], (lane + 9) & 31) + __shfl_sync(0xffffffffu, s0[g], (lane + 18) & 31);
+        s1[g] += __shfl_sync(0xffffffffu, s1[g], (lane + 9) & 31) + __shfl_sync(0xffffffffu, s1[g], (lane + 18) & 31);
+        if (lane < 9) {
+            ws.sums[0][g][lane] = s0[g];
+            ws.sums[1][g][lane] = s1[g];
+        }
+    }
+    __syncwarp();
+    const double *ci = sm.c + ti * (NS * 6 * NCH * NK);   // [neighbour][group][n][k]
+    if (lane < 25) {
+        const int g = lane / NCH, c = lane % NCH;
+        const int grp = g == 0 ? G_R : g + 1;                      // R, EX, DMI, ANI, SIA
+        const int at = g == 0 ? Q_R : Q_EX + (g - 1) * NCH;
+        double v = 0.0;
+#pragma unroll
+        for (int tj = 0; tj < NS; ++tj)
+#pragma unroll
+            for (int k = 0; k < NK; ++k) v += ci[((tj * 6 + grp) * NCH + c) * NK + k] * ws.sums[tj][g][k];
+        ws.q[at + c] = v;
+    }
+    if (lane == 25) ws.q[Q_O] = si.x * si.x + si.y * si.y + si.z * si.z;
+
+    // ---- angular sums: 32 pairs staged at a time (g_n, s g_n, harmonics), summed by 30 lanes:
+    // lane (n, four harmonics)
+    double B[4] = {0, 0, 0, 0}, BS[4] = {0, 0, 0, 0};
+    const int nc = lane / 6, quad = lane % 6;
+    for (int base = 0; base < na; base += 32) {
+        const int cnt = min(32, na - base);
+        if (lane < cnt) {
+            const int p = ws.ang[base + lane], j = neighbour(p), tj = p < m0 ? 0 : 1;
+            const double4 sj = spin[j];
+            double dx, dy, dz;
+            const double d2 = separation(pos[j], dx, dy, dz);
+            const double ir = rsqrt(d2), r = d2 * ir;
+            double f[NK];
+            carrier_f(r, P.inv_rc_a, f);
+            const double s = si.x * sj.x + si.y * sj.y + si.z * sj.z;
+#pragma unroll
+            for (int c = 0; c < NCH; ++c) {
+                double g = 0.0;
+#pragma unroll
+                for (int k = 0; k < NK; ++k) g += ci[((tj * 6 + G_A) * NCH + c) * NK + k] * f[k];
+                ws.stage[c * LD + lane] = g;
+                ws.stage[(NCH + c) * LD + lane] = g * s;
+            }
+            double h[NLM];
+            harm_p(dx * ir, dy * ir, dz * ir, h);
+#pragma unroll
+            for (int lm = 0; lm < NLM; ++lm) ws.stage[(2 * NCH + lm) * LD + lane] = h[lm];
+        }
+        __syncwarp();
+        if (nc < NCH) {
+            for (int at = 0; at < cnt; ++at) {
+                const double g = ws.stage[nc * LD + at], gs = ws.stage[(NCH + nc) * LD + at];
+#pragma unroll
+                for (int x = 0; x < 4; ++x) {
+                    const double h = ws.stage[(2 * NCH + 4 * quad + x) * LD + at];
+                    B[x] = fma(g, h, B[x]);
+                    BS[x] = fma(gs, h, BS[x]);
+                }
+            }
+        }
+        __syncwarp();
+    }
+    if (nc < NCH) {   // the sums take the stage's place: B_n,lm, then BS_n,lm
+#pragma unroll
+        for (int x = 0; x < 4; ++x) {
+            ws.stage[nc * NLM + 4 * quad + x] = B[x];
+            ws.stage[(NCH + nc) * NLM + 4 * quad + x] = BS[x];
+        }
+    }
+    __syncwarp();
+    for (int o = lane; o < 2 * NCH * 4; o += 32) {
+        const int l = o & 3, c = o >> 2;   // c: channel n of A, then of SA
+        const int lm0 = l * (l + 2), lm1 = (l + 1) * (l + 3);   // 0, 3, 8, 15, 24
+        double v = 0.0;
+        for (int lm = lm0; lm < lm1; ++lm) {
+            const double b = ws.stage[c * NLM + lm];
+            v += kappa_of(lm) * b * b;
+        }
+        ws.q[(c < NCH ? Q_A + c * 4 : Q_SA + (c - NCH) * 4) + l] = v;
+    }
+    __syncwarp();
+
+    // ---- outputs and the network, E_i = sum_h w1_h tanh(sum_v W0_hv s_v q_v - b0_h) - b1
+    for (int v = lane; v < DIM; v += 32) {
+        const double x = ws.q[v];
+        if (q_out) q_out[(int64_t)i * DIM + v] = x;
+        ws.q[v] = x * P.scal[v];
+    }
+    __syncwarp();
+    double E = 0.0;
+    if (lane < NH) {
+        double z0 = -P.b0[lane], z1 = 0.0;
+#pragma unroll 6
+        for (int v = 0; v < DIM; v += 2) {
+            z0 = fma(sm.w0[lane * W0_LD + v], ws.q[v], z0);
+            z1 = fma(sm.w0[lane * W0_LD + v + 1], ws.q[v + 1], z1);
+        }
+        E = P.w1[lane] * tanh(z0 + z1);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) E += __shfl_xor_sync(0xffffffffu, E, o);
+    if (lane == 0) e_out[i] = E - P.b1;
 }
+
+constexpr size_t smem_bytes(int n) { return (sizeof(BlockSmem) + 15) / 16 * 16 + sizeof(float4) * (size_t)n; }
+static_assert(2 * smem_bytes(MAX_ATOMS) <= 227 * 1024, "two blocks share an SM at the largest size");
 
 }  // namespace noalloc
 
-// Device address of the scratch array for the current device, looked up once per
-// device (host code cannot use the symbol itself as a device address).
-int noalloc_scratch(void **out) {
+// Device address of the status word for the current device, looked up once per device (host
+// code cannot use the symbol itself as a device address), with the kernel's shared-memory limit.
+static int noalloc_status(int **out) {
     static std::mutex mu;
     static void *addr[128] = {nullptr};
     int dev = 0;
@@ -373,21 +437,23 @@ int noalloc_scratch(void **out) {
     std::lock_guard<std::mutex> lk(mu);
     if (!addr[dev]) {
         void *p = nullptr;
-        if (cudaGetSymbolAddress(&p, noalloc::g_scratch) != cudaSuccess || !p) return -1;
+        if (cudaGetSymbolAddress(&p, noalloc::g_status) != cudaSuccess || !p) return -1;
+        if (cudaFuncSetAttribute(noalloc::k_eval_noalloc, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)noalloc::smem_bytes(noalloc::MAX_ATOMS)) != cudaSuccess)
+            return -1;
         addr[dev] = p;
     }
-    *out = addr[dev];
+    *out = static_cast<int *>(addr[dev]);
     return 0;
 }
 
 int launch_noalloc(const NepDev<double> &P, const double4 *pos, const double4 *spin, const int32_t *species, int n,
                    const BoxDev<double> &box, double *q_out, double *e_out, cudaStream_t stream, int *status_out) {
-    void *scratch = nullptr;
-    if (noalloc_scratch(&scratch)) return -1;
-    int *status = reinterpret_cast<int *>(static_cast<unsigned char *>(scratch) + noalloc::OFF_STATUS);
+    int *status = nullptr;
+    if (noalloc_status(&status)) return -1;
     if (cudaMemsetAsync(status, 0, sizeof(int), stream) != cudaSuccess) return -1;
-    noalloc::k_eval_noalloc<<<(unsigned)((n + 127) / 128), 128, 0, stream>>>(
-        P, pos, spin, species, n, box, static_cast<unsigned char *>(scratch), q_out, e_out);
+    noalloc::k_eval_noalloc<<<(unsigned)((n + noalloc::WARPS - 1) / noalloc::WARPS), noalloc::WARPS * 32,
+                              noalloc::smem_bytes(n), stream>>>(P, pos, spin, species, n, box, status, q_out, e_out);
     if (cudaGetLastError() != cudaSuccess) return -1;
     int st = 0;
     if (cudaMemcpyAsync(&st, status, sizeof(int), cudaMemcpyDeviceToHost, stream) != cudaSuccess) return -1;
