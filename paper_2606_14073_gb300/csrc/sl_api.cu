@@ -142,7 +142,7 @@ void fill_params(sl::NepDev<R> &P, const sl_nep_params *p) {
 void free_sys(sl::Sys &s) {
     void *ptrs[] = {s.pos, s.vel, s.spin, s.spin_prev, s.F, s.H, s.posref, s.posf, s.spinf, s.species, s.orig,
                     s.inv, s.nbr, s.rev, s.nbr_hash, s.cells.posf, s.cells.key, s.seg, s.cells.count, s.cells.start, s.cells.fill, s.cells.atoms,
-                    s.cells.of, s.cells.sub, s.q, s.bsum, s.fp, s.ei, s.pairs, s.clj, s.cls, s.cnt, s.cmask, s.fown, s.gii,
+                    s.cells.of, s.cells.sub, s.q, s.bsum, s.fp, s.ei, s.pairs, s.crow, s.ctab, s.cnt, s.cmask, s.fown, s.gii,
                     s.wpart, s.Fo, s.Ho,
                     s.status, s.rebuild, s.d_step, s.d_par, s.red, s.snap, s.d_builds,
                     s.posmid, s.posmidf, s.mids, s.midsf, s.mx, s.mg, s.aax, s.aag, s.aapart, s.md, s.Bat,
@@ -563,13 +563,14 @@ int sl_create_system(const double *positions, const double *spins, const double 
         (rc = dalloc(&s.cells.of, N)) || (rc = dalloc(&s.cells.sub, (size_t)s.cells.ncell * 8)) || (rc = dalloc((char **)&s.q, R * DIM * (size_t)s.qs)) ||
         (rc = dalloc((char **)&s.bsum, R * NBREC * N)) || (rc = dalloc((char **)&s.fp, R * DIM * N)) ||
         (rc = dalloc((char **)&s.ei, R * N)) || (rc = dalloc((char **)&s.pairs, R * 8 * N * s.cap)) ||
-        (rc = dalloc(&s.clj, N * (size_t)(s.cap + s.cap_ang))) || (rc = dalloc(&s.cls, N * (size_t)(s.cap + s.cap_ang))) ||
+        (rc = dalloc(&s.crow, N * (size_t)(s.cap + s.cap_ang))) ||
         (rc = dalloc(&s.cnt, N)) || (rc = dalloc(&s.cmask, N * (size_t)((s.cap + 31) / 32))) || (rc = dalloc((char **)&s.fown, R * 4 * N)) ||
         (rc = dalloc((char **)&s.gii, R * 4 * N)) || (rc = dalloc((char **)&s.wpart, R * 9 * N)) ||
         (rc = dalloc(&s.Fo, N)) || (rc = dalloc(&s.Ho, N)) || (rc = dalloc(&s.status, 1)) ||
         (rc = dalloc(&s.rebuild, 1)) || (rc = dalloc(&s.d_step, 2)) || (rc = dalloc(&s.d_par, 1)) ||
         (rc = dalloc(&s.red, 256 * 10 + 10)) || (rc = dalloc(&s.snap, 5 * N)) || (rc = dalloc(&s.d_builds, 1)))
         return bail(rc);
+    if (n > 0 && sl::make_coeff_table(s)) return bail(fail(SL_ENOMEM, "the coefficient table could not be made"));
     if (s.prec == SL_PREC_MIXED && n > 0 && sl::make_q_tensor_map(s))
         return bail(fail(SL_ECUDA, "the TMA map of the descriptor array could not be encoded"));
     if (s.prec == SL_PREC_MIXED && n > 0 && sl::make_mlp_image(s))
@@ -969,7 +970,7 @@ int sl_get_neighbors(sl_system *sys, int32_t cap, int32_t *counts_rad, int32_t *
         for (int t = 0; t < seg[i].w; ++t) {
             const int32_t j = orig[nbr[(size_t)i * sl::nbr_stride(s.cap) + t]];
             rad.push_back(j);
-            if (t < seg[i].y) ang.push_back(j);
+            if (t < seg[i].x || (t >= seg[i].y && t < seg[i].z)) ang.push_back(j);
         }
         std::sort(rad.begin(), rad.end());
         std::sort(ang.begin(), ang.end());
@@ -1277,7 +1278,7 @@ int64_t sl_estimate_device_bytes(int64_t n, const sl_options *opt_in) {
     int64_t per = 7 * 32 + 2 * 16                      // state (double4) and FP32 copies
                   + 3 * 4 + 4 + 16 + 16 + 4            // species, caller index maps, list segments, cell copies
                   + 6 * sl::nbr_stride((int)cap)     // candidate lists, reverse slots and index hashes (1 byte each)
-                  + 6 * (ca + cap) + 16                // compact rows, counts
+                  + 8 * (ca + cap) + 16                // compact rows, counts
                   + 4 * ((cap + 31) / 32)              // in-cutoff slot mask
                   + R * (2 * sl::DIM + sl::NBREC + 1 + 9) // q, Fp, angular sums, E_i, virial parts
                   + R * 8 * cap + 2 * R * 4            // pair records, per-atom sums
@@ -1491,7 +1492,7 @@ static int fused_steps(sl_batch *b, const std::vector<int> &active, const int64_
     for (int64_t r = 0; r < most % g; ++r) CK(cudaGraphLaunch(f.graph_1, b->stream));
     b->graph_launches += most / g + most % g;
     b->fused_steps += most;
-    b->kernel_launches += most * sl::FUSED_LAUNCHES_PER_STEP;
+    b->kernel_launches += most * sl::fused_launches_per_step(m.prec);
     ++b->fused_calls;
     CK(cudaEventRecord(b->ev[0], b->stream));
     for (int i : active) CK(cudaStreamWaitEvent(b->sys[i]->s.stream, b->ev[0], 0));   // and each replica waits for it

@@ -23,14 +23,15 @@ namespace sl {
 // kernels of one step, in launch order
 enum FusedKernel {
     FK_FIRST, FK_BIN, FK_SCAN, FK_SCATTER, FK_CELLSORT, FK_LISTS, FK_REV, FK_FINISH,
-    FK_CRAD, FK_ANG, FK_NET, FK_BWD, FK_SECOND, FK_N
+    FK_CRAD, FK_CRADW, FK_ANG, FK_NET, FK_BWD, FK_SECOND, FK_N
 };
-constexpr int FUSED_LAUNCHES_PER_STEP = 1 + FK_N + 1;   // plan, the kernels, the flag clear
+// plan, the kernels (FP64 has the wide radial kernel only), the flag clear
+inline int fused_launches_per_step(int prec) { return 1 + FK_N + 1 - (prec == 0); }
 constexpr int FUSED_MAX_SLOTS = 4096;
 // atoms-per-block classes of the kernels that take one work item per block: the halves (256
-// atoms), the radial kernel and the FP64 network (128), the angular and backward kernels (a
-// quad block's atoms)
-enum { IC_HALF = 0, IC_ATOM = 1, IC_QUAD = 2, IC_N = 3 };
+// atoms), the one-thread-per-atom radial kernel or the FP64 network (128), the angular and
+// backward kernels (a quad block's atoms), the wide radial kernel (8)
+enum { IC_HALF = 0, IC_ATOM = 1, IC_QUAD = 2, IC_OCT = 3, IC_N = 4 };
 
 // what a slot's entries are set up for
 enum SlotKind {
@@ -117,7 +118,7 @@ void launch_rebuild_t(const FusedTables &t, const Launch *L, bool clear, bool lo
 // radial, angular, network, backward; ev (optional, 6 events): recorded before the radial
 // kernel, after it, after the angular kernel, after the network and after the backward
 template <typename R>
-void launch_eval_t(const FusedTables &t, const NepDev<R> &P, const Launch *L /* crad, ang, net, bwd */,
+void launch_eval_t(const FusedTables &t, const NepDev<R> &P, const Launch *L /* crad, ang, net, bwd, wide crad */,
                    cudaStream_t st, cudaEvent_t *ev);
 void launch_net_t_tc(const FusedTables &t, const NepDev<float> &P, const Launch &L, cudaStream_t st);
 void launch_net_t_fp64(const FusedTables &t, const NepDev<double> &P, const Launch &L, cudaStream_t st);

@@ -67,7 +67,7 @@ template <typename R> using v4 = typename V4<R>::t;
 // itself from the pointers.
 __device__ __forceinline__ float4 ro(const float4 *p) { return __ldg(p); }
 __device__ __forceinline__ int4 ro(const int4 *p) { return __ldg(p); }
-__device__ __forceinline__ uchar4 ro(const uchar4 *p) { return __ldg(p); }
+__device__ __forceinline__ int2 ro(const int2 *p) { return __ldg(p); }
 __device__ __forceinline__ int ro(const int *p) { return __ldg(p); }
 __device__ __forceinline__ unsigned ro(const unsigned *p) { return __ldg(p); }
 __device__ __forceinline__ unsigned short ro(const unsigned short *p) { return __ldg(p); }
@@ -86,6 +86,7 @@ __device__ __forceinline__ void stg(unsigned short *p, unsigned short v) { __stw
 __device__ __forceinline__ void stg(float *p, float v) { __stwb(p, v); }
 __device__ __forceinline__ void stg(double *p, double v) { __stwb(p, v); }
 __device__ __forceinline__ void stg(float4 *p, const float4 &v) { __stwb(p, v); }
+__device__ __forceinline__ void stg(int2 *p, const int2 &v) { __stwb(p, v); }
 __device__ __forceinline__ void stg(int4 *p, const int4 &v) { __stwb(p, v); }
 __device__ __forceinline__ void stg(double4 *p, const double4 &v) {
     __stwb(reinterpret_cast<double2 *>(p), make_double2(v.x, v.y));
@@ -99,6 +100,14 @@ __device__ __forceinline__ float rint_<float>(float x) { return rintf(x); }
 template <>
 __device__ __forceinline__ double rint_<double>(double x) { return rint(x); }
 
+// Whole box lengths of a separation.  FP32: the nearest integer by adding and subtracting
+// 1.5 2^23 (one multiply-add and one add, off the conversion pipe; |x/L| < 2^22).
+__device__ __forceinline__ void minimg(const BoxDev<float> &b, float &dx, float &dy, float &dz) {
+    constexpr float big = 12582912.f;
+    dx = fmaf(-b.L[0], __fadd_rn(fmaf(dx, b.invL[0], big), -big), dx);
+    dy = fmaf(-b.L[1], __fadd_rn(fmaf(dy, b.invL[1], big), -big), dy);
+    dz = fmaf(-b.L[2], __fadd_rn(fmaf(dz, b.invL[2], big), -big), dz);
+}
 template <typename R>
 __device__ __forceinline__ void minimg(const BoxDev<R> &b, R &dx, R &dy, R &dz) {
     dx -= b.L[0] * rint_(dx * b.invL[0]);

@@ -9,6 +9,7 @@
 //              neighbour species, and accumulates the radial and pairwise-magnetic basis
 //              sums over them, contracted with the coefficients once per neighbour
 //              species (q^R, q^EX, q^DMI, q^ANI, q^SIA, q^O).
+//   k_crad_wide  the same with sixteen lanes per atom (small systems, and FP64).
 //   k_ang_fwd  four lanes per atom.  Each lane stages one angular pair (carrier, g_n,
 //              spin weight, the 24 solid harmonics) in shared memory; then every lane
 //              accumulates B_nlm, BS_nlm for its 6 harmonics over the staged pairs.
@@ -23,6 +24,7 @@
 // its in-cutoff slots only.
 #include <cstddef>
 #include <mutex>
+#include <vector>
 
 #include "sl_internal.h"
 #include "sl_eval2.cuh"
@@ -106,6 +108,38 @@ __device__ __forceinline__ void sep(const BoxDev<R> &b, const v4<R> &pi, const v
     minimg(b, dx, dy, dz);
 }
 
+// The coefficients of the radial contraction: [centre][neighbour][k][g * 5 + n], rows padded to
+// 32, g in the order R, EX, DMI, ANI, SIA (each lane of k_crad reads its own output's column).
+template <typename R>
+static void fill_ctab(const NepDev<R> &P, std::vector<R> &t) {
+    constexpr int GG[5] = {G_R, G_EX, G_DMI, G_ANI, G_SIA};
+    t.assign((size_t)NS * NS * NK * 32, R(0));
+    for (int x = 0; x < NS; ++x)
+        for (int y = 0; y < NS; ++y)
+            for (int k = 0; k < NK; ++k)
+                for (int o = 0; o < 25; ++o)
+                    t[(size_t)((x * NS + y) * NK + k) * 32 + o] = P.c[x][y][GG[o / NCH]][o % NCH][k];
+}
+int make_coeff_table(Sys &s) {
+    const auto put = [&](const auto &t) {
+        const size_t bytes = t.size() * sizeof(t[0]);
+        if (!s.ctab && cudaMalloc(&s.ctab, bytes) != cudaSuccess) {
+            s.ctab = nullptr;
+            return -1;
+        }
+        if (cudaMemcpyAsync(s.ctab, t.data(), bytes, cudaMemcpyHostToDevice, s.stream) != cudaSuccess) return -1;
+        return cudaStreamSynchronize(s.stream) == cudaSuccess ? 0 : -1;
+    };
+    if (s.prec == 0) {
+        std::vector<double> t;
+        fill_ctab(s.pd, t);
+        return put(t);
+    }
+    std::vector<float> t;
+    fill_ctab(s.pf, t);
+    return put(t);
+}
+
 // per-lane constants of harmonic lm = ql + 4 m (ql = lane in quad)
 __device__ __forceinline__ int lm_of(int ql, int m) { return ql + 4 * m; }
 __device__ __forceinline__ int l_of_lm(int lm) { return lm < 3 ? 1 : lm < 8 ? 2 : lm < 15 ? 3 : 4; }
@@ -137,7 +171,7 @@ __device__ __forceinline__ R kappa_of_lm(int lm) {
 }
 
 // ------------------------------------------------------------------ k_crad
-// One thread per atom, per neighbour species:
+// One thread per atom (mixed precision, larger systems: see crad_is_wide), per neighbour species:
 //  A. the angular candidates (within rc_ang + skin of the list build, so nearly all inside
 //     rc_rad): compaction and the radial and pairwise-magnetic basis sums in one pass;
 //  B. the radial-shell candidates (rc_ang + skin .. rc_rad + skin at the build, fewer than
@@ -145,9 +179,9 @@ __device__ __forceinline__ R kappa_of_lm(int lm) {
 //  C. the basis sums over the rows B produced.
 // Splitting B from C keeps a warp from running the pair arithmetic for every candidate of
 // the shell whenever one of its 32 atoms has that candidate inside the cutoff.  Rows are
-// angular (r < rc_ang) or radial-only (rc_ang <= r < rc_rad), each grouped by neighbour
-// species in candidate order (species 0 from candidate segments 0 and 2, then species 1
-// from 1 and 3), for the angular and backward kernels and the gather.  The sums are
+// angular (r < rc_ang) or radial-only (rc_ang <= r < rc_rad), each in candidate order (the
+// candidates of neighbour species 0 come first in a list, then those of species 1), for the
+// angular and backward kernels and the gather.  The sums are
 // contracted with the coefficients once per neighbour species (q^R, q^EX, q^DMI, q^ANI,
 // q^SIA); q^O = |S|^2.
 
@@ -193,7 +227,7 @@ __device__ __forceinline__ int take_row(const NepDev<R> &P, const Eval2Args<R> &
 }
 
 // in-cutoff slot bits of this thread's atom, in shared memory (column threadIdx.x)
-constexpr int MASKW_MAX = 8;
+constexpr int MASKW_MAX = 8;   // slot-mask words (a list holds at most 256 candidates)
 __device__ __forceinline__ void mark_slot(uint32_t (*sm)[128], int slot) {
     sm[slot >> 5][threadIdx.x] |= 1u << (slot & 31);
 }
@@ -255,8 +289,7 @@ __device__ __forceinline__ void crad_species(const NepDev<R> &P, const Eval2Args
                 if (!(d2 < P.rc_r2)) continue;
                 const int row = take_row(P, a, d2, na, nr, ovf);
                 if (row < 0) continue;
-                stg(a.clj + (int64_t)row * N + i, jj[u]);
-                stg(a.cls + (int64_t)row * N + i, (uint16_t)((c + u) | (tt[u] << 8)));
+                stg(a.crow + (int64_t)row * N + i, make_int2(jj[u], tt[u]));
                 mark_slot(smask, c + u);
                 rad_accumulate(P, si, ss[u], dx, dy, dz, d2, b);
             }
@@ -292,8 +325,7 @@ __device__ __forceinline__ void crad_species(const NepDev<R> &P, const Eval2Args
                 if (!(d2 < P.rc_r2)) continue;
                 const int row = take_row(P, a, d2, na, nr, ovf);
                 if (row < 0) continue;
-                stg(a.clj + (int64_t)row * N + i, jj[u]);
-                stg(a.cls + (int64_t)row * N + i, (uint16_t)((c + u) | (tt[u] << 8)));
+                stg(a.crow + (int64_t)row * N + i, make_int2(jj[u], tt[u]));
                 mark_slot(smask, c + u);
             }
         }
@@ -305,14 +337,14 @@ __device__ __forceinline__ void crad_species(const NepDev<R> &P, const Eval2Args
         auto row_of = [&](int t) { return t < nA ? naB + t : a.cap_ang + nrB + (t - nA); };
         int j1 = 0, j2 = 0;
         v4<R> p1, s1;
-        if (len > 0) j1 = a.clj[(int64_t)row_of(0) * N + i];
-        if (len > 1) j2 = a.clj[(int64_t)row_of(1) * N + i];
+        if (len > 0) j1 = a.crow[(int64_t)row_of(0) * N + i].x;
+        if (len > 1) j2 = a.crow[(int64_t)row_of(1) * N + i].x;
         if (len > 0) { p1 = pos[j1]; s1 = spin[j1]; }
 #pragma unroll 1
         for (int t = 0; t < len; ++t) {
             const v4<R> pj = p1, sj = s1;
             if (t + 1 < len) { p1 = pos[j2]; s1 = spin[j2]; }
-            if (t + 2 < len) j2 = a.clj[(int64_t)row_of(t + 2) * N + i];
+            if (t + 2 < len) j2 = a.crow[(int64_t)row_of(t + 2) * N + i].x;
             R dx, dy, dz;
             sep(a.box, pi, pj, dx, dy, dz);
             rad_accumulate(P, si, sj, dx, dy, dz, dx * dx + dy * dy + dz * dz, b);
@@ -347,9 +379,9 @@ __device__ __forceinline__ void crad_atom(const NepDev<R> &P, const Eval2Args<R>
     int na = 0, nr = 0;
     bool ovf = false;
     for (int w = 0; w < a.maskw; ++w) smask[w][threadIdx.x] = 0u;
-    crad_species<R, TI, 0>(P, a, i, pi, si, 0, sg.x, sg.y, sg.z, na, nr, ovf, smask);
+    crad_species<R, TI, 0>(P, a, i, pi, si, 0, sg.x, sg.x, sg.y, na, nr, ovf, smask);
     const int na0 = na, nr0 = nr;
-    crad_species<R, TI, 1>(P, a, i, pi, si, sg.x, sg.y, sg.z, sg.w, na, nr, ovf, smask);
+    crad_species<R, TI, 1>(P, a, i, pi, si, sg.y, sg.z, sg.z, sg.w, na, nr, ovf, smask);
     if (ovf) atomicOr(a.status, ST_NBR_OVERFLOW);
     stg(a.cnt + i, make_int4(na0, na, nr0, nr));
     for (int w = 0; w < a.maskw; ++w) stg(reinterpret_cast<int *>(a.mask) + (int64_t)w * N + i, (int)smask[w][threadIdx.x]);
@@ -369,6 +401,270 @@ __device__ __forceinline__ void crad_body(const NepDev<R> &P, const Eval2Args<R>
     if (i >= a.n) return;
     if (i < a.n_fe) crad_atom<R, 0>(P, a, i, smask);
     else crad_atom<R, 1>(P, a, i, smask);
+}
+
+// ------------------------------------------------------------------ k_crad_wide
+// Sixteen lanes per atom, two atoms per warp: every FP64 system, and mixed-precision systems of
+// up to CRAD_WIDE_MAX atoms.
+//  A. sixteen candidates at a time, in list order: cutoff test, rows written (ballot/popc), the
+//     neighbour kept in the atom's shared list (grouped by species, as the candidates are);
+//  B. sixteen pairs of that list at a time: each lane takes one pair (geometry, carrier, spin
+//     products) and stages it; then lane (two k's, third) adds every third staged pair into its
+//     ten basis sums (five groups, two k's), one set per neighbour species;
+//  C. the thirds are added, and the lanes contract the 2 x 45 sums with the coefficients.
+// Rows are angular (r < rc_ang) or radial-only, in the angular and backward kernels' order.
+// What bounds it.  FP64: the FP64 pipe (360 warp instructions per atom, as many as one thread per
+// atom takes, but spread over a warp for every two atoms): 512 / 13,824 / 110,592 atoms 45 / 349 /
+// 2,113 us, against 511 / 525 / 2,091 us with one thread per atom.  Mixed precision: instruction
+// issue (1,270 warp instructions per atom against 570 for one thread per atom, whose chain of 110
+// candidates takes 48 us however few the atoms): 512 / 13,824 / 32,768 / 110,592 atoms 15 / 37 / 70 /
+// 189 us, against 51 / 68 / 74 / 161 us.  The line lies at 16,384 atoms, below the crossing: a
+// replica keeps its kernel in a batch (its results are the same there bit for bit), where other
+// replicas fill the GPU and only the instructions count (eight replicas of 4,096 to 65,536 atoms
+// step 2.5% slower with the line at 32,768).
+constexpr int CR_LANES = 16;             // lanes per atom
+constexpr int CR_LD = 20;                // staged pair: f_0..f_8, three pads, sij, dmi, ani, sia, pads
+constexpr int CR_STAGE = CR_LANES * CR_LD + 16;   // the pad puts a warp's two atoms in different banks
+constexpr int CR_NQ = 26;                // descriptor entries an atom gets here
+
+// Test of the candidate pair (i, j): inside rc_rad, inside rc_ang.  FP32: on the FP32
+// positions.  FP64: an FP32 separation decides outside the rounding band around a cutoff and
+// the FP64 test inside it; the FP64 pipe (two lanes per SM and cycle) would otherwise spend a
+// seventh of the kernel on the test.
+template <typename R>
+struct CradTest;
+template <>
+struct CradTest<float> {
+    float4 pi;
+    __device__ __forceinline__ CradTest(const NepDev<float> &, const Eval2Args<float> &a, int64_t i) : pi(a.pos[i]) {}
+    __device__ __forceinline__ void operator()(const NepDev<float> &P, const Eval2Args<float> &a, int j, bool &in,
+                                               bool &ang) const {
+        float dx, dy, dz;
+        sep(a.box, pi, ro(a.pos + j), dx, dy, dz);
+        const float d2 = dx * dx + dy * dy + dz * dz;
+        in = d2 < P.rc_r2;
+        ang = d2 < P.rc_a2;
+    }
+};
+template <>
+struct CradTest<double> {
+    double4 pi;
+    float4 fi;
+    float band;
+    // Band: the FP32 copies are off by 2^-24 of themselves and the separation's own rounding and
+    // minimum image add as much of the coordinates and of a box length, so a component of a
+    // near pair's separation is off by at most E = 2^-24 (8 |x_i| + 4 L + 64) (the pair's other
+    // coordinate is within a box length and a few A of x_i), and d2 by 2 sqrt(3) R E + 3 E^2 and
+    // its sum's 4 2^-24 R^2, R a little beyond the cutoff; the band is twice that.
+    __device__ __forceinline__ CradTest(const NepDev<double> &P, const Eval2Args<double> &a, int64_t i)
+        : pi(a.pos[i]), fi(a.posf[i]) {
+        const float u = 5.9604645e-8f;
+        const float m = fmaxf(fmaxf(fabsf(fi.x), fabsf(fi.y)), fabsf(fi.z));
+        const float L = fmaxf(fmaxf((float)a.box.L[0], (float)a.box.L[1]), (float)a.box.L[2]);
+        const float E = u * (8.f * m + 4.f * L + 64.f), Rc = (float)P.rc_r + 1.f;
+        band = 2.f * (3.4641017f * Rc * E + 3.f * E * E + 4.f * u * Rc * Rc);
+    }
+    __device__ __forceinline__ void operator()(const NepDev<double> &P, const Eval2Args<double> &a, int j, bool &in,
+                                               bool &ang) const {
+        const float4 fj = ro(a.posf + j);
+        float x = fj.x - fi.x, y = fj.y - fi.y, z = fj.z - fi.z;
+        minimg(a.boxf, x, y, z);
+        const float d2f = x * x + y * y + z * z, r2 = (float)P.rc_r2, a2 = (float)P.rc_a2;
+        in = d2f < r2;
+        ang = d2f < a2;
+        // inside a band (or NaN): the FP64 test decides
+        if (!(fabsf(d2f - r2) > band) || !(fabsf(d2f - a2) > band)) {
+            double dx, dy, dz;
+            sep(a.box, pi, ro(a.pos + j), dx, dy, dz);
+            const double d2 = dx * dx + dy * dy + dz * dz;
+            in = d2 < P.rc_r2;
+            ang = d2 < P.rc_a2;
+        }
+    }
+};
+
+template <typename R>
+struct CradSmem {
+    R stage[8][CR_STAGE];                // per atom of the block; afterwards its sums [2][5][10]
+    int list[8][32 * MASKW_MAX + 16];    // in-cutoff neighbours in list order (padded like the stage)
+    uint32_t mask[MASKW_MAX][8];         // in-cutoff candidate slots
+    R q[CR_NQ][8];                       // the block's descriptor entries, written out by rows
+};
+static_assert(CR_STAGE >= 2 * 5 * 10, "the sums take the stage's place");
+
+template <typename R>
+__device__ __forceinline__ void crad_wide_body(const NepDev<R> &P, const Eval2Args<R> &args, int64_t blk,
+                                          CradSmem<R> &sm) {
+    // the arguments as values: read once from the block's copy, so nothing in the loops below
+    // depends on where they are stored
+    const Eval2Args<R> a = args;
+    if (a.skip && *a.skip) return;
+    const int lane = threadIdx.x & (CR_LANES - 1), slot8 = threadIdx.x / CR_LANES;
+    const int half = threadIdx.x & CR_LANES;          // 0 or 16: this atom's lanes in the warp
+    const int per = blockDim.x / CR_LANES;            // atoms of the block
+    const int64_t i = blk * per + slot8;
+    const bool valid = i < a.n;
+    const int64_t N = a.n, at = valid ? i : a.n - 1;
+    const unsigned lt = (1u << lane) - 1u;
+    R *stage = sm.stage[slot8];
+    int *list = sm.list[slot8];
+    if (lane < MASKW_MAX) sm.mask[lane][slot8] = 0u;
+    const v4<R> pi = a.pos[at], si = a.spin[at];
+    const int4 sg = valid ? a.seg[i] : make_int4(0, 0, 0, 0);
+    const CradTest<R> test(P, a, at);
+    const int32_t *__restrict__ nrow = a.nbr + at * a.capr;
+    const uint8_t *__restrict__ rrow = a.rev + at * a.capr;
+    __syncwarp();
+
+    // A
+    int m = 0, m0 = 0, na = 0, na0 = 0;   // pairs found (of species 0), angular ones
+    bool ovf = false;
+    const int steps = __reduce_max_sync(0xffffffffu, sg.w);
+    int jn = lane < sg.w ? nrow[lane] : 0;
+    uint32_t word = 0u;
+    for (int base = 0; base < steps; base += CR_LANES) {
+        const int v = base + lane, j = jn;
+        if (v + CR_LANES < sg.w) jn = nrow[v + CR_LANES];   // the next candidate is in flight
+        bool in = false, ang = false;
+        if (v < sg.w) test(P, a, j, in, ang);
+        const unsigned ha = (__ballot_sync(0xffffffffu, ang) >> half) & 0xffffu;
+        const int ra = na + __popc(ha & lt);
+        if (ang && ra >= a.cap_ang) {   // angular rows full: only after a list overflow
+            ovf = true;
+            in = ang = false;
+        }
+        const unsigned hi = (__ballot_sync(0xffffffffu, in) >> half) & 0xffffu;
+        if (in) {
+            const int c = m + __popc(hi & lt);
+            list[c] = j;
+            stg(a.crow + (int64_t)(ang ? ra : a.cap_ang + (c - ra)) * N + i, make_int2(j, rrow[v]));
+        }
+        word = base & 16 ? word | hi << 16 : hi;
+        if (lane == 0) sm.mask[base >> 5][slot8] = word;
+        if (base < sg.y) {   // species 0 ends at sg.y
+            const unsigned first = base + CR_LANES <= sg.y ? 0xffffu : (1u << (sg.y - base)) - 1u;
+            m0 += __popc(hi & first);
+            na0 = min(na0 + __popc(ha & first), a.cap_ang);
+        }
+        m += __popc(hi);
+        na = min(na + __popc(ha), a.cap_ang);
+    }
+    if (ovf) atomicOr(a.status, ST_NBR_OVERFLOW);
+    if (valid && lane == 0) stg(a.cnt + i, make_int4(na0, na, m0 - na0, m - na));
+    __syncwarp();
+    // B
+    const int kp = lane % 5, third = lane / 5;   // lane 15 is idle in the sums
+    R b0[2][2];
+    v2<R> b12[2][2], b34[2][2];
+#pragma unroll
+    for (int t = 0; t < 2; ++t)
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            b0[t][k] = R(0);
+            b12[t][k] = b34[t][k] = pair2<R>(R(0), R(0));
+        }
+    const int mmax = __reduce_max_sync(0xffffffffu, m);
+    for (int base = 0; base < mmax; base += CR_LANES) {
+        const int cnt = min(m - base, CR_LANES);
+        if (lane < cnt) {
+            const int j = list[base + lane];
+            const v4<R> pj = ro(a.pos + j), sj = ro(a.spin + j);
+            R dx, dy, dz;
+            sep(a.box, pi, pj, dx, dy, dz);
+            const R d2 = dx * dx + dy * dy + dz * dz;
+            const R ir = rsqrt_(d2), r = d2 * ir;
+            const R ux = dx * ir, uy = dy * ir, uz = dz * ir;
+            R f[NK];
+            carrier_f(r, P.inv_rc_r, f);
+            const R siu = si.x * ux + si.y * uy + si.z * uz;
+            const R sju = sj.x * ux + sj.y * uy + sj.z * uz;
+            v4<R> *d = reinterpret_cast<v4<R> *>(stage + lane * CR_LD);
+            v4<R> w;
+            w.x = f[0]; w.y = f[1]; w.z = f[2]; w.w = f[3];
+            d[0] = w;
+            w.x = f[4]; w.y = f[5]; w.z = f[6]; w.w = f[7];
+            d[1] = w;
+            v2<R> w2;
+            w2.x = f[8]; w2.y = R(0);
+            *reinterpret_cast<v2<R> *>(d + 2) = w2;
+            w.x = si.x * sj.x + si.y * sj.y + si.z * sj.z;
+            w.y = (si.y * sj.z - si.z * sj.y) * ux + (si.z * sj.x - si.x * sj.z) * uy + (si.x * sj.y - si.y * sj.x) * uz;
+            w.z = siu * sju;
+            w.w = siu * siu;
+            d[3] = w;
+        }
+        __syncwarp();
+        const int split = min(max(m0 - base, 0), max(cnt, 0));   // staged pairs of species 0
+        if (third < 3) {
+            auto add = [&](int t, int x) {
+                const v2<R> f = *reinterpret_cast<const v2<R> *>(stage + x * CR_LD + 2 * kp);
+                const v4<R> g = *reinterpret_cast<const v4<R> *>(stage + x * CR_LD + 12);
+                b0[t][0] += f.x;
+                b0[t][1] += f.y;
+                b12[t][0] = fma2(pair2<R>(f.x, f.x), pair2<R>(g.x, g.y), b12[t][0]);
+                b34[t][0] = fma2(pair2<R>(f.x, f.x), pair2<R>(g.z, g.w), b34[t][0]);
+                b12[t][1] = fma2(pair2<R>(f.y, f.y), pair2<R>(g.x, g.y), b12[t][1]);
+                b34[t][1] = fma2(pair2<R>(f.y, f.y), pair2<R>(g.z, g.w), b34[t][1]);
+            };
+            for (int x = third; x < split; x += 3) add(0, x);
+            for (int x = split + third; x < cnt; x += 3) add(1, x);
+        }
+        __syncwarp();
+    }
+    // C: the three thirds, then q = sum over species and k
+    R *sums = stage;   // [species][group][10]
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+        R v[5][2];
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            v[0][k] = b0[t][k];
+            v[1][k] = b12[t][k].x;
+            v[2][k] = b12[t][k].y;
+            v[3][k] = b34[t][k].x;
+            v[4][k] = b34[t][k].y;
+        }
+#pragma unroll
+        for (int g = 0; g < 5; ++g) {
+            v2<R> s;
+            s.x = v[g][0] + __shfl_down_sync(0xffffffffu, v[g][0], 5, CR_LANES) +
+                  __shfl_down_sync(0xffffffffu, v[g][0], 10, CR_LANES);
+            s.y = v[g][1] + __shfl_down_sync(0xffffffffu, v[g][1], 5, CR_LANES) +
+                  __shfl_down_sync(0xffffffffu, v[g][1], 10, CR_LANES);
+            if (lane < 5) *reinterpret_cast<v2<R> *>(sums + (t * 5 + g) * 10 + 2 * kp) = s;
+        }
+    }
+    __syncwarp();
+    const R *__restrict__ ct = a.ctab + (at < a.n_fe ? 0 : 1) * (2 * NK * 32);
+    for (int o = lane; o < 25; o += CR_LANES) {
+        const int g = o / NCH;
+        R q = R(0);
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+            const v2<R> *s = reinterpret_cast<const v2<R> *>(sums + (t * 5 + g) * 10);
+#pragma unroll
+            for (int k = 0; k < NK; k += 2) {
+                const v2<R> x = s[k / 2];
+                q += ro(ct + (t * NK + k) * 32 + o) * x.x;
+                if (k + 1 < NK) q += ro(ct + (t * NK + k + 1) * 32 + o) * x.y;
+            }
+        }
+        sm.q[o][slot8] = q;
+    }
+    if (lane == 0) sm.q[25][slot8] = si.x * si.x + si.y * si.y + si.z * si.z;
+    // the block's outputs by rows: its atoms are neighbours in memory
+    __syncthreads();
+    const int64_t i0 = blk * per;
+    for (int e = threadIdx.x; e < (CR_NQ + a.maskw) * per; e += blockDim.x) {
+        const int row = e / per, k = e % per;
+        if (i0 + k >= N) continue;
+        if (row < CR_NQ) {
+            const int v = row < 5 ? Q_R + row : row < 25 ? Q_EX + (row - 5) : Q_O;   // EX, DMI, ANI, SIA in turn
+            stg(a.q + v * a.qs + i0 + k, sm.q[row][k]);
+        } else {
+            stg(reinterpret_cast<int *>(a.mask) + (int64_t)(row - CR_NQ) * N + i0 + k, (int)sm.mask[row - CR_NQ][k]);
+        }
+    }
 }
 
 
@@ -421,7 +717,6 @@ __device__ __forceinline__ void ang_fwd_body(const NepDev<R> &P, const Eval2Args
     const int64_t i = (blk * (blockDim.x >> 5) + warp) * 8 + quad;
     const bool valid = i < a.n;
     R *stage = reinterpret_cast<R *>(smem_raw) + (warp * 8 + quad) * FQUAD;
-    const int64_t N = a.n;
     v4<R> pi, si;
     int na0 = 0, na = 0, ti = 0;
     if (valid) {
@@ -441,17 +736,19 @@ __device__ __forceinline__ void ang_fwd_body(const NepDev<R> &P, const Eval2Args
     // the lane's list entry three rounds ahead and its coordinates two rounds ahead are in flight
     v4<R> pjn, sjn, pjn2, sjn2;
     int jn3 = 0;
+    const int2 *__restrict__ crow = a.crow + i;
+    const int64_t N = a.n;
     if (ql < na) {
-        const int j = a.clj[(int64_t)ql * N + i];
+        const int j = crow[(int64_t)ql * N].x;
         pjn = a.pos[j];
         sjn = a.spin[j];
     }
     if (ql + 4 < na) {
-        const int j = a.clj[(int64_t)(ql + 4) * N + i];
+        const int j = crow[(int64_t)(ql + 4) * N].x;
         pjn2 = a.pos[j];
         sjn2 = a.spin[j];
     }
-    if (ql + 8 < na) jn3 = a.clj[(int64_t)(ql + 8) * N + i];
+    if (ql + 8 < na) jn3 = crow[(int64_t)(ql + 8) * N].x;
     for (int base = 0; base < nmax; base += 4) {
         const int p = base + ql;
         const v4<R> pj = pjn, sj = sjn;
@@ -461,7 +758,7 @@ __device__ __forceinline__ void ang_fwd_body(const NepDev<R> &P, const Eval2Args
             pjn2 = a.pos[jn3];
             sjn2 = a.spin[jn3];
         }
-        if (p + 12 < na) jn3 = a.clj[(int64_t)(p + 12) * N + i];
+        if (p + 12 < na) jn3 = crow[(int64_t)(p + 12) * N].x;
         if (p < na) {
             R *st = stage + ql * FSTAGE;
             if (ti == 0) {
@@ -722,41 +1019,30 @@ __device__ __forceinline__ void bwd_rows(const NepDev<R> &P, const Eval2Args<R> 
                                          int split, const v4<R> &pi, const v4<R> &si, const R *sm,
                                          BwdAcc2<R> &acc) {
     const int64_t N = a.n;
-    int j1 = 0, t1 = 0, j2 = 0, t2 = 0, j3 = 0, t3 = 0;
+    const int2 *__restrict__ crow = a.crow + i;
+    int2 e1 = make_int2(0, 0), e2 = e1, e3 = e1;   // (neighbour, the record's slot in its list)
     v4<R> p1, s1, p2, s2;
+    if (lo < hi) e1 = ro(crow + (int64_t)lo * N);
+    if (lo + 4 < hi) e2 = ro(crow + (int64_t)(lo + 4) * N);
+    if (lo + 8 < hi) e3 = ro(crow + (int64_t)(lo + 8) * N);
     if (lo < hi) {
-        j1 = ro(a.clj + (int64_t)lo * N + i);
-        t1 = ro(a.cls + (int64_t)lo * N + i) >> 8;
+        p1 = ro(a.pos + e1.x);
+        s1 = ro(a.spin + e1.x);
     }
     if (lo + 4 < hi) {
-        j2 = ro(a.clj + (int64_t)(lo + 4) * N + i);
-        t2 = ro(a.cls + (int64_t)(lo + 4) * N + i) >> 8;
-    }
-    if (lo + 8 < hi) {
-        j3 = ro(a.clj + (int64_t)(lo + 8) * N + i);
-        t3 = ro(a.cls + (int64_t)(lo + 8) * N + i) >> 8;
-    }
-    if (lo < hi) {
-        p1 = ro(a.pos + j1);
-        s1 = ro(a.spin + j1);
-    }
-    if (lo + 4 < hi) {
-        p2 = ro(a.pos + j2);
-        s2 = ro(a.spin + j2);
+        p2 = ro(a.pos + e2.x);
+        s2 = ro(a.spin + e2.x);
     }
     for (int row = lo; row < hi; row += 4) {
-        const int j = j1, t = t1;
+        const int j = e1.x, t = e1.y;
         const v4<R> pj = p1, sj = s1;
-        j1 = j2; t1 = t2; p1 = p2; s1 = s2;
-        j2 = j3; t2 = t3;
+        e1 = e2; p1 = p2; s1 = s2;
+        e2 = e3;
         if (row + 8 < hi) {
-            p2 = ro(a.pos + j2);
-            s2 = ro(a.spin + j2);
+            p2 = ro(a.pos + e2.x);
+            s2 = ro(a.spin + e2.x);
         }
-        if (row + 12 < hi) {
-            j3 = ro(a.clj + (int64_t)(row + 12) * N + i);
-            t3 = ro(a.cls + (int64_t)(row + 12) * N + i) >> 8;
-        }
+        if (row + 12 < hi) e3 = ro(crow + (int64_t)(row + 12) * N);
         bwd_pair<R, ANG, VIR>(P, a, ti, row < split ? 0 : 1, pi, si, pj, sj, j, t, sm, acc);
     }
 }
@@ -853,13 +1139,22 @@ __device__ __forceinline__ void bwd_body(const NepDev<R> &P, const Eval2Args<R> 
 // The evaluation kernels over an argument table (sl_batch.h: a system's own table or a
 // batch's).  MINB: the register budget, as the minimum resident blocks per SM.  The
 // mixed-precision kernels default to 4 blocks (128 registers) and have a second budget each,
-// which sl_autotune may choose: radial 3 blocks, angular unconstrained, backward 3 blocks.
-template <typename R, int MINB = sizeof(R) == 4 ? 4 : 2>
-__global__ void __launch_bounds__(128, MINB) k_crad(const __grid_constant__ NepDev<R> P,
-                                                    const Eval2Args<R> *__restrict__ tab, SlotMap sm,
-                                                    const __grid_constant__ Eval2Args<R> solo) {
+// which sl_autotune may choose: radial (one thread per atom) and backward 3 blocks, angular
+// unconstrained.
+template <int MINB = 4>
+__global__ void __launch_bounds__(128, MINB) k_crad(const __grid_constant__ NepDev<float> P,
+                                                    const Eval2Args<float> *__restrict__ tab, SlotMap sm,
+                                                    const __grid_constant__ Eval2Args<float> solo) {
     __shared__ uint32_t smask[MASKW_MAX][128];   // blocks have at most 128 threads
-    one_work(tab, sm, solo, [&](const Eval2Args<R> &a, int64_t blk, int64_t) { crad_body(P, a, blk, smask); });
+    one_work(tab, sm, solo, [&](const Eval2Args<float> &a, int64_t blk, int64_t) { crad_body(P, a, blk, smask); });
+}
+template <typename R>
+__global__ void __launch_bounds__(128, sizeof(R) == 4 ? 8 : 4) k_crad_wide(const __grid_constant__ NepDev<R> P,
+                                                                           const Eval2Args<R> *__restrict__ tab,
+                                                                           SlotMap sm,
+                                                                           const __grid_constant__ Eval2Args<R> solo) {
+    __shared__ __align__(32) CradSmem<R> scratch;   // blocks have at most 128 threads
+    one_work(tab, sm, solo, [&](const Eval2Args<R> &a, int64_t blk, int64_t) { crad_wide_body(P, a, blk, scratch); });
 }
 template <typename R, int MINB = sizeof(R) == 4 ? 4 : 1>
 __global__ void __launch_bounds__(128, MINB) k_ang_fwd(const __grid_constant__ NepDev<R> P,
@@ -887,6 +1182,8 @@ static Eval2Args<R> args2(Sys &s, const EvalAt &at, bool want_virial) {
         a.pos = reinterpret_cast<const v4<R> *>(at.pos ? at.pos : s.pos);
         a.spin = reinterpret_cast<const v4<R> *>(at.spin ? at.spin : s.spin);
         a.box = *reinterpret_cast<const BoxDev<R> *>(&s.boxd);
+        a.posf = at.posf ? at.posf : s.posf;
+        a.boxf = s.boxf;
     } else {
         a.pos = reinterpret_cast<const v4<R> *>(at.posf ? at.posf : s.posf);
         a.spin = reinterpret_cast<const v4<R> *>(at.spinf ? at.spinf : s.spinf);
@@ -895,7 +1192,7 @@ static Eval2Args<R> args2(Sys &s, const EvalAt &at, bool want_virial) {
     a.skip = at.skip;
     a.nbr = s.nbr; a.seg = s.seg; a.rev = s.rev; a.capr = nbr_stride(s.cap); a.n = s.n; a.n_fe = s.n_fe;
     a.cap = s.cap; a.cap_ang = s.cap_ang;
-    a.clj = s.clj; a.cls = s.cls; a.cnt = s.cnt; a.mask = s.cmask; a.maskw = s.maskw;
+    a.crow = s.crow; a.ctab = (const R *)s.ctab; a.cnt = s.cnt; a.mask = s.cmask; a.maskw = s.maskw;
     a.q = (R *)s.q; a.qs = s.qs; a.bsum = (R *)s.bsum; a.fp = (R *)s.fp; a.ei = (R *)s.ei;
     a.pd = (PairRec<R> *)s.pairs; a.fown = (v4<R> *)s.fown; a.gii = (v4<R> *)s.gii;
     a.wpart = (R *)s.wpart; a.want_virial = want_virial; a.status = s.status;
@@ -952,11 +1249,13 @@ void fused_put_eval(Sys &s, int r, int kind, const FusedTables &t, unsigned char
     if (s.prec == 0) reinterpret_cast<Eval2Args<double> *>(img + t.o_eval)[r] = args2<double>(s, at, kind == SK_FULL);
     else reinterpret_cast<Eval2Args<float> *>(img + t.o_eval)[r] = args2<float>(s, at, kind == SK_FULL);
     const int qb = default_quad_block(s.prec);
-    blocks[FK_CRAD] = (s.n + 127) / 128;
+    const bool wide = crad_is_wide(s);
+    blocks[FK_CRAD] = wide ? 0 : (s.n + 127) / 128;
+    blocks[FK_CRADW] = wide ? (s.n + CRAD_WIDE_ATOMS - 1) / CRAD_WIDE_ATOMS : 0;
     blocks[FK_ANG] = blocks[FK_BWD] = (s.n + qb / 4 - 1) / (qb / 4);
 }
 
-// Radial, angular, network and backward over a table, each launch in its own shape
+// Radial, angular, network and backward (and, last, the wide radial kernel) over a table, each launch in its own shape
 // (L[k].block threads, 0: the default) and register budget (L[k].minb, 0: the default).
 template <typename R>
 void launch_eval_t(const FusedTables &t, const NepDev<R> &P, const Launch *L, cudaStream_t st, cudaEvent_t *ev) {
@@ -971,14 +1270,14 @@ void launch_eval_t(const FusedTables &t, const NepDev<R> &P, const Launch *L, cu
     if (ev) cudaEventRecord(ev[0], st);
     // compaction and radial channels in one kernel: the compaction group is empty
     if (ev) cudaEventRecord(ev[1], st);
-    bool variant = false;
+    // a system's own launch has a grid for one of the radial kernels only
     if constexpr (sizeof(R) == 4) {
-        variant = L[0].minb == 3;
-        if (variant) k_crad<R, 3><<<L[0].grid, cb, 0, st>>>(P, tab, s0, so);
+        if (L[0].grid && L[0].minb == 3) k_crad<3><<<L[0].grid, cb, 0, st>>>(P, tab, s0, so);
+        else if (L[0].grid) k_crad<<<L[0].grid, cb, 0, st>>>(P, tab, s0, so);
     }
-    if (!variant) k_crad<R><<<L[0].grid, cb, 0, st>>>(P, tab, s0, so);
+    if (L[4].grid) k_crad_wide<R><<<L[4].grid, L[4].block ? L[4].block : 128, 0, st>>>(P, tab, L[4].slots(), so);
+    bool variant = false;
     if (ev) cudaEventRecord(ev[2], st);
-    variant = false;
     if constexpr (sizeof(R) == 4) {
         variant = L[1].minb == 1;
         if (variant) k_ang_fwd<R, 1><<<L[1].grid, qa, fwd_smem<R>(qa), st>>>(P, tab, s1, so);
@@ -1011,8 +1310,8 @@ template void launch_eval_t<double>(const FusedTables &, const NepDev<double> &,
 void launch_eval(Sys &s, bool want_virial, cudaEvent_t *ev) {
     if (s.n == 0) return;
     const int kind = s.at.pos ? SK_MID : want_virial ? SK_FULL : SK_STEP;
-    const Launch L[4] = {solo_launch(s, FK_CRAD, kind), solo_launch(s, FK_ANG, kind), solo_launch(s, FK_NET, kind),
-                         solo_launch(s, FK_BWD, kind)};
+    const Launch L[5] = {solo_launch(s, FK_CRAD, kind), solo_launch(s, FK_ANG, kind), solo_launch(s, FK_NET, kind),
+                         solo_launch(s, FK_BWD, kind), solo_launch(s, FK_CRADW, kind)};
     if (s.prec == 0) launch_eval_t<double>(s.solo->t, s.pd, L, s.stream, ev);
     else launch_eval_t<float>(s.solo->t, s.pf, L, s.stream, ev);
 }

@@ -27,9 +27,12 @@ struct Eval2Args {
     const int4 *seg;
     int64_t n, n_fe;
     BoxDev<R> box;
+    const float4 *posf;    // FP64 kernels: FP32 copies of pos and box (the cutoff pre-test)
+    BoxDev<float> boxf;
     int cap, cap_ang;
-    int32_t *clj;      // compact in-cutoff rows [cap_ang + cap][n]: neighbour index
-    uint16_t *cls;     // ... its candidate slot s (low byte) and the reverse slot rev[s][i] (high byte)
+    int2 *crow;        // compact in-cutoff rows [cap_ang + cap][n]: angular rows from 0, radial-only rows from
+                       // cap_ang; each the neighbour's index and the atom's slot in the neighbour's list
+    const R *ctab;     // coefficients of the radial contraction (make_coeff_table)
     int4 *cnt;         // (angular rows of species 0, angular rows, radial-only rows of species 0, radial-only rows)
     uint32_t *mask;    // [maskw][n]: bit s of word s/32 set when candidate slot s is inside rc_rad
     int maskw;

@@ -52,7 +52,7 @@ struct MidDev {
 // otherwise).  The per-atom arithmetic does not depend on them, so results are the same
 // for every choice.
 struct LaunchCfg {
-    int crad_block = 128;      // threads per block of k_crad (one atom per thread)
+    int crad_block = 128;      // threads per block of the radial kernel (one per atom, or 16)
     int ang_block = 0;         // threads per block of k_ang_fwd (four per atom); 0: the precision's default
     int bwd_block = 0;         // threads per block of k_bwd
     int mlp_ctas_per_sm = 2;   // persistent CTAs per SM of the tensor-core network
@@ -115,7 +115,7 @@ struct Sys {
     // nbr_hash (an 8-bit hash of each candidate's index: the reverse-slot search's filter)
     int32_t *nbr = nullptr;
     uint8_t *rev = nullptr, *nbr_hash = nullptr;
-    int4 *seg = nullptr;       // per atom: ends of (ang t0, ang t1, rad t0, rad t1)
+    int4 *seg = nullptr;       // per atom: ends of (ang t0, rad t0, ang t1, rad t1)
     Cells cells;
 
     // evaluation buffers (element type = compute precision)
@@ -127,8 +127,8 @@ struct Sys {
     void *fp = nullptr;        // [DIM][n]
     void *ei = nullptr;        // [n]
     void *pairs = nullptr;     // [cap][n] pair records (see sl_eval2.cuh)
-    int32_t *clj = nullptr;    // [cap_ang + cap][n] compact in-cutoff neighbours
-    uint16_t *cls = nullptr;   // [cap_ang + cap][n] candidate slot | reverse slot << 8
+    int2 *crow = nullptr;      // [cap_ang + cap][n] compact in-cutoff rows (see sl_eval2.cuh)
+    void *ctab = nullptr;      // coefficients of the radial contraction (sl_eval2.cu)
     int4 *cnt = nullptr;       // [n] compact row counts
     uint32_t *cmask = nullptr; // [maskw][n] in-cutoff candidate slots (the gather's walk)
     int maskw = 0;             // ceil(cap / 32)
@@ -218,6 +218,12 @@ void solo_free(Sys &s);
 // row stride of the atom-major caller-index copy of the lists: cap rounded up to a multiple
 // of 4 entries, so every row starts on a 16-byte boundary
 inline int nbr_stride(int cap) { return (cap + 31) & ~31; }   // byte rows of 32-byte multiples
+// The radial kernel of a system (fixed by its size, so the same alone and in a batch): sixteen
+// lanes per atom in FP64 and for small systems, else one thread per atom (both timed at
+// k_crad_wide).
+constexpr int64_t CRAD_WIDE_MAX = 16384;
+constexpr int CRAD_WIDE_ATOMS = 8;   // atoms per 128-thread block of k_crad_wide
+inline bool crad_is_wide(const Sys &s) { return s.prec == 0 || s.n <= CRAD_WIDE_MAX; }
 void nbr_setup(Sys &s);
 void launch_rebuild(Sys &s, bool conditional);
 // sl_eval2.cu: the system's evaluation at the state (with the virial parts when asked for), or
@@ -226,6 +232,7 @@ void launch_rebuild(Sys &s, bool conditional);
 void launch_eval(Sys &s, bool want_virial, cudaEvent_t *ev = nullptr);
 void eval2_init();   // dynamic shared-memory limits of the evaluation kernels (once per device)
 int default_quad_block(int prec);   // threads per block of the quad kernels by default
+int make_coeff_table(Sys &s);                    // s.ctab from the model; 0 on success
 int make_q_tensor_map(Sys &s);                   // sl_mlp_tc.cu: the TMA map of s.q; 0 on success
 int make_mlp_image(Sys &s);                      // sl_mlp_tc.cu: s.mlp_img from s.pf; 0 on success
 // first half, rebuild group (7), compaction with radial forward, angular forward, network, backward,

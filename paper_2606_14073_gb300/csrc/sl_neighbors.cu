@@ -9,9 +9,9 @@
 //   d2 = (t_x*t_x + t_y*t_y) + t_z*t_z  <  (rc_rad + skin)^2
 // in FP64 with no contraction.  An FP32 pre-test settles pairs far from the
 // cutoff; only pairs within a margin of it take the exact FP64 test.
-// Each list is split in four segments -- angular candidates (d2 < (rc_ang+skin)^2)
-// of neighbour species 0 and 1, then the remaining radial candidates of species
-// 0 and 1 -- and each segment is in the order of the list build's walk (the half-width
+// Each list is split in four segments -- the angular candidates (d2 < (rc_ang+skin)^2)
+// of neighbour species 0, the remaining radial candidates of species 0, then the two of
+// species 1 -- and each segment is in the order of the list build's walk (the half-width
 // sub-cells around the atom z-major, or the whole stencil's cells z-major in a box with
 // fewer than 3 cells along a periodic axis; each sub-cell's or cell's atoms by species,
 // then caller index), so every per-atom sum runs in an order set by the positions and caller indices
@@ -348,9 +348,9 @@ __device__ __forceinline__ void list_atom(const ListArgs &a, int64_t i, float4 p
     auto append = [&](int f, const float4 &pj, bool in_r, bool in_a) {
         const unsigned mr = __ballot_sync(0xffffffffu, in_r);
         const int pos = m + __popc(mr & lt);
-        // segment (angular? 0 : 2) + species of j in bits 30-31 above the candidate index
+        // segment 2 species of j + (angular? 0 : 1) in bits 30-31 above the candidate index
         if (in_r && pos < SORT_MAX)
-            key[pos] = (((in_a ? 0u : 2u) + ((uint32_t)__float_as_int(pj.w) & 1u)) << 30) | (uint32_t)f;
+            key[pos] = (((in_a ? 0u : 1u) + 2u * ((uint32_t)__float_as_int(pj.w) & 1u)) << 30) | (uint32_t)f;
         m += __popc(mr);
     };
     for (int base = 0; base < nwalk; base += 64) {   // two chunks of 32 candidates at a time
@@ -379,7 +379,7 @@ __device__ __forceinline__ void list_atom(const ListArgs &a, int64_t i, float4 p
 #pragma unroll
         for (int t = 0; t < 4; ++t) cnt4[t] += __popc(__ballot_sync(0xffffffffu, sg == (unsigned)t));
     }
-    const bool overflow = m > a.cap || cnt4[0] + cnt4[1] > a.cap_ang;
+    const bool overflow = m > a.cap || cnt4[0] + cnt4[2] > a.cap_ang;
     int run[4] = {0, cnt4[0], cnt4[0] + cnt4[1], cnt4[0] + cnt4[1] + cnt4[2]};
     const int ends_all[4] = {run[1], run[2], run[3], run[3] + cnt4[3]};
     for (int s0 = 0; s0 < mm; s0 += 32) {
@@ -681,7 +681,7 @@ __device__ __forceinline__ void rev_body(const RevArgs &args, int64_t blk, int64
         for (int p = lane; p < cnt; p += 32) {
             const int s = sm.s[w][p], j = sm.j[w][p];
             const int4 sj = a.seg[j];
-            const int sgi = (s < sg.y ? 0 : 2) + ti;
+            const int sgi = 2 * ti + (s < sg.x || (s >= sg.y && s < sg.z) ? 0 : 1);
             const int lo = sgi == 0 ? 0 : sgi == 1 ? sj.x : sgi == 2 ? sj.y : sj.z;
             const int hi = sgi == 0 ? sj.x : sgi == 1 ? sj.y : sgi == 2 ? sj.z : sj.w;
             const int t = find_slot(a.nbr + (int64_t)j * a.capr, a.hash + (int64_t)j * a.capr, lo, hi, (int)i);
