@@ -571,6 +571,7 @@ int sl_create_system(const double *positions, const double *spins, const double 
         (rc = dalloc(&s.red, 256 * 10 + 10)) || (rc = dalloc(&s.snap, 5 * N)) || (rc = dalloc(&s.d_builds, 1)))
         return bail(rc);
     if (n > 0 && sl::make_coeff_table(s)) return bail(fail(SL_ENOMEM, "the coefficient table could not be made"));
+    if (sl::make_net_table(s)) return bail(fail(SL_ENOMEM, "the network's weight table could not be made"));
     if (s.prec == SL_PREC_MIXED && n > 0 && sl::make_q_tensor_map(s))
         return bail(fail(SL_ECUDA, "the TMA map of the descriptor array could not be encoded"));
     if (s.prec == SL_PREC_MIXED && n > 0 && sl::make_mlp_image(s))

@@ -51,7 +51,7 @@ static int item_class(int k, int prec) {
         case FK_CRAD: return prec == 0 ? -1 : IC_ATOM;   // FP64: the wide kernel only
         case FK_CRADW: return IC_OCT;
         case FK_ANG: case FK_BWD: return IC_QUAD;
-        case FK_NET: return prec == 0 ? IC_ATOM : -1;
+        case FK_NET: return prec == 0 ? IC_OCT : -1;
         default: return -1;
     }
 }
@@ -205,7 +205,7 @@ bool FusedBatch::same_model(const Sys &s) const {
 static int item_kernel_class(const char *name) {
     struct { const char *id; int cls; } const k[] = {
         {"k_first_half", IC_HALF}, {"k_second_half", IC_HALF}, {"k_crad", IC_ATOM}, {"k_crad_wide", IC_OCT},
-        {"k_mlp", IC_ATOM}, {"k_ang_fwd", IC_QUAD}, {"k_bwd", IC_QUAD}};
+        {"k_mlp", IC_OCT}, {"k_ang_fwd", IC_QUAD}, {"k_bwd", IC_QUAD}};
     for (const auto &x : k) {
         const std::string id(x.id);
         const std::string forms[3] = {std::to_string(id.size()) + id + "I", id + "<", id + "("};
@@ -353,7 +353,7 @@ cudaError_t FusedBatch::upload(const int64_t *left, cudaStream_t st) {
     if (dirty || layout_dirty) {
         // block -> slot layout of the one-item-per-block kernels: every occupied slot's blocks in
         // slot order, then no slot (-1) up to the capacity
-        const int kof[IC_N] = {FK_FIRST, t.prec == 0 ? FK_NET : FK_CRAD, FK_ANG, FK_CRADW};
+        const int kof[IC_N] = {FK_FIRST, FK_CRAD, FK_ANG, FK_CRADW};
         for (int c = 0; c < IC_N; ++c) {
             int *it = h_items + item_off[c];
             int64_t o = 0;

@@ -29,8 +29,8 @@ enum FusedKernel {
 inline int fused_launches_per_step(int prec) { return 1 + FK_N + 1 - (prec == 0); }
 constexpr int FUSED_MAX_SLOTS = 4096;
 // atoms-per-block classes of the kernels that take one work item per block: the halves (256
-// atoms), the one-thread-per-atom radial kernel or the FP64 network (128), the angular and
-// backward kernels (a quad block's atoms), the wide radial kernel (8)
+// atoms), the one-thread-per-atom radial kernel (128), the angular and backward kernels (a quad
+// block's atoms), the wide radial kernel and the FP64 network (8)
 enum { IC_HALF = 0, IC_ATOM = 1, IC_QUAD = 2, IC_OCT = 3, IC_N = 4 };
 
 // what a slot's entries are set up for
@@ -121,7 +121,7 @@ template <typename R>
 void launch_eval_t(const FusedTables &t, const NepDev<R> &P, const Launch *L /* crad, ang, net, bwd, wide crad */,
                    cudaStream_t st, cudaEvent_t *ev);
 void launch_net_t_tc(const FusedTables &t, const NepDev<float> &P, const Launch &L, cudaStream_t st);
-void launch_net_t_fp64(const FusedTables &t, const NepDev<double> &P, const Launch &L, cudaStream_t st);
+void launch_net_t_fp64(const FusedTables &t, const Launch &L, cudaStream_t st);
 
 // The fused step of one batch: its tables (device, and a pinned host image of the
 // host-written part), its slots' systems, and two captured graphs over the tables (g steps

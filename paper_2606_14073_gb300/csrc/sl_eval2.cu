@@ -1285,7 +1285,7 @@ void launch_eval_t(const FusedTables &t, const NepDev<R> &P, const Launch *L, cu
     if (!variant) k_ang_fwd<R><<<L[1].grid, qa, fwd_smem<R>(qa), st>>>(P, tab, s1, so);
     if (ev) cudaEventRecord(ev[3], st);
     if constexpr (sizeof(R) == 4) launch_net_t_tc(t, P, L[2], st);
-    else launch_net_t_fp64(t, P, L[2], st);
+    else launch_net_t_fp64(t, L[2], st);
     if (ev) cudaEventRecord(ev[4], st);
     // the virial parts: only a system's own full evaluation asks for them (a batch's slots are
     // set up for the step's evaluation, which has none)

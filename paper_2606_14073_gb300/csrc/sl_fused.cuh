@@ -33,13 +33,14 @@ struct MlpArgs {
 };
 static_assert(alignof(CUtensorMap) >= 64, "tensor maps are 64-byte aligned");
 
-// the CUDA-core network's arguments for one replica
+// the FP64 network's arguments for one replica
 template <typename R>
 struct NetArgs {
     const R *q;
     R *fp, *ei;
     int64_t n, qs;
     const int *skip;     // non-null: the slot's atoms are passed over while *skip
+    const R *wtab;       // the weights (make_net_table)
 };
 
 // the slot of work item w: the last slot r with w0[r] <= w (idle slots before it have

@@ -122,7 +122,7 @@ struct Sys {
     void *q = nullptr;         // [DIM][qs]: descriptor v of atom i at v * qs + i
     int64_t qs = 0;            // row stride of q: n rounded up to a multiple of 4 (16-byte rows)
     CUtensorMap qmap;          // TMA map of q (mixed precision): [DIM] rows x n atoms, 128 x 66 boxes
-    void *mlp_img = nullptr;   // the network weights as the tensor-core kernel's FP16 hi/lo operand images
+    void *mlp_img = nullptr;   // the network weights: the tensor-core kernel's FP16 hi/lo operand images, or the FP64 table
     void *bsum = nullptr;      // [n][NLM][BREC] angular-sum records
     void *fp = nullptr;        // [DIM][n]
     void *ei = nullptr;        // [n]
@@ -234,6 +234,7 @@ void eval2_init();   // dynamic shared-memory limits of the evaluation kernels (
 int default_quad_block(int prec);   // threads per block of the quad kernels by default
 int make_coeff_table(Sys &s);                    // s.ctab from the model; 0 on success
 int make_q_tensor_map(Sys &s);                   // sl_mlp_tc.cu: the TMA map of s.q; 0 on success
+int make_net_table(Sys &s);                      // sl_nep.cu: the FP64 network's weights; 0 on success
 int make_mlp_image(Sys &s);                      // sl_mlp_tc.cu: s.mlp_img from s.pf; 0 on success
 // first half, rebuild group (7), compaction with radial forward, angular forward, network, backward,
 // second half

@@ -17,11 +17,9 @@
 // without atomics (sl_integrate.cu):
 //   F_k = sum_j (dE_k/dr_kj - dE_j/dr_jk),  H_k = -dE_k/dS_k - sum_j dE_j/dS_k + Zeeman.
 //
-// Atoms are stored species-major, so a warp almost always has one centre species;
-// the neighbour list is segmented by neighbour species, so inside a segment both
-// species are compile-time constants and every coefficient is a constant operand.
 #include <cstddef>
 #include <mutex>
+#include <vector>
 
 #include "sl_internal.h"
 #include "sl_batch.h"
@@ -29,52 +27,115 @@
 
 namespace sl {
 
-template <typename R>
-__device__ __forceinline__ R tanh_(R x);
-template <>
-__device__ __forceinline__ float tanh_<float>(float x) { return tanhf(x); }
-template <>
-__device__ __forceinline__ double tanh_<double>(double x) { return tanh(x); }
-
 // ------------------------------------------------------------------ network
 // E_i = sum_h w1_h tanh(z_h) - b1, z_h = sum_v W0_hv s_v q_v - b0_h;
 // Fp_v = s_v sum_h w1_h (1 - tanh^2 z_h) W0_hv.
+// FP64 (the mixed-precision network runs on the tensor cores, sl_mlp_tc.cu): eight atoms per
+// 128-thread block, two per warp.  The weights and the block's descriptors are staged in shared
+// memory; lane h takes hidden unit h of both atoms, then the lanes take the 2 x 66 gradient
+// entries, 32 at a time, and eight lanes share each of the last four.  What bounds it: the FP64
+// pipe (160 warp instructions per atom; one thread per atom took 184, and a serial chain of 4,000
+// multiply-adds however few the atoms): 512 / 13,824 / 110,592 atoms 27 / 154 / 984 us, against
+// 202 / 228 / 1,070.
+constexpr int NET_ATOMS = 8;          // atoms per block
+constexpr int NET_LD = DIM + 1;       // row length of W0 in the table and in shared memory
+// weight table of a system (device): W0 [NH][NET_LD], b0 [NH], w1 [NH], s [DIM], b1
+constexpr int NT_B0 = NH * NET_LD, NT_W1 = NT_B0 + NH, NT_S = NT_W1 + NH, NT_B1 = NT_S + DIM, NT_SIZE = NT_B1 + 1;
+
 template <typename R>
-__device__ __forceinline__ void mlp_atom(const NepDev<R> &P, const R *__restrict__ q, R *__restrict__ fp,
-                                         R *__restrict__ ei, int64_t n, int64_t qs, int64_t i) {
-    R x[DIM];
-#pragma unroll
-    for (int v = 0; v < DIM; ++v) x[v] = q[(int64_t)v * qs + i] * P.scal[v];
-    R t[NH];
-    R E = -P.b1;
-#pragma unroll
-    for (int h = 0; h < NH; ++h) {
-        R z = -P.b0[h];
-#pragma unroll
-        for (int v = 0; v < DIM; ++v) z += P.w0[h][v] * x[v];
-        const R th = tanh_(z);
-        E += P.w1[h] * th;
-        t[h] = P.w1[h] * (R(1) - th * th);
+struct NetSmem {
+    R w[NT_SIZE];
+    R x[DIM][NET_ATOMS];       // s_v q_v, then the gradient entries
+    R t[NET_ATOMS][NH];
+};
+
+template <typename R>
+__device__ __forceinline__ void mlp_body(const NetArgs<R> &a, int64_t blk, NetSmem<R> &sm) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int64_t i0 = blk * NET_ATOMS;
+    for (int k = tid; k < NT_SIZE; k += 128) sm.w[k] = ro(a.wtab + k);
+    for (int k = tid; k < DIM * NET_ATOMS; k += 128) {
+        const int v = k / NET_ATOMS, c = k % NET_ATOMS;
+        const R q = i0 + c < a.n ? a.q[(int64_t)v * a.qs + i0 + c] : R(0);
+        sm.x[v][c] = q * ro(a.wtab + NT_S + v);
     }
+    __syncthreads();
+    const int c0 = 2 * warp, c1 = c0 + 1;   // the warp's atoms
+    R E0 = R(0), E1 = R(0);
+    if (lane < NH) {
+        R z0 = -sm.w[NT_B0 + lane], z1 = z0;
+        const R *w = sm.w + lane * NET_LD;
+#pragma unroll 11
+        for (int v = 0; v < DIM; ++v) {
+            z0 += w[v] * sm.x[v][c0];
+            z1 += w[v] * sm.x[v][c1];
+        }
+        const R t0 = tanh(z0), t1 = tanh(z1), w1 = sm.w[NT_W1 + lane];
+        E0 = w1 * t0;
+        E1 = w1 * t1;
+        sm.t[c0][lane] = w1 * (R(1) - t0 * t0);
+        sm.t[c1][lane] = w1 * (R(1) - t1 * t1);
+    }
+    // both atoms' sums over the units: the lower half of the warp takes the first atom's
+    R E = (lane < 16 ? E0 : E1) + __shfl_xor_sync(0xffffffffu, lane < 16 ? E1 : E0, 16);
 #pragma unroll
-    for (int v = 0; v < DIM; ++v) {
+    for (int o = 8; o > 0; o >>= 1) E += __shfl_xor_sync(0xffffffffu, E, o);
+    const int64_t ie = i0 + c0 + (lane >> 4);
+    if ((lane & 15) == 0 && ie < a.n) a.ei[ie] = E - sm.w[NT_B1];
+    __syncwarp();   // this warp's descriptors are read, its t's written
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {   // 2 x 64 gradient entries
+        const int v = (r & 1) * 32 + lane, c = c0 + (r >> 1);
         R s = R(0);
-#pragma unroll
-        for (int h = 0; h < NH; ++h) s += t[h] * P.w0[h][v];
-        fp[(int64_t)v * n + i] = s * P.scal[v];
+#pragma unroll 10
+        for (int h = 0; h < NH; ++h) s += sm.t[c][h] * sm.w[h * NET_LD + v];
+        sm.x[v][c] = s * sm.w[NT_S + v];
     }
-    ei[i] = E;
+    {   // the last 2 x 2: eight lanes each
+        const int v = 64 + (lane >> 3 & 1), c = c0 + (lane >> 4);
+        R s = R(0);
+        for (int h = lane & 7; h < NH; h += 8) s += sm.t[c][h] * sm.w[h * NET_LD + v];
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if ((lane & 7) == 0) sm.x[v][c] = s * sm.w[NT_S + v];
+    }
+    __syncthreads();
+    for (int k = tid; k < DIM * NET_ATOMS; k += 128) {
+        const int v = k / NET_ATOMS, c = k % NET_ATOMS;
+        if (i0 + c < a.n) a.fp[(int64_t)v * a.n + i0 + c] = sm.x[v][c];
+    }
 }
 
-// over an argument table (sl_batch.h), one 128-thread block per 128 atoms of a slot
+// over an argument table (sl_batch.h)
 template <typename R>
-__global__ void __launch_bounds__(128) k_mlp(const __grid_constant__ NepDev<R> P, const NetArgs<R> *__restrict__ tab,
-                                             SlotMap sm, const __grid_constant__ NetArgs<R> solo) {
-    one_work(tab, sm, solo, [&](const NetArgs<R> &a, int64_t blk, int64_t) {
+__global__ void __launch_bounds__(128) k_mlp(const NetArgs<R> *__restrict__ tab, SlotMap sm,
+                                             const __grid_constant__ NetArgs<R> solo) {
+    __shared__ NetSmem<R> scratch;
+    one_work(tab, sm, solo, [&](const NetArgs<R> &args, int64_t blk, int64_t) {
+        const NetArgs<R> a = args;
         if (a.skip && *a.skip) return;
-        const int64_t i = blk * 128 + threadIdx.x;
-        if (i < a.n) mlp_atom(P, a.q, a.fp, a.ei, a.n, a.qs, i);
+        mlp_body(a, blk, scratch);
     });
+}
+
+// the FP64 network's weight table, from the system's model; 0 on success
+int make_net_table(Sys &s) {
+    if (s.prec != 0 || s.n == 0) return 0;
+    std::vector<double> t(NT_SIZE, 0.0);
+    for (int h = 0; h < NH; ++h) {
+        for (int v = 0; v < DIM; ++v) t[h * NET_LD + v] = s.pd.w0[h][v];
+        t[NT_B0 + h] = s.pd.b0[h];
+        t[NT_W1 + h] = s.pd.w1[h];
+    }
+    for (int v = 0; v < DIM; ++v) t[NT_S + v] = s.pd.scal[v];
+    t[NT_B1] = s.pd.b1;
+    if (!s.mlp_img && cudaMalloc(&s.mlp_img, sizeof(double) * NT_SIZE) != cudaSuccess) {
+        s.mlp_img = nullptr;
+        return -1;
+    }
+    if (cudaMemcpyAsync(s.mlp_img, t.data(), sizeof(double) * NT_SIZE, cudaMemcpyHostToDevice, s.stream) != cudaSuccess)
+        return -1;
+    return cudaStreamSynchronize(s.stream) == cudaSuccess ? 0 : -1;
 }
 
 // ---- argument tables (sl_batch.h): the FP64 network over NetArgs, the mixed one
@@ -89,7 +150,7 @@ void fused_put_net(Sys &s, int r, int kind, const FusedTables &t, unsigned char 
     if (s.prec == 0) {
         NetArgs<double> a;
         a.q = (const double *)s.q; a.fp = (double *)s.fp; a.ei = (double *)s.ei; a.n = s.n; a.qs = s.qs;
-        a.skip = skip;
+        a.skip = skip; a.wtab = (const double *)s.mlp_img;
         reinterpret_cast<NetArgs<double> *>(img + t.o_net)[r] = a;
     } else {
         MlpArgs a;
@@ -97,11 +158,13 @@ void fused_put_net(Sys &s, int r, int kind, const FusedTables &t, unsigned char 
         a.skip = skip; a.wimg = s.mlp_img;
         reinterpret_cast<MlpArgs *>(img + t.o_net)[r] = a;
     }
-    blocks[FK_NET] = (s.n + 127) / 128;   // atoms of 128-thread blocks, or 128-atom tensor-core tiles
+    const int per = s.prec == 0 ? NET_ATOMS : 128;   // atoms of a block, or of a tensor-core tile
+    blocks[FK_NET] = (s.n + per - 1) / per;
 }
 
-void launch_net_t_fp64(const FusedTables &t, const NepDev<double> &P, const Launch &L, cudaStream_t st) {
-    k_mlp<double><<<L.grid, 128, 0, st>>>(P, L.solo ? nullptr : t.at<NetArgs<double>>(t.o_net), L.slots(),
+static_assert(NET_ATOMS == CRAD_WIDE_ATOMS, "one atoms-per-block class in a batch (sl_batch.cu)");
+void launch_net_t_fp64(const FusedTables &t, const Launch &L, cudaStream_t st) {
+    k_mlp<double><<<L.grid, 128, 0, st>>>(L.solo ? nullptr : t.at<NetArgs<double>>(t.o_net), L.slots(),
                                           solo_args<NetArgs<double>>(L));
 }
 
