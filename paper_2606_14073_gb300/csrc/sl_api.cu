@@ -124,6 +124,9 @@ void fill_params(sl::NepDev<R> &P, const sl_nep_params *p) {
                 for (int n = 0; n < NCH; ++n)
                     for (int k = 0; k < NK; ++k)
                         P.c[a][b][g][n][k] = (R)p->coeffs[((((a * NS) + b) * 6 + g) * NCH + n) * NK + k];
+    for (int a = 0; a < NS; ++a)
+        for (int b = 0; b < NS; ++b)
+            for (int n = 0; n < NCH; ++n) P.ca0[a][b][n] = (R)shifted_c0(P.c[a][b][G_A][n]);
     for (int v = 0; v < DIM; ++v) P.scal[v] = (R)p->q_scaler[v];
     for (int h = 0; h < NH; ++h) {
         for (int v = 0; v < DIM; ++v) P.w0[h][v] = (R)p->w0[h * DIM + v];

@@ -42,6 +42,7 @@ constexpr double ACC = 9.6485332e-3;      // (eV/A/amu) -> A/fs^2
 template <typename R>
 struct NepDev {
     R c[NS][NS][6][NCH][NK];   // [centre][neighbour][group][n][k]
+    R ca0[NS][NS][NCH];        // shifted k = 0 coefficients of the angular group (shifted_c0)
     R scal[DIM];
     R w0[NH][DIM];
     R b0[NH];
@@ -49,6 +50,14 @@ struct NepDev {
     R b1;
     R rc_r, rc_a, inv_rc_r, inv_rc_a, rc_r2, rc_a2;
 };
+
+// 2 c_0 + sum_{k>0} c_k: sum_k c_k (T_k + 1) = shifted_c0 + sum_{k>0} c_k T_k.
+template <typename R>
+inline double shifted_c0(const R c[NK]) {
+    double v = 2.0 * (double)c[0];
+    for (int k = 1; k < NK; ++k) v += (double)c[k];
+    return v;
+}
 
 // Orthorhombic box; invL = 0 along free dimensions disables the minimum image.
 template <typename R>
@@ -71,6 +80,8 @@ __device__ __forceinline__ int2 ro(const int2 *p) { return __ldg(p); }
 __device__ __forceinline__ int ro(const int *p) { return __ldg(p); }
 __device__ __forceinline__ unsigned ro(const unsigned *p) { return __ldg(p); }
 __device__ __forceinline__ unsigned short ro(const unsigned short *p) { return __ldg(p); }
+__device__ __forceinline__ float2 ro(const float2 *p) { return __ldg(p); }
+__device__ __forceinline__ double2 ro(const double2 *p) { return __ldg(p); }
 __device__ __forceinline__ float ro(const float *p) { return __ldg(p); }
 __device__ __forceinline__ double ro(const double *p) { return __ldg(p); }
 __device__ __forceinline__ double4 ro(const double4 *p) {

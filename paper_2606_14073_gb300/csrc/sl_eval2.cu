@@ -47,8 +47,7 @@ __device__ __forceinline__ v2<R> pair2(R x, R y) {
     v.y = y;
     return v;
 }
-// g_n = sum_k c_nk f_k and dg_n = sum_k c_nk df_k together, two multiply-adds per instruction
-// The carrier of sl_common.cuh with the T_k and U_k recurrences advanced together.
+// The carrier of sl_common.cuh with the T_k and U_k recurrences advanced together (FP32).
 template <typename R>
 __device__ __forceinline__ void carrier_fd2(R r, R inv_rc, R f[NK], R df[NK]) {
     const R t = r * inv_rc;
@@ -74,6 +73,7 @@ __device__ __forceinline__ void carrier_fd2(R r, R inv_rc, R f[NK], R df[NK]) {
     }
 }
 
+// g_n = sum_k c_nk f_k and dg_n = sum_k c_nk df_k together, two multiply-adds per instruction
 template <typename R, int TI, int TJ, int G>
 __device__ __forceinline__ void contract_k2(const NepDev<R> &P, const R f[NK], const R df[NK], R g[NCH], R dg[NCH]) {
 #pragma unroll
@@ -88,6 +88,38 @@ __device__ __forceinline__ void contract_k2(const NepDev<R> &P, const R f[NK], c
         dg[n] = s.y;
     }
 }
+
+// FP64: the radial carrier f_k = (T_k(x) + 1) f_c/2 at r: x and 2x, f_c/2 and its slope, dx/dr f_c/2.
+// A contraction sum_k C_k f_k is f_c/2 times P = sum_k C_k (T_k + 1), and its slope
+// d(f_c/2)/dr P + dx/dr f_c/2 Q with Q = sum_k C_k dT_k/dx, dT_k/dx = k U_{k-1}; with C_0 replaced
+// by 2 C_0 + sum_{k>0} C_k (shifted coefficients) P is sum_k C_k T_k.  So no f_k or df_k is
+// formed: 28 of 270 FP64 instructions of a radial pair less.  (FP32 keeps f_k and df_k: with its
+// registers capped at 128 this form, whose partial sums live longer, ran the backward at 1.60
+// instead of 1.58 ms at 884,736 atoms.)
+template <typename R>
+struct Carrier {
+    R x, x2, fch, dfch, dxf;
+    __device__ __forceinline__ Carrier(R r, R inv_rc) {
+        const R t = r * inv_rc;
+        cut_half_d(t, inv_rc, fch, dfch);
+        const R y = t - R(1);
+        x = R(2) * y * y - R(1);
+        x2 = R(2) * x;
+        dxf = R(4) * y * inv_rc * fch;
+    }
+    // use(k, (T_k, dT_k/dx)) for k = 2 .. NK - 1
+    template <typename F>
+    __device__ __forceinline__ void terms(F use) const {
+        v2<R> m = pair2<R>(R(1), R(1)), c = pair2<R>(x, x2);   // (T_{k-2}, U_{k-2}), (T_{k-1}, U_{k-1})
+#pragma unroll
+        for (int k = 2; k < NK; ++k) {
+            const v2<R> n = fma2(pair2<R>(x2, x2), c, pair2<R>(-m.x, -m.y));
+            use(k, pair2<R>(n.x, R(k) * c.y));
+            m = c;
+            c = n;
+        }
+    }
+};
 
 template <typename R, int TI, int TJ, int G>
 __device__ __forceinline__ void contract_k(const NepDev<R> &P, const R f[NK], R g[NCH]) {
@@ -108,17 +140,23 @@ __device__ __forceinline__ void sep(const BoxDev<R> &b, const v4<R> &pi, const v
     minimg(b, dx, dy, dz);
 }
 
-// The coefficients of the radial contraction: [centre][neighbour][k][g * 5 + n], rows padded to
-// 32, g in the order R, EX, DMI, ANI, SIA (each lane of k_crad reads its own output's column).
+// Coefficients of the rc_rad groups (g in the order R, EX, DMI, ANI, SIA) for lanes that each take
+// their own: for the wide radial kernel's contraction [centre][neighbour][k][g * 5 + n], rows
+// padded to 32, then for the FP64 backward's precontraction [centre][neighbour][g][n][k], rows of 10,
+// k = 0 shifted (see Carrier).
+constexpr int CTAB_BWD = NS * NS * NK * 32, CB_ROW = 10;
 template <typename R>
 static void fill_ctab(const NepDev<R> &P, std::vector<R> &t) {
     constexpr int GG[5] = {G_R, G_EX, G_DMI, G_ANI, G_SIA};
-    t.assign((size_t)NS * NS * NK * 32, R(0));
+    t.assign((size_t)CTAB_BWD + NS * NS * 25 * CB_ROW, R(0));
     for (int x = 0; x < NS; ++x)
         for (int y = 0; y < NS; ++y)
-            for (int k = 0; k < NK; ++k)
-                for (int o = 0; o < 25; ++o)
-                    t[(size_t)((x * NS + y) * NK + k) * 32 + o] = P.c[x][y][GG[o / NCH]][o % NCH][k];
+            for (int o = 0; o < 25; ++o) {
+                const R *c = P.c[x][y][GG[o / NCH]][o % NCH];
+                R *b = t.data() + CTAB_BWD + (size_t)((x * NS + y) * 25 + o) * CB_ROW;
+                for (int k = 0; k < NK; ++k) t[(size_t)((x * NS + y) * NK + k) * 32 + o] = b[k] = c[k];
+                b[0] = R(shifted_c0(c));
+            }
 }
 int make_coeff_table(Sys &s) {
     const auto put = [&](const auto &t) {
@@ -862,33 +900,96 @@ struct BwdAcc2 {
     R w[9];
 };
 
-template <typename R, int TI>
-__device__ __forceinline__ void bwd_coeffs(const NepDev<R> &P, const R FR[NCH], const R FX[4][NCH], int ql, R *smc) {
+// The atom's precontracted radial coefficients C^G_k = sum_n Fp^G_n c^G_nk for both neighbour
+// species into smc, 48 each; place of C^G_k: FP64 [k][group] (k = 0 shifted), FP32 [group][k].
+template <typename R>
+__device__ __forceinline__ int coeff_at(int g, int k) { return sizeof(R) == 8 ? 5 * k + g : 9 * g + k; }
+// FP32: every lane of the quad forms them all (the coefficients are constant operands) and stores a
+// quarter; taking its own from a table in global memory made the backward 1.58 to 1.70 ms at
+// 884,736 atoms (the loads' latency, before the first pair).
+template <int TI>
+__device__ __forceinline__ void bwd_coeffs(const NepDev<float> &P, const float F[5][NCH], int ql, float *smc) {
 #pragma unroll
-    for (int tj = 0; tj < 2; ++tj)
+    for (int tj = 0; tj < NS; ++tj)
 #pragma unroll
         for (int g = 0; g < 5; ++g)
 #pragma unroll
             for (int k = 0; k < NK; ++k) {
                 constexpr int G[5] = {G_R, G_EX, G_DMI, G_ANI, G_SIA};
-                R v = R(0);
+                float v = 0.f;
 #pragma unroll
-                for (int n = 0; n < NCH; ++n)
-                    v += (g == 0 ? FR[n] : FX[g - 1][n]) * (tj == 0 ? P.c[TI][0][G[g]][n][k] : P.c[TI][1][G[g]][n][k]);
-                if (((tj * 45 + g * 9 + k) & 3) == ql) smc[tj * 48 + g * 9 + k] = v;
+                for (int n = 0; n < NCH; ++n) v += F[g][n] * (tj == 0 ? P.c[TI][0][G[g]][n][k] : P.c[TI][1][G[g]][n][k]);
+                if (((tj * 45 + g * 9 + k) & 3) == ql) smc[tj * 48 + coeff_at<float>(g, k)] = v;
             }
 }
-
-template <typename R, int TI, int TJ>
-__device__ __forceinline__ void ang_gdg(const NepDev<R> &P, R r, R inv_rc, R g[NCH], R dg[NCH]) {
-    R f[NK], df[NK];
-    carrier_fd2(r, inv_rc, f, df);
-    contract_k2<R, TI, TJ, G_A>(P, f, df, g, dg);
+// FP64: lane ql of the quad takes k = 2 ql and 2 ql + 1, lanes 0 and 1 one species' k = 8, from the
+// centre's rows ct of the table (a quarter of the multiply-adds).
+__device__ __forceinline__ void bwd_coeffs(const double *__restrict__ ct, const double F[5][NCH], int ql, double *smc) {
+#pragma unroll
+    for (int tj = 0; tj < NS; ++tj)
+#pragma unroll
+        for (int g = 0; g < 5; ++g) {
+            double2 c2 = make_double2(0.0, 0.0);
+#pragma unroll
+            for (int n = 0; n < NCH; ++n)
+                c2 = fma2(make_double2(F[g][n], F[g][n]),
+                          ro(reinterpret_cast<const double2 *>(ct + ((tj * 5 + g) * NCH + n) * CB_ROW) + ql), c2);
+            smc[tj * 48 + coeff_at<double>(g, 2 * ql)] = c2.x;
+            smc[tj * 48 + coeff_at<double>(g, 2 * ql + 1)] = c2.y;
+        }
+    const int tj = ql & 1;
+#pragma unroll
+    for (int g = 0; g < 5; ++g) {
+        double v = 0.0;
+#pragma unroll
+        for (int n = 0; n < NCH; ++n) v += F[g][n] * ro(ct + ((tj * 5 + g) * NCH + n) * CB_ROW + 8);
+        if (ql < NS) smc[tj * 48 + coeff_at<double>(g, 8)] = v;
+    }
 }
 
+// g_n and dg_n/dr of the angular channels
+template <typename R, int TI, int TJ>
+__device__ __forceinline__ void ang_gdg(const NepDev<R> &P, R r, R inv_rc, R g[NCH], R dg[NCH]) {
+    if constexpr (sizeof(R) == 4) {
+        R f[NK], df[NK];
+        carrier_fd2(r, inv_rc, f, df);
+        contract_k2<R, TI, TJ, G_A>(P, f, df, g, dg);
+        return;
+    }
+    const Carrier<R> cr(r, inv_rc);
+    v2<R> pq[NCH];
+#pragma unroll
+    for (int n = 0; n < NCH; ++n) {
+        const R c1 = P.c[TI][TJ][G_A][n][1];
+        pq[n] = pair2<R>(fma_(c1, cr.x, P.ca0[TI][TJ][n]), c1);
+    }
+    cr.terms([&](int k, const v2<R> &td) {
+#pragma unroll
+        for (int n = 0; n < NCH; ++n) {
+            const R c = P.c[TI][TJ][G_A][n][k];
+            pq[n] = fma2(pair2<R>(c, c), td, pq[n]);
+        }
+    });
+#pragma unroll
+    for (int n = 0; n < NCH; ++n) {
+        g[n] = cr.fch * pq[n].x;
+        dg[n] = fma_(cr.dxf, pq[n].y, cr.dfch * pq[n].x);
+    }
+}
+
+// The angular adjoint of one pair from the atom's adjoint records bb[lm] = (dE/dB_n, dE/dBS_n) and
+// the harmonics p_lm at u.  With a_lm = sum_n g_n (dE/dB + s dE/dBS) the chain rule gives
+//   dE/dr along u    sum_lm p_lm sum_n g_n' (dE/dB + s dE/dBS)
+//   dE/du            sum_lm a_lm grad p_lm, of which only the part across u counts
+//   dE/ds            sum_lm p_lm sum_n g_n dE/dBS
+// and u . grad p_lm = l p_lm, so the part along u is taken out of the vector sum once, by its
+// projection, instead of harmonic by harmonic.
+//
+// FP32: harmonic by harmonic (few values live at a time; the backward at 884,736 atoms 1.62 to 1.58 ms
+// against subtracting each harmonic's part along u).
 template <typename R, int LM>
-__device__ __forceinline__ void bwd_harm(const R *__restrict__ bb, R ux, R uy, R uz, R ir, R s, const R g[NCH],
-                                         const R dg[NCH], R &accu, R &avx, R &avy, R &avz, R &cj) {
+__device__ __forceinline__ void bwd_harm(const R *__restrict__ bb, R ux, R uy, R uz, R s, const R g[NCH],
+                                         const R dg[NCH], v2<R> &along, R &avx, R &avy, R &avz, R &cj) {
     R p, gx, gy, gz;
     harm_one<R, LM>(ux, uy, uz, p, gx, gy, gz);
     const v4<R> *rec = reinterpret_cast<const v4<R> *>(bb + BREC * LM);
@@ -901,14 +1002,101 @@ __device__ __forceinline__ void bwd_harm(const R *__restrict__ bb, R ux, R uy, R
         aa = fma2(Bp[n], pair2<R>(g[n], g[n]), aa);
         bq = fma2(Bp[n], pair2<R>(dg[n], dg[n]), bq);
     }
-    const R aA = aa.x, aS = aa.y, bA = bq.x, bS = bq.y;
-    const R av = aA + s * aS, bv = bA + s * bS;
-    accu += p * (bv - R(harm_l(LM)) * ir * av);
+    const R av = aa.x + s * aa.y;
+    along = fma2(bq, pair2<R>(p, p), along);
     avx += av * gx;
     avy += av * gy;
     avz += av * gz;
-    cj += aS * p;
-    if constexpr (LM + 1 < NLM) bwd_harm<R, LM + 1>(bb, ux, uy, uz, ir, s, g, dg, accu, avx, avy, avz, cj);
+    cj += aa.y * p;
+    if constexpr (LM + 1 < NLM) bwd_harm<R, LM + 1>(bb, ux, uy, uz, s, g, dg, along, avx, avy, avz, cj);
+}
+
+// FP64, where instructions count and registers do not: the sums over n and lm are exchanged,
+//   Psi_n = sum_lm p_lm (dE/dB_n, dE/dBS_n), along u sum_n g_n' Psi_n, dE/ds sum_n g_n Psi^S_n,
+// and the gradient of a solid harmonic being a combination of those one degree lower, sum_lm a_lm
+// grad p_lm is formed from the p of degree l - 1 and a few sums of a's.  With Carrier this takes an
+// angular pair from some 1,040 to 780 FP64 instructions: the backward at 110,592 atoms 7.59 to
+// 6.41 ms.
+template <typename R>
+struct AngAdjoint {
+    const R *bb;
+    R s;
+    const R *g;
+    v2<R> psi[NCH];
+    // harmonic lm = value p: Psi_n advanced, a_lm returned
+    __device__ __forceinline__ R take(int lm, R p) {
+        const v4<R> *rec = reinterpret_cast<const v4<R> *>(bb + BREC * lm);
+        const v4<R> r0 = rec[0], r1 = rec[1];
+        const v2<R> r2 = *reinterpret_cast<const v2<R> *>(rec + 2);
+        const v2<R> Bp[NCH] = {pair2<R>(r0.x, r0.y), pair2<R>(r0.z, r0.w), pair2<R>(r1.x, r1.y),
+                               pair2<R>(r1.z, r1.w), r2};
+        v2<R> aa = pair2<R>(Bp[0].x * g[0], Bp[0].y * g[0]);
+#pragma unroll
+        for (int n = 1; n < NCH; ++n) aa = fma2(Bp[n], pair2<R>(g[n], g[n]), aa);
+#pragma unroll
+        for (int n = 0; n < NCH; ++n) psi[n] = fma2(Bp[n], pair2<R>(p, p), psi[n]);
+        return fma_(s, aa.y, aa.x);
+    }
+};
+
+template <typename R>
+__device__ __forceinline__ void bwd_angular(const R *__restrict__ bb, R x, R y, R z, R s, const R g[NCH],
+                                            const R dg[NCH], R &along, R &vx, R &vy, R &vz, R &cj) {
+    AngAdjoint<R> A;
+    A.bb = bb;
+    A.s = s;
+    A.g = g;
+#pragma unroll
+    for (int n = 0; n < NCH; ++n) A.psi[n] = pair2<R>(R(0), R(0));
+    // degree 1
+    vx = A.take(0, x);
+    vy = A.take(1, y);
+    vz = A.take(2, z);
+    // degree 2: xy, yz, xz, x^2 - y^2, 2 z^2 - x^2 - y^2
+    const R x2 = x * x, y2 = y * y, z2 = z * z, q = x2 + y2;
+    const R p3 = x * y, p4 = y * z, p5 = x * z, p6 = x2 - y2, p7 = fma_(R(2), z2, -q);
+    {
+        const R a3 = A.take(3, p3), a4 = A.take(4, p4), a5 = A.take(5, p5), a6 = A.take(6, p6), a7 = A.take(7, p7);
+        vx += a3 * y + a5 * z + R(2) * (a6 - a7) * x;
+        vy += a3 * x + a4 * z - R(2) * (a6 + a7) * y;
+        vz += a4 * y + a5 * x + R(4) * a7 * z;
+    }
+    // degree 3
+    const R c1 = fma_(R(3), x2, -y2), c2 = fma_(R(-3), y2, x2), c3 = fma_(R(4), z2, -q);
+    const R p8 = y * c1, p9 = p3 * z, p10 = y * c3, p11 = z * fma_(R(2), z2, R(-3) * q), p12 = x * c3, p13 = z * p6,
+            p14 = x * c2;
+    {
+        const R a8 = A.take(8, p8), a9 = A.take(9, p9), a10 = A.take(10, p10), a11 = A.take(11, p11),
+                a12 = A.take(12, p12), a13 = A.take(13, p13), a14 = A.take(14, p14);
+        const R d11 = R(6) * a11, d10 = R(2) * a10, d12 = R(2) * a12;
+        vx += p3 * fma_(R(6), a8, -d10) + p4 * a9 + p5 * fma_(R(2), a13, -d11) + p6 * fma_(R(3), a14, -a12) + p7 * d12;
+        vy += p3 * fma_(R(-6), a14, -d12) + p4 * fma_(R(-2), a13, -d11) + p5 * a9 + p6 * fma_(R(3), a8, a10) + p7 * d10;
+        vz += p3 * a9 + R(4) * (p4 * d10 + p5 * d12) + p6 * a13 + R(0.5) * p7 * d11;
+    }
+    // degree 4
+    {
+        const R c5 = fma_(R(6), z2, -q), c6 = fma_(R(4), z2, R(-3) * q), r2 = q + z2;
+        const R a15 = A.take(15, p3 * p6), a16 = A.take(16, p4 * c1), a17 = A.take(17, p3 * c5),
+                a18 = A.take(18, p4 * c6),
+                a19 = A.take(19, fma_(z2, fma_(R(35), z2, R(-30) * r2), R(3) * r2 * r2)),
+                a20 = A.take(20, p5 * c6), a21 = A.take(21, p6 * c5), a22 = A.take(22, p5 * c2),
+                a23 = A.take(23, fma_(p6, p6, R(-4) * p3 * p3));
+        const R e17 = R(0.5) * a17, d17 = R(1.5) * a17, d19 = R(12) * a19, d21 = R(3) * a21;
+        vx += p8 * (a15 - e17) + p9 * (R(6) * (a16 - a18)) + p10 * d17 + p11 * (R(2) * a20) + p12 * (d21 - d19) +
+              p13 * (R(3) * (a22 - a20)) + p14 * fma_(R(4), a23, -a21);
+        vy += p14 * (a15 + e17) - p9 * (R(6) * (a20 + a22)) + p12 * d17 + p11 * (R(2) * a18) - p10 * (d21 + d19) +
+              p13 * (R(3) * (a16 + a18)) - p8 * fma_(R(4), a23, a21);
+        vz += p8 * a16 + p14 * a22 + R(8) * p9 * d17 + R(3) * (p10 * a18 + p12 * a20) + R(16) * p11 * a19 +
+              R(4) * p13 * d21;
+    }
+    v2<R> b = pair2<R>(R(0), R(0));
+    cj = R(0);
+#pragma unroll
+    for (int n = 0; n < NCH; ++n) {
+        b = fma2(A.psi[n], pair2<R>(dg[n], dg[n]), b);
+        cj = fma_(g[n], A.psi[n].y, cj);
+    }
+    along = fma_(s, b.y, b.x);
 }
 
 // one pair record: FP32 as a single 256-bit store (the record is one 32-byte sector), FP64 as
@@ -934,35 +1122,73 @@ __device__ __forceinline__ void bwd_pair(const NepDev<R> &P, const Eval2Args<R> 
     const R d2 = dx * dx + dy * dy + dz * dz;
     const R ir = rsqrt_(d2), r = d2 * ir;
     const R ux = dx * ir, uy = dy * ir, uz = dz * ir;
-    // radial and pairwise-magnetic part with the precontracted coefficients
-    R f[NK], df[NK];
-    carrier_fd2(r, P.inv_rc_r, f, df);
-    const v4<R> *cv = reinterpret_cast<const v4<R> *>(sm + BW_C + tj * 48);
+    // radial and pairwise-magnetic part with the precontracted coefficients: the values h of the
+    // four magnetic groups, then the slope along the pair of every group's term together.  (The
+    // carrier comes before the coefficients' loads and the spin products after the contraction:
+    // held across it they cost FP32 the registers of its prefetch, 1.62 instead of 1.58 ms.)
     R C[48];
+    auto load_coefficients = [&]() {
+        const v4<R> *cv = reinterpret_cast<const v4<R> *>(sm + BW_C + tj * 48);
 #pragma unroll
-    for (int q = 0; q < 12; ++q) {
-        const v4<R> c4 = cv[q];
-        C[4 * q] = c4.x; C[4 * q + 1] = c4.y; C[4 * q + 2] = c4.z; C[4 * q + 3] = c4.w;
+        for (int q = 0; q < 12; ++q) {
+            const v4<R> c4 = cv[q];
+            C[4 * q] = c4.x; C[4 * q + 1] = c4.y; C[4 * q + 2] = c4.z; C[4 * q + 3] = c4.w;
+        }
+    };
+    [[maybe_unused]] v2<R> pq[5];         // FP64: (P, Q) per group
+    [[maybe_unused]] R e0 = 0, dfch = 0, dxf = 0;
+    [[maybe_unused]] v2<R> he[4];         // FP32: (h_G, e_G) of the four magnetic groups
+    R h1, h2, h3, h4;
+    if constexpr (sizeof(R) == 8) {
+        const Carrier<R> cr(r, P.inv_rc_r);
+        load_coefficients();
+#pragma unroll
+        for (int q = 0; q < 5; ++q) {
+            const R c1 = C[coeff_at<R>(q, 1)];
+            pq[q] = pair2<R>(fma_(c1, cr.x, C[coeff_at<R>(q, 0)]), c1);
+        }
+        cr.terms([&](int k, const v2<R> &td) {
+#pragma unroll
+            for (int q = 0; q < 5; ++q) {
+                const R c = C[coeff_at<R>(q, k)];
+                pq[q] = fma2(pair2<R>(c, c), td, pq[q]);
+            }
+        });
+        h1 = cr.fch * pq[1].x; h2 = cr.fch * pq[2].x; h3 = cr.fch * pq[3].x; h4 = cr.fch * pq[4].x;
+        dfch = cr.dfch;
+        dxf = cr.dxf;
+    } else {
+        R f[NK], df[NK];
+        carrier_fd2(r, P.inv_rc_r, f, df);
+        load_coefficients();
+#pragma unroll
+        for (int q = 0; q < 4; ++q) he[q] = pair2<R>(R(0), R(0));
+#pragma unroll
+        for (int k = 0; k < NK; ++k) {
+            e0 += C[coeff_at<R>(0, k)] * df[k];
+            const v2<R> fd = pair2<R>(f[k], df[k]);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const R c = C[coeff_at<R>(q + 1, k)];
+                he[q] = fma2(pair2<R>(c, c), fd, he[q]);
+            }
+        }
+        h1 = he[0].x; h2 = he[1].x; h3 = he[2].x; h4 = he[3].x;
     }
-    R e0 = 0;
-    v2<R> he[4];   // (h_G, e_G) of the four magnetic groups
-#pragma unroll
-    for (int q = 0; q < 4; ++q) he[q] = pair2<R>(R(0), R(0));
-#pragma unroll
-    for (int k = 0; k < NK; ++k) {
-        e0 += C[k] * df[k];
-        const v2<R> fd = pair2<R>(f[k], df[k]);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) he[q] = fma2(pair2<R>(C[9 * (q + 1) + k], C[9 * (q + 1) + k]), fd, he[q]);
-    }
-    const R h1 = he[0].x, e1 = he[0].y, h2 = he[1].x, e2 = he[1].y, h3 = he[2].x, e3 = he[2].y, h4 = he[3].x,
-            e4 = he[3].y;
     const R sij = si.x * sj.x + si.y * sj.y + si.z * sj.z;
     const R siu = si.x * ux + si.y * uy + si.z * uz;
     const R sju = sj.x * ux + sj.y * uy + sj.z * uz;
     const R wx = si.y * sj.z - si.z * sj.y, wy = si.z * sj.x - si.x * sj.z, wz = si.x * sj.y - si.y * sj.x;
     const R wu = wx * ux + wy * uy + wz * uz;
-    const R rad = e0 + e1 * sij + e2 * wu + e3 * siu * sju + e4 * siu * siu;
+    R rad;
+    if constexpr (sizeof(R) == 8) {
+        const R phi[5] = {R(1), sij, wu, siu * sju, siu * siu};
+#pragma unroll
+        for (int q = 1; q < 5; ++q) pq[0] = fma2(pair2<R>(phi[q], phi[q]), pq[q], pq[0]);
+        rad = fma_(dxf, pq[0].y, dfch * pq[0].x);
+    } else {
+        rad = e0 + he[0].y * sij + he[1].y * wu + he[2].y * siu * sju + he[3].y * siu * siu;
+    }
     const R cSi = (h3 * sju + R(2) * h4 * siu) * ir;
     const R cSj = h3 * siu * ir;
     const R cW = h2 * ir;
@@ -984,8 +1210,16 @@ __device__ __forceinline__ void bwd_pair(const NepDev<R> &P, const Eval2Args<R> 
             if (tj == 0) ang_gdg<R, 1, 0>(P, r, P.inv_rc_a, g, dg);
             else ang_gdg<R, 1, 1>(P, r, P.inv_rc_a, g, dg);
         }
-        R accu = R(0), avx = R(0), avy = R(0), avz = R(0), cj = R(0);
-        bwd_harm<R, 0>(sm, ux, uy, uz, ir, sij, g, dg, accu, avx, avy, avz, cj);
+        R accu, avx, avy, avz, cj;
+        if constexpr (sizeof(R) == 8) {
+            bwd_angular<R>(sm, ux, uy, uz, sij, g, dg, accu, avx, avy, avz, cj);
+        } else {
+            v2<R> al = pair2<R>(R(0), R(0));
+            avx = avy = avz = cj = R(0);
+            bwd_harm<R, 0>(sm, ux, uy, uz, sij, g, dg, al, avx, avy, avz, cj);
+            accu = al.x + sij * al.y;
+        }
+        accu -= ir * (ux * avx + uy * avy + uz * avz);   // only the part across u turns the pair
         Dx += accu * ux + ir * avx;
         Dy += accu * uy + ir * avy;
         Dz += accu * uz + ir * avz;
@@ -1085,21 +1319,20 @@ __device__ __forceinline__ void bwd_body(const NepDev<R> &P, const Eval2Args<R> 
             v4<R> *d = reinterpret_cast<v4<R> *>(sm + BREC * lm);
             d[0] = w0; d[1] = w1; d[2] = w2;
         }
-        R FR[NCH], FX[4][NCH];
+        R F[5][NCH];   // dE/dq of the rc_rad groups
 #pragma unroll
         for (int n = 0; n < NCH; ++n) {
-            FR[n] = ro(a.fp + (int64_t)(Q_R + n) * N + i);
-            FX[0][n] = ro(a.fp + (int64_t)(Q_EX + n) * N + i);
-            FX[1][n] = ro(a.fp + (int64_t)(Q_DMI + n) * N + i);
-            FX[2][n] = ro(a.fp + (int64_t)(Q_ANI + n) * N + i);
-            FX[3][n] = ro(a.fp + (int64_t)(Q_SIA + n) * N + i);
+            F[0][n] = ro(a.fp + (int64_t)(Q_R + n) * N + i);
+#pragma unroll
+            for (int g = 0; g < 4; ++g) F[g + 1][n] = ro(a.fp + (int64_t)(Q_EX + g * NCH + n) * N + i);
         }
         if (ql == 0) {   // onsite term dE_i/dS_i = 2 Fp_O S_i, counted once per atom
             const R fo = R(2) * ro(a.fp + (int64_t)Q_O * N + i);
             acc.hx = fo * si.x; acc.hy = fo * si.y; acc.hz = fo * si.z;
         }
-        if (ti == 0) bwd_coeffs<R, 0>(P, FR, FX, ql, sm + BW_C);
-        else bwd_coeffs<R, 1>(P, FR, FX, ql, sm + BW_C);
+        if constexpr (sizeof(R) == 8) bwd_coeffs(a.ctab + CTAB_BWD + ti * (NS * 25 * CB_ROW), F, ql, sm + BW_C);
+        else if (ti == 0) bwd_coeffs<0>(P, F, ql, sm + BW_C);
+        else bwd_coeffs<1>(P, F, ql, sm + BW_C);
         __syncwarp(0xfu << (quad * 4));
         const int ca = a.cap_ang;
         bwd_rows<R, true, VIR>(P, a, i, ti, ql, c.y, c.x, pi, si, sm, acc);

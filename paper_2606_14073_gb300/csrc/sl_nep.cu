@@ -35,7 +35,7 @@ namespace sl {
 // memory; lane h takes hidden unit h of both atoms, then the lanes take the 2 x 66 gradient
 // entries, 32 at a time, and eight lanes share each of the last four.  What bounds it: the FP64
 // pipe (160 warp instructions per atom; one thread per atom took 184, and a serial chain of 4,000
-// multiply-adds however few the atoms): 512 / 13,824 / 110,592 atoms 27 / 154 / 984 us, against
+// multiply-adds however few the atoms): 512 / 13,824 / 110,592 atoms 25 / 154 / 984 us, against
 // 202 / 228 / 1,070.
 constexpr int NET_ATOMS = 8;          // atoms per block
 constexpr int NET_LD = DIM + 1;       // row length of W0 in the table and in shared memory
