@@ -51,6 +51,7 @@ static int item_class(int k, int prec) {
         case FK_CRAD: return prec == 0 ? -1 : IC_ATOM;   // FP64: the wide kernel only
         case FK_CRADW: return IC_OCT;
         case FK_ANG: case FK_BWD: return IC_QUAD;
+        case FK_ANGW: case FK_BWDW: return IC_WARP;
         case FK_NET: return prec == 0 ? IC_OCT : -1;
         default: return -1;
     }
@@ -78,7 +79,7 @@ void FusedBatch::enqueue(cudaStream_t st) const {
     Launch rb[FK_FINISH - FK_BIN + 1];
     for (int k = FK_BIN; k <= FK_FINISH; ++k) rb[k - FK_BIN] = L(k);
     launch_rebuild_t(t, rb, true, true, st);
-    const Launch ev[5] = {L(FK_CRAD), L(FK_ANG), L(FK_NET), L(FK_BWD), L(FK_CRADW)};
+    const Launch ev[7] = {L(FK_CRAD), L(FK_ANG), L(FK_NET), L(FK_BWD), L(FK_CRADW), L(FK_ANGW), L(FK_BWDW)};
     if (t.prec == 0) launch_eval_t<double>(t, pd, ev, st, nullptr);
     else launch_eval_t<float>(t, pf, ev, st, nullptr);
     launch_second_half_t(t, L(FK_SECOND), true, st);
@@ -205,7 +206,8 @@ bool FusedBatch::same_model(const Sys &s) const {
 static int item_kernel_class(const char *name) {
     struct { const char *id; int cls; } const k[] = {
         {"k_first_half", IC_HALF}, {"k_second_half", IC_HALF}, {"k_crad", IC_ATOM}, {"k_crad_wide", IC_OCT},
-        {"k_mlp", IC_OCT}, {"k_ang_fwd", IC_QUAD}, {"k_bwd", IC_QUAD}};
+        {"k_mlp", IC_OCT}, {"k_ang_fwd", IC_QUAD}, {"k_bwd", IC_QUAD},
+        {"k_ang_wide", IC_WARP}, {"k_bwd_wide", IC_WARP}};
     for (const auto &x : k) {
         const std::string id(x.id);
         const std::string forms[3] = {std::to_string(id.size()) + id + "I", id + "<", id + "("};
@@ -235,9 +237,9 @@ bool FusedBatch::find_item_nodes(cudaGraph_t graph, cudaGraphExec_t exec, int st
         item_nodes.push_back(ItemNode{exec, node, c});
         ++found;
     }
-    // per step: the two halves, the wide radial kernel, the other one (or the FP64 network),
-    // angular, backward
-    return found == (int64_t)steps * 6;
+    // per step: the two halves, the wide radial kernel, the other one (or the FP64 network), the
+    // two angular and the two backward kernels
+    return found == (int64_t)steps * 8;
 }
 
 bool FusedBatch::resize_item_nodes() {
@@ -290,7 +292,7 @@ bool FusedBatch::reserve(int64_t atoms) {
     int64_t c = 1;
     while (c < atoms) c <<= 1;
     const int q = default_quad_block(t.prec);
-    const int64_t per[IC_N] = {256, 128, q / 4, CRAD_WIDE_ATOMS};
+    const int64_t per[IC_N] = {256, 128, q / 4, CRAD_WIDE_ATOMS, q / 32};
     int64_t cap_items[IC_N], total = 0;
     for (int k = 0; k < IC_N; ++k) {
         cap_items[k] = (c + per[k] - 1) / per[k] + t.cap;   // whole blocks, one partial block per slot
@@ -353,7 +355,7 @@ cudaError_t FusedBatch::upload(const int64_t *left, cudaStream_t st) {
     if (dirty || layout_dirty) {
         // block -> slot layout of the one-item-per-block kernels: every occupied slot's blocks in
         // slot order, then no slot (-1) up to the capacity
-        const int kof[IC_N] = {FK_FIRST, FK_CRAD, FK_ANG, FK_CRADW};
+        const int kof[IC_N] = {FK_FIRST, FK_CRAD, FK_ANG, FK_CRADW, FK_ANGW};
         for (int c = 0; c < IC_N; ++c) {
             int *it = h_items + item_off[c];
             int64_t o = 0;
@@ -410,12 +412,13 @@ int solo_refresh(Sys &s) {
         fused_put_net(s, kind, kind, t, img.data(), b[kind]);
     }
     // shape 0: the default threads per block; shape 1: half of them (radial: one or sixteen
-    // threads per atom; angular and backward: four)
+    // threads per atom; angular and backward: four or 32)
     for (int k = 0; k < FK_N; ++k) so.blocks[k][0] = so.blocks[k][1] = b[SK_STEP][k];
     const int q = default_quad_block(s.prec);
     if (crad_is_wide(s)) so.blocks[FK_CRADW][1] = (s.n + CRAD_WIDE_ATOMS / 2 - 1) / (CRAD_WIDE_ATOMS / 2);
     else so.blocks[FK_CRAD][1] = (s.n + 63) / 64;
-    so.blocks[FK_ANG][1] = so.blocks[FK_BWD][1] = (s.n + q / 8 - 1) / (q / 8);
+    if (eval_is_wide(s)) so.blocks[FK_ANGW][1] = so.blocks[FK_BWDW][1] = (s.n + q / 64 - 1) / (q / 64);
+    else so.blocks[FK_ANG][1] = so.blocks[FK_BWD][1] = (s.n + q / 8 - 1) / (q / 8);
     // work maps covering slot `kind` alone
     int64_t *w = reinterpret_cast<int64_t *>(img.data() + t.bytes);
     for (int k = 0; k < FK_N; ++k)
@@ -445,11 +448,11 @@ Launch solo_launch(const Sys &s, int k, int kind) {
         L.block = s.cfg.crad_block;
         L.minb = s.cfg.crad_minb;
         shape = L.block == 128 ? 0 : 1;
-    } else if (k == FK_ANG) {
+    } else if (k == FK_ANG || k == FK_ANGW) {
         L.block = s.cfg.ang_block ? s.cfg.ang_block : q;
         L.minb = s.cfg.ang_minb;
         shape = L.block == q ? 0 : 1;
-    } else if (k == FK_BWD) {
+    } else if (k == FK_BWD || k == FK_BWDW) {
         L.block = s.cfg.bwd_block ? s.cfg.bwd_block : q;
         L.minb = s.cfg.bwd_minb;
         shape = L.block == q ? 0 : 1;
@@ -457,7 +460,8 @@ Launch solo_launch(const Sys &s, int k, int kind) {
     L.m = so.map(k, kind, shape);
     int64_t g = so.blocks[k][shape];
     if (k == FK_NET && s.prec != 0) g = std::min<int64_t>(g, (int64_t)so.sms * s.cfg.mlp_ctas_per_sm);   // persistent
-    L.grid = (unsigned)(k == FK_CRAD || k == FK_CRADW ? g : std::max<int64_t>(g, 1));   // one of the radial kernels only
+    // the radial, angular and backward kernels: one of each kind has blocks
+    L.grid = (unsigned)(k >= FK_CRAD && k <= FK_BWDW && k != FK_NET ? g : std::max<int64_t>(g, 1));
     // the argument block of slot `kind` as the kernel parameter (all but the rebuild group)
     const FusedTables &t = so.t;
     size_t first = 0, second = 0;
@@ -466,7 +470,7 @@ Launch solo_launch(const Sys &s, int k, int kind) {
     switch (k) {
         case FK_FIRST: L.solo = h + t.o_first + kind * first; break;
         case FK_SECOND: L.solo = h + t.o_second + kind * second; break;
-        case FK_CRAD: case FK_CRADW: case FK_ANG: case FK_BWD: L.solo = h + t.o_eval + kind * fused_eval_size(s.prec); break;
+        case FK_CRAD: case FK_CRADW: case FK_ANG: case FK_ANGW: case FK_BWD: case FK_BWDW: L.solo = h + t.o_eval + kind * fused_eval_size(s.prec); break;
         case FK_NET: L.solo = h + t.o_net + kind * fused_net_size(s.prec); break;
         default:   // the rebuild group: a conditional one returns at once on the system's flag
             if (kind != SK_FULL) L.quick = s.rebuild;

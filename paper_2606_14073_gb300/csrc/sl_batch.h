@@ -23,15 +23,16 @@ namespace sl {
 // kernels of one step, in launch order
 enum FusedKernel {
     FK_FIRST, FK_BIN, FK_SCAN, FK_SCATTER, FK_CELLSORT, FK_LISTS, FK_REV, FK_FINISH,
-    FK_CRAD, FK_CRADW, FK_ANG, FK_NET, FK_BWD, FK_SECOND, FK_N
+    FK_CRAD, FK_CRADW, FK_ANG, FK_ANGW, FK_NET, FK_BWD, FK_BWDW, FK_SECOND, FK_N
 };
 // plan, the kernels (FP64 has the wide radial kernel only), the flag clear
 inline int fused_launches_per_step(int prec) { return 1 + FK_N + 1 - (prec == 0); }
 constexpr int FUSED_MAX_SLOTS = 4096;
 // atoms-per-block classes of the kernels that take one work item per block: the halves (256
 // atoms), the one-thread-per-atom radial kernel (128), the angular and backward kernels (a quad
-// block's atoms), the wide radial kernel and the FP64 network (8)
-enum { IC_HALF = 0, IC_ATOM = 1, IC_QUAD = 2, IC_OCT = 3, IC_N = 4 };
+// block's atoms), the wide radial kernel and the FP64 network (8), the wide angular and backward
+// kernels (one per warp of a quad block)
+enum { IC_HALF = 0, IC_ATOM = 1, IC_QUAD = 2, IC_OCT = 3, IC_WARP = 4, IC_N = 5 };
 
 // what a slot's entries are set up for
 enum SlotKind {
@@ -118,7 +119,7 @@ void launch_rebuild_t(const FusedTables &t, const Launch *L, bool clear, bool lo
 // radial, angular, network, backward; ev (optional, 6 events): recorded before the radial
 // kernel, after it, after the angular kernel, after the network and after the backward
 template <typename R>
-void launch_eval_t(const FusedTables &t, const NepDev<R> &P, const Launch *L /* crad, ang, net, bwd, wide crad */,
+void launch_eval_t(const FusedTables &t, const NepDev<R> &P, const Launch *L /* crad, ang, net, bwd, wide crad, ang, bwd */,
                    cudaStream_t st, cudaEvent_t *ev);
 void launch_net_t_tc(const FusedTables &t, const NepDev<float> &P, const Launch &L, cudaStream_t st);
 void launch_net_t_fp64(const FusedTables &t, const Launch &L, cudaStream_t st);

@@ -10,10 +10,10 @@
 //              sums over them, contracted with the coefficients once per neighbour
 //              species (q^R, q^EX, q^DMI, q^ANI, q^SIA, q^O).
 //   k_crad_wide  the same with sixteen lanes per atom (small systems, and FP64).
-//   k_ang_fwd  four lanes per atom.  Each lane stages one angular pair (carrier, g_n,
-//              spin weight, the 24 solid harmonics) in shared memory; then every lane
-//              accumulates B_nlm, BS_nlm for its 6 harmonics over the staged pairs.
-//   k_bwd      four lanes per atom, lanes over pairs.  The angular adjoints
+//   k_ang_fwd  four lanes per atom (k_ang_wide: a warp, in small systems).  Each lane stages one angular pair
+//              (carrier, g_n, spin weight, the 24 solid harmonics) in shared memory; then
+//              every lane accumulates B_nlm, BS_nlm for its 6 harmonics over the staged pairs.
+//   k_bwd      four lanes per atom (k_bwd_wide: a warp), lanes over pairs.  The angular adjoints
 //              dE/dB_nlm = 2 kappa_lm Fp B_nlm and the precontracted radial
 //              coefficients of the atom sit in shared memory; each lane takes whole
 //              pairs (angular rows first, then radial-only rows) and writes the pair
@@ -707,13 +707,21 @@ __device__ __forceinline__ void crad_wide_body(const NepDev<R> &P, const Eval2Ar
 
 
 // ------------------------------------------------------------------ k_ang_fwd
-// stage of one angular pair: (g_n, s g_n) interleaved for n = 0..4, pad (2), then the 24
-// harmonics in lane-major order (position 12 + 6 ql + m holds p_lm of lm = ql + 4 m), so
-// each quad lane reads its six harmonics with three 2-wide loads
+// LPA lanes per atom (4, or 32 in small systems: eval_is_wide): each stages one pair, then each takes the harmonics
+// lm = ql + LPA m.  Stage of one angular pair: (g_n, s g_n) interleaved for n = 0..4, pad (2),
+// then the 24 harmonics in lane-major order, so each lane reads its own from consecutive places.
 constexpr int FSTAGE = 36;
 constexpr int FQUAD = 4 * FSTAGE + 4;   // per quad, padded so quads start in different banks
+template <int LPA>
+struct AngLanes {
+    static constexpr int H = (NLM + LPA - 1) / LPA;     // harmonics per lane
+    static constexpr int FATOM = LPA * FSTAGE + 4;      // an atom's stages
+    static_assert(LPA == 4 || LPA == 8 || LPA == 32, "24 harmonics in equal shares, or one per lane");
+    // harmonic at place t of a stage: lane t / H, its share t % H
+    static constexpr __device__ int lm_at(int t) { return t / H + LPA * (t % H); }
+};
 
-template <typename R, int TI, int TJ>
+template <typename R, int LPA, int TI, int TJ>
 __device__ __forceinline__ void ang_stage_fwd(const NepDev<R> &P, const Eval2Args<R> &a, const v4<R> &pi,
                                               const v4<R> &si, const v4<R> &pj, const v4<R> &sj, R *st) {
     R dx, dy, dz;
@@ -734,27 +742,25 @@ __device__ __forceinline__ void ang_stage_fwd(const NepDev<R> &P, const Eval2Arg
     reinterpret_cast<v2<R> *>(st)[4] = w2;
     R p[NLM];
     harm_p(dx * ir, dy * ir, dz * ir, p);
+    using L = AngLanes<LPA>;
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        v2<R> a0, a1, a2;
-        a0.x = p[q]; a0.y = p[q + 4]; a1.x = p[q + 8]; a1.y = p[q + 12]; a2.x = p[q + 16]; a2.y = p[q + 20];
-        v2<R> *d = reinterpret_cast<v2<R> *>(st + 12 + 6 * q);
-        d[0] = a0; d[1] = a1; d[2] = a2;
-    }
+    for (int t = 0; t < NLM; t += 2) reinterpret_cast<v2<R> *>(st)[6 + t / 2] = pair2<R>(p[L::lm_at(t)], p[L::lm_at(t + 1)]);
 }
 
-template <typename R>
+template <typename R, int LPA>
 __device__ __forceinline__ void ang_fwd_body(const NepDev<R> &P, const Eval2Args<R> &args, int64_t blk,
                                              unsigned char *smem_raw) {
     // the arguments as values: read once from the block's copy, so nothing in the loops below
     // depends on where they are stored
     const Eval2Args<R> a = args;
     if (a.skip && *a.skip) return;
+    using L = AngLanes<LPA>;
+    constexpr int H = L::H, APW = 32 / LPA;   // harmonics per lane, atoms per warp
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int quad = lane >> 2, ql = lane & 3;
-    const int64_t i = (blk * (blockDim.x >> 5) + warp) * 8 + quad;
+    const int grp = lane / LPA, ql = lane % LPA;
+    const int64_t i = (blk * (blockDim.x >> 5) + warp) * APW + grp;
     const bool valid = i < a.n;
-    R *stage = reinterpret_cast<R *>(smem_raw) + (warp * 8 + quad) * FQUAD;
+    R *stage = reinterpret_cast<R *>(smem_raw) + (warp * APW + grp) * L::FATOM;
     v4<R> pi, si;
     int na0 = 0, na = 0, ti = 0;
     if (valid) {
@@ -765,9 +771,9 @@ __device__ __forceinline__ void ang_fwd_body(const NepDev<R> &P, const Eval2Args
         na = c.y;
         ti = i < a.n_fe ? 0 : 1;
     }
-    v2<R> BB[6][NCH];   // (B_nlm, BS_nlm) of the lane's six harmonics
+    v2<R> BB[H][NCH];   // (B_nlm, BS_nlm) of the lane's harmonics
 #pragma unroll
-    for (int m = 0; m < 6; ++m)
+    for (int m = 0; m < H; ++m)
 #pragma unroll
         for (int n = 0; n < NCH; ++n) BB[m][n] = pair2<R>(R(0), R(0));
     const int nmax = __reduce_max_sync(0xffffffffu, na);
@@ -781,34 +787,34 @@ __device__ __forceinline__ void ang_fwd_body(const NepDev<R> &P, const Eval2Args
         pjn = a.pos[j];
         sjn = a.spin[j];
     }
-    if (ql + 4 < na) {
-        const int j = crow[(int64_t)(ql + 4) * N].x;
+    if (ql + LPA < na) {
+        const int j = crow[(int64_t)(ql + LPA) * N].x;
         pjn2 = a.pos[j];
         sjn2 = a.spin[j];
     }
-    if (ql + 8 < na) jn3 = crow[(int64_t)(ql + 8) * N].x;
-    for (int base = 0; base < nmax; base += 4) {
+    if (ql + 2 * LPA < na) jn3 = crow[(int64_t)(ql + 2 * LPA) * N].x;
+    for (int base = 0; base < nmax; base += LPA) {
         const int p = base + ql;
         const v4<R> pj = pjn, sj = sjn;
         pjn = pjn2;
         sjn = sjn2;
-        if (p + 8 < na) {
+        if (p + 2 * LPA < na) {
             pjn2 = a.pos[jn3];
             sjn2 = a.spin[jn3];
         }
-        if (p + 12 < na) jn3 = crow[(int64_t)(p + 12) * N].x;
+        if (p + 3 * LPA < na) jn3 = crow[(int64_t)(p + 3 * LPA) * N].x;
         if (p < na) {
             R *st = stage + ql * FSTAGE;
             if (ti == 0) {
-                if (p < na0) ang_stage_fwd<R, 0, 0>(P, a, pi, si, pj, sj, st);
-                else ang_stage_fwd<R, 0, 1>(P, a, pi, si, pj, sj, st);
+                if (p < na0) ang_stage_fwd<R, LPA, 0, 0>(P, a, pi, si, pj, sj, st);
+                else ang_stage_fwd<R, LPA, 0, 1>(P, a, pi, si, pj, sj, st);
             } else {
-                if (p < na0) ang_stage_fwd<R, 1, 0>(P, a, pi, si, pj, sj, st);
-                else ang_stage_fwd<R, 1, 1>(P, a, pi, si, pj, sj, st);
+                if (p < na0) ang_stage_fwd<R, LPA, 1, 0>(P, a, pi, si, pj, sj, st);
+                else ang_stage_fwd<R, LPA, 1, 1>(P, a, pi, si, pj, sj, st);
             }
         }
         __syncwarp();
-        const int cnt = min(4, na - base);
+        const int cnt = LPA * H > NLM && ql >= NLM ? 0 : min(LPA, na - base);   // lanes without a harmonic
         for (int q = 0; q < cnt; ++q) {
             const R *sp = stage + q * FSTAGE;
             const v4<R> w0 = reinterpret_cast<const v4<R> *>(sp)[0];
@@ -816,11 +822,21 @@ __device__ __forceinline__ void ang_fwd_body(const NepDev<R> &P, const Eval2Args
             const v2<R> w2 = reinterpret_cast<const v2<R> *>(sp)[4];
             const v2<R> gg[NCH] = {pair2<R>(w0.x, w0.y), pair2<R>(w0.z, w0.w), pair2<R>(w1.x, w1.y),
                                    pair2<R>(w1.z, w1.w), w2};
-            const v2<R> *pp = reinterpret_cast<const v2<R> *>(sp + 12 + 6 * ql);
-            const v2<R> p01 = pp[0], p23 = pp[1], p45 = pp[2];
-            const R pv[6] = {p01.x, p01.y, p23.x, p23.y, p45.x, p45.y};
+            R pv[H];
+            if constexpr (LPA == 4) {
+                const v2<R> *pp = reinterpret_cast<const v2<R> *>(sp + 12 + H * ql);
 #pragma unroll
-            for (int m = 0; m < 6; ++m) {
+                for (int m = 0; m < H; m += 2) {
+                    const v2<R> x = pp[m / 2];
+                    pv[m] = x.x;
+                    pv[m + 1] = x.y;
+                }
+            } else {
+#pragma unroll
+                for (int m = 0; m < H; ++m) pv[m] = sp[12 + H * ql + m];
+            }
+#pragma unroll
+            for (int m = 0; m < H; ++m) {
                 const v2<R> pl = pair2<R>(pv[m], pv[m]);
 #pragma unroll
                 for (int n = 0; n < NCH; ++n) BB[m][n] = fma2(gg[n], pl, BB[m][n]);
@@ -828,15 +844,20 @@ __device__ __forceinline__ void ang_fwd_body(const NepDev<R> &P, const Eval2Args
         }
         __syncwarp();
     }
-    // angular sums for the backward pass, and the channel values
-    R qa[NCH][4], qs[NCH][4];
+    // angular sums for the backward pass, and the channel values: with four lanes per atom summed in
+    // registers and over the quad, else through the atom's stage
+    constexpr bool QUAD = LPA == 4;
+    [[maybe_unused]] R qa[QUAD ? NCH : 1][4], qs[QUAD ? NCH : 1][4];
+    if constexpr (QUAD) {
 #pragma unroll
-    for (int n = 0; n < NCH; ++n)
+        for (int n = 0; n < NCH; ++n)
 #pragma unroll
-        for (int l = 0; l < 4; ++l) { qa[n][l] = R(0); qs[n][l] = R(0); }
+            for (int l = 0; l < 4; ++l) { qa[n][l] = R(0); qs[n][l] = R(0); }
+    }
 #pragma unroll
-    for (int m = 0; m < 6; ++m) {
-        const int lm = lm_of(ql, m);
+    for (int m = 0; m < H; ++m) {
+        const int lm = ql + LPA * m;
+        if (!QUAD && lm >= NLM) break;
         const int l = l_of_lm(lm) - 1;
         const R kap = kappa_of_lm<R>(lm);
         if (valid) {   // the harmonic's record: (B_n, BS_n) for n = 0..4, two zeros
@@ -851,35 +872,51 @@ __device__ __forceinline__ void ang_fwd_body(const NepDev<R> &P, const Eval2Args
         for (int n = 0; n < NCH; ++n) {
             const R Bv = BB[m][n].x, BSv = BB[m][n].y;
             const R ka = kap * Bv * Bv, ks = kap * BSv * BSv;
-            // l is 1..4 depending on the lane: add into the matching slot
+            if constexpr (QUAD) {
+                // l is 1..4 depending on the lane: add into the matching slot
 #pragma unroll
-            for (int t = 0; t < 4; ++t) {
-                qa[n][t] += (t == l) ? ka : R(0);
-                qs[n][t] += (t == l) ? ks : R(0);
+                for (int t = 0; t < 4; ++t) {
+                    qa[n][t] += (t == l) ? ka : R(0);
+                    qs[n][t] += (t == l) ? ks : R(0);
+                }
+            } else {   // [lm][2 n + (0: A, 1: SA)]
+                *reinterpret_cast<v2<R> *>(stage + lm * 10 + 2 * n) = pair2<R>(ka, ks);
             }
         }
     }
+    if constexpr (QUAD) {
 #pragma unroll
-    for (int n = 0; n < NCH; ++n)
+        for (int n = 0; n < NCH; ++n)
 #pragma unroll
-        for (int t = 0; t < 4; ++t) {
-            qa[n][t] += __shfl_xor_sync(0xffffffffu, qa[n][t], 1);
-            qa[n][t] += __shfl_xor_sync(0xffffffffu, qa[n][t], 2);
-            qs[n][t] += __shfl_xor_sync(0xffffffffu, qs[n][t], 1);
-            qs[n][t] += __shfl_xor_sync(0xffffffffu, qs[n][t], 2);
-        }
-    if (valid) {
-        // lane ql writes l = ql + 1
-#pragma unroll
-        for (int n = 0; n < NCH; ++n) {
-            R va = qa[n][0], vs = qs[n][0];
-#pragma unroll
-            for (int t = 1; t < 4; ++t) {
-                va = ql == t ? qa[n][t] : va;
-                vs = ql == t ? qs[n][t] : vs;
+            for (int t = 0; t < 4; ++t) {
+                qa[n][t] += __shfl_xor_sync(0xffffffffu, qa[n][t], 1);
+                qa[n][t] += __shfl_xor_sync(0xffffffffu, qa[n][t], 2);
+                qs[n][t] += __shfl_xor_sync(0xffffffffu, qs[n][t], 1);
+                qs[n][t] += __shfl_xor_sync(0xffffffffu, qs[n][t], 2);
             }
-            stg(a.q + (int64_t)(Q_A + n * 4 + ql) * a.qs + i, va);
-            stg(a.q + (int64_t)(Q_SA + n * 4 + ql) * a.qs + i, vs);
+        if (valid) {
+            // lane ql writes l = ql + 1
+#pragma unroll
+            for (int n = 0; n < NCH; ++n) {
+                R va = qa[n][0], vs = qs[n][0];
+#pragma unroll
+                for (int t = 1; t < 4; ++t) {
+                    va = ql == t ? qa[n][t] : va;
+                    vs = ql == t ? qs[n][t] : vs;
+                }
+                stg(a.q + (int64_t)(Q_A + n * 4 + ql) * a.qs + i, va);
+                stg(a.q + (int64_t)(Q_SA + n * 4 + ql) * a.qs + i, vs);
+            }
+        }
+    } else {
+        __syncwarp();
+        if (valid) {   // the lanes take the 40 values
+            for (int o = ql; o < 8 * NCH; o += LPA) {
+                const int l = o & 3, c = o >> 2;   // c: 2 n + (0: A, 1: SA)
+                R v = R(0);
+                for (int lm = l * (l + 2); lm < (l + 1) * (l + 3); ++lm) v += stage[lm * 10 + c];
+                stg(a.q + (int64_t)((c & 1 ? Q_SA : Q_A) + (c >> 1) * 4 + l) * a.qs + i, v);
+            }
         }
     }
 }
@@ -904,10 +941,10 @@ struct BwdAcc2 {
 // species into smc, 48 each; place of C^G_k: FP64 [k][group] (k = 0 shifted), FP32 [group][k].
 template <typename R>
 __device__ __forceinline__ int coeff_at(int g, int k) { return sizeof(R) == 8 ? 5 * k + g : 9 * g + k; }
-// FP32: every lane of the quad forms them all (the coefficients are constant operands) and stores a
-// quarter; taking its own from a table in global memory made the backward 1.58 to 1.70 ms at
+// FP32: every lane of the atom forms them all (the coefficients are constant operands) and stores its
+// share; taking its own from a table in global memory made the backward 1.58 to 1.70 ms at
 // 884,736 atoms (the loads' latency, before the first pair).
-template <int TI>
+template <int TI, int LPA>
 __device__ __forceinline__ void bwd_coeffs(const NepDev<float> &P, const float F[5][NCH], int ql, float *smc) {
 #pragma unroll
     for (int tj = 0; tj < NS; ++tj)
@@ -919,14 +956,18 @@ __device__ __forceinline__ void bwd_coeffs(const NepDev<float> &P, const float F
                 float v = 0.f;
 #pragma unroll
                 for (int n = 0; n < NCH; ++n) v += F[g][n] * (tj == 0 ? P.c[TI][0][G[g]][n][k] : P.c[TI][1][G[g]][n][k]);
-                if (((tj * 45 + g * 9 + k) & 3) == ql) smc[tj * 48 + coeff_at<float>(g, k)] = v;
+                if (((tj * 45 + g * 9 + k) & (LPA - 1)) == ql) smc[tj * 48 + coeff_at<float>(g, k)] = v;
             }
 }
-// FP64: lane ql of the quad takes k = 2 ql and 2 ql + 1, lanes 0 and 1 one species' k = 8, from the
-// centre's rows ct of the table (a quarter of the multiply-adds).
-__device__ __forceinline__ void bwd_coeffs(const double *__restrict__ ct, const double F[5][NCH], int ql, double *smc) {
+// FP64: lane ql of a quad takes k = 2 ql and 2 ql + 1 (with a warp, a quad each species), lanes 0 and
+// 1 one species' k = 8, from the centre's rows ct of the table (a quarter of the multiply-adds).
+template <int LPA>
+__device__ __forceinline__ void bwd_coeffs(const double *__restrict__ ct, const double F[5][NCH], int lane, double *smc) {
+    const int ql = lane & 3;
+    if (LPA > 4 && lane >= 8) return;
 #pragma unroll
-    for (int tj = 0; tj < NS; ++tj)
+    for (int t = 0; t < (LPA == 4 ? NS : 1); ++t) {
+        const int tj = LPA == 4 ? t : lane >> 2;
 #pragma unroll
         for (int g = 0; g < 5; ++g) {
             double2 c2 = make_double2(0.0, 0.0);
@@ -937,13 +978,14 @@ __device__ __forceinline__ void bwd_coeffs(const double *__restrict__ ct, const 
             smc[tj * 48 + coeff_at<double>(g, 2 * ql)] = c2.x;
             smc[tj * 48 + coeff_at<double>(g, 2 * ql + 1)] = c2.y;
         }
-    const int tj = ql & 1;
+    }
+    const int tj = lane & 1;
 #pragma unroll
     for (int g = 0; g < 5; ++g) {
         double v = 0.0;
 #pragma unroll
         for (int n = 0; n < NCH; ++n) v += F[g][n] * ro(ct + ((tj * 5 + g) * NCH + n) * CB_ROW + 8);
-        if (ql < NS) smc[tj * 48 + coeff_at<double>(g, 8)] = v;
+        if (lane < NS) smc[tj * 48 + coeff_at<double>(g, 8)] = v;
     }
 }
 
@@ -1245,10 +1287,10 @@ __device__ __forceinline__ void bwd_pair(const NepDev<R> &P, const Eval2Args<R> 
     store_rec(rec, ra, rb);
 }
 
-// rows lo, lo+4, ... of one range for lane ql.  Two-level prefetch: the list entry of the
+// rows lo, lo + LPA, ... of one range for one lane.  Two-level prefetch: the list entry of the
 // row two steps ahead and the coordinates of the next row are in flight while a pair is
 // computed, so no load waits on a load issued in the same step.
-template <typename R, bool ANG, bool VIR>
+template <typename R, bool ANG, bool VIR, int LPA>
 __device__ __forceinline__ void bwd_rows(const NepDev<R> &P, const Eval2Args<R> &a, int64_t i, int ti, int lo, int hi,
                                          int split, const v4<R> &pi, const v4<R> &si, const R *sm,
                                          BwdAcc2<R> &acc) {
@@ -1257,31 +1299,32 @@ __device__ __forceinline__ void bwd_rows(const NepDev<R> &P, const Eval2Args<R> 
     int2 e1 = make_int2(0, 0), e2 = e1, e3 = e1;   // (neighbour, the record's slot in its list)
     v4<R> p1, s1, p2, s2;
     if (lo < hi) e1 = ro(crow + (int64_t)lo * N);
-    if (lo + 4 < hi) e2 = ro(crow + (int64_t)(lo + 4) * N);
-    if (lo + 8 < hi) e3 = ro(crow + (int64_t)(lo + 8) * N);
+    if (lo + LPA < hi) e2 = ro(crow + (int64_t)(lo + LPA) * N);
+    if (lo + 2 * LPA < hi) e3 = ro(crow + (int64_t)(lo + 2 * LPA) * N);
     if (lo < hi) {
         p1 = ro(a.pos + e1.x);
         s1 = ro(a.spin + e1.x);
     }
-    if (lo + 4 < hi) {
+    if (lo + LPA < hi) {
         p2 = ro(a.pos + e2.x);
         s2 = ro(a.spin + e2.x);
     }
-    for (int row = lo; row < hi; row += 4) {
+#pragma unroll 1
+    for (int row = lo; row < hi; row += LPA) {
         const int j = e1.x, t = e1.y;
         const v4<R> pj = p1, sj = s1;
         e1 = e2; p1 = p2; s1 = s2;
         e2 = e3;
-        if (row + 8 < hi) {
+        if (row + 2 * LPA < hi) {
             p2 = ro(a.pos + e2.x);
             s2 = ro(a.spin + e2.x);
         }
-        if (row + 12 < hi) e3 = ro(crow + (int64_t)(row + 12) * N);
+        if (row + 3 * LPA < hi) e3 = ro(crow + (int64_t)(row + 3 * LPA) * N);
         bwd_pair<R, ANG, VIR>(P, a, ti, row < split ? 0 : 1, pi, si, pj, sj, j, t, sm, acc);
     }
 }
 
-template <typename R, bool VIR>
+template <typename R, bool VIR, int LPA>
 __device__ __forceinline__ void bwd_body(const NepDev<R> &P, const Eval2Args<R> &args, int64_t blk,
                                          unsigned char *smem_raw) {
     // the arguments as values: read once from the block's copy, so nothing in the loops below
@@ -1289,11 +1332,12 @@ __device__ __forceinline__ void bwd_body(const NepDev<R> &P, const Eval2Args<R> 
     const Eval2Args<R> a = args;
     if (a.skip && *a.skip) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int quad = lane >> 2, ql = lane & 3;
-    const int64_t i = (blk * (blockDim.x >> 5) + warp) * 8 + quad;
+    constexpr int APW = 32 / LPA;   // atoms per warp
+    const int grp = lane / LPA, ql = lane % LPA;
+    const int64_t i = (blk * (blockDim.x >> 5) + warp) * APW + grp;
     const bool valid = i < a.n;
     const int64_t N = a.n;
-    R *sm = reinterpret_cast<R *>(smem_raw) + (warp * 8 + quad) * BW_ATOM;
+    R *sm = reinterpret_cast<R *>(smem_raw) + (warp * APW + grp) * BW_ATOM;
     BwdAcc2<R> acc;
     acc.fx = acc.fy = acc.fz = acc.hx = acc.hy = acc.hz = R(0);
 #pragma unroll
@@ -1302,11 +1346,12 @@ __device__ __forceinline__ void bwd_body(const NepDev<R> &P, const Eval2Args<R> 
         const int ti = i < a.n_fe ? 0 : 1;
         const v4<R> pi = ro(a.pos + i), si = ro(a.spin + i);
         const int4 c = ro(a.cnt + i);
-        // angular adjoints of this lane's harmonics lm = ql + 4 m from their records (three
+        // angular adjoints of this lane's harmonics lm = ql + LPA m from their records (three
         // 16-byte loads each), the gradient entries straight from global memory
 #pragma unroll
-        for (int m = 0; m < 6; ++m) {
-            const int lm = lm_of(ql, m);
+        for (int m = 0; m < (NLM + LPA - 1) / LPA; ++m) {
+            const int lm = ql + LPA * m;
+            if (LPA > 8 && lm >= NLM) break;
             const int l = l_of_lm(lm);
             const R k2 = R(2) * kappa_of_lm<R>(lm);
             const v4<R> *src = reinterpret_cast<const v4<R> *>(a.bsum + ((int64_t)i * NLM + lm) * BREC);
@@ -1330,17 +1375,17 @@ __device__ __forceinline__ void bwd_body(const NepDev<R> &P, const Eval2Args<R> 
             const R fo = R(2) * ro(a.fp + (int64_t)Q_O * N + i);
             acc.hx = fo * si.x; acc.hy = fo * si.y; acc.hz = fo * si.z;
         }
-        if constexpr (sizeof(R) == 8) bwd_coeffs(a.ctab + CTAB_BWD + ti * (NS * 25 * CB_ROW), F, ql, sm + BW_C);
-        else if (ti == 0) bwd_coeffs<0>(P, F, ql, sm + BW_C);
-        else bwd_coeffs<1>(P, F, ql, sm + BW_C);
-        __syncwarp(0xfu << (quad * 4));
+        if constexpr (sizeof(R) == 8) bwd_coeffs<LPA>(a.ctab + CTAB_BWD + ti * (NS * 25 * CB_ROW), F, ql, sm + BW_C);
+        else if (ti == 0) bwd_coeffs<0, LPA>(P, F, ql, sm + BW_C);
+        else bwd_coeffs<1, LPA>(P, F, ql, sm + BW_C);
+        __syncwarp(LPA == 32 ? 0xffffffffu : ((1u << (LPA & 31)) - 1u) << (grp * LPA));
         const int ca = a.cap_ang;
-        bwd_rows<R, true, VIR>(P, a, i, ti, ql, c.y, c.x, pi, si, sm, acc);
-        bwd_rows<R, false, VIR>(P, a, i, ti, ca + ql, ca + c.w, ca + c.z, pi, si, sm, acc);
+        bwd_rows<R, true, VIR, LPA>(P, a, i, ti, ql, c.y, c.x, pi, si, sm, acc);
+        bwd_rows<R, false, VIR, LPA>(P, a, i, ti, ca + ql, ca + c.w, ca + c.z, pi, si, sm, acc);
     }
-    // per-atom sums over the quad
+    // per-atom sums over the atom's lanes
 #pragma unroll
-    for (int o = 1; o <= 2; o <<= 1) {
+    for (int o = 1; o < LPA; o <<= 1) {
         acc.fx += __shfl_xor_sync(0xffffffffu, acc.fx, o);
         acc.fy += __shfl_xor_sync(0xffffffffu, acc.fy, o);
         acc.fz += __shfl_xor_sync(0xffffffffu, acc.fz, o);
@@ -1350,10 +1395,9 @@ __device__ __forceinline__ void bwd_body(const NepDev<R> &P, const Eval2Args<R> 
     }
     if constexpr (VIR) {
 #pragma unroll
-        for (int t = 0; t < 9; ++t) {
-            acc.w[t] += __shfl_xor_sync(0xffffffffu, acc.w[t], 1);
-            acc.w[t] += __shfl_xor_sync(0xffffffffu, acc.w[t], 2);
-        }
+        for (int t = 0; t < 9; ++t)
+#pragma unroll
+            for (int o = 1; o < LPA; o <<= 1) acc.w[t] += __shfl_xor_sync(0xffffffffu, acc.w[t], o);
     }
     if (valid && ql == 0) {
         v4<R> f4, g4;
@@ -1395,7 +1439,7 @@ __global__ void __launch_bounds__(128, MINB) k_ang_fwd(const __grid_constant__ N
                                                        const __grid_constant__ Eval2Args<R> solo) {
     extern __shared__ __align__(32) unsigned char smem_raw[];
     one_work(tab, sm, solo,
-             [&](const Eval2Args<R> &a, int64_t blk, int64_t) { ang_fwd_body(P, a, blk, smem_raw); });
+             [&](const Eval2Args<R> &a, int64_t blk, int64_t) { ang_fwd_body<R, 4>(P, a, blk, smem_raw); });
 }
 template <typename R, int MINB = sizeof(R) == 4 ? 4 : 1, bool VIR = false>
 __global__ void __launch_bounds__(128, MINB) k_bwd(const __grid_constant__ NepDev<R> P,
@@ -1403,7 +1447,32 @@ __global__ void __launch_bounds__(128, MINB) k_bwd(const __grid_constant__ NepDe
                                                    const __grid_constant__ Eval2Args<R> solo) {
     extern __shared__ __align__(32) unsigned char smem_raw[];
     one_work(tab, sm, solo,
-             [&](const Eval2Args<R> &a, int64_t blk, int64_t) { bwd_body<R, VIR>(P, a, blk, smem_raw); });
+             [&](const Eval2Args<R> &a, int64_t blk, int64_t) { bwd_body<R, VIR, 4>(P, a, blk, smem_raw); });
+}
+
+// The same with a warp per atom, for systems too small to fill the GPU four lanes per atom (the line
+// in eval_is_wide).  FP64 at 512 / 1,728 / 2,744 atoms: angular 32 / 71 / 110 instead of 117 / 120 / 140
+// us, backward 75 / 198 / 321 instead of 380 / 387 / 398 us (its 21 angular pairs fill two thirds of a
+// round of 32 lanes, so in larger systems four lanes need fewer FP64 instructions).  Mixed precision
+// at 512 / 1,728 / 2,744 / 4,096 atoms: angular 10 / 10 / 14.5 / 16 instead of 12 / 12 / 12 / 12 us,
+// backward 14 / 18 / 25 / 31 instead of 26 / 26 / 26 / 25 us.
+template <typename R>
+__global__ void __launch_bounds__(128, sizeof(R) == 4 ? 4 : 1) k_ang_wide(const __grid_constant__ NepDev<R> P,
+                                                                          const Eval2Args<R> *__restrict__ tab,
+                                                                          SlotMap sm,
+                                                                          const __grid_constant__ Eval2Args<R> solo) {
+    extern __shared__ __align__(32) unsigned char smem_raw[];
+    one_work(tab, sm, solo,
+             [&](const Eval2Args<R> &a, int64_t blk, int64_t) { ang_fwd_body<R, 32>(P, a, blk, smem_raw); });
+}
+template <typename R, bool VIR = false>
+__global__ void __launch_bounds__(128, sizeof(R) == 4 ? 3 : 1) k_bwd_wide(const __grid_constant__ NepDev<R> P,
+                                                                          const Eval2Args<R> *__restrict__ tab,
+                                                                          SlotMap sm,
+                                                                          const __grid_constant__ Eval2Args<R> solo) {
+    extern __shared__ __align__(32) unsigned char smem_raw[];
+    one_work(tab, sm, solo,
+             [&](const Eval2Args<R> &a, int64_t blk, int64_t) { bwd_body<R, VIR, 32>(P, a, blk, smem_raw); });
 }
 
 // ------------------------------------------------------------------ launch
@@ -1438,6 +1507,8 @@ template <typename R>
 static constexpr size_t fwd_smem(int qb = quad_block<R>()) { return (size_t)(qb / 32) * 8 * FQUAD * sizeof(R); }
 template <typename R>
 static constexpr size_t bwdf_smem(int qb = quad_block<R>()) { return (size_t)(qb / 32) * 8 * BW_ATOM * sizeof(R); }
+template <typename R>
+static constexpr size_t bwdw_smem(int qb) { return (size_t)(qb / 32) * BW_ATOM * sizeof(R); }
 
 int default_quad_block(int prec) { return prec == 0 ? quad_block<double>() : quad_block<float>(); }
 
@@ -1460,6 +1531,8 @@ void eval2_init() {
     cudaFuncSetAttribute(k_bwd<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bwdf_smem<double>());
     cudaFuncSetAttribute(k_bwd<double, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)bwdf_smem<double>());
+    cudaFuncSetAttribute(k_ang_wide<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fwd_smem<float>());
+    cudaFuncSetAttribute(k_ang_wide<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fwd_smem<double>());
     if (dev < 64) done |= 1ull << dev;
 }
 
@@ -1485,10 +1558,12 @@ void fused_put_eval(Sys &s, int r, int kind, const FusedTables &t, unsigned char
     const bool wide = crad_is_wide(s);
     blocks[FK_CRAD] = wide ? 0 : (s.n + 127) / 128;
     blocks[FK_CRADW] = wide ? (s.n + CRAD_WIDE_ATOMS - 1) / CRAD_WIDE_ATOMS : 0;
-    blocks[FK_ANG] = blocks[FK_BWD] = (s.n + qb / 4 - 1) / (qb / 4);
+    const bool warp = eval_is_wide(s);   // a warp per atom
+    blocks[FK_ANG] = blocks[FK_BWD] = warp ? 0 : (s.n + qb / 4 - 1) / (qb / 4);
+    blocks[FK_ANGW] = blocks[FK_BWDW] = warp ? (s.n + qb / 32 - 1) / (qb / 32) : 0;
 }
 
-// Radial, angular, network and backward (and, last, the wide radial kernel) over a table, each launch in its own shape
+// Radial, angular, network and backward (and, last, the three wide kernels) over a table, each launch in its own shape
 // (L[k].block threads, 0: the default) and register budget (L[k].minb, 0: the default).
 template <typename R>
 void launch_eval_t(const FusedTables &t, const NepDev<R> &P, const Launch *L, cudaStream_t st, cudaEvent_t *ev) {
@@ -1503,7 +1578,7 @@ void launch_eval_t(const FusedTables &t, const NepDev<R> &P, const Launch *L, cu
     if (ev) cudaEventRecord(ev[0], st);
     // compaction and radial channels in one kernel: the compaction group is empty
     if (ev) cudaEventRecord(ev[1], st);
-    // a system's own launch has a grid for one of the radial kernels only
+    // a system's own launch has a grid for one kernel of each kind only
     if constexpr (sizeof(R) == 4) {
         if (L[0].grid && L[0].minb == 3) k_crad<3><<<L[0].grid, cb, 0, st>>>(P, tab, s0, so);
         else if (L[0].grid) k_crad<<<L[0].grid, cb, 0, st>>>(P, tab, s0, so);
@@ -1512,10 +1587,14 @@ void launch_eval_t(const FusedTables &t, const NepDev<R> &P, const Launch *L, cu
     bool variant = false;
     if (ev) cudaEventRecord(ev[2], st);
     if constexpr (sizeof(R) == 4) {
-        variant = L[1].minb == 1;
+        variant = L[1].minb == 1 && L[1].grid;
         if (variant) k_ang_fwd<R, 1><<<L[1].grid, qa, fwd_smem<R>(qa), st>>>(P, tab, s1, so);
     }
-    if (!variant) k_ang_fwd<R><<<L[1].grid, qa, fwd_smem<R>(qa), st>>>(P, tab, s1, so);
+    if (!variant && L[1].grid) k_ang_fwd<R><<<L[1].grid, qa, fwd_smem<R>(qa), st>>>(P, tab, s1, so);
+    if (L[5].grid) {
+        const int b = L[5].block ? L[5].block : quad_block<R>();
+        k_ang_wide<R><<<L[5].grid, b, fwd_smem<R>(b), st>>>(P, tab, L[5].slots(), so);
+    }
     if (ev) cudaEventRecord(ev[3], st);
     if constexpr (sizeof(R) == 4) launch_net_t_tc(t, P, L[2], st);
     else launch_net_t_fp64(t, L[2], st);
@@ -1523,14 +1602,22 @@ void launch_eval_t(const FusedTables &t, const NepDev<R> &P, const Launch *L, cu
     // the virial parts: only a system's own full evaluation asks for them (a batch's slots are
     // set up for the step's evaluation, which has none)
     const bool vir = L[3].solo && so.want_virial;
-    variant = false;
-    if constexpr (sizeof(R) == 4) {
-        variant = L[3].minb == 3;
-        if (variant && vir) k_bwd<R, 3, true><<<L[3].grid, qw, bwdf_smem<R>(qw), st>>>(P, tab, s3, so);
-        else if (variant) k_bwd<R, 3><<<L[3].grid, qw, bwdf_smem<R>(qw), st>>>(P, tab, s3, so);
+    if (L[3].grid) {
+        variant = false;
+        if constexpr (sizeof(R) == 4) {
+            variant = L[3].minb == 3;
+            if (variant && vir) k_bwd<R, 3, true><<<L[3].grid, qw, bwdf_smem<R>(qw), st>>>(P, tab, s3, so);
+            else if (variant) k_bwd<R, 3><<<L[3].grid, qw, bwdf_smem<R>(qw), st>>>(P, tab, s3, so);
+        }
+        if (!variant && vir)
+            k_bwd<R, sizeof(R) == 4 ? 4 : 1, true><<<L[3].grid, qw, bwdf_smem<R>(qw), st>>>(P, tab, s3, so);
+        else if (!variant) k_bwd<R><<<L[3].grid, qw, bwdf_smem<R>(qw), st>>>(P, tab, s3, so);
     }
-    if (!variant && vir) k_bwd<R, sizeof(R) == 4 ? 4 : 1, true><<<L[3].grid, qw, bwdf_smem<R>(qw), st>>>(P, tab, s3, so);
-    else if (!variant) k_bwd<R><<<L[3].grid, qw, bwdf_smem<R>(qw), st>>>(P, tab, s3, so);
+    if (L[6].grid) {
+        const int b = L[6].block ? L[6].block : quad_block<R>();
+        if (vir) k_bwd_wide<R, true><<<L[6].grid, b, bwdw_smem<R>(b), st>>>(P, tab, L[6].slots(), so);
+        else k_bwd_wide<R><<<L[6].grid, b, bwdw_smem<R>(b), st>>>(P, tab, L[6].slots(), so);
+    }
     if (ev) cudaEventRecord(ev[5], st);
 }
 template void launch_eval_t<float>(const FusedTables &, const NepDev<float> &, const Launch *, cudaStream_t,
@@ -1543,8 +1630,9 @@ template void launch_eval_t<double>(const FusedTables &, const NepDev<double> &,
 void launch_eval(Sys &s, bool want_virial, cudaEvent_t *ev) {
     if (s.n == 0) return;
     const int kind = s.at.pos ? SK_MID : want_virial ? SK_FULL : SK_STEP;
-    const Launch L[5] = {solo_launch(s, FK_CRAD, kind), solo_launch(s, FK_ANG, kind), solo_launch(s, FK_NET, kind),
-                         solo_launch(s, FK_BWD, kind), solo_launch(s, FK_CRADW, kind)};
+    const Launch L[7] = {solo_launch(s, FK_CRAD, kind),  solo_launch(s, FK_ANG, kind),  solo_launch(s, FK_NET, kind),
+                         solo_launch(s, FK_BWD, kind),   solo_launch(s, FK_CRADW, kind), solo_launch(s, FK_ANGW, kind),
+                         solo_launch(s, FK_BWDW, kind)};
     if (s.prec == 0) launch_eval_t<double>(s.solo->t, s.pd, L, s.stream, ev);
     else launch_eval_t<float>(s.solo->t, s.pf, L, s.stream, ev);
 }

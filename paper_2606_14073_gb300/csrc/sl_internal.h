@@ -224,6 +224,10 @@ inline int nbr_stride(int cap) { return (cap + 31) & ~31; }   // byte rows of 32
 constexpr int64_t CRAD_WIDE_MAX = 16384;
 constexpr int CRAD_WIDE_ATOMS = 8;   // atoms per 128-thread block of k_crad_wide
 inline bool crad_is_wide(const Sys &s) { return s.prec == 0 || s.n <= CRAD_WIDE_MAX; }
+// The angular and backward kernels of a system (fixed by its size likewise): a warp per atom in
+// small systems, else four lanes per atom (both timed at k_ang_wide).
+constexpr int64_t EVAL_WIDE_MAX64 = 3040, EVAL_WIDE_MAX32 = 2048;
+inline bool eval_is_wide(const Sys &s) { return s.n <= (s.prec == 0 ? EVAL_WIDE_MAX64 : EVAL_WIDE_MAX32); }
 void nbr_setup(Sys &s);
 void launch_rebuild(Sys &s, bool conditional);
 // sl_eval2.cu: the system's evaluation at the state (with the virial parts when asked for), or
