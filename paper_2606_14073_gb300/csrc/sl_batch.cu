@@ -47,7 +47,9 @@ void launch_fused_plan(const FusedTables &t, cudaStream_t st) {
 // work map: the rebuild group, and the tensor-core network)
 static int item_class(int k, int prec) {
     switch (k) {
-        case FK_FIRST: case FK_SECOND: return IC_HALF;
+        case FK_FIRST: return IC_FIRST;
+        case FK_SECOND: return IC_SECOND;
+        case FK_SECONDW: return IC_GATHER;
         case FK_CRAD: return prec == 0 ? -1 : IC_ATOM;   // FP64: the wide kernel only
         case FK_CRADW: return IC_OCT;
         case FK_ANG: case FK_BWD: return IC_QUAD;
@@ -82,7 +84,7 @@ void FusedBatch::enqueue(cudaStream_t st) const {
     const Launch ev[7] = {L(FK_CRAD), L(FK_ANG), L(FK_NET), L(FK_BWD), L(FK_CRADW), L(FK_ANGW), L(FK_BWDW)};
     if (t.prec == 0) launch_eval_t<double>(t, pd, ev, st, nullptr);
     else launch_eval_t<float>(t, pf, ev, st, nullptr);
-    launch_second_half_t(t, L(FK_SECOND), true, st);
+    launch_second_half_t(t, L(FK_SECOND), L(FK_SECONDW), true, st);
 }
 
 namespace {
@@ -205,7 +207,8 @@ bool FusedBatch::same_model(const Sys &s) const {
 // network, k_mlp_tc, is persistent); -1 for the others.
 static int item_kernel_class(const char *name) {
     struct { const char *id; int cls; } const k[] = {
-        {"k_first_half", IC_HALF}, {"k_second_half", IC_HALF}, {"k_crad", IC_ATOM}, {"k_crad_wide", IC_OCT},
+        {"k_first_half", IC_FIRST}, {"k_second_half", IC_SECOND}, {"k_second_wide", IC_GATHER},
+        {"k_crad", IC_ATOM}, {"k_crad_wide", IC_OCT},
         {"k_mlp", IC_OCT}, {"k_ang_fwd", IC_QUAD}, {"k_bwd", IC_QUAD},
         {"k_ang_wide", IC_WARP}, {"k_bwd_wide", IC_WARP}};
     for (const auto &x : k) {
@@ -237,9 +240,9 @@ bool FusedBatch::find_item_nodes(cudaGraph_t graph, cudaGraphExec_t exec, int st
         item_nodes.push_back(ItemNode{exec, node, c});
         ++found;
     }
-    // per step: the two halves, the wide radial kernel, the other one (or the FP64 network), the
-    // two angular and the two backward kernels
-    return found == (int64_t)steps * 8;
+    // per step: the first half, the wide radial kernel, the other one (or the FP64 network), and two
+    // kernels each of the angular part, the backward and the second half
+    return found == (int64_t)steps * 9;
 }
 
 bool FusedBatch::resize_item_nodes() {
@@ -292,7 +295,7 @@ bool FusedBatch::reserve(int64_t atoms) {
     int64_t c = 1;
     while (c < atoms) c <<= 1;
     const int q = default_quad_block(t.prec);
-    const int64_t per[IC_N] = {256, 128, q / 4, CRAD_WIDE_ATOMS, q / 32};
+    const int64_t per[IC_N] = {256, 128, q / 4, CRAD_WIDE_ATOMS, q / 32, 256, second_wide_atoms(t.prec)};
     int64_t cap_items[IC_N], total = 0;
     for (int k = 0; k < IC_N; ++k) {
         cap_items[k] = (c + per[k] - 1) / per[k] + t.cap;   // whole blocks, one partial block per slot
@@ -355,7 +358,7 @@ cudaError_t FusedBatch::upload(const int64_t *left, cudaStream_t st) {
     if (dirty || layout_dirty) {
         // block -> slot layout of the one-item-per-block kernels: every occupied slot's blocks in
         // slot order, then no slot (-1) up to the capacity
-        const int kof[IC_N] = {FK_FIRST, FK_CRAD, FK_ANG, FK_CRADW, FK_ANGW};
+        const int kof[IC_N] = {FK_FIRST, FK_CRAD, FK_ANG, FK_CRADW, FK_ANGW, FK_SECOND, FK_SECONDW};
         for (int c = 0; c < IC_N; ++c) {
             int *it = h_items + item_off[c];
             int64_t o = 0;
@@ -460,8 +463,8 @@ Launch solo_launch(const Sys &s, int k, int kind) {
     L.m = so.map(k, kind, shape);
     int64_t g = so.blocks[k][shape];
     if (k == FK_NET && s.prec != 0) g = std::min<int64_t>(g, (int64_t)so.sms * s.cfg.mlp_ctas_per_sm);   // persistent
-    // the radial, angular and backward kernels: one of each kind has blocks
-    L.grid = (unsigned)(k >= FK_CRAD && k <= FK_BWDW && k != FK_NET ? g : std::max<int64_t>(g, 1));
+    // the radial, angular and backward kernels and the second half: one of each kind has blocks
+    L.grid = (unsigned)(k >= FK_CRAD && k <= FK_SECONDW && k != FK_NET ? g : std::max<int64_t>(g, 1));
     // the argument block of slot `kind` as the kernel parameter (all but the rebuild group)
     const FusedTables &t = so.t;
     size_t first = 0, second = 0;
@@ -469,7 +472,7 @@ Launch solo_launch(const Sys &s, int k, int kind) {
     const unsigned char *h = so.host.data();
     switch (k) {
         case FK_FIRST: L.solo = h + t.o_first + kind * first; break;
-        case FK_SECOND: L.solo = h + t.o_second + kind * second; break;
+        case FK_SECOND: case FK_SECONDW: L.solo = h + t.o_second + kind * second; break;
         case FK_CRAD: case FK_CRADW: case FK_ANG: case FK_ANGW: case FK_BWD: case FK_BWDW: L.solo = h + t.o_eval + kind * fused_eval_size(s.prec); break;
         case FK_NET: L.solo = h + t.o_net + kind * fused_net_size(s.prec); break;
         default:   // the rebuild group: a conditional one returns at once on the system's flag

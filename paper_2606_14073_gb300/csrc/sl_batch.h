@@ -23,16 +23,17 @@ namespace sl {
 // kernels of one step, in launch order
 enum FusedKernel {
     FK_FIRST, FK_BIN, FK_SCAN, FK_SCATTER, FK_CELLSORT, FK_LISTS, FK_REV, FK_FINISH,
-    FK_CRAD, FK_CRADW, FK_ANG, FK_ANGW, FK_NET, FK_BWD, FK_BWDW, FK_SECOND, FK_N
+    FK_CRAD, FK_CRADW, FK_ANG, FK_ANGW, FK_NET, FK_BWD, FK_BWDW, FK_SECOND, FK_SECONDW,
+    FK_N
 };
 // plan, the kernels (FP64 has the wide radial kernel only), the flag clear
 inline int fused_launches_per_step(int prec) { return 1 + FK_N + 1 - (prec == 0); }
 constexpr int FUSED_MAX_SLOTS = 4096;
-// atoms-per-block classes of the kernels that take one work item per block: the halves (256
+// atoms-per-block classes of the kernels that take one work item per block: the first half (256
 // atoms), the one-thread-per-atom radial kernel (128), the angular and backward kernels (a quad
 // block's atoms), the wide radial kernel and the FP64 network (8), the wide angular and backward
-// kernels (one per warp of a quad block)
-enum { IC_HALF = 0, IC_ATOM = 1, IC_QUAD = 2, IC_OCT = 3, IC_WARP = 4, IC_N = 5 };
+// kernels (one per warp of a quad block), the second half (256) and its wide form
+enum { IC_FIRST = 0, IC_ATOM = 1, IC_QUAD = 2, IC_OCT = 3, IC_WARP = 4, IC_SECOND = 5, IC_GATHER = 6, IC_N = 7 };
 
 // what a slot's entries are set up for
 enum SlotKind {
@@ -91,6 +92,7 @@ A solo_args(const Launch &L) {
     return a;
 }
 
+int64_t second_wide_atoms(int prec);   // atoms per block of the wide second half (sl_integrate.cu)
 // sizes of the per-slot argument blocks (sl_integrate.cu, sl_eval2.cu, sl_nep.cu)
 void fused_half_sizes(int prec, size_t *first, size_t *second);
 size_t fused_eval_size(int prec);
@@ -111,7 +113,7 @@ void fused_grid_net(FusedTables &t);
 // launches over a table
 void launch_fused_plan(const FusedTables &t, cudaStream_t st);
 void launch_first_half_t(const FusedTables &t, const Launch &L, cudaStream_t st);
-void launch_second_half_t(const FusedTables &t, const Launch &L, bool spin, cudaStream_t st);
+void launch_second_half_t(const FusedTables &t, const Launch &L, const Launch &W, bool spin, cudaStream_t st);
 // the rebuild group: L[0 .. 5] for the binning, scan, scatter, lists, reverse slots and finish
 // kernels; clear: then the flags of the conditional slots in L[0]'s map are cleared; loop: the
 // persistent form (a batch's), else one work item per block (a system's own launches)

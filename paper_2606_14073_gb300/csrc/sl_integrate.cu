@@ -132,17 +132,17 @@ __device__ __forceinline__ void first_half_body(const IntArgs &a, int64_t blk) {
 
 // SPIN = false (midpoint mode): the spins were already advanced by the midpoint
 // iteration; only the gather, the final kick and the carried F, H remain.
-template <typename R, bool MIXED, bool SPIN = true>
-__device__ __forceinline__ void second_half_body(const IntArgs &a, const GatherArgs<R> &g, int64_t blk) {
-    const int64_t i = blk * (int64_t)blockDim.x + threadIdx.x;
+template <typename R, bool MIXED, int W, bool SPIN = true>
+__device__ __forceinline__ void second_half_body(const IntArgs &a, const GatherArgs<R> &g, int64_t blk,
+                                                 GatherSmem<R, W> &sm) {
+    double Fs[3], Hs[3];
+    const int64_t i = gather_block<R, W>(g, blk, sm, Fs, Hs);
     if (i == 0) a.step[0] = a.step[1] + 1;
-    if (i >= a.n) return;
+    if (i < 0) return;
     const StepDev &P = *a.par;
     const int t = i < a.n_fe ? 0 : 1;
     const uint64_t id = (uint64_t)a.orig[i];
     const unsigned long long st = a.step[1];
-    double Fs[3], Hs[3];
-    gather<R>(g, i, Fs, Hs);
     Hs[0] += P.zee[t][0]; Hs[1] += P.zee[t][1]; Hs[2] += P.zee[t][2];
     if (a.Bat) {
         const double4 b = a.Bat[i];
@@ -213,7 +213,7 @@ __device__ __forceinline__ void second_half_body(const IntArgs &a, const GatherA
 }
 
 // The halves over an argument table (sl_batch.h: a system's own table or a batch's), one
-// 256-thread block per 256 atoms of a slot.
+// 256-thread block per 256 atoms of a slot (second half: gather_atoms).
 template <typename R>
 struct HalfArgs {
     IntArgs a;
@@ -227,20 +227,31 @@ __global__ void __launch_bounds__(256) k_first_half(const IntArgs *__restrict__ 
 template <typename R, bool MIXED, bool SPIN>
 __global__ void __launch_bounds__(256) k_second_half(const HalfArgs<R> *__restrict__ tab, SlotMap sm,
                                                      const __grid_constant__ HalfArgs<R> solo) {
-    one_work(tab, sm, solo,
-             [](const HalfArgs<R> &h, int64_t blk, int64_t) { second_half_body<R, MIXED, SPIN>(h.a, h.g, blk); });
+    __shared__ GatherSmem<R, 1> scratch;
+    one_work(tab, sm, solo, [&](const HalfArgs<R> &h, int64_t blk, int64_t) {
+        second_half_body<R, MIXED, 1, SPIN>(h.a, h.g, blk, scratch);
+    });
+}
+// the same with several lanes per atom in the gather (gather_is_wide)
+template <typename R, bool MIXED, bool SPIN>
+__global__ void __launch_bounds__(256) k_second_wide(const HalfArgs<R> *__restrict__ tab, SlotMap sm,
+                                                     const __grid_constant__ HalfArgs<R> solo) {
+    __shared__ GatherSmem<R, GATHER_WIDE<R>> scratch;
+    one_work(tab, sm, solo, [&](const HalfArgs<R> &h, int64_t blk, int64_t) {
+        second_half_body<R, MIXED, GATHER_WIDE<R>, SPIN>(h.a, h.g, blk, scratch);
+    });
 }
 
 // Forces and fields at the current state into (Fo, Ho).
-template <typename R>
+template <typename R, int W>
 __global__ void __launch_bounds__(256) k_gather_only(GatherArgs<R> g, const StepDev *par, int64_t n_fe,
                                                      double4 *Fo, double4 *Ho, int *status, const double4 *Bat,
                                                      const double4 *spin) {
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= g.n) return;
-    const int t = i < n_fe ? 0 : 1;
+    __shared__ GatherSmem<R, W> sm;
     double Fs[3], Hs[3];
-    gather<R>(g, i, Fs, Hs);
+    const int64_t i = gather_block<R, W>(g, blockIdx.x, sm, Fs, Hs);
+    if (i < 0) return;
+    const int t = i < n_fe ? 0 : 1;
     Hs[0] += par->zee[t][0]; Hs[1] += par->zee[t][1]; Hs[2] += par->zee[t][2];
     if (Bat) {
         const double4 b = Bat[i];
@@ -259,16 +270,16 @@ __global__ void __launch_bounds__(256) k_gather_only(GatherArgs<R> g, const Step
 // FP64; eta is the step's thermal field (the spin stream's normals of this step, as in the
 // predictor-corrector).  The field is gathered from the pair records of the evaluation just
 // made; spins of other colours are left alone.
-template <typename R, bool MIXED>
+template <typename R, bool MIXED, int W>
 __global__ void __launch_bounds__(256) k_sweep_rotate(IntArgs a, GatherArgs<R> g, const int32_t *colour, int c) {
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= a.n || colour[i] != c) return;
+    __shared__ GatherSmem<R, W> sm;
+    double Fs[3], Hs[3];
+    const int64_t i = gather_block<R, W>(g, blockIdx.x, sm, Fs, Hs);
+    if (i < 0 || colour[i] != c) return;
     const StepDev &P = *a.par;
     const int t = i < a.n_fe ? 0 : 1;
     const uint64_t id = (uint64_t)a.orig[i];
     const unsigned long long st = a.step[1];
-    double Fs[3], Hs[3];
-    gather<R>(g, i, Fs, Hs);
     Hs[0] += P.zee[t][0]; Hs[1] += P.zee[t][1]; Hs[2] += P.zee[t][2];
     if (a.Bat) {
         const double4 b = a.Bat[i];
@@ -329,44 +340,53 @@ void launch_first_half_t(const FusedTables &t, const Launch &L, cudaStream_t st)
     else k_first_half<true><<<L.grid, 256, 0, st>>>(tab, L.slots(), so);
 }
 
+// L, W: the launches of the one-lane and the wide form (a grid of 0: not launched)
 template <typename R, bool MIXED>
-static void second_half_t(const FusedTables &t, const Launch &L, bool spin, cudaStream_t st) {
+static void second_half_t(const FusedTables &t, const Launch &L, const Launch &W, bool spin, cudaStream_t st) {
     const HalfArgs<R> *tab = L.solo ? nullptr : t.at<HalfArgs<R>>(t.o_second);
     const HalfArgs<R> so = solo_args<HalfArgs<R>>(L);
-    if (spin) k_second_half<R, MIXED, true><<<L.grid, 256, 0, st>>>(tab, L.slots(), so);
-    else k_second_half<R, MIXED, false><<<L.grid, 256, 0, st>>>(tab, L.slots(), so);
+    if (L.grid && spin) k_second_half<R, MIXED, true><<<L.grid, 256, 0, st>>>(tab, L.slots(), so);
+    else if (L.grid) k_second_half<R, MIXED, false><<<L.grid, 256, 0, st>>>(tab, L.slots(), so);
+    if (W.grid && spin) k_second_wide<R, MIXED, true><<<W.grid, 256, 0, st>>>(tab, W.slots(), so);
+    else if (W.grid) k_second_wide<R, MIXED, false><<<W.grid, 256, 0, st>>>(tab, W.slots(), so);
 }
-void launch_second_half_t(const FusedTables &t, const Launch &L, bool spin, cudaStream_t st) {
-    if (t.prec == 0) second_half_t<double, false>(t, L, spin, st);
-    else second_half_t<float, true>(t, L, spin, st);
+void launch_second_half_t(const FusedTables &t, const Launch &L, const Launch &W, bool spin, cudaStream_t st) {
+    if (t.prec == 0) second_half_t<double, false>(t, L, W, spin, st);
+    else second_half_t<float, true>(t, L, W, spin, st);
 }
 
 // a system's own launches, over its table
 void launch_first_half(Sys &s) { launch_first_half_t(s.solo->t, solo_launch(s, FK_FIRST, SK_STEP), s.stream); }
 void launch_second_half(Sys &s) {
-    launch_second_half_t(s.solo->t, solo_launch(s, FK_SECOND, SK_STEP), true, s.stream);
+    launch_second_half_t(s.solo->t, solo_launch(s, FK_SECOND, SK_STEP), solo_launch(s, FK_SECONDW, SK_STEP), true,
+                         s.stream);
 }
 void launch_second_half_nospin(Sys &s) {
-    launch_second_half_t(s.solo->t, solo_launch(s, FK_SECOND, SK_STEP), false, s.stream);
+    launch_second_half_t(s.solo->t, solo_launch(s, FK_SECOND, SK_STEP), solo_launch(s, FK_SECONDW, SK_STEP), false,
+                         s.stream);
 }
 
+template <typename R, bool MIXED, int W>
+static void sweep_rotate(Sys &s, int c) {
+    k_sweep_rotate<R, MIXED, W><<<nblk(s.n, gather_atoms(W)), 256, 0, s.stream>>>(int_args(s), gather_args<R>(s),
+                                                                                 s.colour, c);
+}
 void launch_sweep_rotate(Sys &s, int c) {
-    if (s.prec == 0)
-        k_sweep_rotate<double, false><<<nblk(s.n, 256), 256, 0, s.stream>>>(int_args(s), gather_args<double>(s),
-                                                                            s.colour, c);
-    else
-        k_sweep_rotate<float, true><<<nblk(s.n, 256), 256, 0, s.stream>>>(int_args(s), gather_args<float>(s),
-                                                                          s.colour, c);
+    const bool wide = gather_is_wide(s);
+    if (s.prec == 0) wide ? sweep_rotate<double, false, GATHER_WIDE<double>>(s, c) : sweep_rotate<double, false, 1>(s, c);
+    else wide ? sweep_rotate<float, true, GATHER_WIDE<float>>(s, c) : sweep_rotate<float, true, 1>(s, c);
 }
 
+template <typename R, int W>
+static void gather_only(Sys &s, double4 *Fo, double4 *Ho) {
+    k_gather_only<R, W><<<nblk(s.n, gather_atoms(W)), 256, 0, s.stream>>>(gather_args<R>(s), s.d_par, s.n_fe, Fo, Ho,
+                                                                          s.status, s.Bat, s.spin);
+}
 void launch_gather(Sys &s, bool carried) {
     double4 *Fo = carried ? s.F : s.Fo, *Ho = carried ? s.H : s.Ho;
-    if (s.prec == 0)
-        k_gather_only<double><<<nblk(s.n, 256), 256, 0, s.stream>>>(gather_args<double>(s), s.d_par, s.n_fe, Fo, Ho,
-                                                                    s.status, s.Bat, s.spin);
-    else
-        k_gather_only<float><<<nblk(s.n, 256), 256, 0, s.stream>>>(gather_args<float>(s), s.d_par, s.n_fe, Fo, Ho,
-                                                                   s.status, s.Bat, s.spin);
+    const bool wide = gather_is_wide(s);
+    if (s.prec == 0) wide ? gather_only<double, GATHER_WIDE<double>>(s, Fo, Ho) : gather_only<double, 1>(s, Fo, Ho);
+    else wide ? gather_only<float, GATHER_WIDE<float>>(s, Fo, Ho) : gather_only<float, 1>(s, Fo, Ho);
 }
 
 // Sets *diff when the evaluation outputs (Fo, Ho) differ in any bit from ref ([n] forces,
@@ -386,6 +406,7 @@ __global__ void k_compare_bits(const double4 *__restrict__ Fo, const double4 *__
 }
 
 // ---- fused batch step (sl_batch.h)
+int64_t second_wide_atoms(int prec) { return gather_atoms(prec == 0 ? GATHER_WIDE<double> : GATHER_WIDE<float>); }
 void fused_half_sizes(int prec, size_t *first, size_t *second) {
     *first = sizeof(IntArgs);
     *second = prec == 0 ? sizeof(HalfArgs<double>) : sizeof(HalfArgs<float>);
@@ -396,7 +417,9 @@ void fused_put_half(Sys &s, int r, const FusedTables &t, unsigned char *img, int
     reinterpret_cast<IntArgs *>(img + t.o_first)[r] = a;
     if (s.prec == 0) reinterpret_cast<HalfArgs<double> *>(img + t.o_second)[r] = HalfArgs<double>{a, gather_args<double>(s)};
     else reinterpret_cast<HalfArgs<float> *>(img + t.o_second)[r] = HalfArgs<float>{a, gather_args<float>(s)};
-    blocks[FK_FIRST] = blocks[FK_SECOND] = nblk(s.n, 256);
+    blocks[FK_FIRST] = nblk(s.n, 256);
+    blocks[FK_SECOND] = gather_is_wide(s) ? 0 : nblk(s.n, gather_atoms(1));
+    blocks[FK_SECONDW] = gather_is_wide(s) ? nblk(s.n, second_wide_atoms(s.prec)) : 0;
 }
 
 void launch_compare_bits(Sys &s, const double4 *ref, int *diff) {

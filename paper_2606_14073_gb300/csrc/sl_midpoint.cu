@@ -82,15 +82,15 @@ __global__ void __launch_bounds__(256) k_mid_prep(MidArgs a, int m) {
     a.midsf[i] = make_float4((float)(mx * inv), (float)(my * inv), (float)(mz * inv), 0.f);
 }
 
-template <typename R, bool MIXED>
+template <typename R, bool MIXED, int W>
 __global__ void __launch_bounds__(256) k_mid_update(MidArgs a, GatherArgs<R> g, int m) {
     if (a.md->converged) return;
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= a.n) return;
+    __shared__ GatherSmem<R, W> sm;
+    double Fs[3], Hs[3];
+    const int64_t i = gather_block<R, W>(g, blockIdx.x, sm, Fs, Hs);
+    if (i < 0) return;
     const StepDev &P = *a.par;
     const int t = i < a.n_fe ? 0 : 1;
-    double Fs[3], Hs[3];
-    gather<R>(g, i, Fs, Hs);
     Hs[0] += P.zee[t][0]; Hs[1] += P.zee[t][1]; Hs[2] += P.zee[t][2];
     if (a.Bat) {
         const double4 b = a.Bat[i];
@@ -299,10 +299,16 @@ int midpoint_kernels_per_step(const Sys &s) {
 
 size_t midpoint_scratch_doubles() { return (size_t)AA_BLOCKS * AA_VALS; }
 
+template <typename R, bool MIXED, int W>
+static void mid_update(Sys &s, const MidArgs &a, int m) {
+    k_mid_update<R, MIXED, W><<<nblk(s.n, gather_atoms(W)), 256, 0, s.stream>>>(a, mid_gather_args<R>(s), m);
+}
+
 int launch_midpoint(Sys &s) {
     if (s.mid_iters <= 0 || s.n == 0) return 0;
     const MidArgs a = mid_args(s);
     const unsigned nb = nblk(s.n, 256);
+    const bool wide = gather_is_wide(s);
     k_mid_start<<<1, 64, 0, s.stream>>>(s.md, s.mid_iters);
     EvalAt at;
     at.pos = s.posmid; at.posf = s.posmidf; at.spin = s.mids; at.spinf = s.midsf;
@@ -312,8 +318,8 @@ int launch_midpoint(Sys &s) {
         s.at = at;
         launch_eval(s, false);
         s.at = EvalAt();
-        if (s.prec == 0) k_mid_update<double, false><<<nb, 256, 0, s.stream>>>(a, mid_gather_args<double>(s), m);
-        else k_mid_update<float, true><<<nb, 256, 0, s.stream>>>(a, mid_gather_args<float>(s), m);
+        if (s.prec == 0) wide ? mid_update<double, false, GATHER_WIDE<double>>(s, a, m) : mid_update<double, false, 1>(s, a, m);
+        else wide ? mid_update<float, true, GATHER_WIDE<float>>(s, a, m) : mid_update<float, true, 1>(s, a, m);
         k_mid_check<<<1, 1, 0, s.stream>>>(s.md, m, s.mid_iters, s.mid_tol);
         if (s.aa_depth > 0) {
             k_aa_dots<<<AA_BLOCKS, 256, 0, s.stream>>>(a, m);

@@ -6,6 +6,7 @@
 
 #include "sl_common.cuh"
 #include "sl_eval2.cuh"
+#include "sl_internal.h"
 
 namespace sl {
 
@@ -64,29 +65,80 @@ __device__ __forceinline__ void omega_of_f(float sx, float sy, float sz, float h
 }
 
 // F_k = sum_j dE_k/dr_kj - sum_j dE_j/dr_jk, H_k = -dE_k/dS_k - sum_j dE_j/dS_k: the
-// records (dE_j/dr_jk, dE_j/dS_k) sit in k's own in-cutoff candidate slots.  The slots
-// are walked in order by the whole warp at once, so the records that neighbouring atoms
-// read at one slot are neighbours in memory (slot-major layout).
+// records (dE_j/dr_jk, dE_j/dS_k) sit in k's own in-cutoff candidate slots.  W lanes take an atom;
+// lane q walks the slots s = q mod W in order with the other lanes of its warp, so the records
+// that neighbouring atoms read at one slot are neighbours in memory (slot-major layout); the
+// lanes' sums are added in a fixed order.  What bounds it: the records' DRAM traffic in large systems (two 16-byte loads per
+// record), and in small ones the chain of a lane's slots, a few loads in flight at a time: so a
+// small system (gather_is_wide) takes several lanes per atom, a larger one one.  Second half, mixed
+// precision, 512 / 13,824 / 32,768 / 110,592 atoms: 17 / 21 / 32 / 89 us with four lanes, 29 / 34 / 45 / 85
+// with one; FP64, 512 / 13,824 / 32,768 atoms: 32 / 54 / 121 us with eight, 90 / 109 / 121 with one.
 template <typename R>
-__device__ __forceinline__ void gather(const GatherArgs<R> &g, int64_t k, double F[3], double H[3]) {
-    const v4<R> fo = ro(g.fown + k), gi = ro(g.gii + k);
-    R fx = fo.x, fy = fo.y, fz = fo.z, hx = -gi.x, hy = -gi.y, hz = -gi.z;
+constexpr int GATHER_WIDE = sizeof(R) == 4 ? 4 : 8;
+constexpr int gather_atoms(int W) { return 256 / W; }   // atoms per 256-thread block
+inline bool gather_is_wide(const Sys &s) { return s.n <= (s.prec == 0 ? 16384 : 65536); }
+
+template <typename R, int W>
+struct GatherSmem {
+    R v[W == 1 ? 1 : 6][W == 1 ? 1 : gather_atoms(W)];   // (unused with one lane per atom)
+};
+
+// Sums of one atom's own part and records, its lane q of W.
+template <typename R, int W>
+__device__ __forceinline__ void gather_lane(const GatherArgs<R> &g, int64_t k, int q, R v[6]) {
     const int64_t N = g.n;
+#pragma unroll
+    for (int c = 0; c < 6; ++c) v[c] = R(0);
+    if (q == 0) {
+        const v4<R> fo = ro(g.fown + k), gi = ro(g.gii + k);
+        v[0] = fo.x; v[1] = fo.y; v[2] = fo.z;
+        v[3] = -gi.x; v[4] = -gi.y; v[5] = -gi.z;
+    }
 #pragma unroll 1
     for (int w = 0; w < g.maskw; ++w) {
         const uint32_t word = ro(g.mask + (int64_t)w * N + k);
 #pragma unroll 4
-        for (int b = 0; b < 32; ++b) {
+        for (int b = q; b < 32; b += W) {
             if ((word >> b) & 1u) {
                 const PairRec<R> *e = g.pd + (int64_t)(w * 32 + b) * N + k;
                 const v4<R> ea = ro(&e->a), eb = ro(&e->b);
-                fx -= ea.x; fy -= ea.y; fz -= ea.z;
-                hx -= ea.w; hy -= eb.x; hz -= eb.y;
+                v[0] -= ea.x; v[1] -= ea.y; v[2] -= ea.z;
+                v[3] -= ea.w; v[4] -= eb.x; v[5] -= eb.y;
             }
         }
     }
-    F[0] = (double)fx; F[1] = (double)fy; F[2] = (double)fz;
-    H[0] = (double)hx; H[1] = (double)hy; H[2] = (double)hz;
+}
+
+// The atoms of block blk of 256 threads: the atom of this thread (-1: none) and its sums F, H.
+template <typename R, int W>
+__device__ __forceinline__ int64_t gather_block(const GatherArgs<R> &g, int64_t blk, GatherSmem<R, W> &sm, double F[3],
+                                                double H[3]) {
+    const int64_t i = blk * gather_atoms(W) + threadIdx.x;   // the thread's atom afterwards
+    R v[6];
+    if constexpr (W == 1) {
+        if (i >= g.n) return -1;
+        gather_lane<R, 1>(g, i, 0, v);
+    } else {
+        const int at = threadIdx.x / W, q = threadIdx.x % W;
+        const int64_t k = blk * gather_atoms(W) + at;
+        gather_lane<R, W>(g, k < g.n ? k : g.n - 1, q, v);
+#pragma unroll
+        for (int c = 0; c < 6; ++c) {
+#pragma unroll
+            for (int o = 1; o < W; o <<= 1) v[c] += __shfl_xor_sync(0xffffffffu, v[c], o);
+            if (q == 0) sm.v[c][at] = v[c];
+        }
+        __syncthreads();
+        if (threadIdx.x >= gather_atoms(W) || i >= g.n) return -1;
+#pragma unroll
+        for (int c = 0; c < 6; ++c) v[c] = sm.v[c][threadIdx.x];
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        F[c] = (double)v[c];
+        H[c] = (double)v[3 + c];
+    }
+    return i;
 }
 
 }  // namespace sl
