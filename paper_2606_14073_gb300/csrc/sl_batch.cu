@@ -442,6 +442,16 @@ void solo_free(Sys &s) {
     s.solo = nullptr;
 }
 
+// Threads per block of a half of the step over `threads` threads: 256, or fewer (at least `least`) while
+// that leaves SMs without a block.  The halves' FP64 state arithmetic occupies an SM's pipe for 64
+// cycles a warp instruction and scheduler, so a small system's few warps are spread: first half at
+// 512 atoms 10 instead of 12 us mixed and 21 instead of 36 us FP64, second half 28 instead of 32 us FP64.
+static int half_block(int64_t threads, int sms, int least) {
+    int b = 256;
+    while (b > least && threads < (int64_t)b * sms) b >>= 1;
+    return b;
+}
+
 Launch solo_launch(const Sys &s, int k, int kind) {
     const SoloTables &so = *s.solo;
     Launch L;
@@ -462,6 +472,14 @@ Launch solo_launch(const Sys &s, int k, int kind) {
     }
     L.m = so.map(k, kind, shape);
     int64_t g = so.blocks[k][shape];
+    if (k == FK_FIRST) {
+        L.block = half_block(s.n, so.sms, 32);
+        g = (s.n + L.block - 1) / L.block;
+    } else if (k == FK_SECONDW && g > 0) {
+        const int64_t lanes = 256 / second_wide_atoms(s.prec);
+        L.block = half_block(s.n * lanes, so.sms, 64);
+        g = (s.n * lanes + L.block - 1) / L.block;
+    }
     if (k == FK_NET && s.prec != 0) g = std::min<int64_t>(g, (int64_t)so.sms * s.cfg.mlp_ctas_per_sm);   // persistent
     // the radial, angular and backward kernels and the second half: one of each kind has blocks
     L.grid = (unsigned)(k >= FK_CRAD && k <= FK_SECONDW && k != FK_NET ? g : std::max<int64_t>(g, 1));

@@ -213,7 +213,8 @@ __device__ __forceinline__ void second_half_body(const IntArgs &a, const GatherA
 }
 
 // The halves over an argument table (sl_batch.h: a system's own table or a batch's), one
-// 256-thread block per 256 atoms of a slot (second half: gather_atoms).
+// 256-thread block per 256 atoms of a slot (second half: gather_atoms; a small system's own launches:
+// smaller blocks, solo_launch).
 template <typename R>
 struct HalfArgs {
     IntArgs a;
@@ -336,8 +337,9 @@ static inline unsigned nblk(int64_t n, int t) { return (unsigned)((n + t - 1) / 
 void launch_first_half_t(const FusedTables &t, const Launch &L, cudaStream_t st) {
     const IntArgs *tab = L.solo ? nullptr : t.at<IntArgs>(t.o_first);
     const IntArgs so = solo_args<IntArgs>(L);
-    if (t.prec == 0) k_first_half<false><<<L.grid, 256, 0, st>>>(tab, L.slots(), so);
-    else k_first_half<true><<<L.grid, 256, 0, st>>>(tab, L.slots(), so);
+    const int b = L.block ? L.block : 256;
+    if (t.prec == 0) k_first_half<false><<<L.grid, b, 0, st>>>(tab, L.slots(), so);
+    else k_first_half<true><<<L.grid, b, 0, st>>>(tab, L.slots(), so);
 }
 
 // L, W: the launches of the one-lane and the wide form (a grid of 0: not launched)
@@ -347,8 +349,9 @@ static void second_half_t(const FusedTables &t, const Launch &L, const Launch &W
     const HalfArgs<R> so = solo_args<HalfArgs<R>>(L);
     if (L.grid && spin) k_second_half<R, MIXED, true><<<L.grid, 256, 0, st>>>(tab, L.slots(), so);
     else if (L.grid) k_second_half<R, MIXED, false><<<L.grid, 256, 0, st>>>(tab, L.slots(), so);
-    if (W.grid && spin) k_second_wide<R, MIXED, true><<<W.grid, 256, 0, st>>>(tab, W.slots(), so);
-    else if (W.grid) k_second_wide<R, MIXED, false><<<W.grid, 256, 0, st>>>(tab, W.slots(), so);
+    const int b = W.block ? W.block : 256;
+    if (W.grid && spin) k_second_wide<R, MIXED, true><<<W.grid, b, 0, st>>>(tab, W.slots(), so);
+    else if (W.grid) k_second_wide<R, MIXED, false><<<W.grid, b, 0, st>>>(tab, W.slots(), so);
 }
 void launch_second_half_t(const FusedTables &t, const Launch &L, const Launch &W, bool spin, cudaStream_t st) {
     if (t.prec == 0) second_half_t<double, false>(t, L, W, spin, st);

@@ -109,18 +109,19 @@ __device__ __forceinline__ void gather_lane(const GatherArgs<R> &g, int64_t k, i
     }
 }
 
-// The atoms of block blk of 256 threads: the atom of this thread (-1: none) and its sums F, H.
+// The atoms of block blk (blockDim.x / W of them): the atom of this thread (-1: none) and its sums F, H.
 template <typename R, int W>
 __device__ __forceinline__ int64_t gather_block(const GatherArgs<R> &g, int64_t blk, GatherSmem<R, W> &sm, double F[3],
                                                 double H[3]) {
-    const int64_t i = blk * gather_atoms(W) + threadIdx.x;   // the thread's atom afterwards
+    const int per = blockDim.x / W;
+    const int64_t i = blk * per + threadIdx.x;   // the thread's atom afterwards
     R v[6];
     if constexpr (W == 1) {
         if (i >= g.n) return -1;
         gather_lane<R, 1>(g, i, 0, v);
     } else {
         const int at = threadIdx.x / W, q = threadIdx.x % W;
-        const int64_t k = blk * gather_atoms(W) + at;
+        const int64_t k = blk * per + at;
         gather_lane<R, W>(g, k < g.n ? k : g.n - 1, q, v);
 #pragma unroll
         for (int c = 0; c < 6; ++c) {
@@ -129,7 +130,7 @@ __device__ __forceinline__ int64_t gather_block(const GatherArgs<R> &g, int64_t 
             if (q == 0) sm.v[c][at] = v[c];
         }
         __syncthreads();
-        if (threadIdx.x >= gather_atoms(W) || i >= g.n) return -1;
+        if (threadIdx.x >= per || i >= g.n) return -1;
 #pragma unroll
         for (int c = 0; c < 6; ++c) v[c] = sm.v[c][threadIdx.x];
     }
