@@ -149,7 +149,7 @@ void free_sys(sl::Sys &s) {
                     s.wpart, s.Fo, s.Ho,
                     s.status, s.rebuild, s.d_step, s.d_par, s.red, s.snap, s.d_builds,
                     s.posmid, s.posmidf, s.mids, s.midsf, s.mx, s.mg, s.aax, s.aag, s.aapart, s.md, s.Bat,
-                    s.tex_acc, s.tex_m, s.tex_part, s.colour, s.mlp_img};
+                    s.tex_acc, s.tex_m, s.tex_part, s.colour, s.mlp_img, s.rb_count};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     sl::solo_free(s);
@@ -214,7 +214,9 @@ void enqueue_step(sl::Sys &s) {
     }
 }
 
-int64_t kernels_per_step(const sl::Sys &s) { return sl::KERNELS_PER_STEP + sl::midpoint_kernels_per_step(s); }
+// (a one-launch rebuild takes one of the eight launches of its group)
+int64_t step_kernels(const sl::Sys &s) { return sl::KERNELS_PER_STEP - (s.rb_count ? 7 : 0); }
+int64_t kernels_per_step(const sl::Sys &s) { return step_kernels(s) + sl::midpoint_kernels_per_step(s); }
 
 // Evaluate at the current state: optional unconditional rebuild, eval, gather.
 int evaluate(sl::Sys &s, bool rebuild, bool carried, bool want_virial) {
@@ -236,7 +238,10 @@ int check_status(sl::Sys &s) {
     if (st & sl::ST_NBR_OVERFLOW)
         return fail(SL_ENBR_OVERFLOW, "neighbour list capacity exceeded (caps %d/%d)", s.cap, s.cap_ang);
     if (st & sl::ST_NONFINITE) return fail(SL_ENONFINITE, "non-finite force or field");
-    if (st & sl::ST_TIMEOUT) return fail(SL_ETIMEOUT, "a bounded device wait gave up (tensor-core network)");
+    if (st & sl::ST_TIMEOUT) {
+        if (s.rb_count) CK(cudaMemsetAsync(s.rb_count, 0, sizeof(unsigned long long), s.stream));
+        return fail(SL_ETIMEOUT, "a bounded device wait gave up (tensor-core network or list rebuild)");
+    }
     if (st & sl::ST_MID_RANGE)
         return fail(SL_ENBR_OVERFLOW, "midpoint configuration moved beyond skin/2 of the list positions");
     return SL_OK;
@@ -573,6 +578,7 @@ int sl_create_system(const double *positions, const double *spins, const double 
         (rc = dalloc(&s.rebuild, 1)) || (rc = dalloc(&s.d_step, 2)) || (rc = dalloc(&s.d_par, 1)) ||
         (rc = dalloc(&s.red, 256 * 10 + 10)) || (rc = dalloc(&s.snap, 5 * N)) || (rc = dalloc(&s.d_builds, 1)))
         return bail(rc);
+    if (sl::make_rebuild_one(s)) return bail(fail(SL_ENOMEM, "the rebuild's barrier count"));
     if (n > 0 && sl::make_coeff_table(s)) return bail(fail(SL_ENOMEM, "the coefficient table could not be made"));
     if (sl::make_net_table(s)) return bail(fail(SL_ENOMEM, "the network's weight table could not be made"));
     if (s.prec == SL_PREC_MIXED && n > 0 && sl::make_q_tensor_map(s))
@@ -780,7 +786,7 @@ static int sweep_step(sl::Sys &s) {
     sl::launch_second_half_nospin(s);
     CK(cudaGetLastError());
     s.sweep_evaluations += 2 * C + 1;
-    s.n_launches += sl::KERNELS_PER_STEP + (int64_t)2 * C * 5;
+    s.n_launches += step_kernels(s) + (int64_t)2 * C * 5;
     return SL_OK;
 }
 

@@ -137,6 +137,10 @@ struct Sys {
     void *wpart = nullptr;     // [9][n] per-atom virial parts
     double4 *Fo = nullptr, *Ho = nullptr;   // evaluation outputs (not the carried F, H)
 
+    // the one-launch rebuild (sl_neighbors.cu; null: the kernels one by one): its barrier's count, its grid
+    unsigned long long *rb_count = nullptr;
+    int rb_grid = 0;
+
     // control
     int *status = nullptr;     // device status bits
     int *rebuild = nullptr;    // device rebuild flag
@@ -228,6 +232,9 @@ inline bool crad_is_wide(const Sys &s) { return s.prec == 0 || s.n <= CRAD_WIDE_
 // small systems, else four lanes per atom (both timed at k_ang_wide).
 constexpr int64_t EVAL_WIDE_MAX64 = 3040, EVAL_WIDE_MAX32 = 2048;
 inline bool eval_is_wide(const Sys &s) { return s.n <= (s.prec == 0 ? EVAL_WIDE_MAX64 : EVAL_WIDE_MAX32); }
+// The largest system whose own rebuilds take one launch (both timed at k_rebuild_one).
+constexpr int64_t REBUILD_ONE_MAX = 131072;
+int make_rebuild_one(Sys &s);
 void nbr_setup(Sys &s);
 void launch_rebuild(Sys &s, bool conditional);
 // sl_eval2.cu: the system's evaluation at the state (with the virial parts when asked for), or

@@ -19,6 +19,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
+#include <cstring>
 
 #include "sl_internal.h"
 #include "sl_batch.h"
@@ -76,8 +77,8 @@ __device__ __forceinline__ void bin_body(const BinArgs &r, int64_t blk, int64_t 
 // shared memory, for the starts it writes (a shuffle scan per 32 cells with a running carry).
 __device__ __forceinline__ void scan_body(const BinArgs &r, int *s_part) {
     if (r.flag && *r.flag == 0) return;
-    const int *__restrict__ count = r.count;
-    int *__restrict__ start = r.start;
+    const int *count = r.count;   // (not restrict: k_rebuild_one reads what another block of it wrote)
+    int *start = r.start;
     const int m = r.ncell, lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int chunk = ((m + nw - 1) / nw + 31) & ~31;
     const int b0 = min(wid * chunk, m), b1 = min(b0 + chunk, m);
@@ -407,7 +408,8 @@ __device__ __forceinline__ void list_atom(const ListArgs &a, int64_t i, float4 p
     __syncwarp();
 }
 
-// Cells blk, blk + nblk, ... of the grid (a block-uniform loop).
+// Items blk, blk + nblk, ... (a block-uniform loop): part k of a.parts of a cell's atoms (every part
+// stages the stencil; more than one part where a box has fewer cells than the GPU has SMs).
 __device__ __forceinline__ void lists_body(const ListArgs &args, int64_t blk, int64_t nblk, ListSmem &sm) {
     const ListArgs a = args;   // as values: the stores below cannot make the compiler re-read them
     if (a.flag && *a.flag == 0) return;
@@ -419,7 +421,9 @@ __device__ __forceinline__ void lists_body(const ListArgs &args, int64_t blk, in
 #pragma unroll
     for (int d = 0; d < 3; ++d) image_placed = image_placed && (!a.g.per[d] || a.g.nc[d] >= 3);
     const float4 far = make_float4(1e30f, 1e30f, 1e30f, 0.f);
-    for (int64_t c = blk; c < ncell; c += nblk) {
+    for (int64_t item = blk; item < (int64_t)ncell * a.parts; item += nblk) {
+        const int64_t c = (uint32_t)item / (uint32_t)a.parts;
+        const int part = (int)((uint32_t)item % (uint32_t)a.parts);
         // the stencil and each cell's offset in it (warp 0): the 27 cells around (an empty one
         // past a non-periodic face) when the images are placed, else lo..hi per axis, z-major
         if (w == 0) {
@@ -548,7 +552,7 @@ __device__ __forceinline__ void lists_body(const ListArgs &args, int64_t blk, in
         };
         // the cell's own atoms, one per warp
         const int c0 = a.cell_start[c], nc0 = a.cell_start[c + 1] - c0;
-        for (int q = w; q < nc0; q += LB_WARPS) {
+        for (int q = w + LB_WARPS * part; q < nc0; q += LB_WARPS * a.parts) {
             const int64_t i = a.cell_atoms[c0 + q];
             const float4 pfi = a.cposf[c0 + q];
             auto jof = [&](int f) { return sm.j[f]; };
@@ -615,7 +619,7 @@ __device__ __forceinline__ uint32_t zero_bytes4(uint32_t x) {
 // search runs the atom is in the segment unless a list was cut at its capacity (which the list
 // build has already reported): so a window that holds the whole segment and a single candidate
 // gives the slot; otherwise each candidate's entry is compared, in order.
-__device__ __forceinline__ int find_slot(const int32_t *__restrict__ row, const uint8_t *__restrict__ hrow, int lo,
+__device__ __forceinline__ int find_slot(const int32_t *row, const uint8_t *hrow, int lo,
                                          int hi, int ai) {
     const uint32_t hh = index_hash8(ai) * 0x01010101u;
     for (int b = lo & ~31; b < hi; b += 64) {
@@ -725,6 +729,10 @@ __device__ __forceinline__ void rebuild_items(const A *__restrict__ tab, const W
     else map_item(tab, m, body);
 }
 
+// parts of a cell's atoms in the list build at most: a cell of the densest boxes holds some 64 atoms, four
+// for each part's warps
+constexpr int LISTS_PARTS_MAX = 16;
+
 // register budget of a system's own list build (its 29 KB of staging allow 7 blocks per SM)
 constexpr int LISTS_MINB = 6;
 
@@ -773,6 +781,73 @@ __global__ void k_finish(const BinArgs *__restrict__ tab, WorkMap m, const int *
 __global__ void k_clear_flags(const BinArgs *__restrict__ tab, WorkMap m) {
     for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < m.nrep; r += gridDim.x * blockDim.x)
         if (m.w0[r + 1] > m.w0[r] && tab[r].flag) *tab[r].rebuild = 0;
+}
+
+// The whole group in one launch, for a system's own rebuild in a small system: a cooperative grid
+// whose blocks meet at a barrier between the phases.  In the steps without a rebuild, most of
+// them, it costs one empty launch instead of eight in a row: a step of 512 / 13,824 / 110,592 atoms 50 / 111 /
+// 549 instead of 56 / 122 / 558 us; with a build in every step 74 / 161 / 790 instead of 92 / 165 / 786 us
+// (beyond, the separate kernels' own block shapes pay more than the launches).  The lists are the same:
+// integer work, and every phase the same body.
+struct RebuildArgs {
+    const int *flag;   // null: unconditional; else nothing is done unless *flag
+    BinArgs bin;       // (their own flags null)
+    ListArgs lists;
+    RevArgs rev;
+};
+constexpr int ONE_THREADS = 128;
+static_assert(ONE_THREADS == LB_WARPS * 32 && ONE_THREADS == REV_WARPS * 32, "one block shape for every phase");
+
+// Every block of the grid has arrived (thread 0 of each counts it; the count starts at a multiple
+// of the grid).  False when the wait gave up.
+__device__ __forceinline__ bool grid_barrier(unsigned long long *count, int *s_ok) {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        const unsigned long long t = atomicAdd(count, 1ull), target = (t / gridDim.x + 1ull) * gridDim.x;
+        int ok = 0;
+        for (int it = 0; it < (1 << 22) && !ok; ++it) {
+            unsigned long long v;
+            asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(count) : "memory");
+            ok = v >= target;
+        }
+        __threadfence();
+        *s_ok = ok;
+    }
+    __syncthreads();
+    return *s_ok != 0;
+}
+
+__global__ void __launch_bounds__(ONE_THREADS, LISTS_MINB) k_rebuild_one(const __grid_constant__ RebuildArgs A,
+                                                                         unsigned long long *count) {
+    __shared__ union {
+        ListSmem lists;
+        RevSmem rev;
+        int scan[32];
+    } sm;
+    __shared__ int s_ok;
+    const BinArgs &r = A.bin;
+    if (A.flag && *A.flag == 0) return;   // the flag is cleared below, after a barrier: every block has read it
+    const int64_t b = blockIdx.x, nb = gridDim.x;
+    bool ok = true;
+    auto meet = [&]() { ok = ok && grid_barrier(count, &s_ok); };
+    bin_body(r, b, nb);
+    meet();
+    if (ok && b == 0) scan_body(r, sm.scan);
+    meet();
+    if (ok) scatter_body(r, b, nb);
+    meet();
+    if (ok) cellsort_body(r, b, nb);
+    meet();
+    if (ok) lists_body(A.lists, b, nb, sm.lists);
+    meet();
+    if (!ok) {
+        if (threadIdx.x == 0) atomicOr(A.lists.status, ST_TIMEOUT);
+        return;
+    }
+    rev_body(A.rev, b, nb, sm.rev);
+    finish_body(r, b, nb);
+    if (b == 0 && threadIdx.x == 0) *r.rebuild = 0;
 }
 
 inline unsigned blocks(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
@@ -856,16 +931,60 @@ RebuildPlan rebuild_plan(Sys &s, bool conditional) {
     pl.blocks[RB_SCAN] = 1;
     pl.blocks[RB_SCATTER] = capped(n, RB_THREADS);
     pl.blocks[RB_CELLSORT] = capped(s.cells.ncell, RB_THREADS / 32);   // a warp per cell
-    pl.blocks[RB_LISTS] = capped(s.cells.ncell, 1);   // one cell per block and item
+    // one item per block: the atoms of a cell in parts while there are fewer cells than SMs
+    la.parts = std::max(1, std::min(LISTS_PARTS_MAX, 2 * sms / std::max(1, s.cells.ncell)));
+    pl.blocks[RB_LISTS] = capped((int64_t)s.cells.ncell * la.parts, 1);
     pl.blocks[RB_REV] = capped(n, REV_WARPS);
     pl.blocks[RB_FINISH] = capped(m, RB_THREADS);
     return pl;
+}
+
+// Whether the system's own rebuilds take the one-launch form: its barrier count (device, zero) and
+// its grid, a block for each item of the list build as far as they fit on the GPU at once.  0 on
+// success.
+int make_rebuild_one(Sys &s) {
+    if (s.n == 0 || s.n > REBUILD_ONE_MAX) return 0;
+    int sms = 0, coop = 0, per = 0;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, s.device);
+    cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, s.device);
+    if (!coop || cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_rebuild_one, ONE_THREADS, 0) != cudaSuccess || per < 1) {
+        cudaGetLastError();
+        return 0;
+    }
+    if (cudaMalloc(&s.rb_count, sizeof(unsigned long long)) != cudaSuccess) {
+        s.rb_count = nullptr;
+        return -1;
+    }
+    const RebuildPlan pl = rebuild_plan(s, false);
+    s.rb_grid = (int)std::min<int64_t>((int64_t)sms * per, std::max<int64_t>(sms, pl.blocks[RB_LISTS]));
+    return cudaMemsetAsync(s.rb_count, 0, sizeof(unsigned long long), s.stream) == cudaSuccess ? 0 : -1;
 }
 
 // The system's own rebuild group: conditional (a step's, on the flag the first half raised;
 // the flag is cleared afterwards) or unconditional.
 void launch_rebuild(Sys &s, bool conditional) {
     const int kind = conditional ? SK_STEP : SK_FULL;
+    if (s.rb_count) {
+        const FusedTables &t = s.solo->t;
+        const unsigned char *h = s.solo->host.data();
+        RebuildArgs A;
+        std::memcpy(&A.bin, h + t.o_bin + kind * sizeof(BinArgs), sizeof(BinArgs));
+        std::memcpy(&A.lists, h + t.o_lists + kind * sizeof(ListArgs), sizeof(ListArgs));
+        std::memcpy(&A.rev, h + t.o_rev + kind * sizeof(RevArgs), sizeof(RevArgs));
+        A.flag = conditional ? s.rebuild : nullptr;
+        A.bin.flag = A.lists.flag = A.rev.flag = nullptr;   // tested once, at the start
+        cudaLaunchAttribute attr;
+        attr.id = cudaLaunchAttributeCooperative;
+        attr.val.cooperative = 1;
+        cudaLaunchConfig_t c = {};
+        c.gridDim = dim3((unsigned)s.rb_grid);
+        c.blockDim = dim3(ONE_THREADS);
+        c.stream = s.stream;
+        c.attrs = &attr;
+        c.numAttrs = 1;
+        cudaLaunchKernelEx(&c, k_rebuild_one, A, s.rb_count);
+        return;
+    }
     Launch L[RB_KERNELS];
     for (int k = 0; k < RB_KERNELS; ++k) L[k] = solo_launch(s, FK_BIN + k, kind);
     launch_rebuild_t(s.solo->t, L, conditional, false, s.stream);

@@ -39,6 +39,7 @@ struct ListArgs {
     const int *cell_start, *cell_atoms, *cell_sub;
     const float4 *cposf;      // cell-ordered FP32 positions relative to each cell's corner, species and sub-cell bits in w
     int cap, cap_ang, capr;
+    int parts;                // parts of a cell's atoms (see lists_body)
     double cut_r2, cut_a2;
     float cut_r2f_lo, cut_r2f_hi, cut_a2f_lo, cut_a2f_hi;   // FP32 pre-test band
     float wf[3];              // cell widths in FP32 (the stencil cells' corner offsets)

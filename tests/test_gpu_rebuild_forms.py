@@ -1,0 +1,32 @@
+"""Neighbour lists on both sides of the size where a system's own rebuild goes from one cooperative
+launch to its kernels one by one (131,072 atoms), and with cells split into parts (few cells)."""
+import numpy as np
+import pytest
+
+from oracle import oracle as O
+from paper_2606_14073_gb300 import nep_params, spinlat as S, workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("shape,drop", [((3, 3, 3), 0), ((3, 3, 3), 5), ((3, 6, 12), 1), ((9, 9, 9), 2),
+                                        ((32, 32, 16), 0), ((33, 32, 16), 4095)])
+def test_lists_equal_the_oracle(shape, drop):
+    rng = np.random.default_rng(shape[0] + drop)
+    pos, species, box = W.b20_lattice(*shape)
+    per = np.ones(3, np.int32)
+    keep = np.sort(rng.permutation(len(pos))[drop:])
+    pos = W.wrap(pos + rng.normal(0.0, 0.05, pos.shape), box, per)[keep]
+    n = len(pos)
+    s = S.System(pos, W.random_unit_vectors(rng, n), box, per, species[keep], nep_params.load(),
+                 precision=S.SL_PREC_MIXED)
+    s.step(30, 1.0, 300.0)     # builds triggered on the device, too
+    pos = s.get_state()["positions"]
+    rad, ang = s.get_neighbors()
+    builds = s.info()["n_builds"]
+    s.destroy()
+    method = 0 if n <= 2000 else 1
+    for lists, cut in ((rad, 7.0), (ang, 5.0)):
+        ref = O.neighbors(pos, box, per, cut, method=method)
+        assert all(np.array_equal(a, b) for a, b in zip(lists, ref))
+    assert builds >= 2
