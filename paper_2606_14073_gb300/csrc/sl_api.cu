@@ -12,6 +12,7 @@
 #include <cstddef>
 #include <cstdio>
 #include <cstring>
+#include <initializer_list>
 #include <map>
 #include <mutex>
 #include <new>
@@ -247,15 +248,6 @@ int check_status(sl::Sys &s) {
     return SL_OK;
 }
 
-// Pinned staging buffer of n records for state transfers (allocated once per system).
-static double4 *stage_buffer(const sl::Sys &s) {
-    if (!s.h_stage && cudaMallocHost((void **)&s.h_stage, sizeof(double4) * (size_t)s.n) != cudaSuccess) {
-        s.h_stage = nullptr;
-        return nullptr;
-    }
-    return s.h_stage;
-}
-
 // fn(lo, hi) over [0, n) in contiguous chunks on up to 8 host threads (one thread for small n);
 // every index is handled by exactly one thread, so results do not depend on the split.
 template <typename F>
@@ -280,9 +272,155 @@ static void parallel_chunks(int64_t n, F fn) {
     for (auto &x : th) x.join();
 }
 
+// ------------------------------------------------------------------ results to the host
+// Results leave the device in caller order: a kernel permutes them into the pair records' buffer
+// (scratch between evaluations, 32 bytes per atom and slot or more), and they cross in pieces
+// through pinned memory, each piece copied on by the host thread that asked for it, so that the
+// copies into the caller's (often untouched) pages overlap each other and the transfers.
+
+// Up to six vector arrays, permuted: out[k][orig[i]][0..2] = src[k][i].xyz
+constexpr int PACK_MAX = 6;
+struct PackArgs {
+    const double4 *src[PACK_MAX];
+    const int32_t *orig;
+    int64_t n;
+    double *out;   // [k][n][3]
+};
+__global__ void __launch_bounds__(256) k_pack_vectors(PackArgs a) {
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i >= a.n) return;
+    const double4 v = a.src[blockIdx.y][i];
+    double *o = a.out + ((int64_t)blockIdx.y * a.n + a.orig[i]) * 3;
+    o[0] = v.x;
+    o[1] = v.y;
+    o[2] = v.z;
+}
+
+// Descriptors, permuted and transposed: out[orig[i]][v] = q[v][i], 32 atoms per block through shared
+// memory; then out_e[orig[i]] = e[i].
+template <typename R>
+__global__ void __launch_bounds__(256) k_pack_descriptors(const R *q, int64_t qs, const R *e, const int32_t *orig,
+                                                          int64_t n, double *out, double *out_e) {
+    __shared__ R t[sl::DIM][33];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t i0 = blockIdx.x * (int64_t)32;
+    if (i0 + lane < n)
+        for (int v = w; v < sl::DIM; v += 8) t[v][lane] = q[(int64_t)v * qs + i0 + lane];
+    __syncthreads();
+    for (int a = w; a < 32 && i0 + a < n; a += 8) {
+        const int64_t c = orig[i0 + a];
+        for (int v = lane; v < sl::DIM; v += 32) out[c * sl::DIM + v] = (double)t[v][a];
+        if (lane == 0) out_e[c] = (double)e[i0 + a];
+    }
+}
+
+constexpr size_t PIECE = 4u << 20;       // bytes of one piece of a transfer
+constexpr unsigned COPY_THREADS = 8;     // at most; one per MiB
+
+// Pinned memory of at least `bytes` (kept by the system, grown on demand).
+static char *stage_buffer(const sl::Sys &s, size_t bytes) {
+    if (s.h_stage_bytes < bytes) {
+        if (s.h_stage) cudaFreeHost(s.h_stage);
+        s.h_stage_bytes = 0;
+        if (cudaMallocHost((void **)&s.h_stage, bytes) != cudaSuccess) {
+            cudaGetLastError();
+            s.h_stage = nullptr;
+            return nullptr;
+        }
+        s.h_stage_bytes = bytes;
+    }
+    return s.h_stage;
+}
+
+struct Segment {
+    void *dst;       // null: not wanted
+    size_t bytes;
+};
+
+// The consecutive segments of device memory at `src` into host memory, ordered after the work on
+// the system's stream; returns when they have arrived.
+static int copy_out(const sl::Sys &s, const char *src, const std::vector<Segment> &segs) {
+    size_t total = 0;
+    for (const Segment &g : segs) total += g.bytes;
+    const unsigned hw = std::max(1u, std::thread::hardware_concurrency());
+    const unsigned nt = (unsigned)std::min<size_t>(std::min(hw, COPY_THREADS), total / (1u << 20) + 1);
+    const size_t piece = std::min(PIECE, (total / nt + 4096) & ~(size_t)4095);
+    char *stage = stage_buffer(s, piece * nt);
+    if (!stage) return fail(SL_ENOMEM, "pinned staging buffer allocation failed");
+    const size_t pieces = (total + piece - 1) / piece;
+    std::atomic<int> err{(int)cudaSuccess};
+    // thread t moves pieces t, t + nt, ... through its own part of the staging memory
+    auto work = [&](unsigned t) {
+        cudaError_t e = cudaSetDevice(s.device);
+        cudaEvent_t ev = nullptr;
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
+        char *h = stage + piece * t;
+        for (size_t p = t; p < pieces && e == cudaSuccess; p += nt) {
+            const size_t off = p * piece, len = std::min(piece, total - off);
+            e = cudaMemcpyAsync(h, src + off, len, cudaMemcpyDeviceToHost, s.stream);
+            if (e == cudaSuccess) e = cudaEventRecord(ev, s.stream);
+            if (e == cudaSuccess) e = cudaEventSynchronize(ev);
+            if (e != cudaSuccess) break;
+            size_t at = 0;   // where the segment begins
+            for (const Segment &g : segs) {
+                const size_t lo = std::max(at, off), hi = std::min(at + g.bytes, off + len);
+                if (lo < hi && g.dst) std::memcpy(static_cast<char *>(g.dst) + (lo - at), h + (lo - off), hi - lo);
+                at += g.bytes;
+            }
+        }
+        if (ev) cudaEventDestroy(ev);
+        if (e != cudaSuccess) err.store((int)e);
+    };
+    // a thread that cannot be created leaves its share, and every later one's, to the calling
+    // thread: no exception crosses the ABI
+    std::vector<std::thread> th;
+    unsigned started = 1;
+    try {
+        th.reserve(nt - 1);
+        for (; started < nt; ++started) th.emplace_back(work, started);
+    } catch (...) {
+    }
+    work(0);
+    for (unsigned t = started; t < nt; ++t) work(t);
+    for (auto &x : th) x.join();
+    if (err.load() != (int)cudaSuccess) return cuda_fail((cudaError_t)err.load(), "copy to the host");
+    return SL_OK;
+}
+
+struct VecOut {
+    const double4 *src;
+    double *dst;     // null: not wanted
+};
+
+// Vector arrays (internal order) into host arrays [n][3] in caller order.
+static int download_vecs(const sl::Sys &s, std::initializer_list<VecOut> outs) {
+    const size_t bytes = sizeof(double) * 3 * (size_t)s.n;
+    const size_t room = (s.prec == 0 ? 8u : 4u) * 8u * (size_t)s.n * s.cap;   // the pair records' buffer
+    const size_t most = std::min<size_t>(PACK_MAX, room / bytes);             // at least one array fits
+    auto it = outs.begin();
+    while (it != outs.end()) {
+        PackArgs a;
+        std::vector<Segment> segs;
+        for (; it != outs.end() && segs.size() < most; ++it)
+            if (it->dst) {
+                a.src[segs.size()] = it->src;
+                segs.push_back(Segment{it->dst, bytes});
+            }
+        if (segs.empty()) break;
+        a.orig = s.orig;
+        a.n = s.n;
+        a.out = static_cast<double *>(s.pairs);
+        k_pack_vectors<<<dim3((unsigned)((s.n + 255) / 256), (unsigned)segs.size()), 256, 0, s.stream>>>(a);
+        CK(cudaGetLastError());
+        int rc;
+        if ((rc = copy_out(s, reinterpret_cast<const char *>(s.pairs), segs))) return rc;
+    }
+    return SL_OK;
+}
+
 // host (caller order) -> device (internal order), through the pinned staging buffer
 int upload_vec(sl::Sys &s, double4 *dst, const double *src, bool normalise) {
-    double4 *h = stage_buffer(s);
+    double4 *h = reinterpret_cast<double4 *>(stage_buffer(s, sizeof(double4) * (size_t)s.n));
     if (!h) return fail(SL_ENOMEM, "pinned staging buffer allocation failed");
     // the buffer may still be read by an earlier copy on this stream
     CK(cudaStreamSynchronize(s.stream));
@@ -311,21 +449,6 @@ int upload_vec(sl::Sys &s, double4 *dst, const double *src, bool normalise) {
     // ordered on the system's stream; synchronised before the staging buffer is reused
     CK(cudaMemcpyAsync(dst, h, sizeof(double4) * s.n, cudaMemcpyHostToDevice, s.stream));
     CK(cudaStreamSynchronize(s.stream));
-    return SL_OK;
-}
-
-int download_vec(const sl::Sys &s, const double4 *src, double *dst) {
-    double4 *h = stage_buffer(s);
-    if (!h) return fail(SL_ENOMEM, "pinned staging buffer allocation failed");
-    CK(cudaMemcpyAsync(h, src, sizeof(double4) * s.n, cudaMemcpyDeviceToHost, s.stream));
-    CK(cudaStreamSynchronize(s.stream));
-    const int32_t *orig = s.h_orig.data();
-    parallel_chunks(s.n, [&](int64_t lo, int64_t hi) {
-        for (int64_t i = lo; i < hi; ++i) {
-            double *p = dst + 3 * (int64_t)orig[i];
-            p[0] = h[i].x; p[1] = h[i].y; p[2] = h[i].z;
-        }
-    });
     return SL_OK;
 }
 
@@ -867,9 +990,7 @@ int sl_energy_forces_fields(sl_system *sys, double *energy, double *forces, doub
     if (sl::reduce_energy_virial(s, &E, W, virial != nullptr)) return fail(SL_ECUDA, "reduction failed");
     if (energy) *energy = E;
     if (virial) std::memcpy(virial, W, sizeof W);
-    if (forces && (rc = download_vec(s, s.Fo, forces))) return rc;
-    if (fields && (rc = download_vec(s, s.Ho, fields))) return rc;
-    return SL_OK;
+    return download_vecs(s, {{s.Fo, forces}, {s.Ho, fields}});
 }
 
 int sl_get_descriptors(sl_system *sys, double *q, double *atom_energy) {
@@ -878,23 +999,32 @@ int sl_get_descriptors(sl_system *sys, double *q, double *atom_energy) {
     cudaSetDevice(s.device);
     if (s.n == 0) return SL_OK;
     int rc;
-    if ((rc = evaluate(s, false, false, false))) return rc;
-    const size_t N = (size_t)s.n, R = s.prec == 0 ? 8 : 4, QS = (size_t)s.qs;
-    std::vector<char> hq(R * sl::DIM * QS), he(R * N);
-    std::vector<int32_t> orig(N);
-    CK(cudaMemcpyAsync(hq.data(), s.q, hq.size(), cudaMemcpyDeviceToHost, s.stream));
-    CK(cudaMemcpyAsync(he.data(), s.ei, he.size(), cudaMemcpyDeviceToHost, s.stream));
-    CK(cudaMemcpyAsync(orig.data(), s.orig, sizeof(int32_t) * N, cudaMemcpyDeviceToHost, s.stream));
-    CK(cudaStreamSynchronize(s.stream));
-    auto get = [&](const std::vector<char> &b, size_t idx) {
-        return R == 8 ? ((const double *)b.data())[idx] : (double)((const float *)b.data())[idx];
-    };
-    for (size_t i = 0; i < N; ++i) {
-        if (q)
-            for (int v = 0; v < sl::DIM; ++v) q[(size_t)orig[i] * sl::DIM + v] = get(hq, (size_t)v * QS + i);
-        if (atom_energy) atom_energy[orig[i]] = get(he, i);
+    sl::launch_eval(s, false, nullptr, true);   // descriptors and network only
+    CK(cudaGetLastError());
+    const size_t N = (size_t)s.n, bq = sizeof(double) * sl::DIM * N, be = sizeof(double) * N;
+    // into the pair records' buffer, or (very short lists) memory of its own
+    const size_t room = (s.prec == 0 ? 8u : 4u) * 8u * N * s.cap;
+    char *buf = static_cast<char *>(s.pairs), *own = nullptr;
+    if (room < bq + be) {
+        if ((rc = dalloc(&own, bq + be))) return rc;
+        buf = own;
     }
-    return SL_OK;
+    double *dq = reinterpret_cast<double *>(buf), *de = reinterpret_cast<double *>(buf + bq);
+    const unsigned nb = (unsigned)((N + 31) / 32);
+    if (s.prec == 0)
+        k_pack_descriptors<double><<<nb, 256, 0, s.stream>>>((const double *)s.q, s.qs, (const double *)s.ei, s.orig, s.n, dq, de);
+    else
+        k_pack_descriptors<float><<<nb, 256, 0, s.stream>>>((const float *)s.q, s.qs, (const float *)s.ei, s.orig, s.n, dq, de);
+    const cudaError_t e = cudaGetLastError();
+    rc = e != cudaSuccess ? cuda_fail(e, "descriptor transpose")
+         : q              ? copy_out(s, buf, {Segment{q, bq}, Segment{atom_energy, be}})
+         : atom_energy    ? copy_out(s, buf + bq, {Segment{atom_energy, be}})
+                          : SL_OK;
+    if (own) {
+        cudaStreamSynchronize(s.stream);
+        cudaFree(own);
+    }
+    return rc;
 }
 
 int sl_get_state(const sl_system *sys, double *pos, double *vel, double *spins, double *forces, double *fields,
@@ -904,12 +1034,8 @@ int sl_get_state(const sl_system *sys, double *pos, double *vel, double *spins, 
     cudaSetDevice(s.device);
     int rc;
     if (s.n > 0) {
-        if (pos && (rc = download_vec(s, s.pos, pos))) return rc;
-        if (vel && (rc = download_vec(s, s.vel, vel))) return rc;
-        if (spins && (rc = download_vec(s, s.spin, spins))) return rc;
-        if (forces && (rc = download_vec(s, s.F, forces))) return rc;
-        if (fields && (rc = download_vec(s, s.H, fields))) return rc;
-        if (ref && (rc = download_vec(s, s.posref, ref))) return rc;
+        if ((rc = download_vecs(s, {{s.pos, pos}, {s.vel, vel}, {s.spin, spins}, {s.F, forces}, {s.H, fields}, {s.posref, ref}})))
+            return rc;
     }
     if (step) *step = s.step;
     return SL_OK;

@@ -1627,12 +1627,13 @@ template void launch_eval_t<double>(const FusedTables &, const NepDev<double> &,
 
 // The system's own evaluation: at the midpoint point while s.at is set (the midpoint
 // iteration), else at the state, with the virial parts when asked for.
-void launch_eval(Sys &s, bool want_virial, cudaEvent_t *ev) {
+void launch_eval(Sys &s, bool want_virial, cudaEvent_t *ev, bool forward_only) {
     if (s.n == 0) return;
     const int kind = s.at.pos ? SK_MID : want_virial ? SK_FULL : SK_STEP;
-    const Launch L[7] = {solo_launch(s, FK_CRAD, kind),  solo_launch(s, FK_ANG, kind),  solo_launch(s, FK_NET, kind),
-                         solo_launch(s, FK_BWD, kind),   solo_launch(s, FK_CRADW, kind), solo_launch(s, FK_ANGW, kind),
-                         solo_launch(s, FK_BWDW, kind)};
+    Launch L[7] = {solo_launch(s, FK_CRAD, kind), solo_launch(s, FK_ANG, kind),   solo_launch(s, FK_NET, kind),
+                   solo_launch(s, FK_BWD, kind),  solo_launch(s, FK_CRADW, kind), solo_launch(s, FK_ANGW, kind),
+                   solo_launch(s, FK_BWDW, kind)};
+    if (forward_only) L[3].grid = L[6].grid = 0;
     if (s.prec == 0) launch_eval_t<double>(s.solo->t, s.pd, L, s.stream, ev);
     else launch_eval_t<float>(s.solo->t, s.pf, L, s.stream, ev);
 }

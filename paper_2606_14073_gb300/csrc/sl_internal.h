@@ -156,9 +156,10 @@ struct Sys {
     double *red = nullptr;     // reduction scratch (device)
     double *h_red = nullptr;   // pinned
     // host side of state transfers: the internal -> caller order permutation (fixed at
-    // creation) and a pinned staging buffer of n records, allocated on first use
+    // creation) and a pinned staging buffer, allocated on first use and grown on demand
     std::vector<int32_t> h_orig;
-    mutable double4 *h_stage = nullptr;
+    mutable char *h_stage = nullptr;
+    mutable size_t h_stage_bytes = 0;
 
     cudaGraphExec_t graph = nullptr;
     int graph_steps = 0;
@@ -239,8 +240,9 @@ void nbr_setup(Sys &s);
 void launch_rebuild(Sys &s, bool conditional);
 // sl_eval2.cu: the system's evaluation at the state (with the virial parts when asked for), or
 // at the midpoint point while s.at is set; ev (optional, 6 events): recorded before the
-// radial kernel, after it, after the angular kernel, the network and the backward.
-void launch_eval(Sys &s, bool want_virial, cudaEvent_t *ev = nullptr);
+// radial kernel, after it, after the angular kernel, the network and the backward; forward_only:
+// no backward (descriptors and network outputs only).
+void launch_eval(Sys &s, bool want_virial, cudaEvent_t *ev = nullptr, bool forward_only = false);
 void eval2_init();   // dynamic shared-memory limits of the evaluation kernels (once per device)
 int default_quad_block(int prec);   // threads per block of the quad kernels by default
 int make_coeff_table(Sys &s);                    // s.ctab from the model; 0 on success
