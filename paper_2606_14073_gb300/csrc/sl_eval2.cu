@@ -709,16 +709,28 @@ __device__ __forceinline__ void crad_wide_body(const NepDev<R> &P, const Eval2Ar
 // ------------------------------------------------------------------ k_ang_fwd
 // LPA lanes per atom (4, or 32 in small systems: eval_is_wide): each stages one pair, then each takes the harmonics
 // lm = ql + LPA m.  Stage of one angular pair: (g_n, s g_n) interleaved for n = 0..4, pad (2),
-// then the 24 harmonics in lane-major order, so each lane reads its own from consecutive places.
+// then the 24 harmonics in lane-major order, so each lane reads its own from consecutive places (four
+// lanes: the first four of each lane's six, then the last two of each).
 constexpr int FSTAGE = 36;
-constexpr int FQUAD = 4 * FSTAGE + 4;   // per quad, padded so quads start in different banks
+constexpr int FWARP = 32 * FSTAGE + 20;   // a warp's stages
 template <int LPA>
 struct AngLanes {
     static constexpr int H = (NLM + LPA - 1) / LPA;     // harmonics per lane
-    static constexpr int FATOM = LPA * FSTAGE + 4;      // an atom's stages
-    static_assert(LPA == 4 || LPA == 8 || LPA == 32, "24 harmonics in equal shares, or one per lane");
-    // harmonic at place t of a stage: lane t / H, its share t % H
-    static constexpr __device__ int lm_at(int t) { return t / H + LPA * (t % H); }
+    static_assert(LPA == 4 || LPA == 32, "24 harmonics in equal shares, or one per lane");
+    // harmonic at place t of a stage
+    static constexpr __device__ int lm_at(int t) {
+        if (LPA == 32) return t;
+        return t < 16 ? t / 4 + 4 * (t % 4) : (t - 16) / 2 + 4 * (4 + t % 2);
+    }
+    // Atom grp's stages in its warp's.  With four lanes per atom (FP32) the eight atoms start in different
+    // groups of four banks, 16 banks apart within a pair of atoms and 8 between pairs, so that eight
+    // lanes writing their stages, a quad reading one together and the lanes reading their own
+    // harmonics meet no bank twice.  What bounds the kernel is the shared-memory and L1 data path (74%
+    // busy); with the quads 4 words apart a third of the shared-memory wavefronts were bank
+    // conflicts: 519 to 493 us at 884,736 atoms, 79 to 75 us at 110,592.
+    static __device__ int stage_at(int grp) {
+        return LPA == 32 ? 0 : grp * (4 * FSTAGE) + 8 * ((grp >> 1) & 1) + 12 * (grp >> 2);
+    }
 };
 
 template <typename R, int LPA, int TI, int TJ>
@@ -760,7 +772,7 @@ __device__ __forceinline__ void ang_fwd_body(const NepDev<R> &P, const Eval2Args
     const int grp = lane / LPA, ql = lane % LPA;
     const int64_t i = (blk * (blockDim.x >> 5) + warp) * APW + grp;
     const bool valid = i < a.n;
-    R *stage = reinterpret_cast<R *>(smem_raw) + (warp * APW + grp) * L::FATOM;
+    R *stage = reinterpret_cast<R *>(smem_raw) + warp * FWARP + L::stage_at(grp);
     v4<R> pi, si;
     int na0 = 0, na = 0, ti = 0;
     if (valid) {
@@ -824,13 +836,9 @@ __device__ __forceinline__ void ang_fwd_body(const NepDev<R> &P, const Eval2Args
                                    pair2<R>(w1.z, w1.w), w2};
             R pv[H];
             if constexpr (LPA == 4) {
-                const v2<R> *pp = reinterpret_cast<const v2<R> *>(sp + 12 + H * ql);
-#pragma unroll
-                for (int m = 0; m < H; m += 2) {
-                    const v2<R> x = pp[m / 2];
-                    pv[m] = x.x;
-                    pv[m + 1] = x.y;
-                }
+                const v4<R> x = *reinterpret_cast<const v4<R> *>(sp + 12 + 4 * ql);
+                const v2<R> y = *reinterpret_cast<const v2<R> *>(sp + 28 + 2 * ql);
+                pv[0] = x.x; pv[1] = x.y; pv[2] = x.z; pv[3] = x.w; pv[4] = y.x; pv[5] = y.y;
             } else {
 #pragma unroll
                 for (int m = 0; m < H; ++m) pv[m] = sp[12 + H * ql + m];
@@ -1504,7 +1512,7 @@ static Eval2Args<R> args2(Sys &s, const EvalAt &at, bool want_virial) {
 template <typename R>
 static constexpr int quad_block() { return sizeof(R) == 8 ? 64 : 128; }
 template <typename R>
-static constexpr size_t fwd_smem(int qb = quad_block<R>()) { return (size_t)(qb / 32) * 8 * FQUAD * sizeof(R); }
+static constexpr size_t fwd_smem(int qb = quad_block<R>()) { return (size_t)(qb / 32) * FWARP * sizeof(R); }
 template <typename R>
 static constexpr size_t bwdf_smem(int qb = quad_block<R>()) { return (size_t)(qb / 32) * 8 * BW_ATOM * sizeof(R); }
 template <typename R>
