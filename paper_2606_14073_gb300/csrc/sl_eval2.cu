@@ -142,20 +142,20 @@ __device__ __forceinline__ void sep(const BoxDev<R> &b, const v4<R> &pi, const v
 
 // Coefficients of the rc_rad groups (g in the order R, EX, DMI, ANI, SIA) for lanes that each take
 // their own: for the wide radial kernel's contraction [centre][neighbour][k][g * 5 + n], rows
-// padded to 32, then for the FP64 backward's precontraction [centre][neighbour][g][n][k], rows of 10,
-// k = 0 shifted (see Carrier).
-constexpr int CTAB_BWD = NS * NS * NK * 32, CB_ROW = 10;
+// padded to 32, then for the backward's precontraction [centre][neighbour][n][group][k], rows of 12, the
+// groups in the order EX, DMI, ANI, SIA, R (FP64: k = 0 shifted, see Carrier).
+constexpr int CTAB_BWD = NS * NS * NK * 32, CB_ROW = 12, CB_CENTRE = NS * NCH * 5 * CB_ROW;
 template <typename R>
 static void fill_ctab(const NepDev<R> &P, std::vector<R> &t) {
     constexpr int GG[5] = {G_R, G_EX, G_DMI, G_ANI, G_SIA};
-    t.assign((size_t)CTAB_BWD + NS * NS * 25 * CB_ROW, R(0));
+    t.assign((size_t)CTAB_BWD + NS * CB_CENTRE, R(0));
     for (int x = 0; x < NS; ++x)
         for (int y = 0; y < NS; ++y)
             for (int o = 0; o < 25; ++o) {
                 const R *c = P.c[x][y][GG[o / NCH]][o % NCH];
-                R *b = t.data() + CTAB_BWD + (size_t)((x * NS + y) * 25 + o) * CB_ROW;
+                R *b = t.data() + CTAB_BWD + (size_t)(((x * NS + y) * NCH + o % NCH) * 5 + (o / NCH + 4) % 5) * CB_ROW;
                 for (int k = 0; k < NK; ++k) t[(size_t)((x * NS + y) * NK + k) * 32 + o] = b[k] = c[k];
-                b[0] = R(shifted_c0(c));
+                if (sizeof(R) == 8) b[0] = R(shifted_c0(c));
             }
 }
 int make_coeff_table(Sys &s) {
@@ -945,55 +945,48 @@ struct BwdAcc2 {
     R w[9];
 };
 
-// The atom's precontracted radial coefficients C^G_k = sum_n Fp^G_n c^G_nk for both neighbour
-// species into smc, 48 each; place of C^G_k: FP64 [k][group] (k = 0 shifted), FP32 [group][k].
-template <typename R>
-__device__ __forceinline__ int coeff_at(int g, int k) { return sizeof(R) == 8 ? 5 * k + g : 9 * g + k; }
-// FP32: every lane of the atom forms them all (the coefficients are constant operands) and stores its
-// share; taking its own from a table in global memory made the backward 1.58 to 1.70 ms at
-// 884,736 atoms (the loads' latency, before the first pair).
-template <int TI, int LPA>
-__device__ __forceinline__ void bwd_coeffs(const NepDev<float> &P, const float F[5][NCH], int ql, float *smc) {
+// The atom's precontracted radial coefficients C^G_k = sum_n Fp^G_n c^G_nk for both neighbour species
+// into smc, 48 each: [k][EX, DMI, ANI, SIA], then R by k.  Lane ql of four takes group ql of the four
+// magnetic ones (fm: its five gradient entries) and k = 2 ql, 2 ql + 1 of group R (fr), lane 0 also R's
+// k = 8, from the centre's rows ct of the table; species tj0 .. tj0 + NT - 1.  (FP32 had every lane form
+// all 90 from constant operands, and every lane fetch the entries of its own harmonics: with the
+// shares here and the entries handed round through shared memory the backward at 884,736 atoms takes
+// 1.55 instead of 1.69 ms, at 110,592 227 instead of 248 us, with a warp per atom at 512 12.5 instead of
+// 14.0 us.  Fetching the entries' records with asynchronous copies instead: 1.62 ms.)
+constexpr int BW_CR = 4 * NK;   // group R's place
+__device__ __forceinline__ constexpr int coeff_at(int g, int k) { return g == 0 ? BW_CR + k : 4 * k + g - 1; }
+template <typename R, int NT>
+__device__ __forceinline__ void bwd_coeffs(const R *__restrict__ ct, const R fm[NCH], const R fr[NCH], int ql, int tj0,
+                                           R *smc) {
 #pragma unroll
-    for (int tj = 0; tj < NS; ++tj)
+    for (int t = 0; t < NT; ++t) {
+        const R *__restrict__ row = ct + (tj0 + t) * (NCH * 5 * CB_ROW);
+        v2<R> c[4], cr = pair2<R>(R(0), R(0));
+        R c8 = R(0), cr8 = R(0);
 #pragma unroll
-        for (int g = 0; g < 5; ++g)
+        for (int q = 0; q < 4; ++q) c[q] = pair2<R>(R(0), R(0));
 #pragma unroll
-            for (int k = 0; k < NK; ++k) {
-                constexpr int G[5] = {G_R, G_EX, G_DMI, G_ANI, G_SIA};
-                float v = 0.f;
-#pragma unroll
-                for (int n = 0; n < NCH; ++n) v += F[g][n] * (tj == 0 ? P.c[TI][0][G[g]][n][k] : P.c[TI][1][G[g]][n][k]);
-                if (((tj * 45 + g * 9 + k) & (LPA - 1)) == ql) smc[tj * 48 + coeff_at<float>(g, k)] = v;
-            }
-}
-// FP64: lane ql of a quad takes k = 2 ql and 2 ql + 1 (with a warp, a quad each species), lanes 0 and
-// 1 one species' k = 8, from the centre's rows ct of the table (a quarter of the multiply-adds).
-template <int LPA>
-__device__ __forceinline__ void bwd_coeffs(const double *__restrict__ ct, const double F[5][NCH], int lane, double *smc) {
-    const int ql = lane & 3;
-    if (LPA > 4 && lane >= 8) return;
-#pragma unroll
-    for (int t = 0; t < (LPA == 4 ? NS : 1); ++t) {
-        const int tj = LPA == 4 ? t : lane >> 2;
-#pragma unroll
-        for (int g = 0; g < 5; ++g) {
-            double2 c2 = make_double2(0.0, 0.0);
-#pragma unroll
-            for (int n = 0; n < NCH; ++n)
-                c2 = fma2(make_double2(F[g][n], F[g][n]),
-                          ro(reinterpret_cast<const double2 *>(ct + ((tj * 5 + g) * NCH + n) * CB_ROW) + ql), c2);
-            smc[tj * 48 + coeff_at<double>(g, 2 * ql)] = c2.x;
-            smc[tj * 48 + coeff_at<double>(g, 2 * ql + 1)] = c2.y;
+        for (int n = 0; n < NCH; ++n, row += 5 * CB_ROW) {
+            const R *m = row + ql * CB_ROW, *r = row + 4 * CB_ROW;
+            const v4<R> a = *reinterpret_cast<const v4<R> *>(m), b = *reinterpret_cast<const v4<R> *>(m + 4);
+            const v2<R> f2 = pair2<R>(fm[n], fm[n]);
+            c[0] = fma2(f2, pair2<R>(a.x, a.y), c[0]);
+            c[1] = fma2(f2, pair2<R>(a.z, a.w), c[1]);
+            c[2] = fma2(f2, pair2<R>(b.x, b.y), c[2]);
+            c[3] = fma2(f2, pair2<R>(b.z, b.w), c[3]);
+            c8 = fma_(fm[n], m[8], c8);
+            cr = fma2(pair2<R>(fr[n], fr[n]), *reinterpret_cast<const v2<R> *>(r + 2 * ql), cr);
+            cr8 = fma_(fr[n], r[8], cr8);
         }
-    }
-    const int tj = lane & 1;
+        R *d = smc + (tj0 + t) * 48;
 #pragma unroll
-    for (int g = 0; g < 5; ++g) {
-        double v = 0.0;
-#pragma unroll
-        for (int n = 0; n < NCH; ++n) v += F[g][n] * ro(ct + ((tj * 5 + g) * NCH + n) * CB_ROW + 8);
-        if (lane < NS) smc[tj * 48 + coeff_at<double>(g, 8)] = v;
+        for (int q = 0; q < 4; ++q) {
+            d[8 * q + ql] = c[q].x;
+            d[8 * q + 4 + ql] = c[q].y;
+        }
+        d[32 + ql] = c8;
+        *reinterpret_cast<v2<R> *>(d + BW_CR + 2 * ql) = cr;
+        if (ql == 0) d[BW_CR + 8] = cr8;
     }
 }
 
@@ -1194,13 +1187,13 @@ __device__ __forceinline__ void bwd_pair(const NepDev<R> &P, const Eval2Args<R> 
         load_coefficients();
 #pragma unroll
         for (int q = 0; q < 5; ++q) {
-            const R c1 = C[coeff_at<R>(q, 1)];
-            pq[q] = pair2<R>(fma_(c1, cr.x, C[coeff_at<R>(q, 0)]), c1);
+            const R c1 = C[coeff_at(q, 1)];
+            pq[q] = pair2<R>(fma_(c1, cr.x, C[coeff_at(q, 0)]), c1);
         }
         cr.terms([&](int k, const v2<R> &td) {
 #pragma unroll
             for (int q = 0; q < 5; ++q) {
-                const R c = C[coeff_at<R>(q, k)];
+                const R c = C[coeff_at(q, k)];
                 pq[q] = fma2(pair2<R>(c, c), td, pq[q]);
             }
         });
@@ -1215,11 +1208,11 @@ __device__ __forceinline__ void bwd_pair(const NepDev<R> &P, const Eval2Args<R> 
         for (int q = 0; q < 4; ++q) he[q] = pair2<R>(R(0), R(0));
 #pragma unroll
         for (int k = 0; k < NK; ++k) {
-            e0 += C[coeff_at<R>(0, k)] * df[k];
+            e0 += C[coeff_at(0, k)] * df[k];
             const v2<R> fd = pair2<R>(f[k], df[k]);
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                const R c = C[coeff_at<R>(q + 1, k)];
+                const R c = C[coeff_at(q + 1, k)];
                 he[q] = fma2(pair2<R>(c, c), fd, he[q]);
             }
         }
@@ -1346,6 +1339,16 @@ __device__ __forceinline__ void bwd_body(const NepDev<R> &P, const Eval2Args<R> 
     const bool valid = i < a.n;
     const int64_t N = a.n;
     R *sm = reinterpret_cast<R *>(smem_raw) + (warp * APW + grp) * BW_ATOM;
+    // the atom's lanes
+    [[maybe_unused]] const unsigned quad = LPA == 32 ? 0xffffffffu : ((1u << (LPA & 31)) - 1u) << (grp * LPA);
+    // FP32, four lanes per atom: both centres' coefficients in shared memory, after the atoms' (read
+    // from global memory where they are used they came to 1.70 ms at 884,736 atoms)
+    [[maybe_unused]] R *ctab = reinterpret_cast<R *>(smem_raw) + (blockDim.x >> 5) * APW * BW_ATOM;
+    if constexpr (sizeof(R) == 4 && LPA == 4) {
+        const v4<R> *src = reinterpret_cast<const v4<R> *>(a.ctab + CTAB_BWD);
+        for (int e = threadIdx.x; e < NS * CB_CENTRE / 4; e += blockDim.x) reinterpret_cast<v4<R> *>(ctab)[e] = ro(src + e);
+        __syncthreads();
+    }
     BwdAcc2<R> acc;
     acc.fx = acc.fy = acc.fz = acc.hx = acc.hy = acc.hz = R(0);
 #pragma unroll
@@ -1354,8 +1357,34 @@ __device__ __forceinline__ void bwd_body(const NepDev<R> &P, const Eval2Args<R> 
         const int ti = i < a.n_fe ? 0 : 1;
         const v4<R> pi = ro(a.pos + i), si = ro(a.spin + i);
         const int4 c = ro(a.cnt + i);
+        // the lane's gradient entries: of group R and of its own magnetic group (bwd_coeffs)
+        const int qg = ql & 3;
+        R fr[NCH], fm[NCH];
+#pragma unroll
+        for (int n = 0; n < NCH; ++n) {
+            fr[n] = ro(a.fp + (int64_t)(Q_R + n) * N + i);
+            fm[n] = ro(a.fp + (int64_t)(Q_EX + qg * NCH + n) * N + i);
+        }
+        // the angular channels' entries (dE/dq_A, dE/dq_SA)_n of degree l; four lanes per atom: lane
+        // l - 1 fetches them for the others
+        auto angular_entries = [&](int l, v4<R> &x0, v4<R> &x1, v2<R> &x2) {
+            const R *fa = a.fp + (int64_t)(Q_A + l - 1) * N + i, *fs = a.fp + (int64_t)(Q_SA + l - 1) * N + i;
+            x0.x = ro(fa); x0.y = ro(fs); x0.z = ro(fa + 4 * N); x0.w = ro(fs + 4 * N);
+            x1.x = ro(fa + 8 * N); x1.y = ro(fs + 8 * N); x1.z = ro(fa + 12 * N); x1.w = ro(fs + 12 * N);
+            x2.x = ro(fa + 16 * N); x2.y = ro(fs + 16 * N);
+        };
+        if constexpr (LPA == 4) {
+            v4<R> x0, x1;
+            v2<R> x2;
+            angular_entries(ql + 1, x0, x1, x2);
+            R *d = sm + BW_C + 12 * ql;
+            reinterpret_cast<v4<R> *>(d)[0] = x0;
+            reinterpret_cast<v4<R> *>(d)[1] = x1;
+            *reinterpret_cast<v2<R> *>(d + 8) = x2;
+            __syncwarp(quad);
+        }
         // angular adjoints of this lane's harmonics lm = ql + LPA m from their records (three
-        // 16-byte loads each), the gradient entries straight from global memory
+        // 16-byte loads each)
 #pragma unroll
         for (int m = 0; m < (NLM + LPA - 1) / LPA; ++m) {
             const int lm = ql + LPA * m;
@@ -1363,30 +1392,36 @@ __device__ __forceinline__ void bwd_body(const NepDev<R> &P, const Eval2Args<R> 
             const int l = l_of_lm(lm);
             const R k2 = R(2) * kappa_of_lm<R>(lm);
             const v4<R> *src = reinterpret_cast<const v4<R> *>(a.bsum + ((int64_t)i * NLM + lm) * BREC);
-            v4<R> w0 = ro(src), w1 = ro(src + 1), w2 = ro(src + 2);
-            const R *fa = a.fp + (int64_t)(Q_A + l - 1) * N + i, *fs = a.fp + (int64_t)(Q_SA + l - 1) * N + i;
-            w0.x *= k2 * ro(fa); w0.y *= k2 * ro(fs); w0.z *= k2 * ro(fa + 4 * N); w0.w *= k2 * ro(fs + 4 * N);
-            w1.x *= k2 * ro(fa + 8 * N); w1.y *= k2 * ro(fs + 8 * N); w1.z *= k2 * ro(fa + 12 * N);
-            w1.w *= k2 * ro(fs + 12 * N);
-            w2.x *= k2 * ro(fa + 16 * N); w2.y *= k2 * ro(fs + 16 * N); w2.z = R(0); w2.w = R(0);
+            v4<R> w0 = ro(src), w1 = ro(src + 1), w2 = ro(src + 2), x0, x1;
+            v2<R> x2;
+            if constexpr (LPA == 4) {
+                const R *e = sm + BW_C + 12 * (l - 1);
+                x0 = reinterpret_cast<const v4<R> *>(e)[0];
+                x1 = reinterpret_cast<const v4<R> *>(e)[1];
+                x2 = *reinterpret_cast<const v2<R> *>(e + 8);
+            } else {
+                angular_entries(l, x0, x1, x2);
+            }
+            w0.x *= k2 * x0.x; w0.y *= k2 * x0.y; w0.z *= k2 * x0.z; w0.w *= k2 * x0.w;
+            w1.x *= k2 * x1.x; w1.y *= k2 * x1.y; w1.z *= k2 * x1.z; w1.w *= k2 * x1.w;
+            w2.x *= k2 * x2.x; w2.y *= k2 * x2.y; w2.z = R(0); w2.w = R(0);
             v4<R> *d = reinterpret_cast<v4<R> *>(sm + BREC * lm);
             d[0] = w0; d[1] = w1; d[2] = w2;
         }
-        R F[5][NCH];   // dE/dq of the rc_rad groups
-#pragma unroll
-        for (int n = 0; n < NCH; ++n) {
-            F[0][n] = ro(a.fp + (int64_t)(Q_R + n) * N + i);
-#pragma unroll
-            for (int g = 0; g < 4; ++g) F[g + 1][n] = ro(a.fp + (int64_t)(Q_EX + g * NCH + n) * N + i);
-        }
+        if constexpr (LPA == 4) __syncwarp(quad);   // the entries are read: the coefficients take their place
         if (ql == 0) {   // onsite term dE_i/dS_i = 2 Fp_O S_i, counted once per atom
             const R fo = R(2) * ro(a.fp + (int64_t)Q_O * N + i);
             acc.hx = fo * si.x; acc.hy = fo * si.y; acc.hz = fo * si.z;
         }
-        if constexpr (sizeof(R) == 8) bwd_coeffs<LPA>(a.ctab + CTAB_BWD + ti * (NS * 25 * CB_ROW), F, ql, sm + BW_C);
-        else if (ti == 0) bwd_coeffs<0, LPA>(P, F, ql, sm + BW_C);
-        else bwd_coeffs<1, LPA>(P, F, ql, sm + BW_C);
-        __syncwarp(LPA == 32 ? 0xffffffffu : ((1u << (LPA & 31)) - 1u) << (grp * LPA));
+        if constexpr (LPA == 4) {
+            if constexpr (sizeof(R) == 4)
+                bwd_coeffs<R, NS>(ctab + ti * CB_CENTRE, fm, fr, ql, 0, sm + BW_C);
+            else
+                bwd_coeffs<R, NS>(a.ctab + CTAB_BWD + ti * CB_CENTRE, fm, fr, ql, 0, sm + BW_C);
+        } else if (ql < 4 * NS) {   // four lanes per neighbour species
+            bwd_coeffs<R, 1>(a.ctab + CTAB_BWD + ti * CB_CENTRE, fm, fr, qg, ql >> 2, sm + BW_C);
+        }
+        __syncwarp(quad);
         const int ca = a.cap_ang;
         bwd_rows<R, true, VIR, LPA>(P, a, i, ti, ql, c.y, c.x, pi, si, sm, acc);
         bwd_rows<R, false, VIR, LPA>(P, a, i, ti, ca + ql, ca + c.w, ca + c.z, pi, si, sm, acc);
@@ -1514,7 +1549,9 @@ static constexpr int quad_block() { return sizeof(R) == 8 ? 64 : 128; }
 template <typename R>
 static constexpr size_t fwd_smem(int qb = quad_block<R>()) { return (size_t)(qb / 32) * FWARP * sizeof(R); }
 template <typename R>
-static constexpr size_t bwdf_smem(int qb = quad_block<R>()) { return (size_t)(qb / 32) * 8 * BW_ATOM * sizeof(R); }
+static constexpr size_t bwdf_smem(int qb = quad_block<R>()) {
+    return ((size_t)(qb / 32) * 8 * BW_ATOM + (sizeof(R) == 4 ? NS * CB_CENTRE : 0)) * sizeof(R);
+}
 template <typename R>
 static constexpr size_t bwdw_smem(int qb) { return (size_t)(qb / 32) * BW_ATOM * sizeof(R); }
 
