@@ -47,6 +47,27 @@ __device__ __forceinline__ v2<R> pair2(R x, R y) {
     v.y = y;
     return v;
 }
+// FP32: the carrier f_k = (T_k(x) + 1) f_c/2 as pairs of neighbouring k, k = 8 last: T_{k+2} = 2 T_2 T_k -
+// T_{k-2} advances two k's per packed multiply-add, and sums over pairs by k need no f_k twice in a
+// register pair.  (T_4 .. T_7 are carried negated, which saves the recurrence its sign changes.)
+struct CarrierPairs {
+    float2 f[4];
+    float f8;
+    __device__ __forceinline__ CarrierPairs(float r, float inv_rc) {
+        const float t = r * inv_rc, fch = cut_half(t);
+        const float y = t - 1.f, x = fma_(2.f * y, y, -1.f), x2 = 2.f * x;
+        const float t2 = fma_(x2, x, -1.f), w = 2.f * t2;
+        const float2 s0 = make_float2(1.f, x), s1 = make_float2(t2, fma_(x2, t2, -x));
+        const float2 s2 = fma2(make_float2(-w, -w), s1, s0), s3 = fma2(make_float2(w, w), s2, s1);
+        const float2 F = make_float2(fch, fch), Fm = make_float2(-fch, -fch);
+        f[0] = make_float2(fch + fch, fma_(x, fch, fch));
+        f[1] = fma2(s1, F, F);
+        f[2] = fma2(s2, Fm, F);
+        f[3] = fma2(s3, Fm, F);
+        f8 = fma_(fma_(-w, s3.x, s2.x), fch, fch);
+    }
+};
+
 // The carrier of sl_common.cuh with the T_k and U_k recurrences advanced together (FP32).
 template <typename R>
 __device__ __forceinline__ void carrier_fd2(R r, R inv_rc, R f[NK], R df[NK]) {
@@ -222,30 +243,36 @@ __device__ __forceinline__ R kappa_of_lm(int lm) {
 // angular and backward kernels and the gather.  The sums are
 // contracted with the coefficients once per neighbour species (q^R, q^EX, q^DMI, q^ANI,
 // q^SIA); q^O = |S|^2.
+// What bounds it: latency, at 16 warps per SM (the sums take 45 of 128 registers): 53% of issue slots, no
+// unit above 66%.  So the loads are kept in flight: the next candidate's coordinates in A, the next
+// four's in B, the next row's in C, and the first species' 25 values all at once before the second's
+// are stored (each load behind the store before it cost 25 trips to the L2 cache): 921 to 881 us at
+// 884,736 atoms, 161 to 147 us at 110,592 (two candidates ahead in A: 898 and 147 us; A as four at a
+// time, loaded where they are used: 926 and 150 us).  Lists tiled so that a warp's list loads are
+// consecutive changed nothing (936 us).
 
-template <typename R>
 struct RadSums {
-    R b0[NK];
-    v2<R> b12[NK], b34[NK];   // (EX, DMI) and (ANI, SIA) sums, two per packed multiply-add
+    float2 b[5][4];   // R, EX, DMI, ANI, SIA sums of k = 0 .. 7, two per packed multiply-add
+    float b8[5];      // k = 8
+    __device__ __forceinline__ float at(int g, int k) const { return k == 8 ? b8[g] : k & 1 ? b[g][k / 2].y : b[g][k / 2].x; }
 };
 
-template <typename R>
-__device__ __forceinline__ void rad_accumulate(const NepDev<R> &P, const v4<R> &si, const v4<R> &cs, R dx, R dy,
-                                               R dz, R d2, RadSums<R> &b) {
-    const R ir = rsqrt_(d2), r = d2 * ir;
-    const R ux = dx * ir, uy = dy * ir, uz = dz * ir;
-    R f[NK];
-    carrier_f(r, P.inv_rc_r, f);
-    const R sij = si.x * cs.x + si.y * cs.y + si.z * cs.z;
-    const R siu = si.x * ux + si.y * uy + si.z * uz;
-    const R sju = cs.x * ux + cs.y * uy + cs.z * uz;
-    const R dmi = (si.y * cs.z - si.z * cs.y) * ux + (si.z * cs.x - si.x * cs.z) * uy + (si.x * cs.y - si.y * cs.x) * uz;
-    const R ani = siu * sju, sia = siu * siu;
+__device__ __forceinline__ void rad_accumulate(const NepDev<float> &P, const float4 &si, const float4 &cs, float dx,
+                                               float dy, float dz, float d2, RadSums &b) {
+    const float ir = rsqrt_(d2), r = d2 * ir;
+    const float ux = dx * ir, uy = dy * ir, uz = dz * ir;
+    const CarrierPairs cr(r, P.inv_rc_r);
+    const float sij = si.x * cs.x + si.y * cs.y + si.z * cs.z;
+    const float siu = si.x * ux + si.y * uy + si.z * uz;
+    const float sju = cs.x * ux + cs.y * uy + cs.z * uz;
+    const float dmi = (si.y * cs.z - si.z * cs.y) * ux + (si.z * cs.x - si.x * cs.z) * uy + (si.x * cs.y - si.y * cs.x) * uz;
+    const float h[5] = {1.f, sij, dmi, siu * sju, siu * siu};
 #pragma unroll
-    for (int k = 0; k < NK; ++k) {
-        b.b0[k] += f[k];
-        b.b12[k] = fma2(pair2<R>(f[k], f[k]), pair2<R>(sij, dmi), b.b12[k]);
-        b.b34[k] = fma2(pair2<R>(f[k], f[k]), pair2<R>(ani, sia), b.b34[k]);
+    for (int g = 0; g < 5; ++g) {
+#pragma unroll
+        for (int p = 0; p < 4; ++p)
+            b.b[g][p] = g == 0 ? __fadd2_rn(cr.f[p], b.b[g][p]) : fma2(cr.f[p], make_float2(h[g], h[g]), b.b[g][p]);
+        b.b8[g] = g == 0 ? b.b8[g] + cr.f8 : fma_(cr.f8, h[g], b.b8[g]);
     }
 }
 
@@ -274,11 +301,12 @@ template <typename R, int TI, int TJ>
 __device__ __forceinline__ void crad_species(const NepDev<R> &P, const Eval2Args<R> &a, int64_t i, const v4<R> &pi,
                                              const v4<R> &si, int lo0, int hi0, int lo1, int hi1, int &na, int &nr,
                                              bool &ovf, uint32_t (*smask)[128]) {
-    RadSums<R> b;
+    RadSums b;
 #pragma unroll
-    for (int k = 0; k < NK; ++k) {
-        b.b0[k] = R(0);
-        b.b12[k] = b.b34[k] = pair2<R>(R(0), R(0));
+    for (int g = 0; g < 5; ++g) {
+        b.b8[g] = 0.f;
+#pragma unroll
+        for (int p = 0; p < 4; ++p) b.b[g][p] = make_float2(0.f, 0.f);
     }
     const int64_t N = a.n;
     // this atom's candidate list and reverse slots: one row each, read in aligned chunks of 4
@@ -294,46 +322,44 @@ __device__ __forceinline__ void crad_species(const NepDev<R> &P, const Eval2Args
         }
     };
 
-    // A: angular candidates, compaction and sums
+    // A: angular candidates, compaction and sums; the coordinates of the next candidate are in flight
+    // while one is computed
     {
         int4 jq1 = make_int4(-1, -1, -1, -1), jq2 = jq1;
         uchar4 tq1 = make_uchar4(0, 0, 0, 0), tq2 = tq1;
         const int c0 = lo0 & ~3;
         chunk(c0, hi0, jq1, tq1);
         chunk(c0 + 4, hi0, jq2, tq2);
+        auto pick = [&](int c, int j) { return c >= lo0 && c < hi0 ? j : (int)i; };   // not another segment's entry
+        const int ja = pick(c0, jq1.x);
+        v4<R> p1 = pos[ja], s1 = spin[ja];
 #pragma unroll 1
         for (int c = c0; c < hi0; c += 4) {
-            int jj[4] = {jq1.x, jq1.y, jq1.z, jq1.w};
+            const int jj[5] = {jq1.x, jq1.y, jq1.z, jq1.w, jq2.x};
             const int tt[4] = {tq1.x, tq1.y, tq1.z, tq1.w};
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-                if (c + u < lo0 || c + u >= hi0) jj[u] = -1;   // another segment's entry
-            v4<R> pp[4], ss[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int j = jj[u] >= 0 ? jj[u] : (int)i;
-                pp[u] = pos[j];
-                ss[u] = spin[j];
-            }
             jq1 = jq2;
             tq1 = tq2;
             chunk(c + 8, hi0, jq2, tq2);
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                if (jj[u] < 0) continue;
+                const v4<R> pu = p1, su = s1;
+                const int jn = pick(c + u + 1, jj[u + 1]);
+                p1 = pos[jn];
+                s1 = spin[jn];
+                if (c + u < lo0 || c + u >= hi0) continue;
                 R dx, dy, dz;
-                sep(a.box, pi, pp[u], dx, dy, dz);
+                sep(a.box, pi, pu, dx, dy, dz);
                 const R d2 = dx * dx + dy * dy + dz * dz;
                 if (!(d2 < P.rc_r2)) continue;
                 const int row = take_row(P, a, d2, na, nr, ovf);
                 if (row < 0) continue;
                 stg(a.crow + (int64_t)row * N + i, make_int2(jj[u], tt[u]));
                 mark_slot(smask, c + u);
-                rad_accumulate(P, si, ss[u], dx, dy, dz, d2, b);
+                rad_accumulate(P, si, su, dx, dy, dz, d2, b);
             }
         }
     }
-    // B: radial-shell candidates, compaction only
+    // B: radial-shell candidates, compaction only; the next four candidates' positions are in flight
     const int naB = na, nrB = nr;
     {
         int4 jq1 = make_int4(-1, -1, -1, -1), jq2 = jq1;
@@ -341,24 +367,27 @@ __device__ __forceinline__ void crad_species(const NepDev<R> &P, const Eval2Args
         const int c0 = lo1 & ~3;
         chunk(c0, hi1, jq1, tq1);
         chunk(c0 + 4, hi1, jq2, tq2);
+        auto pick = [&](int c, int j) { return c >= lo1 && c < hi1 ? j : (int)i; };
+        v4<R> pn[4];
+        {
+            const int j[4] = {jq1.x, jq1.y, jq1.z, jq1.w};
+#pragma unroll
+            for (int u = 0; u < 4; ++u) pn[u] = pos[pick(c0 + u, j[u])];
+        }
 #pragma unroll 1
         for (int c = c0; c < hi1; c += 4) {
-            int jj[4] = {jq1.x, jq1.y, jq1.z, jq1.w};
+            const int jj[4] = {jq1.x, jq1.y, jq1.z, jq1.w}, jx[4] = {jq2.x, jq2.y, jq2.z, jq2.w};
             const int tt[4] = {tq1.x, tq1.y, tq1.z, tq1.w};
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-                if (c + u < lo1 || c + u >= hi1) jj[u] = -1;
-            v4<R> pp[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) pp[u] = pos[jj[u] >= 0 ? jj[u] : (int)i];
             jq1 = jq2;
             tq1 = tq2;
             chunk(c + 8, hi1, jq2, tq2);
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                if (jj[u] < 0) continue;
+                const v4<R> pu = pn[u];
+                pn[u] = pos[pick(c + 4 + u, jx[u])];
+                if (c + u < lo1 || c + u >= hi1) continue;
                 R dx, dy, dz;
-                sep(a.box, pi, pp[u], dx, dy, dz);
+                sep(a.box, pi, pu, dx, dy, dz);
                 const R d2 = dx * dx + dy * dy + dz * dz;
                 if (!(d2 < P.rc_r2)) continue;
                 const int row = take_row(P, a, d2, na, nr, ovf);
@@ -392,17 +421,18 @@ __device__ __forceinline__ void crad_species(const NepDev<R> &P, const Eval2Args
     // values in q (the same thread wrote them), so no accumulator lives across the loops
     constexpr int GQ[5] = {Q_R, Q_EX, Q_DMI, Q_ANI, Q_SIA};
     constexpr int GG[5] = {G_R, G_EX, G_DMI, G_ANI, G_SIA};
+    R first[5][NCH];   // all loads before the first store: the stores keep their order
+#pragma unroll
+    for (int g = 0; g < 5; ++g)
+#pragma unroll
+        for (int n = 0; n < NCH; ++n) first[g][n] = TJ == 0 ? R(0) : a.q[(GQ[g] + n) * a.qs + i];
 #pragma unroll
     for (int g = 0; g < 5; ++g) {
 #pragma unroll
         for (int n = 0; n < NCH; ++n) {
-            R v = TJ == 0 ? R(0) : a.q[(GQ[g] + n) * a.qs + i];
+            R v = first[g][n];
 #pragma unroll
-            for (int k = 0; k < NK; ++k) {
-                const R bgk = g == 0 ? b.b0[k] : g == 1 ? b.b12[k].x : g == 2 ? b.b12[k].y : g == 3 ? b.b34[k].x
-                                                                                                 : b.b34[k].y;
-                v += P.c[TI][TJ][GG[g]][n][k] * bgk;
-            }
+            for (int k = 0; k < NK; ++k) v += P.c[TI][TJ][GG[g]][n][k] * b.at(g, k);
             stg(a.q + (GQ[g] + n) * a.qs + i, v);
         }
     }
@@ -455,8 +485,8 @@ __device__ __forceinline__ void crad_body(const NepDev<R> &P, const Eval2Args<R>
 // atom takes, but spread over a warp for every two atoms): 512 / 13,824 / 110,592 atoms 45 / 349 /
 // 2,113 us, against 511 / 525 / 2,091 us with one thread per atom.  Mixed precision: instruction
 // issue (1,270 warp instructions per atom against 570 for one thread per atom, whose chain of 110
-// candidates takes 48 us however few the atoms): 512 / 13,824 / 32,768 / 110,592 atoms 15 / 37 / 70 /
-// 189 us, against 51 / 68 / 74 / 161 us.  The line lies at 16,384 atoms, below the crossing: a
+// candidates takes 47 us however few the atoms): 512 / 13,824 / 32,768 / 110,592 atoms 15 / 37 / 70 /
+// 202 us, against 47 / 64 / 72 / 148 us.  The line lies at 16,384 atoms, below the crossing: a
 // replica keeps its kernel in a batch (its results are the same there bit for bit), where other
 // replicas fill the GPU and only the instructions count (eight replicas of 4,096 to 65,536 atoms
 // step 2.5% slower with the line at 32,768).
@@ -1498,7 +1528,7 @@ __global__ void __launch_bounds__(128, MINB) k_bwd(const __grid_constant__ NepDe
 // us, backward 75 / 198 / 321 instead of 380 / 387 / 398 us (its 21 angular pairs fill two thirds of a
 // round of 32 lanes, so in larger systems four lanes need fewer FP64 instructions).  Mixed precision
 // at 512 / 1,728 / 2,744 / 4,096 atoms: angular 10 / 10 / 14.5 / 16 instead of 12 / 12 / 12 / 12 us,
-// backward 14 / 18 / 25 / 31 instead of 26 / 26 / 26 / 25 us.
+// backward 12 / 15 / 20 / 27 instead of 23 / 24 / 24 / 25 us.
 template <typename R>
 __global__ void __launch_bounds__(128, sizeof(R) == 4 ? 4 : 1) k_ang_wide(const __grid_constant__ NepDev<R> P,
                                                                           const Eval2Args<R> *__restrict__ tab,
