@@ -68,11 +68,14 @@ __device__ __forceinline__ void omega_of_f(float sx, float sy, float sz, float h
 // records (dE_j/dr_jk, dE_j/dS_k) sit in k's own in-cutoff candidate slots.  W lanes take an atom;
 // lane q walks the slots s = q mod W in order with the other lanes of its warp, so the records
 // that neighbouring atoms read at one slot are neighbours in memory (slot-major layout); the
-// lanes' sums are added in a fixed order.  What bounds it: the records' DRAM traffic in large systems (two 16-byte loads per
-// record), and in small ones the chain of a lane's slots, a few loads in flight at a time: so a
+// lanes' sums are added in a fixed order.  What bounds it: the records' DRAM traffic in large FP32 systems
+// (2.3 GB in 470 us at 884,736 atoms), and elsewhere the chain of a lane's slots, a few loads in flight
+// at a time: so eight slots' records are loaded together, without branches (FP64 at 32,768 atoms 92 instead
+// of 120 us a second half, FP32 at 110,592 83 instead of 85), and a
 // small system (gather_is_wide) takes several lanes per atom, a larger one one.  Second half, mixed
-// precision, 512 / 13,824 / 32,768 / 110,592 atoms: 17 / 21 / 32 / 89 us with four lanes, 29 / 34 / 45 / 85
-// with one; FP64, 512 / 13,824 / 32,768 atoms: 32 / 54 / 121 us with eight, 90 / 109 / 121 with one.
+// precision, 512 / 13,824 / 32,768 / 64,000 / 110,592 atoms: 17 / 21 / 32 / 59 / 89 us with four lanes, 27 / 31 /
+// 43 / 59 / 83 with one; FP64, 512 / 13,824 / 21,952 / 32,768 atoms: 27 / 49 / 77 / 114 us with eight, 83 / 87 /
+// 88 / 92 with one.
 template <typename R>
 constexpr int GATHER_WIDE = sizeof(R) == 4 ? 4 : 8;
 constexpr int gather_atoms(int W) { return 256 / W; }   // atoms per 256-thread block
@@ -82,6 +85,24 @@ template <typename R, int W>
 struct GatherSmem {
     R v[W == 1 ? 1 : 6][W == 1 ? 1 : gather_atoms(W)];   // (unused with one lane per atom)
 };
+
+// The record at p where it is set, else zeros, without a branch, so the loads of several slots are in
+// flight together: FP32 in one 256-bit load, FP64 in two.
+__device__ __forceinline__ PairRec<float> rec_if(const PairRec<float> *p, uint32_t set) {
+    PairRec<float> e = {};
+    asm("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %9, 0;\n\t@p ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];\n\t}"
+        : "+f"(e.a.x), "+f"(e.a.y), "+f"(e.a.z), "+f"(e.a.w), "+f"(e.b.x), "+f"(e.b.y), "+f"(e.b.z), "+f"(e.b.w)
+        : "l"(p), "r"(set));
+    return e;
+}
+__device__ __forceinline__ PairRec<double> rec_if(const PairRec<double> *p, uint32_t set) {
+    PairRec<double> e = {};
+    asm("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %7, 0;\n\t@p ld.global.v4.f64 {%0, %1, %2, %3}, [%6];\n\t"
+        "@p ld.global.v2.f64 {%4, %5}, [%6 + 32];\n\t}"
+        : "+d"(e.a.x), "+d"(e.a.y), "+d"(e.a.z), "+d"(e.a.w), "+d"(e.b.x), "+d"(e.b.y)
+        : "l"(p), "r"(set));
+    return e;
+}
 
 // Sums of one atom's own part and records, its lane q of W.
 template <typename R, int W>
@@ -97,13 +118,18 @@ __device__ __forceinline__ void gather_lane(const GatherArgs<R> &g, int64_t k, i
 #pragma unroll 1
     for (int w = 0; w < g.maskw; ++w) {
         const uint32_t word = ro(g.mask + (int64_t)w * N + k);
-#pragma unroll 4
-        for (int b = q; b < 32; b += W) {
-            if ((word >> b) & 1u) {
-                const PairRec<R> *e = g.pd + (int64_t)(w * 32 + b) * N + k;
-                const v4<R> ea = ro(&e->a), eb = ro(&e->b);
-                v[0] -= ea.x; v[1] -= ea.y; v[2] -= ea.z;
-                v[3] -= ea.w; v[4] -= eb.x; v[5] -= eb.y;
+constexpr int U = 4 * W <= 16 ? 8 : 4;   // slots at a time
+#pragma unroll 1
+        for (int b = q; b < 32; b += U * W) {
+            if ((word >> b) == 0u) break;
+            PairRec<R> e[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                e[u] = rec_if(g.pd + (int64_t)(w * 32 + b + u * W) * N + k, (word >> (b + u * W)) & 1u);
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                v[0] -= e[u].a.x; v[1] -= e[u].a.y; v[2] -= e[u].a.z;
+                v[3] -= e[u].a.w; v[4] -= e[u].b.x; v[5] -= e[u].b.y;
             }
         }
     }
