@@ -18,11 +18,11 @@ constexpr int NH = 30;    // hidden units
 constexpr int NLM = 24;   // real solid harmonics, l = 1..4
 constexpr int DIM = 66;   // descriptor length
 constexpr int NB = 2 * NCH * NLM;   // 240 angular sums kept for the backward pass
-// The angular sums are stored atom-major as one 12-entry record per harmonic lm:
-// (B_0lm, BS_0lm, B_1lm, BS_1lm, ..., B_4lm, BS_4lm, 0, 0), 48 bytes in FP32 (three
-// 16-byte words), the layout the backward kernel keeps its adjoints in.
-constexpr int BREC = 12;
-constexpr int NBREC = NLM * BREC;   // 288 stored entries per atom
+// The angular sums are stored atom-major as one 10-entry record per harmonic lm:
+// (B_0lm, BS_0lm, B_1lm, BS_1lm, ..., B_4lm, BS_4lm), so two neighbouring harmonics are 80 bytes in
+// FP32 (five 16-byte words), the layout the backward kernel keeps its adjoints in.
+constexpr int BREC = 10;
+constexpr int NBREC = NLM * BREC;   // 240 stored entries per atom
 
 // coefficient groups
 constexpr int G_R = 0, G_A = 1, G_EX = 2, G_DMI = 3, G_ANI = 4, G_SIA = 5;
@@ -97,6 +97,8 @@ __device__ __forceinline__ void stg(unsigned short *p, unsigned short v) { __stw
 __device__ __forceinline__ void stg(float *p, float v) { __stwb(p, v); }
 __device__ __forceinline__ void stg(double *p, double v) { __stwb(p, v); }
 __device__ __forceinline__ void stg(float4 *p, const float4 &v) { __stwb(p, v); }
+__device__ __forceinline__ void stg(float2 *p, const float2 &v) { __stwb(p, v); }
+__device__ __forceinline__ void stg(double2 *p, const double2 &v) { __stwb(p, v); }
 __device__ __forceinline__ void stg(int2 *p, const int2 &v) { __stwb(p, v); }
 __device__ __forceinline__ void stg(int4 *p, const int4 &v) { __stwb(p, v); }
 __device__ __forceinline__ void stg(double4 *p, const double4 &v) {

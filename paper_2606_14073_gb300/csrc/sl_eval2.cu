@@ -68,6 +68,12 @@ struct CarrierPairs {
     }
 };
 
+template <typename R>
+__device__ __forceinline__ v4<R> quad4(const v2<R> &a, const v2<R> &b) {
+    v4<R> v;
+    v.x = a.x; v.y = a.y; v.z = b.x; v.w = b.y;
+    return v;
+}
 // The carrier of sl_common.cuh with the T_k and U_k recurrences advanced together (FP32).
 template <typename R>
 __device__ __forceinline__ void carrier_fd2(R r, R inv_rc, R f[NK], R df[NK]) {
@@ -199,8 +205,13 @@ int make_coeff_table(Sys &s) {
     return put(t);
 }
 
-// per-lane constants of harmonic lm = ql + 4 m (ql = lane in quad)
-__device__ __forceinline__ int lm_of(int ql, int m) { return ql + 4 * m; }
+// harmonic m of lane ql of an atom's LPA: four lanes take neighbouring pairs (2 ql, 2 ql + 1, then eight
+// further, so that a pair of records is whole 16-byte pieces), a warp one each
+template <int LPA>
+__device__ __forceinline__ constexpr int lm_of(int ql, int m) {
+    static_assert(LPA == 4 || LPA == 32, "24 harmonics in equal shares, or one per lane");
+    return LPA == 4 ? 2 * ql + (m & 1) + 8 * (m >> 1) : ql;
+}
 __device__ __forceinline__ int l_of_lm(int lm) { return lm < 3 ? 1 : lm < 8 ? 2 : lm < 15 ? 3 : 4; }
 template <typename R>
 __device__ __forceinline__ R kappa_of_lm(int lm) {
@@ -738,7 +749,7 @@ __device__ __forceinline__ void crad_wide_body(const NepDev<R> &P, const Eval2Ar
 
 // ------------------------------------------------------------------ k_ang_fwd
 // LPA lanes per atom (4, or 32 in small systems: eval_is_wide): each stages one pair, then each takes the harmonics
-// lm = ql + LPA m.  Stage of one angular pair: (g_n, s g_n) interleaved for n = 0..4, pad (2),
+// of lm_of.  Stage of one angular pair: (g_n, s g_n) interleaved for n = 0..4, pad (2),
 // then the 24 harmonics in lane-major order, so each lane reads its own from consecutive places (four
 // lanes: the first four of each lane's six, then the last two of each).
 constexpr int FSTAGE = 36;
@@ -750,7 +761,7 @@ struct AngLanes {
     // harmonic at place t of a stage
     static constexpr __device__ int lm_at(int t) {
         if (LPA == 32) return t;
-        return t < 16 ? t / 4 + 4 * (t % 4) : (t - 16) / 2 + 4 * (4 + t % 2);
+        return t < 16 ? lm_of<4>(t / 4, t % 4) : lm_of<4>((t - 16) / 2, 4 + t % 2);
     }
     // Atom grp's stages in its warp's.  With four lanes per atom (FP32) the eight atoms start in different
     // groups of four banks, 16 banks apart within a pair of atoms and 8 between pairs, so that eight
@@ -894,17 +905,21 @@ __device__ __forceinline__ void ang_fwd_body(const NepDev<R> &P, const Eval2Args
     }
 #pragma unroll
     for (int m = 0; m < H; ++m) {
-        const int lm = ql + LPA * m;
+        const int lm = lm_of<LPA>(ql, m);
         if (!QUAD && lm >= NLM) break;
         const int l = l_of_lm(lm) - 1;
         const R kap = kappa_of_lm<R>(lm);
-        if (valid) {   // the harmonic's record: (B_n, BS_n) for n = 0..4, two zeros
-            v4<R> *rec = reinterpret_cast<v4<R> *>(a.bsum + ((int64_t)i * NLM + lm) * BREC);
-            v4<R> w0, w1, w2;
-            w0.x = BB[m][0].x; w0.y = BB[m][0].y; w0.z = BB[m][1].x; w0.w = BB[m][1].y;
-            w1.x = BB[m][2].x; w1.y = BB[m][2].y; w1.z = BB[m][3].x; w1.w = BB[m][3].y;
-            w2.x = BB[m][4].x; w2.y = BB[m][4].y; w2.z = R(0); w2.w = R(0);
-            stg(rec, w0); stg(rec + 1, w1); stg(rec + 2, w2);
+        if (valid) {   // the harmonic's record: (B_n, BS_n) for n = 0..4; two harmonics' in five pieces
+            R *rec = a.bsum + ((int64_t)i * NLM + lm) * BREC;
+            if constexpr (!QUAD) {
+#pragma unroll
+                for (int n = 0; n < NCH; ++n) stg(reinterpret_cast<v2<R> *>(rec) + n, BB[m][n]);
+            } else if (m % 2 == 0) {
+                const v2<R> *p = BB[m], *q = BB[m + (H > 1 ? 1 : 0)];
+                v4<R> *rec4 = reinterpret_cast<v4<R> *>(rec);
+                stg(rec4, quad4<R>(p[0], p[1])); stg(rec4 + 1, quad4<R>(p[2], p[3])); stg(rec4 + 2, quad4<R>(p[4], q[0]));
+                stg(rec4 + 3, quad4<R>(q[1], q[2])); stg(rec4 + 4, quad4<R>(q[3], q[4]));
+            }
         }
 #pragma unroll
         for (int n = 0; n < NCH; ++n) {
@@ -962,12 +977,19 @@ __device__ __forceinline__ void ang_fwd_body(const NepDev<R> &P, const Eval2Args
 
 // ------------------------------------------------------------------ k_bwd (fused)
 // Quad per atom, lanes over pairs.  Shared memory per atom: the angular adjoints
-// dE/dB_nlm, dE/dBS_nlm as 24 records of 12 ((dE/dB, dE/dBS) interleaved per n, pad), then the precontracted
+// dE/dB_nlm, dE/dBS_nlm as 24 records of 10 ((dE/dB, dE/dBS) interleaved per n), then the precontracted
 // radial coefficients C^G_k = sum_n Fp^G_n c^G_{n k t_i t_j} for both neighbour
-// species (2 x 48).  Stride 388: 388 mod 32 = 4, so the eight atoms of a warp read
-// disjoint bank groups.
-constexpr int BW_C = 292;
-constexpr int BW_ATOM = 388;
+// species (2 x 48).  336 mod 32 = 16 and four words more every second atom: the eight atoms of a warp
+// read disjoint groups of four banks, and two atoms' lanes storing their records meet no bank twice.
+// What bounds the FP32 kernel is its loads, of which the records' (60 16-byte words an angular pair)
+// are most of the shared-memory ones: without the two pads a 12-word record had, the backward at
+// 884,736 atoms takes 1.49 instead of 1.55 ms and the angular kernel, which writes them, 483 instead of
+// 493 us (110,592: 220 / 73.5 instead of 227 / 75 us; FP64 unchanged).
+constexpr int BW_C = NLM * BREC;
+constexpr int BW_ATOM = BW_C + 96;
+constexpr int BW_WARP = 8 * BW_ATOM + 16;
+template <int LPA>
+__device__ __forceinline__ int bwd_at(int grp) { return LPA == 4 ? grp * BW_ATOM + 4 * (grp >> 1) : 0; }
 
 template <typename R>
 struct BwdAcc2 {
@@ -1062,13 +1084,22 @@ __device__ __forceinline__ void ang_gdg(const NepDev<R> &P, R r, R inv_rc, R g[N
 // against subtracting each harmonic's part along u).
 template <typename R, int LM>
 __device__ __forceinline__ void bwd_harm(const R *__restrict__ bb, R ux, R uy, R uz, R s, const R g[NCH],
-                                         const R dg[NCH], v2<R> &along, R &avx, R &avy, R &avz, R &cj) {
+                                         const R dg[NCH], v2<R> &along, R &avx, R &avy, R &avz, R &cj, v4<R> &mid) {
     R p, gx, gy, gz;
     harm_one<R, LM>(ux, uy, uz, p, gx, gy, gz);
-    const v4<R> *rec = reinterpret_cast<const v4<R> *>(bb + BREC * LM);
-    const v4<R> r0 = rec[0], r1 = rec[1], r2 = rec[2];
-    const v2<R> Bp[NCH] = {pair2<R>(r0.x, r0.y), pair2<R>(r0.z, r0.w), pair2<R>(r1.x, r1.y), pair2<R>(r1.z, r1.w),
-                           pair2<R>(r2.x, r2.y)};   // (dE/dB_n, dE/dBS_n)
+    // (dE/dB_n, dE/dBS_n); the records of harmonics 2 k and 2 k + 1 are five 16-byte pieces
+    const v4<R> *rec = reinterpret_cast<const v4<R> *>(bb + BREC * (LM & ~1));
+    v2<R> Bp[NCH];
+    if constexpr (LM % 2 == 0) {
+        const v4<R> r0 = rec[0], r1 = rec[1];
+        mid = rec[2];
+        Bp[0] = pair2<R>(r0.x, r0.y); Bp[1] = pair2<R>(r0.z, r0.w); Bp[2] = pair2<R>(r1.x, r1.y);
+        Bp[3] = pair2<R>(r1.z, r1.w); Bp[4] = pair2<R>(mid.x, mid.y);
+    } else {
+        const v4<R> r3 = rec[3], r4 = rec[4];
+        Bp[0] = pair2<R>(mid.z, mid.w); Bp[1] = pair2<R>(r3.x, r3.y); Bp[2] = pair2<R>(r3.z, r3.w);
+        Bp[3] = pair2<R>(r4.x, r4.y); Bp[4] = pair2<R>(r4.z, r4.w);
+    }
     v2<R> aa = pair2<R>(R(0), R(0)), bq = pair2<R>(R(0), R(0));
 #pragma unroll
     for (int n = 0; n < NCH; ++n) {
@@ -1081,7 +1112,7 @@ __device__ __forceinline__ void bwd_harm(const R *__restrict__ bb, R ux, R uy, R
     avy += av * gy;
     avz += av * gz;
     cj += aa.y * p;
-    if constexpr (LM + 1 < NLM) bwd_harm<R, LM + 1>(bb, ux, uy, uz, s, g, dg, along, avx, avy, avz, cj);
+    if constexpr (LM + 1 < NLM) bwd_harm<R, LM + 1>(bb, ux, uy, uz, s, g, dg, along, avx, avy, avz, cj, mid);
 }
 
 // FP64, where instructions count and registers do not: the sums over n and lm are exchanged,
@@ -1098,11 +1129,8 @@ struct AngAdjoint {
     v2<R> psi[NCH];
     // harmonic lm = value p: Psi_n advanced, a_lm returned
     __device__ __forceinline__ R take(int lm, R p) {
-        const v4<R> *rec = reinterpret_cast<const v4<R> *>(bb + BREC * lm);
-        const v4<R> r0 = rec[0], r1 = rec[1];
-        const v2<R> r2 = *reinterpret_cast<const v2<R> *>(rec + 2);
-        const v2<R> Bp[NCH] = {pair2<R>(r0.x, r0.y), pair2<R>(r0.z, r0.w), pair2<R>(r1.x, r1.y),
-                               pair2<R>(r1.z, r1.w), r2};
+        const v2<R> *rec = reinterpret_cast<const v2<R> *>(bb + BREC * lm);
+        const v2<R> Bp[NCH] = {rec[0], rec[1], rec[2], rec[3], rec[4]};
         v2<R> aa = pair2<R>(Bp[0].x * g[0], Bp[0].y * g[0]);
 #pragma unroll
         for (int n = 1; n < NCH; ++n) aa = fma2(Bp[n], pair2<R>(g[n], g[n]), aa);
@@ -1289,7 +1317,8 @@ __device__ __forceinline__ void bwd_pair(const NepDev<R> &P, const Eval2Args<R> 
         } else {
             v2<R> al = pair2<R>(R(0), R(0));
             avx = avy = avz = cj = R(0);
-            bwd_harm<R, 0>(sm, ux, uy, uz, sij, g, dg, al, avx, avy, avz, cj);
+            v4<R> mid;
+            bwd_harm<R, 0>(sm, ux, uy, uz, sij, g, dg, al, avx, avy, avz, cj, mid);
             accu = al.x + sij * al.y;
         }
         accu -= ir * (ux * avx + uy * avy + uz * avz);   // only the part across u turns the pair
@@ -1368,12 +1397,12 @@ __device__ __forceinline__ void bwd_body(const NepDev<R> &P, const Eval2Args<R> 
     const int64_t i = (blk * (blockDim.x >> 5) + warp) * APW + grp;
     const bool valid = i < a.n;
     const int64_t N = a.n;
-    R *sm = reinterpret_cast<R *>(smem_raw) + (warp * APW + grp) * BW_ATOM;
+    R *sm = reinterpret_cast<R *>(smem_raw) + warp * (LPA == 4 ? BW_WARP : BW_ATOM) + bwd_at<LPA>(grp);
     // the atom's lanes
     [[maybe_unused]] const unsigned quad = LPA == 32 ? 0xffffffffu : ((1u << (LPA & 31)) - 1u) << (grp * LPA);
     // FP32, four lanes per atom: both centres' coefficients in shared memory, after the atoms' (read
     // from global memory where they are used they came to 1.70 ms at 884,736 atoms)
-    [[maybe_unused]] R *ctab = reinterpret_cast<R *>(smem_raw) + (blockDim.x >> 5) * APW * BW_ATOM;
+    [[maybe_unused]] R *ctab = reinterpret_cast<R *>(smem_raw) + (blockDim.x >> 5) * BW_WARP;
     if constexpr (sizeof(R) == 4 && LPA == 4) {
         const v4<R> *src = reinterpret_cast<const v4<R> *>(a.ctab + CTAB_BWD);
         for (int e = threadIdx.x; e < NS * CB_CENTRE / 4; e += blockDim.x) reinterpret_cast<v4<R> *>(ctab)[e] = ro(src + e);
@@ -1417,26 +1446,46 @@ __device__ __forceinline__ void bwd_body(const NepDev<R> &P, const Eval2Args<R> 
         // 16-byte loads each)
 #pragma unroll
         for (int m = 0; m < (NLM + LPA - 1) / LPA; ++m) {
-            const int lm = ql + LPA * m;
+            const int lm = lm_of<LPA>(ql, m);
             if (LPA > 8 && lm >= NLM) break;
-            const int l = l_of_lm(lm);
-            const R k2 = R(2) * kappa_of_lm<R>(lm);
-            const v4<R> *src = reinterpret_cast<const v4<R> *>(a.bsum + ((int64_t)i * NLM + lm) * BREC);
-            v4<R> w0 = ro(src), w1 = ro(src + 1), w2 = ro(src + 2), x0, x1;
+            const int64_t at = ((int64_t)i * NLM + lm) * BREC;
+            v4<R> x0, x1;
             v2<R> x2;
-            if constexpr (LPA == 4) {
-                const R *e = sm + BW_C + 12 * (l - 1);
-                x0 = reinterpret_cast<const v4<R> *>(e)[0];
-                x1 = reinterpret_cast<const v4<R> *>(e)[1];
-                x2 = *reinterpret_cast<const v2<R> *>(e + 8);
+            if constexpr (LPA == 4) {   // with its neighbour's record, in five pieces
+                if (m % 2) continue;
+                v4<R> w[5];
+#pragma unroll
+                for (int q = 0; q < 5; ++q) w[q] = ro(reinterpret_cast<const v4<R> *>(a.bsum + at) + q);
+                auto entries = [&](int l) {
+                    const R *e = sm + BW_C + 12 * (l - 1);
+                    x0 = reinterpret_cast<const v4<R> *>(e)[0];
+                    x1 = reinterpret_cast<const v4<R> *>(e)[1];
+                    x2 = *reinterpret_cast<const v2<R> *>(e + 8);
+                };
+                entries(l_of_lm(lm));
+                const R k2 = R(2) * kappa_of_lm<R>(lm), k3 = R(2) * kappa_of_lm<R>(lm + 1);
+                w[0].x *= k2 * x0.x; w[0].y *= k2 * x0.y; w[0].z *= k2 * x0.z; w[0].w *= k2 * x0.w;
+                w[1].x *= k2 * x1.x; w[1].y *= k2 * x1.y; w[1].z *= k2 * x1.z; w[1].w *= k2 * x1.w;
+                w[2].x *= k2 * x2.x; w[2].y *= k2 * x2.y;
+                entries(l_of_lm(lm + 1));
+                w[2].z *= k3 * x0.x; w[2].w *= k3 * x0.y;
+                w[3].x *= k3 * x0.z; w[3].y *= k3 * x0.w; w[3].z *= k3 * x1.x; w[3].w *= k3 * x1.y;
+                w[4].x *= k3 * x1.z; w[4].y *= k3 * x1.w; w[4].z *= k3 * x2.x; w[4].w *= k3 * x2.y;
+                v4<R> *d = reinterpret_cast<v4<R> *>(sm + BREC * lm);
+#pragma unroll
+                for (int q = 0; q < 5; ++q) d[q] = w[q];
             } else {
-                angular_entries(l, x0, x1, x2);
+                angular_entries(l_of_lm(lm), x0, x1, x2);
+                const R k2 = R(2) * kappa_of_lm<R>(lm);
+                const v2<R> e[NCH] = {pair2<R>(x0.x, x0.y), pair2<R>(x0.z, x0.w), pair2<R>(x1.x, x1.y),
+                                      pair2<R>(x1.z, x1.w), x2};
+#pragma unroll
+                for (int n = 0; n < NCH; ++n) {
+                    v2<R> w = ro(reinterpret_cast<const v2<R> *>(a.bsum + at) + n);
+                    w.x *= k2 * e[n].x; w.y *= k2 * e[n].y;
+                    reinterpret_cast<v2<R> *>(sm + BREC * lm)[n] = w;
+                }
             }
-            w0.x *= k2 * x0.x; w0.y *= k2 * x0.y; w0.z *= k2 * x0.z; w0.w *= k2 * x0.w;
-            w1.x *= k2 * x1.x; w1.y *= k2 * x1.y; w1.z *= k2 * x1.z; w1.w *= k2 * x1.w;
-            w2.x *= k2 * x2.x; w2.y *= k2 * x2.y; w2.z = R(0); w2.w = R(0);
-            v4<R> *d = reinterpret_cast<v4<R> *>(sm + BREC * lm);
-            d[0] = w0; d[1] = w1; d[2] = w2;
         }
         if constexpr (LPA == 4) __syncwarp(quad);   // the entries are read: the coefficients take their place
         if (ql == 0) {   // onsite term dE_i/dS_i = 2 Fp_O S_i, counted once per atom
@@ -1580,7 +1629,7 @@ template <typename R>
 static constexpr size_t fwd_smem(int qb = quad_block<R>()) { return (size_t)(qb / 32) * FWARP * sizeof(R); }
 template <typename R>
 static constexpr size_t bwdf_smem(int qb = quad_block<R>()) {
-    return ((size_t)(qb / 32) * 8 * BW_ATOM + (sizeof(R) == 4 ? NS * CB_CENTRE : 0)) * sizeof(R);
+    return ((size_t)(qb / 32) * BW_WARP + (sizeof(R) == 4 ? NS * CB_CENTRE : 0)) * sizeof(R);
 }
 template <typename R>
 static constexpr size_t bwdw_smem(int qb) { return (size_t)(qb / 32) * BW_ATOM * sizeof(R); }
