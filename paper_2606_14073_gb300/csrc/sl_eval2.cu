@@ -774,6 +774,48 @@ struct AngLanes {
     }
 };
 
+// g_n of the angular channels and the harmonics at u.  FP64, bound by its pipe: the contraction without
+// the f_k (see Carrier) and the harmonics from shared products, some 25 of 150 FP64 instructions of a
+// staged pair less (1,719 to 1,652 us at 110,592 atoms); FP32, which the shared-memory path
+// bounds, gains nothing from either (518 to 520 us at 884,736 atoms).
+template <typename R, int TI, int TJ>
+__device__ __forceinline__ void ang_g(const NepDev<R> &P, R r, R inv_rc, R g[NCH]) {
+    if constexpr (sizeof(R) == 4) {
+        R f[NK];
+        carrier_f(r, inv_rc, f);
+        contract_k<R, TI, TJ, G_A>(P, f, g);
+    } else {
+        const R t = r * inv_rc, fch = cut_half(t), y = t - R(1), x = fma_(R(2) * y, y, R(-1)), x2 = R(2) * x;
+        R pn[NCH], m = R(1), c = x;
+#pragma unroll
+        for (int n = 0; n < NCH; ++n) pn[n] = fma_(P.c[TI][TJ][G_A][n][1], x, P.ca0[TI][TJ][n]);
+#pragma unroll
+        for (int k = 2; k < NK; ++k) {
+            const R tk = fma_(x2, c, -m);
+#pragma unroll
+            for (int n = 0; n < NCH; ++n) pn[n] = fma_(P.c[TI][TJ][G_A][n][k], tk, pn[n]);
+            m = c;
+            c = tk;
+        }
+#pragma unroll
+        for (int n = 0; n < NCH; ++n) g[n] = fch * pn[n];
+    }
+}
+__device__ __forceinline__ void ang_harm(float x, float y, float z, float p[NLM]) { harm_p(x, y, z, p); }
+__device__ __forceinline__ void ang_harm(double x, double y, double z, double p[NLM]) {
+    const double x2 = x * x, y2 = y * y, z2 = z * z, q = x2 + y2, r2 = q + z2;
+    const double xy = x * y, yz = y * z, xz = x * z, d = x2 - y2;
+    const double c1 = fma(3.0, x2, -y2), c2 = fma(-3.0, y2, x2), c3 = fma(4.0, z2, -q);
+    const double c5 = fma(6.0, z2, -q), c6 = fma(4.0, z2, -3.0 * q);
+    p[0] = x; p[1] = y; p[2] = z;
+    p[3] = xy; p[4] = yz; p[5] = xz; p[6] = d; p[7] = fma(2.0, z2, -q);
+    p[8] = y * c1; p[9] = xy * z; p[10] = y * c3; p[11] = z * fma(2.0, z2, -3.0 * q); p[12] = x * c3; p[13] = z * d;
+    p[14] = x * c2;
+    p[15] = xy * d; p[16] = yz * c1; p[17] = xy * c5; p[18] = yz * c6;
+    p[19] = fma(z2, fma(35.0, z2, -30.0 * r2), 3.0 * r2 * r2);
+    p[20] = xz * c6; p[21] = d * c5; p[22] = xz * c2; p[23] = fma(d, d, -4.0 * xy * xy);
+}
+
 template <typename R, int LPA, int TI, int TJ>
 __device__ __forceinline__ void ang_stage_fwd(const NepDev<R> &P, const Eval2Args<R> &a, const v4<R> &pi,
                                               const v4<R> &si, const v4<R> &pj, const v4<R> &sj, R *st) {
@@ -781,9 +823,8 @@ __device__ __forceinline__ void ang_stage_fwd(const NepDev<R> &P, const Eval2Arg
     sep(a.box, pi, pj, dx, dy, dz);
     const R d2 = dx * dx + dy * dy + dz * dz;
     const R ir = rsqrt_(d2), r = d2 * ir;
-    R f[NK], g[NCH];
-    carrier_f(r, P.inv_rc_a, f);
-    contract_k<R, TI, TJ, G_A>(P, f, g);
+    R g[NCH];
+    ang_g<R, TI, TJ>(P, r, P.inv_rc_a, g);
     const R s = si.x * sj.x + si.y * sj.y + si.z * sj.z;
     v4<R> w0, w1;
     v2<R> w2;
@@ -794,7 +835,7 @@ __device__ __forceinline__ void ang_stage_fwd(const NepDev<R> &P, const Eval2Arg
     reinterpret_cast<v4<R> *>(st)[1] = w1;
     reinterpret_cast<v2<R> *>(st)[4] = w2;
     R p[NLM];
-    harm_p(dx * ir, dy * ir, dz * ir, p);
+    ang_harm(dx * ir, dy * ir, dz * ir, p);
     using L = AngLanes<LPA>;
 #pragma unroll
     for (int t = 0; t < NLM; t += 2) reinterpret_cast<v2<R> *>(st)[6 + t / 2] = pair2<R>(p[L::lm_at(t)], p[L::lm_at(t + 1)]);
