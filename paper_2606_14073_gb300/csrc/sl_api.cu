@@ -144,12 +144,12 @@ void fill_params(sl::NepDev<R> &P, const sl_nep_params *p) {
 }
 
 void free_sys(sl::Sys &s) {
-    void *ptrs[] = {s.pos, s.vel, s.spin, s.spin_prev, s.F, s.H, s.posref, s.posf, s.spinf, s.species, s.orig,
+    void *ptrs[] = {s.pos, s.vel, s.spin, s.spin_prev, s.F, s.H, s.posref, s.posf, s.psf, s.species, s.orig,
                     s.inv, s.nbr, s.rev, s.nbr_hash, s.cells.posf, s.cells.key, s.seg, s.cells.count, s.cells.start, s.cells.fill, s.cells.atoms,
                     s.cells.of, s.cells.sub, s.q, s.bsum, s.fp, s.ei, s.pairs, s.crow, s.ctab, s.cnt, s.cmask, s.fown, s.gii,
                     s.wpart, s.Fo, s.Ho,
                     s.status, s.rebuild, s.d_step, s.d_par, s.red, s.snap, s.d_builds,
-                    s.posmid, s.posmidf, s.mids, s.midsf, s.mx, s.mg, s.aax, s.aag, s.aapart, s.md, s.Bat,
+                    s.posmid, s.midposf, s.midpsf, s.mids, s.mx, s.mg, s.aax, s.aag, s.aapart, s.md, s.Bat,
                     s.tex_acc, s.tex_m, s.tex_part, s.colour, s.mlp_img, s.rb_count};
     for (void *p : ptrs)
         if (p) cudaFree(p);
@@ -452,7 +452,7 @@ int upload_vec(sl::Sys &s, double4 *dst, const double *src, bool normalise) {
     return SL_OK;
 }
 
-__global__ void k_wrap_and_copy(double4 *pos, float4 *posf, const double4 *spin, float4 *spinf, int64_t n,
+__global__ void k_wrap_and_copy(double4 *pos, const double4 *spin, float4 *posf, float4 *psf, int64_t n,
                                 sl::BoxDev<double> b, int px, int py, int pz) {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= n) return;
@@ -461,14 +461,17 @@ __global__ void k_wrap_and_copy(double4 *pos, float4 *posf, const double4 *spin,
     if (py) r.y = r.y - b.L[1] * floor(r.y / b.L[1]);
     if (pz) r.z = r.z - b.L[2] * floor(r.z / b.L[2]);
     pos[i] = r;
-    posf[i] = make_float4((float)r.x, (float)r.y, (float)r.z, 0.f);
+    const float4 rf = make_float4((float)r.x, (float)r.y, (float)r.z, 0.f);
+    posf[i] = rf;
+    if (!psf) return;
+    psf[2 * i] = rf;
     const double4 S = spin[i];
-    spinf[i] = make_float4((float)S.x, (float)S.y, (float)S.z, 0.f);
+    psf[2 * i + 1] = make_float4((float)S.x, (float)S.y, (float)S.z, 0.f);
 }
 
 int refresh_copies(sl::Sys &s) {
     if (s.n == 0) return SL_OK;
-    k_wrap_and_copy<<<(unsigned)((s.n + 255) / 256), 256, 0, s.stream>>>(s.pos, s.posf, s.spin, s.spinf, s.n, s.boxd,
+    k_wrap_and_copy<<<(unsigned)((s.n + 255) / 256), 256, 0, s.stream>>>(s.pos, s.spin, s.posf, s.psf, s.n, s.boxd,
                                                                          s.per[0], s.per[1], s.per[2]);
     CK(cudaGetLastError());
     return SL_OK;
@@ -684,7 +687,7 @@ int sl_create_system(const double *positions, const double *spins, const double 
     s.qs = (n + 3) & ~(int64_t)3;
     if ((rc = dalloc(&s.pos, N)) || (rc = dalloc(&s.vel, N)) || (rc = dalloc(&s.spin, N)) ||
         (rc = dalloc(&s.spin_prev, N)) || (rc = dalloc(&s.F, N)) || (rc = dalloc(&s.H, N)) ||
-        (rc = dalloc(&s.posref, N)) || (rc = dalloc(&s.posf, N)) || (rc = dalloc(&s.spinf, N)) ||
+        (rc = dalloc(&s.posref, N)) || (rc = dalloc(&s.posf, N)) || (s.prec != SL_PREC_FP64 && (rc = dalloc(&s.psf, 2 * N))) ||
         (rc = dalloc(&s.species, N)) || (rc = dalloc(&s.orig, N)) || (rc = dalloc(&s.inv, N)) ||
         (rc = dalloc(&s.nbr, N * sl::nbr_stride(s.cap))) || (rc = dalloc(&s.rev, N * sl::nbr_stride(s.cap))) ||
         (rc = dalloc(&s.nbr_hash, N * sl::nbr_stride(s.cap))) ||
@@ -710,8 +713,8 @@ int sl_create_system(const double *positions, const double *spins, const double 
         return bail(fail(SL_ENOMEM, "the network weights' operand images could not be made"));
     if (s.mid_iters > 0) {
         const size_t ring = (size_t)(s.aa_depth > 0 ? s.aa_depth + 1 : 0) * N;
-        if ((rc = dalloc(&s.posmid, N)) || (rc = dalloc(&s.posmidf, N)) || (rc = dalloc(&s.mids, N)) ||
-            (rc = dalloc(&s.midsf, N)) || (rc = dalloc(&s.mx, N)) || (rc = dalloc(&s.mg, N)) ||
+        if ((rc = dalloc(&s.posmid, N)) || (rc = dalloc(&s.midposf, N)) || (s.prec != SL_PREC_FP64 && (rc = dalloc(&s.midpsf, 2 * N))) || (rc = dalloc(&s.mids, N)) ||
+            (rc = dalloc(&s.mx, N)) || (rc = dalloc(&s.mg, N)) ||
             (rc = dalloc(&s.aax, ring)) || (rc = dalloc(&s.aag, ring)) ||
             (rc = dalloc(&s.aapart, sl::midpoint_scratch_doubles())) || (rc = dalloc(&s.md, 1)))
             return bail(rc);
@@ -1411,7 +1414,8 @@ int64_t sl_estimate_device_bytes(int64_t n, const sl_options *opt_in) {
     if (n < 0) return -1;
     const int64_t R = opt.precision == SL_PREC_FP64 ? 8 : 4;
     const int64_t cap = opt.nbr_cap_rad, ca = opt.nbr_cap_ang;
-    int64_t per = 7 * 32 + 2 * 16                      // state (double4) and FP32 copies
+    const int64_t copies = R == 4 ? 48 : 16;           // FP32 copies of positions and spins
+    int64_t per = 7 * 32 + copies                      // state (double4) and FP32 copies
                   + 3 * 4 + 4 + 16 + 16 + 4            // species, caller index maps, list segments, cell copies
                   + 6 * sl::nbr_stride((int)cap)     // candidate lists, reverse slots and index hashes (1 byte each)
                   + 8 * (ca + cap) + 16                // compact rows, counts
@@ -1420,7 +1424,7 @@ int64_t sl_estimate_device_bytes(int64_t n, const sl_options *opt_in) {
                   + R * 8 * cap + 2 * R * 4            // pair records, per-atom sums
                   + 2 * 32 + 5 * 32 + 4 * 4;           // evaluation outputs, snapshot, cell arrays
     if (opt.midpoint_iters > 0)                        // midpoint positions and spins, iterate, image, rings
-        per += 4 * 32 + 2 * 16 + (opt.anderson_depth > 0 ? 2 * 32 * (opt.anderson_depth + 1) : 0);
+        per += 4 * 32 + copies + (opt.anderson_depth > 0 ? 2 * 32 * (opt.anderson_depth + 1) : 0);
     return n * per + (1 << 20);
 }
 

@@ -20,14 +20,14 @@ struct PairRec {
 
 template <typename R>
 struct Eval2Args {
-    const v4<R> *pos, *spin;
+    const v4<R> *pos, *spin;   // FP32: psf and psf + 1 (atom j at 2 j; pair_at)
     const int32_t *nbr;   // [n][capr] candidate list of atom i (internal indices), atom-major
     const uint8_t *rev;   // [n][capr] rev[i][s] = slot of i in the list of nbr[i][s]
     int capr;             // row stride of nbr and rev: cap rounded up to a multiple of 32
     const int4 *seg;
     int64_t n, n_fe;
     BoxDev<R> box;
-    const float4 *posf;    // FP64 kernels: FP32 copies of pos and box (the cutoff pre-test)
+    const float4 *posf;    // FP32 copies of the positions, and of the box (the cutoff tests)
     BoxDev<float> boxf;
     int cap, cap_ang;
     int2 *crow;        // compact in-cutoff rows [cap_ang + cap][n]: angular rows from 0, radial-only rows from

@@ -27,9 +27,9 @@ namespace sl {
 
 struct IntArgs {
     double4 *pos, *vel, *spin, *spin_prev, *F, *H, *posref;
-    float4 *posf, *spinf;
+    float4 *posf, *psf; // FP32 copies (Sys::posf, psf)
     double4 *posmid;    // non-null in the midpoint mode: lattice midpoint of the step
-    float4 *posmidf;
+    float4 *midposf, *midpsf;
     const double4 *Bat; // non-null: per-atom part of the external field (tesla)
     const int32_t *orig;
     int64_t n, n_fe;
@@ -94,7 +94,9 @@ __device__ __forceinline__ void first_half_body(const IntArgs &a, int64_t blk) {
         for (int d = 0; d < 3; ++d)
             if (a.per[d]) m3[d] = m3[d] - a.bd.L[d] * floor(m3[d] * a.bd.invL[d]);
         a.posmid[i] = make_double4(m3[0], m3[1], m3[2], 0.0);
-        a.posmidf[i] = make_float4((float)m3[0], (float)m3[1], (float)m3[2], 0.f);
+        const float4 mf = make_float4((float)m3[0], (float)m3[1], (float)m3[2], 0.f);
+        a.midposf[i] = mf;
+        if constexpr (MIXED) a.midpsf[2 * i] = mf;
     }
     // wrapped, x - L floor(x / L) on the periodic axes: seen on the quotients' high words, floor is 0
     // (every quotient at least 0 and below 1) for nearly every atom
@@ -135,8 +137,12 @@ __device__ __forceinline__ void first_half_body(const IntArgs &a, int64_t blk) {
     a.vel[i] = v;
     a.spin_prev[i] = S;
     a.spin[i] = make_double4(Sp[0], Sp[1], Sp[2], 0.0);
-    a.posf[i] = make_float4((float)r.x, (float)r.y, (float)r.z, 0.f);
-    a.spinf[i] = make_float4((float)Sp[0], (float)Sp[1], (float)Sp[2], 0.f);
+    const float4 rf = make_float4((float)r.x, (float)r.y, (float)r.z, 0.f);
+    a.posf[i] = rf;
+    if constexpr (MIXED) {
+        a.psf[2 * i] = rf;
+        a.psf[2 * i + 1] = make_float4((float)Sp[0], (float)Sp[1], (float)Sp[2], 0.f);
+    }
     // rebuild trigger: displacement since the last build beyond skin/2
     const double4 p0 = a.posref[i];
     double dx = r.x - p0.x, dy = r.y - p0.y, dz = r.z - p0.z;
@@ -218,7 +224,7 @@ __device__ __forceinline__ void second_half_body(const IntArgs &a, const GatherA
     v.x += hdt * Fs[0] * am; v.y += hdt * Fs[1] * am; v.z += hdt * Fs[2] * am;
     a.vel[i] = v;
     a.spin[i] = make_double4(Sn[0], Sn[1], Sn[2], 0.0);
-    a.spinf[i] = make_float4((float)Sn[0], (float)Sn[1], (float)Sn[2], 0.f);
+    if constexpr (MIXED) a.psf[2 * i + 1] = make_float4((float)Sn[0], (float)Sn[1], (float)Sn[2], 0.f);
     a.F[i] = make_double4(Fs[0], Fs[1], Fs[2], 0.0);
     a.H[i] = make_double4(Hs[0], Hs[1], Hs[2], 0.0);
     if (!(isfinite(Fs[0]) && isfinite(Fs[1]) && isfinite(Fs[2]) && isfinite(Hs[0]) && isfinite(Hs[1]) &&
@@ -320,20 +326,21 @@ __global__ void __launch_bounds__(256) k_sweep_rotate(IntArgs a, GatherArgs<R> g
     const double inn = 1.0 / sqrt(Sn[0] * Sn[0] + Sn[1] * Sn[1] + Sn[2] * Sn[2]);
     Sn[0] *= inn; Sn[1] *= inn; Sn[2] *= inn;
     a.spin[i] = make_double4(Sn[0], Sn[1], Sn[2], 0.0);
-    a.spinf[i] = make_float4((float)Sn[0], (float)Sn[1], (float)Sn[2], 0.f);
+    if constexpr (MIXED) a.psf[2 * i + 1] = make_float4((float)Sn[0], (float)Sn[1], (float)Sn[2], 0.f);
     if (!(isfinite(Hs[0]) && isfinite(Hs[1]) && isfinite(Hs[2]))) atomicOr(a.status, ST_NONFINITE);
 }
 
 static IntArgs int_args(Sys &s) {
     IntArgs a;
     a.pos = s.pos; a.vel = s.vel; a.spin = s.spin; a.spin_prev = s.spin_prev; a.F = s.F; a.H = s.H;
-    a.posref = s.posref; a.posf = s.posf; a.spinf = s.spinf; a.orig = s.orig; a.n = s.n; a.n_fe = s.n_fe;
+    a.posref = s.posref; a.posf = s.posf; a.psf = s.psf; a.orig = s.orig; a.n = s.n; a.n_fe = s.n_fe;
     a.bd = s.boxd;
     for (int d = 0; d < 3; ++d) a.per[d] = s.per[d];
     a.par = s.d_par; a.step = s.d_step; a.rebuild = s.rebuild; a.status = s.status;
     a.seed = s.seed; a.replica = s.replica;
     a.posmid = s.mid_iters > 0 ? s.posmid : nullptr;
-    a.posmidf = s.mid_iters > 0 ? s.posmidf : nullptr;
+    a.midposf = s.mid_iters > 0 ? s.midposf : nullptr;
+    a.midpsf = s.mid_iters > 0 ? s.midpsf : nullptr;
     a.Bat = s.Bat;
     return a;
 }
@@ -444,7 +451,7 @@ void launch_compare_bits(Sys &s, const double4 *ref, int *diff) {
 }
 
 // Unit length for every spin (leaving the longitudinal mode), FP64.
-__global__ void k_normalise_spins(double4 *spin, float4 *spinf, int64_t n, int *status) {
+__global__ void k_normalise_spins(double4 *spin, float4 *psf, int64_t n, int *status) {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= n) return;
     const double4 S = spin[i];
@@ -455,11 +462,11 @@ __global__ void k_normalise_spins(double4 *spin, float4 *spinf, int64_t n, int *
     }
     const double inn = 1.0 / sqrt(n2);
     spin[i] = make_double4(S.x * inn, S.y * inn, S.z * inn, 0.0);
-    spinf[i] = make_float4((float)(S.x * inn), (float)(S.y * inn), (float)(S.z * inn), 0.f);
+    if (psf) psf[2 * i + 1] = make_float4((float)(S.x * inn), (float)(S.y * inn), (float)(S.z * inn), 0.f);
 }
 
 void launch_normalise_spins(Sys &s) {
-    if (s.n > 0) k_normalise_spins<<<nblk(s.n, 256), 256, 0, s.stream>>>(s.spin, s.spinf, s.n, s.status);
+    if (s.n > 0) k_normalise_spins<<<nblk(s.n, 256), 256, 0, s.stream>>>(s.spin, s.psf, s.n, s.status);
 }
 
 

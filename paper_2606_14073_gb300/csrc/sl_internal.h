@@ -67,7 +67,7 @@ struct LaunchCfg {
 // optional device flag that makes the evaluation kernels return at once.
 struct EvalAt {
     const double4 *pos = nullptr, *spin = nullptr;
-    const float4 *posf = nullptr, *spinf = nullptr;
+    const float4 *posf = nullptr, *psf = nullptr;   // FP32 copies (Sys::posf, psf)
     const int *skip = nullptr;
 };
 
@@ -106,7 +106,8 @@ struct Sys {
     // state, internal atom order (species-major, then spatial cell order)
     double4 *pos = nullptr, *vel = nullptr, *spin = nullptr, *spin_prev = nullptr;
     double4 *F = nullptr, *H = nullptr, *posref = nullptr;
-    float4 *posf = nullptr, *spinf = nullptr;
+    float4 *posf = nullptr;    // FP32 positions (cutoff tests)
+    float4 *psf = nullptr;     // mixed precision: [n][2] FP32 position and spin, next to each other (one 32-byte sector)
     int32_t *species = nullptr, *orig = nullptr, *inv = nullptr;
     int64_t n_fe = 0;          // atoms [0, n_fe) are species 0
 
@@ -205,9 +206,8 @@ struct Sys {
     int mid_iters = 0, aa_depth = 0;
     double mid_tol = 0.0, aa_reg = 1e-10;
     double4 *posmid = nullptr;   // lattice midpoint of the step
-    float4 *posmidf = nullptr;
+    float4 *midposf = nullptr, *midpsf = nullptr;   // FP32 copies of the midpoint point (as posf and psf)
     double4 *mids = nullptr;     // midpoint spins (evaluation point of the iteration)
-    float4 *midsf = nullptr;
     double4 *mx = nullptr, *mg = nullptr;        // iterate X and its image G
     double4 *aax = nullptr, *aag = nullptr;      // Anderson rings [(depth + 1)][n]
     double *aapart = nullptr;                    // Anderson partial sums [AA_BLOCKS][...]

@@ -31,9 +31,8 @@ constexpr int AA_VALS = AA_MAX_DEPTH * AA_MAX_DEPTH + AA_MAX_DEPTH;
 struct MidArgs {
     const double4 *spin_prev;          // S_n
     double4 *spin;                     // state spins: X_0 on entry, S_{n+1} at the end
-    float4 *spinf;
+    float4 *psf, *midpsf;              // mixed precision: FP32 copies (Sys::psf), else null
     double4 *mids;                     // midpoint spins M_m
-    float4 *midsf;
     double4 *X, *G;                    // iterate and its image
     double4 *Xh, *Gh;                  // Anderson rings [(depth + 1)][n]
     double *part;                      // [AA_BLOCKS][AA_VALS]
@@ -79,7 +78,7 @@ __global__ void __launch_bounds__(256) k_mid_prep(MidArgs a, int m) {
     const double mx = S0.x + X.x, my = S0.y + X.y, mz = S0.z + X.z;
     const double inv = 1.0 / sqrt(mx * mx + my * my + mz * mz);
     a.mids[i] = make_double4(mx * inv, my * inv, mz * inv, 0.0);
-    a.midsf[i] = make_float4((float)(mx * inv), (float)(my * inv), (float)(mz * inv), 0.f);
+    if (a.midpsf) a.midpsf[2 * i + 1] = make_float4((float)(mx * inv), (float)(my * inv), (float)(mz * inv), 0.f);
 }
 
 template <typename R, bool MIXED, int W>
@@ -267,13 +266,13 @@ __global__ void __launch_bounds__(256) k_mid_final(MidArgs a) {
     const double inv = 1.0 / sqrt(G.x * G.x + G.y * G.y + G.z * G.z);
     const double sx = G.x * inv, sy = G.y * inv, sz = G.z * inv;
     a.spin[i] = make_double4(sx, sy, sz, 0.0);
-    a.spinf[i] = make_float4((float)sx, (float)sy, (float)sz, 0.f);
+    if (a.psf) a.psf[2 * i + 1] = make_float4((float)sx, (float)sy, (float)sz, 0.f);
 }
 
 MidArgs mid_args(Sys &s) {
     MidArgs a;
-    a.spin_prev = s.spin_prev; a.spin = s.spin; a.spinf = s.spinf;
-    a.mids = s.mids; a.midsf = s.midsf; a.X = s.mx; a.G = s.mg; a.Xh = s.aax; a.Gh = s.aag; a.part = s.aapart;
+    a.spin_prev = s.spin_prev; a.spin = s.spin; a.psf = s.psf;
+    a.mids = s.mids; a.midpsf = s.midpsf; a.X = s.mx; a.G = s.mg; a.Xh = s.aax; a.Gh = s.aag; a.part = s.aapart;
     a.posmid = s.posmid; a.posref = s.posref; a.Bat = s.Bat; a.orig = s.orig; a.n = s.n; a.n_fe = s.n_fe; a.bd = s.boxd;
     a.par = s.d_par; a.step = s.d_step; a.status = s.status; a.md = s.md; a.seed = s.seed; a.replica = s.replica;
     a.cap = s.mid_iters; a.depth = s.aa_depth; a.tol = s.mid_tol; a.reg = s.aa_reg;
@@ -311,7 +310,7 @@ int launch_midpoint(Sys &s) {
     const bool wide = gather_is_wide(s);
     k_mid_start<<<1, 64, 0, s.stream>>>(s.md, s.mid_iters);
     EvalAt at;
-    at.pos = s.posmid; at.posf = s.posmidf; at.spin = s.mids; at.spinf = s.midsf;
+    at.pos = s.posmid; at.spin = s.mids; at.posf = s.midposf; at.psf = s.midpsf;
     at.skip = reinterpret_cast<const int *>(reinterpret_cast<const char *>(s.md) + offsetof(MidDev, converged));
     for (int m = 0; m < s.mid_iters; ++m) {
         k_mid_prep<<<nb, 256, 0, s.stream>>>(a, m);
