@@ -202,22 +202,30 @@ int upload_params(sl::Sys &s, double dt, double T, const double B[3]) {
     return SL_OK;
 }
 
-void enqueue_step(sl::Sys &s) {
-    sl::launch_first_half(s);
-    sl::launch_rebuild(s, true);
-    if (s.mid_iters > 0) {          // self-consistent midpoint spin update, then the end state
-        sl::launch_midpoint(s);
-        sl::launch_eval(s, false);
-        sl::launch_second_half_nospin(s);
-    } else {
-        sl::launch_eval(s, false);
-        sl::launch_second_half(s);
+// n steps in a row; the second half of one and the first half of the next share a launch
+void enqueue_steps(sl::Sys &s, int64_t n) {
+    for (int64_t t = 0; t < n; ++t) {
+        if (t == 0 || s.mid_iters > 0) sl::launch_first_half(s);
+        sl::launch_rebuild(s, true);
+        if (s.mid_iters > 0) {      // self-consistent midpoint spin update, then the end state
+            sl::launch_midpoint(s);
+            sl::launch_eval(s, false);
+            sl::launch_second_half_nospin(s);
+        } else {
+            sl::launch_eval(s, false);
+            if (t + 1 < n) sl::launch_halves(s, t);
+            else sl::launch_second_half(s);
+        }
     }
 }
 
 // (a one-launch rebuild takes one of the eight launches of its group)
 int64_t step_kernels(const sl::Sys &s) { return sl::KERNELS_PER_STEP - (s.rb_count ? 7 : 0); }
 int64_t kernels_per_step(const sl::Sys &s) { return step_kernels(s) + sl::midpoint_kernels_per_step(s); }
+// of `queues` queues of n steps each (enqueue_steps)
+int64_t queue_kernels(const sl::Sys &s, int64_t queues, int64_t n) {
+    return queues * (n * kernels_per_step(s) - (s.mid_iters > 0 || n == 0 ? 0 : n - 1));
+}
 
 // Evaluate at the current state: optional unconditional rebuild, eval, gather.
 int evaluate(sl::Sys &s, bool rebuild, bool carried, bool want_virial) {
@@ -484,7 +492,7 @@ int capture_graph(sl::Sys &s, int k) {
     }
     cudaGraph_t g;
     CK(cudaStreamBeginCapture(s.stream, cudaStreamCaptureModeThreadLocal));
-    for (int t = 0; t < k; ++t) enqueue_step(s);
+    enqueue_steps(s, k);
     cudaError_t e = cudaStreamEndCapture(s.stream, &g);
     if (e != cudaSuccess) return cuda_fail(e, "graph capture");
     e = cudaGraphInstantiate(&s.graph, g, 0);
@@ -930,9 +938,10 @@ static int queue_steps(sl::Sys &s, int64_t n_steps) {
             left -= k;
         }
     }
-    for (; left > 0; --left) enqueue_step(s);
+    enqueue_steps(s, left);
     CK(cudaGetLastError());
-    s.n_launches += n_steps * kernels_per_step(s);
+    if (k > 0) s.n_launches += queue_kernels(s, (n_steps - left) / k, k);
+    s.n_launches += queue_kernels(s, 1, left);
     return SL_OK;
 }
 
@@ -1568,7 +1577,7 @@ static int batch_graph(sl_batch *b, int g) {
         if (!b->sys[i]) continue;
         sl::Sys &s = b->sys[i]->s;
         CK(cudaStreamWaitEvent(s.stream, b->ev[0], 0));
-        for (int t = 0; t < g; ++t) enqueue_step(s);
+        enqueue_steps(s, g);
         CK(cudaEventRecord(b->ev[1 + i], s.stream));
         CK(cudaStreamWaitEvent(b->stream, b->ev[1 + i], 0));
     }
@@ -1668,16 +1677,17 @@ static int replica_steps(sl_batch *b, const std::vector<int> &active, const int6
         for (int i : active) {   // and each replica's stream waits for the batch
             sl::Sys &s = b->sys[i]->s;
             CK(cudaStreamWaitEvent(s.stream, b->ev[0], 0));
-            s.n_launches += rounds * g * kernels_per_step(s);
-            b->kernel_launches += rounds * g * kernels_per_step(s);
+            s.n_launches += queue_kernels(s, rounds, g);
+            b->kernel_launches += queue_kernels(s, rounds, g);
         }
     }
     for (int i : active) {
         sl::Sys &s = b->sys[i]->s;
         const int64_t left = n_steps[i] - rounds * g;
         if (left > 0) {
+            const int64_t before = s.n_launches;
             if ((rc = queue_steps(s, left))) return rc;
-            b->kernel_launches += left * kernels_per_step(s);
+            b->kernel_launches += s.n_launches - before;
         }
     }
     ++b->replica_calls;

@@ -43,11 +43,10 @@ struct IntArgs {
 
 // Landau onsite field -(2a + 4b|S|^2) S of atom i (species t), added to H.
 __device__ __forceinline__ void add_landau(const StepDev &P, int t, const double4 S, double H[3]) {
-    const double m2 = S.x * S.x + S.y * S.y + S.z * S.z;
-    const double k = -(2.0 * P.landau[t][0] + 4.0 * P.landau[t][1] * m2);
-    H[0] += k * S.x; H[1] += k * S.y; H[2] += k * S.z;
+    const double m2 = dot3_(S.x, S.y, S.z, S.x, S.y, S.z);
+    const double k = -fma_(mul_(4.0, P.landau[t][1]), m2, mul_(2.0, P.landau[t][0]));
+    H[0] = fma_(k, S.x, H[0]); H[1] = fma_(k, S.y, H[1]); H[2] = fma_(k, S.z, H[2]);
 }
-
 
 
 // Whether the high word (under mask) of a component times 1/L reaches `from`.
@@ -60,17 +59,12 @@ __device__ __forceinline__ bool outside(double x, double y, double z, const BoxD
     return max(max(hx, hy), hz) >= from;
 }
 
+// First half of step st of atom i (species t, stream id) from its velocity, force, field and spin.
 template <bool MIXED>
-__device__ __forceinline__ void first_half_body(const IntArgs &a, int64_t blk) {
-    const int64_t i = blk * (int64_t)blockDim.x + threadIdx.x;
-    const unsigned long long st = a.step[0];
-    if (i == 0) a.step[1] = st;
-    if (i >= a.n) return;
+__device__ __forceinline__ void first_half_atom(const IntArgs &a, int64_t i, unsigned long long st, int t, uint64_t id,
+                                                double4 v, const double4 &F, const double4 &H, const double4 &S) {
     const StepDev &P = *a.par;
-    const int t = i < a.n_fe ? 0 : 1;
-    const uint64_t id = (uint64_t)a.orig[i];
-    double4 r = a.pos[i], v = a.vel[i];
-    const double4 F = a.F[i], H = a.H[i], S = a.spin[i];
+    double4 r = a.pos[i];
     const double hdt = P.half_dt, am = P.acc_m[t];
     double xi[3], ze[3];
     if constexpr (MIXED) {
@@ -83,11 +77,13 @@ __device__ __forceinline__ void first_half_body(const IntArgs &a, int64_t blk) {
         gauss3(st, id, 2, a.seed, a.replica, ze);
     }
     const double4 r0 = r;
-    v.x += hdt * F.x * am; v.y += hdt * F.y * am; v.z += hdt * F.z * am;
-    r.x += hdt * v.x; r.y += hdt * v.y; r.z += hdt * v.z;
+    auto kick = [&](double &x, double f) { x = fma_(mul_(hdt, f), am, x); };
+    auto drift = [&]() { r.x = fma_(hdt, v.x, r.x); r.y = fma_(hdt, v.y, r.y); r.z = fma_(hdt, v.z, r.z); };
+    kick(v.x, F.x); kick(v.y, F.y); kick(v.z, F.z);
+    drift();
     const double c = P.c_fric, sv = P.sig_v[t];
-    v.x = c * v.x + sv * xi[0]; v.y = c * v.y + sv * xi[1]; v.z = c * v.z + sv * xi[2];
-    r.x += hdt * v.x; r.y += hdt * v.y; r.z += hdt * v.z;
+    v.x = fma_(c, v.x, mul_(sv, xi[0])); v.y = fma_(c, v.y, mul_(sv, xi[1])); v.z = fma_(c, v.z, mul_(sv, xi[2]));
+    drift();
     if (a.posmid) {   // lattice midpoint r0 + (r - r0)/2 of the unwrapped step, then wrapped
         double m3[3] = {r0.x + 0.5 * (r.x - r0.x), r0.y + 0.5 * (r.y - r0.y), r0.z + 0.5 * (r.z - r0.z)};
 #pragma unroll
@@ -101,9 +97,9 @@ __device__ __forceinline__ void first_half_body(const IntArgs &a, int64_t blk) {
     // wrapped, x - L floor(x / L) on the periodic axes: seen on the quotients' high words, floor is 0
     // (every quotient at least 0 and below 1) for nearly every atom
     if (outside(r.x, r.y, r.z, a.bd, 0xFFFFFFFFu, 0x3FF00000u)) {
-        if (a.per[0]) r.x = r.x - a.bd.L[0] * floor(r.x * a.bd.invL[0]);
-        if (a.per[1]) r.y = r.y - a.bd.L[1] * floor(r.y * a.bd.invL[1]);
-        if (a.per[2]) r.z = r.z - a.bd.L[2] * floor(r.z * a.bd.invL[2]);
+        if (a.per[0]) r.x = fma_(-a.bd.L[0], floor(mul_(r.x, a.bd.invL[0])), r.x);
+        if (a.per[1]) r.y = fma_(-a.bd.L[1], floor(mul_(r.y, a.bd.invL[1])), r.y);
+        if (a.per[2]) r.z = fma_(-a.bd.L[2], floor(mul_(r.z, a.bd.invL[2])), r.z);
     }
     const double se = P.sig_eta;
     double Sp[3];
@@ -112,25 +108,25 @@ __device__ __forceinline__ void first_half_body(const IntArgs &a, int64_t blk) {
     } else if constexpr (MIXED) {
         float w[3], d[3];
         const float fse = (float)se;
-        omega_of_f((float)S.x, (float)S.y, (float)S.z, (float)H.x + fse * (float)ze[0],
-                   (float)H.y + fse * (float)ze[1], (float)H.z + fse * (float)ze[2], (float)P.lambda,
-                   (float)P.wscale, w);
+        omega_of((float)S.x, (float)S.y, (float)S.z, fma_(fse, (float)ze[0], (float)H.x),
+                 fma_(fse, (float)ze[1], (float)H.y), fma_(fse, (float)ze[2], (float)H.z), (float)P.lambda,
+                 (float)P.wscale, w);
         rotate_delta_f((float)S.x, (float)S.y, (float)S.z, w[0], w[1], w[2], (float)P.dt, d);
         if (P.lng) {
             const float kd = (float)P.lng_drift, ks = (float)P.lng_sig;
-            d[0] += kd * (float)H.x + ks * (float)ze[0];
-            d[1] += kd * (float)H.y + ks * (float)ze[1];
-            d[2] += kd * (float)H.z + ks * (float)ze[2];
+            d[0] += fma_(kd, (float)H.x, mul_(ks, (float)ze[0]));
+            d[1] += fma_(kd, (float)H.y, mul_(ks, (float)ze[1]));
+            d[2] += fma_(kd, (float)H.z, mul_(ks, (float)ze[2]));
         }
         Sp[0] = S.x + (double)d[0]; Sp[1] = S.y + (double)d[1]; Sp[2] = S.z + (double)d[2];
     } else {
         double w[3];
-        omega_of(S.x, S.y, S.z, H.x + se * ze[0], H.y + se * ze[1], H.z + se * ze[2], P.lambda, P.wscale, w);
+        omega_of(S.x, S.y, S.z, fma_(se, ze[0], H.x), fma_(se, ze[1], H.y), fma_(se, ze[2], H.z), P.lambda, P.wscale, w);
         rotate(S.x, S.y, S.z, w, P.dt, Sp);
         if (P.lng) {
-            Sp[0] += P.lng_drift * H.x + P.lng_sig * ze[0];
-            Sp[1] += P.lng_drift * H.y + P.lng_sig * ze[1];
-            Sp[2] += P.lng_drift * H.z + P.lng_sig * ze[2];
+            Sp[0] += fma_(P.lng_drift, H.x, mul_(P.lng_sig, ze[0]));
+            Sp[1] += fma_(P.lng_drift, H.y, mul_(P.lng_sig, ze[1]));
+            Sp[2] += fma_(P.lng_drift, H.z, mul_(P.lng_sig, ze[2]));
         }
     }
     a.pos[i] = r;
@@ -146,27 +142,49 @@ __device__ __forceinline__ void first_half_body(const IntArgs &a, int64_t blk) {
     // rebuild trigger: displacement since the last build beyond skin/2
     const double4 p0 = a.posref[i];
     double dx = r.x - p0.x, dy = r.y - p0.y, dz = r.z - p0.z;
-    if (outside(dx, dy, dz, a.bd, 0x7FFFFFFFu, 0x3FE00000u)) minimg(a.bd, dx, dy, dz);   // a quotient of 1/2 or more
-    if (dx * dx + dy * dy + dz * dz > P.disp2) *a.rebuild = 1;
+    if (outside(dx, dy, dz, a.bd, 0x7FFFFFFFu, 0x3FE00000u)) {   // a quotient of 1/2 or more
+        dx = fma_(-a.bd.L[0], rint(mul_(dx, a.bd.invL[0])), dx);
+        dy = fma_(-a.bd.L[1], rint(mul_(dy, a.bd.invL[1])), dy);
+        dz = fma_(-a.bd.L[2], rint(mul_(dz, a.bd.invL[2])), dz);
+    }
+    if (dot3_(dx, dy, dz, dx, dy, dz) > P.disp2) *a.rebuild = 1;
+}
+
+template <bool MIXED>
+__device__ __forceinline__ void first_half_body(const IntArgs &a, int64_t blk) {
+    const int64_t i = blk * (int64_t)blockDim.x + threadIdx.x;
+    const unsigned long long st = a.step[0];
+    if (i == 0) a.step[1] = st;
+    if (i >= a.n) return;
+    first_half_atom<MIXED>(a, i, st, i < a.n_fe ? 0 : 1, (uint64_t)a.orig[i], a.vel[i], a.F[i], a.H[i], a.spin[i]);
+}
+
+// Values as the compiler cannot trace them, so what is computed from them is computed as from loads.
+__device__ __forceinline__ double4 opaque(double x, double y, double z) {
+    asm volatile("" : "+d"(x), "+d"(y), "+d"(z));
+    return make_double4(x, y, z, 0.0);
 }
 
 // SPIN = false (midpoint mode): the spins were already advanced by the midpoint
 // iteration; only the gather, the final kick and the carried F, H remain.
-template <typename R, bool MIXED, int W, bool SPIN = true>
+// NEXT: followed by the first half of the next step, the same operations in the same order (k_halves).
+// Step counters: step[0] is the step that a queue of k_halves launches starts from, which the last second
+// half moves on, and step[1] the step being taken; ahead is the launch's place in its queue.
+template <typename R, bool MIXED, int W, bool SPIN = true, bool NEXT = false>
 __device__ __forceinline__ void second_half_body(const IntArgs &a, const GatherArgs<R> &g, int64_t blk,
-                                                 GatherSmem<R, W> &sm) {
+                                                 GatherSmem<R, W> &sm, unsigned long long ahead = 0) {
     double Fs[3], Hs[3];
     const int64_t i = gather_block<R, W>(g, blk, sm, Fs, Hs);
-    if (i == 0) a.step[0] = a.step[1] + 1;
+    const unsigned long long st = NEXT ? a.step[0] + ahead : a.step[1];
+    if (i == 0) a.step[NEXT ? 1 : 0] = st + 1;
     if (i < 0) return;
     const StepDev &P = *a.par;
     const int t = i < a.n_fe ? 0 : 1;
     const uint64_t id = (uint64_t)a.orig[i];
-    const unsigned long long st = a.step[1];
     Hs[0] += P.zee[t][0]; Hs[1] += P.zee[t][1]; Hs[2] += P.zee[t][2];
     if (a.Bat) {
         const double4 b = a.Bat[i];
-        Hs[0] += P.mom[t] * b.x; Hs[1] += P.mom[t] * b.y; Hs[2] += P.mom[t] * b.z;
+        Hs[0] = fma_(P.mom[t], b.x, Hs[0]); Hs[1] = fma_(P.mom[t], b.y, Hs[1]); Hs[2] = fma_(P.mom[t], b.z, Hs[2]);
     }
     if (P.lng) add_landau(P, t, a.spin[i], Hs);
     if constexpr (!SPIN) {
@@ -188,48 +206,58 @@ __device__ __forceinline__ void second_half_body(const IntArgs &a, const GatherA
         float ze[3], w0[3], w1[3], d[3];
         gauss3f(st, id, 2, a.seed, a.replica, ze);
         const float fse = (float)se, lam = (float)P.lambda, k = (float)P.wscale;
-        omega_of_f((float)S0.x, (float)S0.y, (float)S0.z, (float)H0.x + fse * ze[0], (float)H0.y + fse * ze[1],
-                   (float)H0.z + fse * ze[2], lam, k, w0);
-        omega_of_f((float)S1.x, (float)S1.y, (float)S1.z, (float)Hs[0] + fse * ze[0], (float)Hs[1] + fse * ze[1],
-                   (float)Hs[2] + fse * ze[2], lam, k, w1);
-        rotate_delta_f((float)S0.x, (float)S0.y, (float)S0.z, 0.5f * (w0[0] + w1[0]), 0.5f * (w0[1] + w1[1]),
-                       0.5f * (w0[2] + w1[2]), (float)P.dt, d);
+        omega_of((float)S0.x, (float)S0.y, (float)S0.z, fma_(fse, ze[0], (float)H0.x), fma_(fse, ze[1], (float)H0.y),
+                 fma_(fse, ze[2], (float)H0.z), lam, k, w0);
+        omega_of((float)S1.x, (float)S1.y, (float)S1.z, fma_(fse, ze[0], (float)Hs[0]), fma_(fse, ze[1], (float)Hs[1]),
+                 fma_(fse, ze[2], (float)Hs[2]), lam, k, w1);
+        rotate_delta_f((float)S0.x, (float)S0.y, (float)S0.z, mul_(0.5f, w0[0] + w1[0]),
+                       mul_(0.5f, w0[1] + w1[1]), mul_(0.5f, w0[2] + w1[2]), (float)P.dt, d);
         if (P.lng) {
             const float kd = (float)P.lng_drift, ks = (float)P.lng_sig;
-            d[0] += kd * (0.5f * ((float)H0.x + (float)Hs[0])) + ks * ze[0];
-            d[1] += kd * (0.5f * ((float)H0.y + (float)Hs[1])) + ks * ze[1];
-            d[2] += kd * (0.5f * ((float)H0.z + (float)Hs[2])) + ks * ze[2];
+            d[0] += fma_(kd, mul_(0.5f, (float)H0.x + (float)Hs[0]), mul_(ks, ze[0]));
+            d[1] += fma_(kd, mul_(0.5f, (float)H0.y + (float)Hs[1]), mul_(ks, ze[1]));
+            d[2] += fma_(kd, mul_(0.5f, (float)H0.z + (float)Hs[2]), mul_(ks, ze[2]));
         }
         Sn[0] = S0.x + (double)d[0]; Sn[1] = S0.y + (double)d[1]; Sn[2] = S0.z + (double)d[2];
     } else {
         double ze[3], w0[3], w1[3], w[3];
         gauss3(st, id, 2, a.seed, a.replica, ze);
-        omega_of(S0.x, S0.y, S0.z, H0.x + se * ze[0], H0.y + se * ze[1], H0.z + se * ze[2], P.lambda, P.wscale, w0);
-        omega_of(S1.x, S1.y, S1.z, Hs[0] + se * ze[0], Hs[1] + se * ze[1], Hs[2] + se * ze[2], P.lambda, P.wscale,
-                 w1);
-        w[0] = 0.5 * (w0[0] + w1[0]); w[1] = 0.5 * (w0[1] + w1[1]); w[2] = 0.5 * (w0[2] + w1[2]);
+        omega_of(S0.x, S0.y, S0.z, fma_(se, ze[0], H0.x), fma_(se, ze[1], H0.y), fma_(se, ze[2], H0.z), P.lambda,
+                 P.wscale, w0);
+        omega_of(S1.x, S1.y, S1.z, fma_(se, ze[0], Hs[0]), fma_(se, ze[1], Hs[1]), fma_(se, ze[2], Hs[2]), P.lambda,
+                 P.wscale, w1);
+        w[0] = mul_(0.5, w0[0] + w1[0]); w[1] = mul_(0.5, w0[1] + w1[1]); w[2] = mul_(0.5, w0[2] + w1[2]);
         rotate(S0.x, S0.y, S0.z, w, P.dt, Sn);
         if (P.lng) {
-            Sn[0] += P.lng_drift * (0.5 * (H0.x + Hs[0])) + P.lng_sig * ze[0];
-            Sn[1] += P.lng_drift * (0.5 * (H0.y + Hs[1])) + P.lng_sig * ze[1];
-            Sn[2] += P.lng_drift * (0.5 * (H0.z + Hs[2])) + P.lng_sig * ze[2];
+            Sn[0] += fma_(P.lng_drift, mul_(0.5, H0.x + Hs[0]), mul_(P.lng_sig, ze[0]));
+            Sn[1] += fma_(P.lng_drift, mul_(0.5, H0.y + Hs[1]), mul_(P.lng_sig, ze[1]));
+            Sn[2] += fma_(P.lng_drift, mul_(0.5, H0.z + Hs[2]), mul_(P.lng_sig, ze[2]));
         }
     }
     if (!P.lng) {   // renormalisation in FP64 after every rotation
-        const double inn = 1.0 / sqrt(Sn[0] * Sn[0] + Sn[1] * Sn[1] + Sn[2] * Sn[2]);
-        Sn[0] *= inn; Sn[1] *= inn; Sn[2] *= inn;
+        const double inn = 1.0 / sqrt(dot3_(Sn[0], Sn[1], Sn[2], Sn[0], Sn[1], Sn[2]));
+        Sn[0] = mul_(Sn[0], inn); Sn[1] = mul_(Sn[1], inn); Sn[2] = mul_(Sn[2], inn);
     }
     double4 v = a.vel[i];
     const double hdt = P.half_dt, am = P.acc_m[t];
-    v.x += hdt * Fs[0] * am; v.y += hdt * Fs[1] * am; v.z += hdt * Fs[2] * am;
+    v.x = fma_(mul_(hdt, Fs[0]), am, v.x);
+    v.y = fma_(mul_(hdt, Fs[1]), am, v.y);
+    v.z = fma_(mul_(hdt, Fs[2]), am, v.z);
+    if (!(isfinite(Fs[0]) && isfinite(Fs[1]) && isfinite(Fs[2]) && isfinite(Hs[0]) && isfinite(Hs[1]) &&
+          isfinite(Hs[2])))
+        atomicOr(a.status, ST_NONFINITE);
+    if constexpr (NEXT) {
+        const double4 H = opaque(Hs[0], Hs[1], Hs[2]);
+        a.H[i] = H;
+        first_half_atom<MIXED>(a, i, st + 1, t, id, opaque(v.x, v.y, v.z), opaque(Fs[0], Fs[1], Fs[2]), H,
+                               opaque(Sn[0], Sn[1], Sn[2]));
+        return;
+    }
     a.vel[i] = v;
     a.spin[i] = make_double4(Sn[0], Sn[1], Sn[2], 0.0);
     if constexpr (MIXED) a.psf[2 * i + 1] = make_float4((float)Sn[0], (float)Sn[1], (float)Sn[2], 0.f);
     a.F[i] = make_double4(Fs[0], Fs[1], Fs[2], 0.0);
     a.H[i] = make_double4(Hs[0], Hs[1], Hs[2], 0.0);
-    if (!(isfinite(Fs[0]) && isfinite(Fs[1]) && isfinite(Fs[2]) && isfinite(Hs[0]) && isfinite(Hs[1]) &&
-          isfinite(Hs[2])))
-        atomicOr(a.status, ST_NONFINITE);
 }
 
 // The halves over an argument table (sl_batch.h: a system's own table or a batch's), one
@@ -261,6 +289,18 @@ __global__ void __launch_bounds__(256) k_second_wide(const HalfArgs<R> *__restri
     one_work(tab, sm, solo, [&](const HalfArgs<R> &h, int64_t blk, int64_t) {
         second_half_body<R, MIXED, GATHER_WIDE<R>, SPIN>(h.a, h.g, blk, scratch);
     });
+}
+
+// The second half of a step and the first half of the next in one launch, between two steps of one queue
+// (a system's own launches): velocity, force, field and spin stay in registers, a launch and its ramp less.
+// A step of 512 / 13,824 / 32,768 / 110,592 / 884,736 atoms, mixed precision: 47.2 / 106.2 / 192.6 / 484.6 / 3,285 to
+// 44.7 / 103.0 / 189.0 / 480.1 / 3,214 us; FP64, 512 / 32,768: 189.5 to 186.2, 3,485 to 3,474 us.  Four blocks of
+// an SM in mixed precision (64 registers): with three, 32,768 atoms' 512 blocks took a second wave
+// (200 us a step).
+template <typename R, bool MIXED, int W>
+__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 3) k_halves(const __grid_constant__ HalfArgs<R> h, unsigned long long ahead) {
+    __shared__ GatherSmem<R, W> scratch;
+    second_half_body<R, MIXED, W, true, true>(h.a, h.g, blockIdx.x, scratch, ahead);
 }
 
 // Forces and fields at the current state into (Fo, Ho).
@@ -313,7 +353,7 @@ __global__ void __launch_bounds__(256) k_sweep_rotate(IntArgs a, GatherArgs<R> g
         float ze[3], w[3], d[3];
         gauss3f(st, id, 2, a.seed, a.replica, ze);
         const float fse = (float)se;
-        omega_of_f((float)S.x, (float)S.y, (float)S.z, (float)Hs[0] + fse * ze[0], (float)Hs[1] + fse * ze[1],
+        omega_of((float)S.x, (float)S.y, (float)S.z, (float)Hs[0] + fse * ze[0], (float)Hs[1] + fse * ze[1],
                    (float)Hs[2] + fse * ze[2], (float)P.lambda, (float)P.wscale, w);
         rotate_delta_f((float)S.x, (float)S.y, (float)S.z, w[0], w[1], w[2], (float)P.half_dt, d);
         Sn[0] = S.x + (double)d[0]; Sn[1] = S.y + (double)d[1]; Sn[2] = S.z + (double)d[2];
@@ -384,6 +424,17 @@ void launch_first_half(Sys &s) { launch_first_half_t(s.solo->t, solo_launch(s, F
 void launch_second_half(Sys &s) {
     launch_second_half_t(s.solo->t, solo_launch(s, FK_SECOND, SK_STEP), solo_launch(s, FK_SECONDW, SK_STEP), true,
                          s.stream);
+}
+template <typename R, bool MIXED>
+static void halves(Sys &s, unsigned long long ahead) {
+    const Launch L = solo_launch(s, FK_SECOND, SK_STEP), W = solo_launch(s, FK_SECONDW, SK_STEP);
+    const HalfArgs<R> so = solo_args<HalfArgs<R>>(L);
+    if (L.grid) k_halves<R, MIXED, 1><<<L.grid, 256, 0, s.stream>>>(so, ahead);
+    if (W.grid) k_halves<R, MIXED, GATHER_WIDE<R>><<<W.grid, W.block, 0, s.stream>>>(so, ahead);
+}
+void launch_halves(Sys &s, int64_t ahead) {
+    if (s.prec == 0) halves<double, false>(s, (unsigned long long)ahead);
+    else halves<float, true>(s, (unsigned long long)ahead);
 }
 void launch_second_half_nospin(Sys &s) {
     launch_second_half_t(s.solo->t, solo_launch(s, FK_SECOND, SK_STEP), solo_launch(s, FK_SECONDW, SK_STEP), false,

@@ -255,6 +255,7 @@ constexpr int KERNELS_PER_STEP = 1 + 8 + 2 + 1 + 1 + 1;
 // sl_integrate.cu
 void launch_first_half(Sys &s);
 void launch_second_half(Sys &s);
+void launch_halves(Sys &s, int64_t ahead);   // second half, and first half of the next step
 void launch_second_half_nospin(Sys &s);   // gather and final kick only (midpoint mode)
 void launch_sweep_rotate(Sys &s, int c);  // coloured sweep: half-step rotation of the spins of colour c
 // sl_midpoint.cu: the iteration of one step between the first half and the final evaluation;

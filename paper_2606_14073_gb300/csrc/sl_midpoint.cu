@@ -105,7 +105,7 @@ __global__ void __launch_bounds__(256) k_mid_update(MidArgs a, GatherArgs<R> g, 
         float ze[3], w[3], d[3];
         gauss3f(st, id, 2, a.seed, a.replica, ze);
         const float fse = (float)se;
-        omega_of_f((float)M.x, (float)M.y, (float)M.z, (float)Hs[0] + fse * ze[0], (float)Hs[1] + fse * ze[1],
+        omega_of((float)M.x, (float)M.y, (float)M.z, (float)Hs[0] + fse * ze[0], (float)Hs[1] + fse * ze[1],
                    (float)Hs[2] + fse * ze[2], (float)P.lambda, (float)P.wscale, w);
         rotate_delta_f((float)S0.x, (float)S0.y, (float)S0.z, w[0], w[1], w[2], (float)P.dt, d);
         Gn[0] = S0.x + (double)d[0]; Gn[1] = S0.y + (double)d[1]; Gn[2] = S0.z + (double)d[2];

@@ -19,49 +19,51 @@ struct GatherArgs {
     int64_t n;
 };
 
-__device__ __forceinline__ void omega_of(double sx, double sy, double sz, double hx, double hy, double hz,
-                                         double lam, double k, double w[3]) {
-    w[0] = (hx + lam * (sy * hz - sz * hy)) * k;
-    w[1] = (hy + lam * (sz * hx - sx * hz)) * k;
-    w[2] = (hz + lam * (sx * hy - sy * hx)) * k;
+// The state arithmetic of a step names its multiply-adds: k_halves and the separate halves inline it, and a
+// step's bits must not depend on which of them ran it (the compiler fuses a product and a sum as the code
+// around them allows).
+__device__ __forceinline__ double mul_(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float mul_(float a, float b) { return __fmul_rn(a, b); }
+template <typename R>
+__device__ __forceinline__ R cross_(R a, R b, R c, R d) { return fma_(a, b, -mul_(c, d)); }   // a b - c d
+template <typename R>
+__device__ __forceinline__ R dot3_(R ax, R ay, R az, R bx, R by, R bz) { return fma_(az, bz, fma_(ay, by, mul_(ax, bx))); }
+
+template <typename R>
+__device__ __forceinline__ void omega_of(R sx, R sy, R sz, R hx, R hy, R hz, R lam, R k, R w[3]) {
+    w[0] = mul_(fma_(lam, cross_(sy, hz, sz, hy), hx), k);
+    w[1] = mul_(fma_(lam, cross_(sz, hx, sx, hz), hy), k);
+    w[2] = mul_(fma_(lam, cross_(sx, hy, sy, hx), hz), k);
 }
 
 __device__ __forceinline__ void rotate(double sx, double sy, double sz, const double w[3], double dt, double out[3]) {
-    const double wn2 = w[0] * w[0] + w[1] * w[1] + w[2] * w[2];
+    const double wn2 = dot3_(w[0], w[1], w[2], w[0], w[1], w[2]);
     if (wn2 == 0.0) { out[0] = sx; out[1] = sy; out[2] = sz; return; }
     const double wn = sqrt(wn2);
     const double ax = w[0] / wn, ay = w[1] / wn, az = w[2] / wn;
     double s, c;
-    sincos(wn * dt, &s, &c);
-    const double as = ax * sx + ay * sy + az * sz;
-    const double cx = ay * sz - az * sy, cy = az * sx - ax * sz, cz = ax * sy - ay * sx;
-    out[0] = sx * c + cx * s + ax * as * (1.0 - c);
-    out[1] = sy * c + cy * s + ay * as * (1.0 - c);
-    out[2] = sz * c + cz * s + az * as * (1.0 - c);
+    sincos(mul_(wn, dt), &s, &c);
+    const double p = mul_(dot3_(ax, ay, az, sx, sy, sz), 1.0 - c);
+    out[0] = fma_(ax, p, fma_(cross_(ay, sz, az, sy), s, mul_(sx, c)));
+    out[1] = fma_(ay, p, fma_(cross_(az, sx, ax, sz), s, mul_(sy, c)));
+    out[2] = fma_(az, p, fma_(cross_(ax, sy, ay, sx), s, mul_(sz, c)));
 }
 
 // Rotation increment dS = Rot(S, w dt) - S in FP32 (added to the FP64 spin by the
 // caller): dS = (a x S) sin(th) - 2 sin^2(th/2) (S - a (a.S)), th = |w| dt.
 __device__ __forceinline__ void rotate_delta_f(float sx, float sy, float sz, float wx, float wy, float wz, float dt,
                                                float d[3]) {
-    const float wn2 = wx * wx + wy * wy + wz * wz;
+    const float wn2 = dot3_(wx, wy, wz, wx, wy, wz);
     if (wn2 == 0.0f) { d[0] = d[1] = d[2] = 0.0f; return; }
     const float iw = rsqrtf(wn2);
-    const float ax = wx * iw, ay = wy * iw, az = wz * iw;
+    const float ax = mul_(wx, iw), ay = mul_(wy, iw), az = mul_(wz, iw);
     float sh, ch;
-    sincosf(0.5f * wn2 * iw * dt, &sh, &ch);
-    const float sn = 2.0f * sh * ch, omc = 2.0f * sh * sh;
-    const float as = ax * sx + ay * sy + az * sz;
-    d[0] = (ay * sz - az * sy) * sn - omc * (sx - ax * as);
-    d[1] = (az * sx - ax * sz) * sn - omc * (sy - ay * as);
-    d[2] = (ax * sy - ay * sx) * sn - omc * (sz - az * as);
-}
-
-__device__ __forceinline__ void omega_of_f(float sx, float sy, float sz, float hx, float hy, float hz, float lam,
-                                           float k, float w[3]) {
-    w[0] = (hx + lam * (sy * hz - sz * hy)) * k;
-    w[1] = (hy + lam * (sz * hx - sx * hz)) * k;
-    w[2] = (hz + lam * (sx * hy - sy * hx)) * k;
+    sincosf(mul_(mul_(mul_(0.5f, wn2), iw), dt), &sh, &ch);
+    const float sn = mul_(2.0f * sh, ch), omc = mul_(2.0f * sh, sh);
+    const float as = dot3_(ax, ay, az, sx, sy, sz);
+    d[0] = cross_(cross_(ay, sz, az, sy), sn, omc, fma_(-ax, as, sx));
+    d[1] = cross_(cross_(az, sx, ax, sz), sn, omc, fma_(-ay, as, sy));
+    d[2] = cross_(cross_(ax, sy, ay, sx), sn, omc, fma_(-az, as, sz));
 }
 
 // F_k = sum_j dE_k/dr_kj - sum_j dE_j/dr_jk, H_k = -dE_k/dS_k - sum_j dE_j/dS_k: the
