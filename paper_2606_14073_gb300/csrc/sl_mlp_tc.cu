@@ -11,8 +11,8 @@
 // is split into hi = fp16(x), lo = fp16(x - hi) and each GEMM accumulates
 // hi.hi + hi.lo + lo.hi in FP32 in tensor memory, which keeps the network within
 // ~1e-6 relative of FP32 arithmetic.  One thread issues the MMAs; completion is
-// signalled through an mbarrier (tcgen05.commit); the 128 threads read their
-// atom's row back with tcgen05.ld (TMEM lane = atom row).  Persistent CTAs loop
+// signalled through an mbarrier (tcgen05.commit); two threads to an atom read its
+// row back with tcgen05.ld (TMEM lane = atom row).  Persistent CTAs loop
 // over tiles; the weights are staged once per CTA; each tile's 66 x 128 descriptors arrive
 // by one TMA tile load (cp.async.bulk.tensor) issued while the previous tile is in the
 // tensor cores.  Every wait is bounded: on timeout the kernel raises ST_TIMEOUT, waits for
@@ -61,7 +61,15 @@ constexpr uint32_t OFF_TMEM = OFF_BARQ + 8;               // tensor-memory base 
 // brought in by one TMA tile load while the current tile is in the tensor cores
 constexpr uint32_t OFF_Q = (OFF_TMEM + 8 + 127) & ~127u;
 constexpr uint32_t SZ_Q = DIM * TM * 4;                   // 33792, the TMA transaction size
-constexpr uint32_t SMEM_BYTES = OFF_Q + SZ_Q;
+// Threads per atom row.  A tile's time is its row's staging, tanh layer and results, a chain of some 2,500
+// instructions for one thread (the MMAs are a few hundred cycles), so two threads share a row, each half
+// of its columns (a warp reads the tensor-memory lanes of its place in its group of four warps): at
+// 884,736 / 110,592 / 512 atoms 117.5 / 24.8 / 10.4 instead of 129 / 26.7 / 11.4 us, the last together with the
+// descriptors' load issued before the weights' copy (four threads: 123 / 24.9 / 10.5).
+constexpr int RT = 2, NT = TM * RT;
+constexpr int HC = N1 / RT;                               // hidden columns of a thread
+constexpr uint32_t OFF_E = OFF_Q + SZ_Q;                  // the row's RT partial energies
+constexpr uint32_t SMEM_BYTES = OFF_E + RT * TM * 4;
 
 // byte offset of element (row, k) of a [rows x K] 16-bit operand in the canonical
 // no-swizzle K-major layout: core matrix = 8 rows x 8 elements (128 B, row stride 16 B),
@@ -128,6 +136,15 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float v[16]) {
         : "r"(taddr));
 #pragma unroll
     for (int t = 0; t < 16; ++t) v[t] = __uint_as_float(r[t]);
+}
+
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float v[8]) {
+    uint32_t r[8];
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr));
+#pragma unroll
+    for (int t = 0; t < 8; ++t) v[t] = __uint_as_float(r[t]);
 }
 
 // One TMA tile load of the descriptor box (atoms x0 .. x0+127, all 66 rows) into shared
@@ -217,19 +234,36 @@ __device__ __forceinline__ void mlp_tc_body(const NepDev<float> &P, int64_t ntil
                                             Src src) {
     extern __shared__ __align__(1024) unsigned char smem[];
     const int tid = threadIdx.x, warp = tid >> 5;
+    const int row = tid % TM, part = tid / TM;   // the thread's atom of the tile and its share of the columns
     const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(smem);
     const uint32_t bar = sbase + OFF_BAR, barq = sbase + OFF_BARQ;
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(smem + OFF_TMEM);
 
+    // the next tile's source, read while the current tile is in the tensor cores; one thread of the
+    // last warp issues the loads and acquires each tensor map it has not used yet before the first copy through it
+    const CUtensorMap *acquired = nullptr;
+    auto issue = [&](const MlpTile &t) {
+        if (t.gmem_map && t.qmap != acquired) {
+            tensormap_acquire(t.qmap);
+            acquired = t.qmap;
+        }
+        tma_load_q(sbase + OFF_Q, t.qmap, t.x0, barq);
+    };
+    // the first tile's descriptors are on their way before anything else (the other warps meanwhile
+    // copy the weights and allocate the tensor memory)
+    MlpTile nxt;
+    if (blockIdx.x < ntiles) nxt = src(blockIdx.x);
+    if (tid == NT - 32) {
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(barq) : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        fence_async_smem();
+        if (blockIdx.x < ntiles) issue(nxt);
+    }
     // weights, once per CTA: a coalesced copy of the images (the same bytes the split of P.w0
     // gives, made once per system by k_weight_images)
     for (int k = tid; k < (int)(SZ_W / 16); k += blockDim.x)
         reinterpret_cast<uint4 *>(smem + OFF_B1H)[k] = __ldg(wimg + k);
-    if (tid == 0) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(barq) : "memory");
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(sbase + OFF_TMEM),
                      "r"(TMEM_COLS)
@@ -241,7 +275,7 @@ __device__ __forceinline__ void mlp_tc_body(const NepDev<float> &P, int64_t ntil
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
     const uint32_t t_z = tmem, t_g = tmem + N1;
-    const uint32_t lane_off = (uint32_t)(warp * 32) << 16;   // this warp's TMEM lane quadrant
+    const uint32_t lane_off = (uint32_t)(warp % 4 * 32) << 16;   // this warp's TMEM lane quadrant
     constexpr uint32_t IDESC1 = instr_desc(TM, N1), IDESC2 = instr_desc(TM, N2);
     uint32_t phase = 0, phase_q = 0;
     bool ok = true;
@@ -249,27 +283,13 @@ __device__ __forceinline__ void mlp_tc_body(const NepDev<float> &P, int64_t ntil
     int *status = nullptr;   // the status word of the last tile's system (timeouts are reported there)
 
     const float *stage = reinterpret_cast<const float *>(smem + OFF_Q);
-    // the next tile's source, read while the current tile is in the tensor cores; thread 0
-    // acquires each tensor map it has not used yet before the first copy through it
-    const CUtensorMap *acquired = nullptr;
-    auto issue = [&](const MlpTile &t) {
-        if (t.gmem_map && t.qmap != acquired) {
-            tensormap_acquire(t.qmap);
-            acquired = t.qmap;
-        }
-        tma_load_q(sbase + OFF_Q, t.qmap, t.x0, barq);
-    };
-    MlpTile nxt;
-    if (blockIdx.x < ntiles) {
-        nxt = src(blockIdx.x);
-        if (tid == 0) issue(nxt);
-    }
+    [[maybe_unused]] float *energy = reinterpret_cast<float *>(smem + OFF_E);
     q_in_flight = blockIdx.x < ntiles;
 
     for (int64_t tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
         const MlpTile cur = nxt;
         status = cur.status;
-        const int64_t i = cur.x0 + tid;
+        const int64_t i = cur.x0 + row;
         const bool valid = i < cur.n;
         float *__restrict__ fp = cur.fp;
         float *__restrict__ ei = cur.ei;
@@ -280,17 +300,19 @@ __device__ __forceinline__ void mlp_tc_body(const NepDev<float> &P, int64_t ntil
         q_in_flight = false;
         // A1 row: s_v q_v, hi/lo
 #pragma unroll
-        for (int c = 0; c < K1 / 8; ++c) {
+        for (int k = 0; k < (K1 / 8 + RT - 1) / RT; ++k) {
+            const int c = k * RT + part;
+            if (K1 / 8 % RT && c >= K1 / 8) break;
             float x[8];
 #pragma unroll
             for (int t = 0; t < 8; ++t) {
                 const int v = c * 8 + t;
-                x[t] = v < DIM ? P.scal[v] * stage[v * TM + tid] : 0.f;
+                x[t] = v < DIM ? P.scal[v] * stage[v * TM + row] : 0.f;
             }
             uint4 hi, lo;
             split8(x, hi, lo);
-            *reinterpret_cast<uint4 *>(smem + OFF_A1H + cm_off(tid, c * 8, K1)) = hi;
-            *reinterpret_cast<uint4 *>(smem + OFF_A1L + cm_off(tid, c * 8, K1)) = lo;
+            *reinterpret_cast<uint4 *>(smem + OFF_A1H + cm_off(row, c * 8, K1)) = hi;
+            *reinterpret_cast<uint4 *>(smem + OFF_A1L + cm_off(row, c * 8, K1)) = lo;
         }
         // every thread's reads of the stage are ordered before the next tile load, which
         // overlaps this tile's MMAs
@@ -299,7 +321,7 @@ __device__ __forceinline__ void mlp_tc_body(const NepDev<float> &P, int64_t ntil
         __syncthreads();
         if (tile + gridDim.x < ntiles) {
             nxt = src(tile + gridDim.x);
-            if (tid == 0) issue(nxt);
+            if (tid == NT - 32) issue(nxt);
             q_in_flight = true;
         }
         if (tid == 0) {
@@ -324,29 +346,34 @@ __device__ __forceinline__ void mlp_tc_body(const NepDev<float> &P, int64_t ntil
         phase ^= 1u;
         tc_fence_after();
         // epilogue 1: tanh layer, E_i, t_h into the A2 tile
-        float z[N1];
-        tmem_ld16(t_z + lane_off, z);
-        tmem_ld16(t_z + lane_off + 16, z + 16);
-        tmem_wait_ld();
-        float tt[N1];
-        float E = -P.b1;
+        float z[HC], tt[HC];
+        const int h0 = part * HC;
+        if constexpr (HC == 8) {
+            tmem_ld8(t_z + lane_off + h0, z);
+        } else {
 #pragma unroll
-        for (int h = 0; h < N1; ++h) {
+            for (int c = 0; c < HC; c += 16) tmem_ld16(t_z + lane_off + h0 + c, z + c);
+        }
+        tmem_wait_ld();
+        float E = part == 0 ? -P.b1 : 0.f;
+#pragma unroll
+        for (int k = 0; k < HC; ++k) {
+            const int h = h0 + k;
             if (h < NH) {
-                const float a = tanhf(z[h] - P.b0[h]);
+                const float a = tanhf(z[k] - P.b0[h]);
                 E += P.w1[h] * a;
-                tt[h] = P.w1[h] * (1.f - a * a);
+                tt[k] = P.w1[h] * (1.f - a * a);
             } else {
-                tt[h] = 0.f;
+                tt[k] = 0.f;
             }
         }
-        if (valid) ei[i] = E;
+        if constexpr (RT > 1) energy[part * TM + row] = E;
 #pragma unroll
-        for (int c = 0; c < K2 / 8; ++c) {
+        for (int c = 0; c < HC / 8; ++c) {
             uint4 hi, lo;
             split8(tt + 8 * c, hi, lo);
-            *reinterpret_cast<uint4 *>(smem + OFF_A2H + cm_off(tid, c * 8, K2)) = hi;
-            *reinterpret_cast<uint4 *>(smem + OFF_A2L + cm_off(tid, c * 8, K2)) = lo;
+            *reinterpret_cast<uint4 *>(smem + OFF_A2H + cm_off(row, h0 + c * 8, K2)) = hi;
+            *reinterpret_cast<uint4 *>(smem + OFF_A2L + cm_off(row, h0 + c * 8, K2)) = lo;
         }
         fence_async_smem();
         tc_fence_before();
@@ -366,12 +393,19 @@ __device__ __forceinline__ void mlp_tc_body(const NepDev<float> &P, int64_t ntil
             }
             mma_commit(bar);
         }
+        if (part == 0 && valid) {   // the row's energy, its parts in order
+#pragma unroll
+            for (int k = 1; k < RT; ++k) E += energy[k * TM + row];
+            ei[i] = E;
+        }
         if (!__syncthreads_and(mbar_wait(bar, phase))) { ok = false; break; }
         phase ^= 1u;
         tc_fence_after();
         // epilogue 2: Fp_v = s_v G_v
 #pragma unroll
-        for (int c = 0; c < N2 / 16; ++c) {
+        for (int k = 0; k < (N2 / 16 + RT - 1) / RT; ++k) {
+            const int c = k * RT + part;   // uniform in a warp
+            if (N2 / 16 % RT && c >= N2 / 16) break;
             float g[16];
             tmem_ld16(t_g + lane_off + 16 * c, g);
             tmem_wait_ld();
@@ -404,10 +438,11 @@ __device__ __forceinline__ void mlp_tc_body(const NepDev<float> &P, int64_t ntil
 // The network over the 128-atom tiles of a work map (sl_batch.h): a batch's (tab non-null;
 // each slot's arguments and TMA map from the table, in global memory) or a system's own (tab
 // null; its arguments, map included, as the kernel parameter solo).
-__global__ void __launch_bounds__(128, 2) k_mlp_tc(const __grid_constant__ NepDev<float> P,
+__global__ void __launch_bounds__(NT, 2) k_mlp_tc(const __grid_constant__ NepDev<float> P,
                                                    const MlpArgs *__restrict__ tab, WorkMap m,
                                                    const __grid_constant__ MlpArgs solo) {
-    const int64_t total = __ldg(m.w0 + m.nrep);
+    // (a system's own launch: its tiles are known without the map)
+    const int64_t total = tab ? __ldg(m.w0 + m.nrep) : (solo.n + TM - 1) / TM;
     // the skip flag (the midpoint iteration's own launches only): uniform for the whole CTA and
     // before any shared-memory or TMEM use
     if (!tab && solo.skip && *solo.skip) return;
@@ -416,11 +451,11 @@ __global__ void __launch_bounds__(128, 2) k_mlp_tc(const __grid_constant__ NepDe
     // the slots taking part share the model: the weight images of the slot of this CTA's first tile
     const void *wimg = tab ? tab[work_replica(m, blockIdx.x)].wimg : solo.wimg;
     mlp_tc_body(P, total, reinterpret_cast<const uint4 *>(wimg), [&](int64_t g) {
-        const int r = work_replica(m, g);
+        const int r = tab ? work_replica(m, g) : 0;
         const MlpArgs &a = tab ? tab[r] : solo;
         MlpTile t;
         t.qmap = &a.qmap;
-        t.x0 = (int)((g - __ldg(m.w0 + r)) * TM);
+        t.x0 = (int)((tab ? g - __ldg(m.w0 + r) : g) * TM);
         t.n = a.n;
         t.fp = a.fp;
         t.ei = a.ei;
@@ -516,7 +551,7 @@ void launch_net_t_tc(const FusedTables &t, const NepDev<float> &P, const Launch 
     int dev = 0;
     cudaGetDevice(&dev);
     tc_smem_attribute(dev);
-    tc::k_mlp_tc<<<L.grid, 128, tc::SMEM_BYTES, st>>>(P, L.solo ? nullptr : t.at<MlpArgs>(t.o_net), L.m,
+    tc::k_mlp_tc<<<L.grid, tc::NT, tc::SMEM_BYTES, st>>>(P, L.solo ? nullptr : t.at<MlpArgs>(t.o_net), L.m,
                                                        solo_args<MlpArgs>(L));
 }
 
