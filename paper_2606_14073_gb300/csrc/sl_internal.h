@@ -43,6 +43,7 @@ constexpr int AA_MAX_DEPTH = 8;      // largest accepted Anderson history
 struct MidDev {
     int converged;                                   // set once the step's iteration has stopped
     int fallback;                                    // Anderson solve unusable this iteration
+    unsigned blocks_done;                            // blocks of the running update that have finished
     unsigned long long resid[MID_MAX_ITERS];         // max_i |G_i - X_i| per iteration (FP64 bits)
     unsigned long long iters;                        // midpoint evaluations executed, all steps
     double gamma[AA_MAX_DEPTH];                      // Anderson coefficients of the current iteration
