@@ -79,12 +79,15 @@ void FusedBatch::enqueue(cudaStream_t st) const {
     launch_fused_plan(t, st);
     launch_first_half_t(t, L(FK_FIRST), st);
     Launch rb[FK_FINISH - FK_BIN + 1];
-    for (int k = FK_BIN; k <= FK_FINISH; ++k) rb[k - FK_BIN] = L(k);
+    for (int k = FK_BIN; k <= FK_FINISH; ++k) {
+        rb[k - FK_BIN] = L(k);
+        rb[k - FK_BIN].quick = t.any();
+    }
     launch_rebuild_t(t, rb, true, true, st);
     const Launch ev[7] = {L(FK_CRAD), L(FK_ANG), L(FK_NET), L(FK_BWD), L(FK_CRADW), L(FK_ANGW), L(FK_BWDW)};
-    if (t.prec == 0) launch_eval_t<double>(t, pd, ev, st, nullptr);
-    else launch_eval_t<float>(t, pf, ev, st, nullptr);
-    launch_second_half_t(t, L(FK_SECOND), L(FK_SECONDW), true, st);
+    if (t.prec == 0) launch_eval_t<double>(t, pd, ev, st, nullptr, fork);
+    else launch_eval_t<float>(t, pf, ev, st, nullptr, fork);
+    launch_second_half_t(t, L(FK_SECOND), L(FK_SECONDW), true, st, fork);
 }
 
 namespace {
@@ -112,6 +115,7 @@ void fused_layout(FusedTables &t, int prec, int cap) {
     take(t.o_net, fused_net_size(prec) * cap);
     t.upload_bytes = o;
     take(t.o_w0, sizeof(int64_t) * FK_N * (cap + 1));
+    take(t.o_any, sizeof(int));
     t.bytes = o;
 }
 
@@ -143,6 +147,10 @@ void FusedBatch::release() {
     release_items();
     if (t.dev) cudaFree(t.dev);
     if (img) cudaFreeHost(img);
+    if (fork.out) cudaEventDestroy(fork.out);
+    if (fork.back) cudaEventDestroy(fork.back);
+    if (fork.st) cudaStreamDestroy(fork.st);
+    fork = Fork();
     t = FusedTables();
     img = nullptr;
     dev_ = -1;
@@ -160,6 +168,7 @@ bool FusedBatch::setup(int prec, int cap, int device) {
     release();
     if (cap < 1 || cap > FUSED_MAX_SLOTS) return false;
     fused_layout(t, prec, cap);
+    t.batch = true;
     if (cudaMalloc((void **)&t.dev, t.bytes) != cudaSuccess) {
         t.dev = nullptr;
         release();
@@ -172,6 +181,12 @@ bool FusedBatch::setup(int prec, int cap, int device) {
     }
     std::memset(img, 0, t.upload_bytes);
     if (cudaMemset(t.dev, 0, t.bytes) != cudaSuccess) {
+        release();
+        return false;
+    }
+    if (cudaStreamCreateWithFlags(&fork.st, cudaStreamNonBlocking) != cudaSuccess ||
+        cudaEventCreateWithFlags(&fork.out, cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&fork.back, cudaEventDisableTiming) != cudaSuccess) {
         release();
         return false;
     }

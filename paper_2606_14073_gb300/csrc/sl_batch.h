@@ -52,6 +52,8 @@ struct FusedTables {
     size_t o_left = 0;     // int64 [cap]: steps left (set per call, counted down by the plan kernel)
     size_t o_first = 0, o_second = 0, o_bin = 0, o_lists = 0, o_rev = 0, o_eval = 0, o_net = 0;
     size_t o_w0 = 0;       // int64 [FK_N][cap + 1]: the current step's work maps (batches)
+    size_t o_any = 0;      // int: whether any slot's rebuild is due (batches: set by the first half)
+    bool batch = false;
     size_t upload_bytes = 0;   // the host-written part: [0, upload_bytes)
     size_t bytes = 0;
     unsigned char *dev = nullptr;   // device base
@@ -59,6 +61,7 @@ struct FusedTables {
 
     template <typename T>
     const T *at(size_t off) const { return reinterpret_cast<const T *>(dev + off); }
+    int *any() const { return batch ? reinterpret_cast<int *>(dev + o_any) : nullptr; }
     WorkMap map(int k) const {
         return WorkMap{reinterpret_cast<const int64_t *>(dev + o_w0) + (size_t)k * (cap + 1), cap};
     }
@@ -76,7 +79,7 @@ struct Launch {
     const int *item_slot = nullptr;
     const int64_t *start = nullptr;
     const void *solo = nullptr;
-    const int *quick = nullptr;   // a system's own conditional rebuild: its flag (see sl_neighbors.cu)
+    const int *quick = nullptr;   // conditional rebuild: the system's flag, or the batch's (see sl_neighbors.cu)
     unsigned grid = 0;
     int block = 0;
     int minb = 0;
@@ -113,7 +116,27 @@ void fused_grid_net(FusedTables &t);
 // launches over a table
 void launch_fused_plan(const FusedTables &t, cudaStream_t st);
 void launch_first_half_t(const FusedTables &t, const Launch &L, cudaStream_t st);
-void launch_second_half_t(const FusedTables &t, const Launch &L, const Launch &W, bool spin, cudaStream_t st);
+// A second stream for the launch group's kernel of the other width, which takes other slots: forked from the
+// group's stream and joined to it by the events.  Without one the two run one after the other.
+// (Eight replicas of 5,832 to 64,000 atoms, mixed precision, 20 steps: 17.6 to 17.3 ms, together with a rebuild
+// group that returns at once on the batch's word when no slot's rebuild is due, 48 us a step before.)
+struct Fork {
+    cudaStream_t st = nullptr;
+    cudaEvent_t out = nullptr, back = nullptr;
+    cudaStream_t open(cudaStream_t from) const {
+        if (!st) return from;
+        cudaEventRecord(out, from);
+        cudaStreamWaitEvent(st, out, 0);
+        return st;
+    }
+    void close(cudaStream_t to) const {
+        if (!st) return;
+        cudaEventRecord(back, st);
+        cudaStreamWaitEvent(to, back, 0);
+    }
+};
+void launch_second_half_t(const FusedTables &t, const Launch &L, const Launch &W, bool spin, cudaStream_t st,
+                          const Fork &fork = Fork());
 // the rebuild group: L[0 .. 5] for the binning, scan, scatter, lists, reverse slots and finish
 // kernels; clear: then the flags of the conditional slots in L[0]'s map are cleared; loop: the
 // persistent form (a batch's), else one work item per block (a system's own launches)
@@ -122,7 +145,7 @@ void launch_rebuild_t(const FusedTables &t, const Launch *L, bool clear, bool lo
 // kernel, after it, after the angular kernel, after the network and after the backward
 template <typename R>
 void launch_eval_t(const FusedTables &t, const NepDev<R> &P, const Launch *L /* crad, ang, net, bwd, wide crad, ang, bwd */,
-                   cudaStream_t st, cudaEvent_t *ev);
+                   cudaStream_t st, cudaEvent_t *ev, const Fork &fork = Fork());
 void launch_net_t_tc(const FusedTables &t, const NepDev<float> &P, const Launch &L, cudaStream_t st);
 void launch_net_t_fp64(const FusedTables &t, const Launch &L, cudaStream_t st);
 
@@ -163,6 +186,7 @@ public:
     void enqueue(cudaStream_t st) const;
 
     FusedTables t;
+    Fork fork;   // of the captured steps
     cudaGraphExec_t graph_g = nullptr, graph_1 = nullptr;
     int g = 0;
     int64_t captures = 0;

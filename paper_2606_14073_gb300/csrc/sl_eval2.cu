@@ -1740,7 +1740,8 @@ void fused_put_eval(Sys &s, int r, int kind, const FusedTables &t, unsigned char
 // Radial, angular, network and backward (and, last, the three wide kernels) over a table, each launch in its own shape
 // (L[k].block threads, 0: the default) and register budget (L[k].minb, 0: the default).
 template <typename R>
-void launch_eval_t(const FusedTables &t, const NepDev<R> &P, const Launch *L, cudaStream_t st, cudaEvent_t *ev) {
+void launch_eval_t(const FusedTables &t, const NepDev<R> &P, const Launch *L, cudaStream_t st, cudaEvent_t *ev,
+                   const Fork &fork) {
     // a system's own launch passes its argument block as a kernel parameter; a batch's reads
     // the table (the same for the four kernels of one launch group)
     const Eval2Args<R> *tab = L[0].solo ? nullptr : t.at<Eval2Args<R>>(t.o_eval);
@@ -1752,14 +1753,18 @@ void launch_eval_t(const FusedTables &t, const NepDev<R> &P, const Launch *L, cu
     if (ev) cudaEventRecord(ev[0], st);
     // compaction and radial channels in one kernel: the compaction group is empty
     if (ev) cudaEventRecord(ev[1], st);
-    // a system's own launch has a grid for one kernel of each kind only
+    // a system's own launch has a grid for one kernel of each kind only; a batch's two, over different
+    // slots, run side by side (the wider ones on the fork's stream)
+    cudaStream_t side = fork.open(st);
     if constexpr (sizeof(R) == 4) {
         if (L[0].grid && L[0].minb == 3) k_crad<3><<<L[0].grid, cb, 0, st>>>(P, tab, s0, so);
         else if (L[0].grid) k_crad<<<L[0].grid, cb, 0, st>>>(P, tab, s0, so);
     }
-    if (L[4].grid) k_crad_wide<R><<<L[4].grid, L[4].block ? L[4].block : 128, 0, st>>>(P, tab, L[4].slots(), so);
+    if (L[4].grid) k_crad_wide<R><<<L[4].grid, L[4].block ? L[4].block : 128, 0, side>>>(P, tab, L[4].slots(), so);
+    fork.close(st);
     bool variant = false;
     if (ev) cudaEventRecord(ev[2], st);
+    side = fork.open(st);
     if constexpr (sizeof(R) == 4) {
         variant = L[1].minb == 1 && L[1].grid;
         if (variant) k_ang_fwd<R, 1><<<L[1].grid, qa, fwd_smem<R>(qa), st>>>(P, tab, s1, so);
@@ -1767,8 +1772,9 @@ void launch_eval_t(const FusedTables &t, const NepDev<R> &P, const Launch *L, cu
     if (!variant && L[1].grid) k_ang_fwd<R><<<L[1].grid, qa, fwd_smem<R>(qa), st>>>(P, tab, s1, so);
     if (L[5].grid) {
         const int b = L[5].block ? L[5].block : quad_block<R>();
-        k_ang_wide<R><<<L[5].grid, b, fwd_smem<R>(b), st>>>(P, tab, L[5].slots(), so);
+        k_ang_wide<R><<<L[5].grid, b, fwd_smem<R>(b), side>>>(P, tab, L[5].slots(), so);
     }
+    fork.close(st);
     if (ev) cudaEventRecord(ev[3], st);
     if constexpr (sizeof(R) == 4) launch_net_t_tc(t, P, L[2], st);
     else launch_net_t_fp64(t, L[2], st);
@@ -1776,6 +1782,7 @@ void launch_eval_t(const FusedTables &t, const NepDev<R> &P, const Launch *L, cu
     // the virial parts: only a system's own full evaluation asks for them (a batch's slots are
     // set up for the step's evaluation, which has none)
     const bool vir = L[3].solo && so.want_virial;
+    side = fork.open(st);
     if (L[3].grid) {
         variant = false;
         if constexpr (sizeof(R) == 4) {
@@ -1789,15 +1796,16 @@ void launch_eval_t(const FusedTables &t, const NepDev<R> &P, const Launch *L, cu
     }
     if (L[6].grid) {
         const int b = L[6].block ? L[6].block : quad_block<R>();
-        if (vir) k_bwd_wide<R, true><<<L[6].grid, b, bwdw_smem<R>(b), st>>>(P, tab, L[6].slots(), so);
-        else k_bwd_wide<R><<<L[6].grid, b, bwdw_smem<R>(b), st>>>(P, tab, L[6].slots(), so);
+        if (vir) k_bwd_wide<R, true><<<L[6].grid, b, bwdw_smem<R>(b), side>>>(P, tab, L[6].slots(), so);
+        else k_bwd_wide<R><<<L[6].grid, b, bwdw_smem<R>(b), side>>>(P, tab, L[6].slots(), so);
     }
+    fork.close(st);
     if (ev) cudaEventRecord(ev[5], st);
 }
 template void launch_eval_t<float>(const FusedTables &, const NepDev<float> &, const Launch *, cudaStream_t,
-                                   cudaEvent_t *);
+                                   cudaEvent_t *, const Fork &);
 template void launch_eval_t<double>(const FusedTables &, const NepDev<double> &, const Launch *, cudaStream_t,
-                                    cudaEvent_t *);
+                                    cudaEvent_t *, const Fork &);
 
 // The system's own evaluation: at the midpoint point while s.at is set (the midpoint
 // iteration), else at the state, with the virial parts when asked for.

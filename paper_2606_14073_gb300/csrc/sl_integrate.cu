@@ -38,6 +38,7 @@ struct IntArgs {
     const StepDev *par;
     unsigned long long *step;
     int *rebuild, *status;
+    int *any;           // a batch's word: a rebuild is due in one of its slots (null: a system's own step)
     uint64_t seed, replica;
 };
 
@@ -147,14 +148,20 @@ __device__ __forceinline__ void first_half_atom(const IntArgs &a, int64_t i, uns
         dy = fma_(-a.bd.L[1], rint(mul_(dy, a.bd.invL[1])), dy);
         dz = fma_(-a.bd.L[2], rint(mul_(dz, a.bd.invL[2])), dz);
     }
-    if (dot3_(dx, dy, dz, dx, dy, dz) > P.disp2) *a.rebuild = 1;
+    if (dot3_(dx, dy, dz, dx, dy, dz) > P.disp2) {
+        *a.rebuild = 1;
+        if (a.any) *a.any = 1;
+    }
 }
 
 template <bool MIXED>
 __device__ __forceinline__ void first_half_body(const IntArgs &a, int64_t blk) {
     const int64_t i = blk * (int64_t)blockDim.x + threadIdx.x;
     const unsigned long long st = a.step[0];
-    if (i == 0) a.step[1] = st;
+    if (i == 0) {
+        a.step[1] = st;
+        if (a.any && *a.rebuild) *a.any = 1;
+    }
     if (i >= a.n) return;
     first_half_atom<MIXED>(a, i, st, i < a.n_fe ? 0 : 1, (uint64_t)a.orig[i], a.vel[i], a.F[i], a.H[i], a.spin[i]);
 }
@@ -376,7 +383,7 @@ static IntArgs int_args(Sys &s) {
     a.posref = s.posref; a.posf = s.posf; a.psf = s.psf; a.orig = s.orig; a.n = s.n; a.n_fe = s.n_fe;
     a.bd = s.boxd;
     for (int d = 0; d < 3; ++d) a.per[d] = s.per[d];
-    a.par = s.d_par; a.step = s.d_step; a.rebuild = s.rebuild; a.status = s.status;
+    a.par = s.d_par; a.step = s.d_step; a.rebuild = s.rebuild; a.any = nullptr; a.status = s.status;
     a.seed = s.seed; a.replica = s.replica;
     a.posmid = s.mid_iters > 0 ? s.posmid : nullptr;
     a.midposf = s.mid_iters > 0 ? s.midposf : nullptr;
@@ -405,18 +412,22 @@ void launch_first_half_t(const FusedTables &t, const Launch &L, cudaStream_t st)
 
 // L, W: the launches of the one-lane and the wide form (a grid of 0: not launched)
 template <typename R, bool MIXED>
-static void second_half_t(const FusedTables &t, const Launch &L, const Launch &W, bool spin, cudaStream_t st) {
+static void second_half_t(const FusedTables &t, const Launch &L, const Launch &W, bool spin, cudaStream_t st,
+                          const Fork &fork) {
     const HalfArgs<R> *tab = L.solo ? nullptr : t.at<HalfArgs<R>>(t.o_second);
     const HalfArgs<R> so = solo_args<HalfArgs<R>>(L);
+    const cudaStream_t side = fork.open(st);
     if (L.grid && spin) k_second_half<R, MIXED, true><<<L.grid, 256, 0, st>>>(tab, L.slots(), so);
     else if (L.grid) k_second_half<R, MIXED, false><<<L.grid, 256, 0, st>>>(tab, L.slots(), so);
     const int b = W.block ? W.block : 256;
-    if (W.grid && spin) k_second_wide<R, MIXED, true><<<W.grid, b, 0, st>>>(tab, W.slots(), so);
-    else if (W.grid) k_second_wide<R, MIXED, false><<<W.grid, b, 0, st>>>(tab, W.slots(), so);
+    if (W.grid && spin) k_second_wide<R, MIXED, true><<<W.grid, b, 0, side>>>(tab, W.slots(), so);
+    else if (W.grid) k_second_wide<R, MIXED, false><<<W.grid, b, 0, side>>>(tab, W.slots(), so);
+    fork.close(st);
 }
-void launch_second_half_t(const FusedTables &t, const Launch &L, const Launch &W, bool spin, cudaStream_t st) {
-    if (t.prec == 0) second_half_t<double, false>(t, L, W, spin, st);
-    else second_half_t<float, true>(t, L, W, spin, st);
+void launch_second_half_t(const FusedTables &t, const Launch &L, const Launch &W, bool spin, cudaStream_t st,
+                          const Fork &fork) {
+    if (t.prec == 0) second_half_t<double, false>(t, L, W, spin, st, fork);
+    else second_half_t<float, true>(t, L, W, spin, st, fork);
 }
 
 // a system's own launches, over its table
@@ -488,7 +499,8 @@ void fused_half_sizes(int prec, size_t *first, size_t *second) {
 }
 
 void fused_put_half(Sys &s, int r, const FusedTables &t, unsigned char *img, int64_t *blocks) {
-    const IntArgs a = int_args(s);
+    IntArgs a = int_args(s);
+    a.any = t.any();
     reinterpret_cast<IntArgs *>(img + t.o_first)[r] = a;
     if (s.prec == 0) reinterpret_cast<HalfArgs<double> *>(img + t.o_second)[r] = HalfArgs<double>{a, gather_args<double>(s)};
     else reinterpret_cast<HalfArgs<float> *>(img + t.o_second)[r] = HalfArgs<float>{a, gather_args<float>(s)};

@@ -778,7 +778,14 @@ __global__ void k_finish(const BinArgs *__restrict__ tab, WorkMap m, const int *
 }
 // clears the rebuild flag of every slot with a conditional rebuild in the launch (after the
 // whole group has read it); m is the binning kernel's map, in which every such slot has blocks
-__global__ void k_clear_flags(const BinArgs *__restrict__ tab, WorkMap m) {
+// (any: a batch's word that a rebuild is due, cleared with them)
+__global__ void k_clear_flags(const BinArgs *__restrict__ tab, WorkMap m, int *any) {
+    if (any) {   // one block: the word is read by all of it, then cleared
+        const int due = *any;
+        __syncthreads();
+        if (due == 0) return;
+        if (threadIdx.x == 0) *any = 0;
+    }
     for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < m.nrep; r += gridDim.x * blockDim.x)
         if (m.w0[r + 1] > m.w0[r] && tab[r].flag) *tab[r].rebuild = 0;
 }
@@ -1029,7 +1036,7 @@ static void rebuild_t(const FusedTables &t, const Launch *L, bool clear, cudaStr
                                                               L[RB_LISTS].quick);
     k_rev<LOOP><<<L[RB_REV].grid, REV_WARPS * 32, 0, st>>>(t.at<RevArgs>(t.o_rev), L[RB_REV].m, L[RB_REV].quick);
     k_finish<LOOP><<<L[RB_FINISH].grid, RB_THREADS, 0, st>>>(bin, L[RB_FINISH].m, L[RB_FINISH].quick);
-    if (clear) k_clear_flags<<<1, 128, 0, st>>>(bin, L[RB_BIN].m);
+    if (clear) k_clear_flags<<<1, 128, 0, st>>>(bin, L[RB_BIN].m, t.any());
 }
 void launch_rebuild_t(const FusedTables &t, const Launch *L, bool clear, bool loop, cudaStream_t st) {
     if (loop) rebuild_t<true>(t, L, clear, st);

@@ -1,0 +1,29 @@
+"""A batch's two kernels of a launch group (a width each) run side by side over their own slots, and
+its rebuild group returns at once unless a slot's rebuild is due: replicas on both sides of the
+widths, some rebuilding often and some never, step bit for bit as alone."""
+import numpy as np
+import pytest
+
+from paper_2606_14073_gb300 import nep_params, spinlat as S, workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("prec,cells,skins", [(S.SL_PREC_MIXED, (4, 7, 13), (1.0, 0.02, 1.0)),
+                                              (S.SL_PREC_MIXED, (13, 5), (0.02, 1.0)),
+                                              (S.SL_PREC_FP64, (4, 8, 13), (0.05, 1.0, 0.02))])
+def test_widths_side_by_side(prec, cells, skins):
+    make = lambda: [S.system_from_workload(W.fege_cube(c, T=300.0, seed=c), nep_params.load(), precision=prec,  # noqa: E731
+                                           skin=k, seed=c, steps_per_graph=3) for c, k in zip(cells, skins)]
+    alone, together = make(), make()
+    steps = [8 - i for i in range(len(cells))]
+    for s, n in zip(alone, steps):
+        s.step(n, 1.0, 300.0)
+    b = S.Batch(together)
+    k = len(cells)
+    b.step(steps, [1.0] * k, [300.0] * k, [(0.0, 0.0, 0.0)] * k)
+    assert max(s.info()["n_builds"] for s in together) > 1
+    for x, y in zip(alone, together):
+        p, q = x.get_state(), y.get_state()
+        for k in ("positions", "velocities", "spins", "forces", "fields"):
+            assert np.array_equal(p[k], q[k]), k
