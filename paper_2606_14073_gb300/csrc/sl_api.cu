@@ -220,7 +220,7 @@ void enqueue_steps(sl::Sys &s, int64_t n) {
 }
 
 // (a one-launch rebuild takes one of the eight launches of its group)
-int64_t step_kernels(const sl::Sys &s) { return sl::KERNELS_PER_STEP - (s.rb_count ? 7 : 0); }
+int64_t step_kernels(const sl::Sys &s) { return sl::KERNELS_PER_STEP - (s.rb_count ? 7 : 0) + sl::crad_is_split(s); }
 int64_t kernels_per_step(const sl::Sys &s) { return step_kernels(s) + sl::midpoint_kernels_per_step(s); }
 // of `queues` queues of n steps each (enqueue_steps)
 int64_t queue_kernels(const sl::Sys &s, int64_t queues, int64_t n) {

@@ -85,8 +85,8 @@ void FusedBatch::enqueue(cudaStream_t st) const {
     }
     launch_rebuild_t(t, rb, true, true, st);
     const Launch ev[7] = {L(FK_CRAD), L(FK_ANG), L(FK_NET), L(FK_BWD), L(FK_CRADW), L(FK_ANGW), L(FK_BWDW)};
-    if (t.prec == 0) launch_eval_t<double>(t, pd, ev, st, nullptr, fork);
-    else launch_eval_t<float>(t, pf, ev, st, nullptr, fork);
+    if (t.prec == 0) launch_eval_t<double>(t, pd, ev, st, nullptr, fork, fork2);
+    else launch_eval_t<float>(t, pf, ev, st, nullptr, fork, fork2);
     launch_second_half_t(t, L(FK_SECOND), L(FK_SECONDW), true, st, fork);
 }
 
@@ -119,6 +119,21 @@ void fused_layout(FusedTables &t, int prec, int cap) {
     t.bytes = o;
 }
 
+bool Fork::make() {
+    if (cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking) == cudaSuccess &&
+        cudaEventCreateWithFlags(&out, cudaEventDisableTiming) == cudaSuccess &&
+        cudaEventCreateWithFlags(&back, cudaEventDisableTiming) == cudaSuccess)
+        return true;
+    free();
+    return false;
+}
+void Fork::free() {
+    if (out) cudaEventDestroy(out);
+    if (back) cudaEventDestroy(back);
+    if (st) cudaStreamDestroy(st);
+    *this = Fork();
+}
+
 FusedBatch::~FusedBatch() { release(); }
 
 void FusedBatch::release_graphs() {
@@ -147,10 +162,8 @@ void FusedBatch::release() {
     release_items();
     if (t.dev) cudaFree(t.dev);
     if (img) cudaFreeHost(img);
-    if (fork.out) cudaEventDestroy(fork.out);
-    if (fork.back) cudaEventDestroy(fork.back);
-    if (fork.st) cudaStreamDestroy(fork.st);
-    fork = Fork();
+    fork.free();
+    fork2.free();
     t = FusedTables();
     img = nullptr;
     dev_ = -1;
@@ -184,9 +197,7 @@ bool FusedBatch::setup(int prec, int cap, int device) {
         release();
         return false;
     }
-    if (cudaStreamCreateWithFlags(&fork.st, cudaStreamNonBlocking) != cudaSuccess ||
-        cudaEventCreateWithFlags(&fork.out, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&fork.back, cudaEventDisableTiming) != cudaSuccess) {
+    if (!fork.make() || !fork2.make()) {
         release();
         return false;
     }
@@ -220,17 +231,20 @@ bool FusedBatch::same_model(const Sys &s) const {
 // after its length; demangled: the identifier before its template or parameter list): the
 // halves, the radial, angular and backward kernels and the FP64 network (the tensor-core
 // network, k_mlp_tc, is persistent); -1 for the others.
-static int item_kernel_class(const char *name) {
-    struct { const char *id; int cls; } const k[] = {
-        {"k_first_half", IC_FIRST}, {"k_second_half", IC_SECOND}, {"k_second_wide", IC_GATHER},
-        {"k_crad", IC_ATOM}, {"k_crad_wide", IC_OCT},
-        {"k_mlp", IC_OCT}, {"k_ang_fwd", IC_QUAD}, {"k_bwd", IC_QUAD},
-        {"k_ang_wide", IC_WARP}, {"k_bwd_wide", IC_WARP}};
+static int item_kernel_class(const char *name, int whole, int split, int &bit) {
+    struct { const char *id; int cls, bit; } const k[] = {
+        {"k_first_half", IC_FIRST, -1}, {"k_second_half", IC_SECOND, FK_SECOND}, {"k_second_wide", IC_GATHER, FK_SECONDW},
+        {"k_crad", IC_ATOM, FK_CRAD}, {"k_crad_wide", IC_OCT, whole}, {"k_crad_rows", IC_OCT, split},
+        {"k_crad_sums", IC_OCT, split}, {"k_mlp", IC_OCT, -1}, {"k_ang_fwd", IC_QUAD, FK_ANG}, {"k_bwd", IC_QUAD, FK_BWD},
+        {"k_ang_wide", IC_WARP, FK_ANGW}, {"k_bwd_wide", IC_WARP, FK_BWDW}};
     for (const auto &x : k) {
         const std::string id(x.id);
         const std::string forms[3] = {std::to_string(id.size()) + id + "I", id + "<", id + "("};
         for (const std::string &f : forms)
-            if (std::strstr(name, f.c_str())) return x.cls;
+            if (std::strstr(name, f.c_str())) {
+                bit = x.bit;
+                return x.cls;
+            }
     }
     return -1;
 }
@@ -249,15 +263,22 @@ bool FusedBatch::find_item_nodes(cudaGraph_t graph, cudaGraphExec_t exec, int st
         if (cudaGraphKernelNodeGetParams(node, &p) != cudaSuccess) return false;
         const char *name = nullptr;
         if (cudaFuncGetName(&name, p.func) != cudaSuccess || !name) return false;
-        const int c = item_kernel_class(name);
+        int bit = -1;
+        const int c = item_kernel_class(name, BIT_WHOLE, BIT_SPLIT, bit);
         if (c < 0) continue;
         if ((int64_t)p.gridDim.x != std::max<int64_t>(grid_items[c], 1)) return false;
-        item_nodes.push_back(ItemNode{exec, node, c});
+        item_nodes.push_back(ItemNode{exec, node, c, bit});
         ++found;
     }
-    // per step: the first half, the wide radial kernel, the other one (or the FP64 network), and two
-    // kernels each of the angular part, the backward and the second half
-    return found == (int64_t)steps * 9;
+    // per step: the first half, four radial kernels (FP64: three, and the network), and two kernels each of
+    // the angular part, the backward and the second half
+    return found == (int64_t)steps * 11;
+}
+
+void FusedBatch::switch_nodes() {
+    for (const ItemNode &x : item_nodes)
+        if (x.bit >= 0 && cudaGraphNodeSetEnabled(x.exec, x.node, taken >> x.bit & 1u) != cudaSuccess)
+            cudaGetLastError();   // (stays as it is: without blocks of its own it returns at once)
 }
 
 bool FusedBatch::resize_item_nodes() {
@@ -300,6 +321,7 @@ bool FusedBatch::graphs(int steps, const Sys &m, cudaStream_t st) {
             return graphs(steps, m, st);
         }
     }
+    switch_nodes();
     g = steps;
     ++captures;
     return true;
@@ -367,8 +389,17 @@ cudaError_t FusedBatch::upload(const int64_t *left, cudaStream_t st) {
         dirty = true;
     }
     int64_t atoms = 0;
-    for (int r = 0; r < t.cap; ++r)
-        if (slot[(size_t)r]) atoms += slot[(size_t)r]->n;
+    uint32_t now = 0;
+    for (int r = 0; r < t.cap; ++r) {
+        const Sys *s = slot[(size_t)r];
+        if (!s) continue;
+        atoms += s->n;
+        for (int k = 0; k < FK_N; ++k)
+            if (blocks[(size_t)k * t.cap + r] > 0) now |= 1u << k;
+        if (crad_is_wide(*s)) now |= 1u << (crad_is_split(*s) ? BIT_SPLIT : BIT_WHOLE);
+    }
+    const bool other = now != taken;
+    taken = now;
     if (!reserve(atoms)) return cudaErrorMemoryAllocation;
     if (dirty || layout_dirty) {
         // block -> slot layout of the one-item-per-block kernels: every occupied slot's blocks in
@@ -396,6 +427,7 @@ cudaError_t FusedBatch::upload(const int64_t *left, cudaStream_t st) {
             release_graphs();
         }
     }
+    if (other && graph_g) switch_nodes();
     std::memcpy(img + t.o_left, left, sizeof(int64_t) * t.cap);
     if (dirty) e = cudaMemcpyAsync(t.dev, img, t.upload_bytes, cudaMemcpyHostToDevice, st);
     else e = cudaMemcpyAsync(t.dev + t.o_left, img + t.o_left, sizeof(int64_t) * t.cap, cudaMemcpyHostToDevice, st);
@@ -410,6 +442,7 @@ int solo_refresh(Sys &s) {
         if (!s.solo) return -1;
     }
     SoloTables &so = *s.solo;
+    if (crad_is_split(s) && !so.fork.st && !so.fork.make()) return -1;
     FusedTables &t = so.t;
     const size_t w0_bytes = sizeof(int64_t) * FK_N * SK_N * 2 * (SK_N + 1);
     if (!t.dev) {
@@ -453,6 +486,7 @@ int solo_refresh(Sys &s) {
 void solo_free(Sys &s) {
     if (!s.solo) return;
     if (s.solo->t.dev) cudaFree(s.solo->t.dev);
+    s.solo->fork.free();
     delete s.solo;
     s.solo = nullptr;
 }

@@ -26,8 +26,8 @@ enum FusedKernel {
     FK_CRAD, FK_CRADW, FK_ANG, FK_ANGW, FK_NET, FK_BWD, FK_BWDW, FK_SECOND, FK_SECONDW,
     FK_N
 };
-// plan, the kernels (FP64 has the wide radial kernel only), the flag clear
-inline int fused_launches_per_step(int prec) { return 1 + FK_N + 1 - (prec == 0); }
+// plan, the kernels (FP64 has the wide radial kernel only; that is three, in both its forms), the flag clear
+inline int fused_launches_per_step(int prec) { return 1 + FK_N + 2 + 1 - (prec == 0); }
 constexpr int FUSED_MAX_SLOTS = 4096;
 // atoms-per-block classes of the kernels that take one work item per block: the first half (256
 // atoms), the one-thread-per-atom radial kernel (128), the angular and backward kernels (a quad
@@ -134,6 +134,8 @@ struct Fork {
         cudaEventRecord(back, st);
         cudaStreamWaitEvent(to, back, 0);
     }
+    bool make();    // false on failure (then free())
+    void free();
 };
 void launch_second_half_t(const FusedTables &t, const Launch &L, const Launch &W, bool spin, cudaStream_t st,
                           const Fork &fork = Fork());
@@ -145,7 +147,7 @@ void launch_rebuild_t(const FusedTables &t, const Launch *L, bool clear, bool lo
 // kernel, after it, after the angular kernel, after the network and after the backward
 template <typename R>
 void launch_eval_t(const FusedTables &t, const NepDev<R> &P, const Launch *L /* crad, ang, net, bwd, wide crad, ang, bwd */,
-                   cudaStream_t st, cudaEvent_t *ev, const Fork &fork = Fork());
+                   cudaStream_t st, cudaEvent_t *ev, const Fork &fork = Fork(), const Fork &fork2 = Fork());
 void launch_net_t_tc(const FusedTables &t, const NepDev<float> &P, const Launch &L, cudaStream_t st);
 void launch_net_t_fp64(const FusedTables &t, const Launch &L, cudaStream_t st);
 
@@ -186,7 +188,7 @@ public:
     void enqueue(cudaStream_t st) const;
 
     FusedTables t;
-    Fork fork;   // of the captured steps
+    Fork fork, fork2;   // of the captured steps
     cudaGraphExec_t graph_g = nullptr, graph_1 = nullptr;
     int g = 0;
     int64_t captures = 0;
@@ -210,8 +212,14 @@ private:
         cudaGraphExec_t exec;
         cudaGraphNode_t node;   // in tmpl[...], which stays alive with the executable graph
         int cls;
+        int bit;   // of `taken` (-1: every step's)
     };
     std::vector<ItemNode> item_nodes;
+    // Kernels that some slot takes: bit k of kernel k, and of the wide radial kernel's forms.  The others' nodes
+    // are switched off in the executable graphs, an empty launch less each.
+    static constexpr int BIT_WHOLE = FK_N, BIT_SPLIT = FK_N + 1;
+    uint32_t taken = 0;
+    void switch_nodes();
     cudaGraph_t tmpl[2] = {};
     int64_t atom_cap = 0;
     // block -> slot layout per atoms-per-block class (device; pinned host copy), and each
@@ -241,6 +249,7 @@ struct SoloTables {
     int64_t *w0 = nullptr;            // device [FK_N][SK_N][2][SK_N + 1] (in t's allocation)
     int64_t blocks[FK_N][2] = {};     // block count of each kernel per shape
     int sms = 148;                    // the device's SM count (persistent network grid)
+    Fork fork;                        // of the system's evaluation
     WorkMap map(int k, int kind, int shape) const {
         return WorkMap{w0 + (((size_t)k * SK_N + kind) * 2 + shape) * (SK_N + 1), SK_N};
     }

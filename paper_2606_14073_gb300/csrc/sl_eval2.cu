@@ -519,7 +519,7 @@ constexpr int CR_LD = 20;                // staged pair: f_0..f_8, three pads, s
 constexpr int CR_STAGE = CR_LANES * CR_LD + 16;   // the pad puts a warp's two atoms in different banks
 constexpr int CR_NQ = 26;                // descriptor entries an atom gets here
 
-// Test of the candidate pair (i, j): inside rc_rad, inside rc_ang.  FP32: on the FP32
+// Test of the candidate pair (i, j), j's FP32 position at hand: inside rc_rad, inside rc_ang.  FP32: on the FP32
 // positions.  FP64: an FP32 separation decides outside the rounding band around a cutoff and
 // the FP64 test inside it; the FP64 pipe (two lanes per SM and cycle) would otherwise spend a
 // seventh of the kernel on the test.
@@ -529,10 +529,10 @@ template <>
 struct CradTest<float> {
     float4 pi;
     __device__ __forceinline__ CradTest(const NepDev<float> &, const Eval2Args<float> &a, int64_t i) : pi(a.posf[i]) {}
-    __device__ __forceinline__ void operator()(const NepDev<float> &P, const Eval2Args<float> &a, int j, bool &in,
-                                               bool &ang) const {
+    __device__ __forceinline__ void operator()(const NepDev<float> &P, const Eval2Args<float> &a, int, const float4 &fj,
+                                               bool &in, bool &ang) const {
         float dx, dy, dz;
-        sep(a.box, pi, ro(a.posf + j), dx, dy, dz);
+        sep(a.box, pi, fj, dx, dy, dz);
         const float d2 = dx * dx + dy * dy + dz * dz;
         in = d2 < P.rc_r2;
         ang = d2 < P.rc_a2;
@@ -556,9 +556,8 @@ struct CradTest<double> {
         const float E = u * (8.f * m + 4.f * L + 64.f), Rc = (float)P.rc_r + 1.f;
         band = 2.f * (3.4641017f * Rc * E + 3.f * E * E + 4.f * u * Rc * Rc);
     }
-    __device__ __forceinline__ void operator()(const NepDev<double> &P, const Eval2Args<double> &a, int j, bool &in,
-                                               bool &ang) const {
-        const float4 fj = ro(a.posf + j);
+    __device__ __forceinline__ void operator()(const NepDev<double> &P, const Eval2Args<double> &a, int j, const float4 &fj,
+                                               bool &in, bool &ang) const {
         float x = fj.x - fi.x, y = fj.y - fi.y, z = fj.z - fi.z;
         minimg(a.boxf, x, y, z);
         const float d2f = x * x + y * y + z * z, r2 = (float)P.rc_r2, a2 = (float)P.rc_a2;
@@ -578,48 +577,57 @@ struct CradTest<double> {
 template <typename R>
 struct CradSmem {
     R stage[8][CR_STAGE];                // per atom of the block; afterwards its sums [2][5][10]
-    int list[8][32 * MASKW_MAX + 16];    // in-cutoff neighbours in list order (padded like the stage)
-    uint32_t mask[MASKW_MAX][8];         // in-cutoff candidate slots
     R q[CR_NQ][8];                       // the block's descriptor entries, written out by rows
 };
-static_assert(CR_STAGE >= 2 * 5 * 10, "the sums take the stage's place");
+struct CradRowsSmem {
+    uint32_t mask[MASKW_MAX][8];         // in-cutoff candidate slots of the block's atoms
+};
+struct CradLists {                       // the one-kernel form: in-cutoff neighbours in list order
+    int list[8][32 * MASKW_MAX + 16];    // (padded like the stage)
+};
 
+// Where a lane of a wide radial kernel works: 16 lanes per atom, two atoms per warp.
 template <typename R>
-__device__ __forceinline__ void crad_wide_body(const NepDev<R> &P, const Eval2Args<R> &args, int64_t blk,
-                                          CradSmem<R> &sm) {
-    // the arguments as values: read once from the block's copy, so nothing in the loops below
-    // depends on where they are stored
-    const Eval2Args<R> a = args;
-    if (a.skip && *a.skip) return;
-    const int lane = threadIdx.x & (CR_LANES - 1), slot8 = threadIdx.x / CR_LANES;
-    const int half = threadIdx.x & CR_LANES;          // 0 or 16: this atom's lanes in the warp
-    const int per = blockDim.x / CR_LANES;            // atoms of the block
-    const int64_t i = blk * per + slot8;
-    const bool valid = i < a.n;
-    const int64_t N = a.n, at = valid ? i : a.n - 1;
+struct CradPlace {
+    int lane, slot8, half, per;   // lane of the atom, atom of the block, its lanes' shift in the warp, atoms per block
+    int64_t blk, i, at;           // i: the atom; at: the last one for lanes past it
+    bool valid;
+    __device__ __forceinline__ CradPlace(const Eval2Args<R> &a, int64_t block)
+        : lane(threadIdx.x & (CR_LANES - 1)), slot8(threadIdx.x / CR_LANES), half(threadIdx.x & CR_LANES),
+          per(blockDim.x / CR_LANES), blk(block), i(block * (blockDim.x / CR_LANES) + threadIdx.x / CR_LANES),
+          at(i < a.n ? i : a.n - 1), valid(i < a.n) {}
+};
+
+// A: rows, in-cutoff slots and counts of the atom; list: its in-cutoff neighbours (null: not kept).
+// Returns the pairs found, m0 of them of species 0.
+template <typename R>
+__device__ __forceinline__ int crad_rows(const NepDev<R> &P, const Eval2Args<R> &a, const CradPlace<R> &w,
+                                         CradRowsSmem &sm, int *list, int &m0) {
+    const int lane = w.lane, half = w.half, slot8 = w.slot8;
+    const int64_t N = a.n, i = w.i, at = w.at;
     const unsigned lt = (1u << lane) - 1u;
-    R *stage = sm.stage[slot8];
-    int *list = sm.list[slot8];
     if (lane < MASKW_MAX) sm.mask[lane][slot8] = 0u;
-    v4<R> pi, si;
-    pair_at(a, at, pi, si);
-    const int4 sg = valid ? a.seg[i] : make_int4(0, 0, 0, 0);
+    const int4 sg = w.valid ? a.seg[i] : make_int4(0, 0, 0, 0);
     const CradTest<R> test(P, a, at);
     const int32_t *__restrict__ nrow = a.nbr + at * a.capr;
     const uint8_t *__restrict__ rrow = a.rev + at * a.capr;
     __syncwarp();
-
-    // A
-    int m = 0, m0 = 0, na = 0, na0 = 0;   // pairs found (of species 0), angular ones
+    int m = 0, na = 0, na0 = 0;   // pairs found, angular ones (of species 0)
+    m0 = 0;
     bool ovf = false;
     const int steps = __reduce_max_sync(0xffffffffu, sg.w);
-    int jn = lane < sg.w ? nrow[lane] : 0;
+    // the next candidate's FP32 position and the one after it are in flight
+    int jn = lane < sg.w ? nrow[lane] : 0, jn2 = lane + CR_LANES < sg.w ? nrow[lane + CR_LANES] : 0;
+    float4 pn = a.posf[lane < sg.w ? jn : at];
     uint32_t word = 0u;
     for (int base = 0; base < steps; base += CR_LANES) {
         const int v = base + lane, j = jn;
-        if (v + CR_LANES < sg.w) jn = nrow[v + CR_LANES];   // the next candidate is in flight
+        const float4 pj = pn;
+        jn = jn2;
+        if (v + CR_LANES < sg.w) pn = a.posf[jn];
+        if (v + 2 * CR_LANES < sg.w) jn2 = nrow[v + 2 * CR_LANES];
         bool in = false, ang = false;
-        if (v < sg.w) test(P, a, j, in, ang);
+        if (v < sg.w) test(P, a, j, pj, in, ang);
         const unsigned ha = (__ballot_sync(0xffffffffu, ang) >> half) & 0xffffu;
         const int ra = na + __popc(ha & lt);
         if (ang && ra >= a.cap_ang) {   // angular rows full: only after a list overflow
@@ -629,7 +637,7 @@ __device__ __forceinline__ void crad_wide_body(const NepDev<R> &P, const Eval2Ar
         const unsigned hi = (__ballot_sync(0xffffffffu, in) >> half) & 0xffffu;
         if (in) {
             const int c = m + __popc(hi & lt);
-            list[c] = j;
+            if (list) list[c] = j;
             stg(a.crow + (int64_t)(ang ? ra : a.cap_ang + (c - ra)) * N + i, make_int2(j, rrow[v]));
         }
         word = base & 16 ? word | hi << 16 : hi;
@@ -643,9 +651,40 @@ __device__ __forceinline__ void crad_wide_body(const NepDev<R> &P, const Eval2Ar
         na = min(na + __popc(ha), a.cap_ang);
     }
     if (ovf) atomicOr(a.status, ST_NBR_OVERFLOW);
-    if (valid && lane == 0) stg(a.cnt + i, make_int4(na0, na, m0 - na0, m - na));
+    if (w.valid && lane == 0) stg(a.cnt + i, make_int4(na0, na, m0 - na0, m - na));
     __syncwarp();
-    // B
+    return m;
+}
+
+// The block's slot masks by words, its descriptor entries by rows: its atoms are neighbours in memory.
+template <typename R>
+__device__ __forceinline__ void crad_store_masks(const Eval2Args<R> &a, const CradPlace<R> &w, const CradRowsSmem &sm) {
+    for (int e = threadIdx.x; e < a.maskw * w.per; e += blockDim.x) {
+        const int word = e / w.per, k = e % w.per;
+        const int64_t i = w.blk * w.per + k;
+        if (i < a.n) stg(reinterpret_cast<int *>(a.mask) + (int64_t)word * a.n + i, (int)sm.mask[word][k]);
+    }
+}
+template <typename R>
+__device__ __forceinline__ void crad_store_q(const Eval2Args<R> &a, const CradPlace<R> &w, const CradSmem<R> &sm) {
+    for (int e = threadIdx.x; e < CR_NQ * w.per; e += blockDim.x) {
+        const int row = e / w.per, k = e % w.per;
+        const int64_t i = w.blk * w.per + k;
+        const int v = row < 5 ? Q_R + row : row < 25 ? Q_EX + (row - 5) : Q_O;   // EX, DMI, ANI, SIA in turn
+        if (i < a.n) stg(a.q + v * a.qs + i, sm.q[row][k]);
+    }
+}
+
+// B, C: the sums of the atom's m pairs (m0 of species 0 first) and its descriptor entries; neighbour(base): the
+// neighbour of the lane's pair of the round from base on.
+template <typename R, typename Neighbour>
+__device__ __forceinline__ void crad_sums(const NepDev<R> &P, const Eval2Args<R> &a, const CradPlace<R> &w, int m, int m0,
+                                          CradSmem<R> &sm, Neighbour neighbour) {
+    const int lane = w.lane, slot8 = w.slot8;
+    const int64_t at = w.at;
+    R *stage = sm.stage[slot8];
+    v4<R> pi, si;
+    pair_at(a, at, pi, si);
     const int kp = lane % 5, third = lane / 5;   // lane 15 is idle in the sums
     R b0[2][2];
     v2<R> b12[2][2], b34[2][2];
@@ -660,7 +699,7 @@ __device__ __forceinline__ void crad_wide_body(const NepDev<R> &P, const Eval2Ar
     for (int base = 0; base < mmax; base += CR_LANES) {
         const int cnt = min(m - base, CR_LANES);
         if (lane < cnt) {
-            const int j = list[base + lane];
+            const int j = neighbour(base);
             v4<R> pj, sj;
             pair_at(a, j, pj, sj);
             R dx, dy, dz;
@@ -746,19 +785,62 @@ __device__ __forceinline__ void crad_wide_body(const NepDev<R> &P, const Eval2Ar
         sm.q[o][slot8] = q;
     }
     if (lane == 0) sm.q[25][slot8] = si.x * si.x + si.y * si.y + si.z * si.z;
-    // the block's outputs by rows: its atoms are neighbours in memory
+}
+
+// In one kernel.
+template <typename R>
+__device__ __forceinline__ void crad_wide_body(const NepDev<R> &P, const Eval2Args<R> &args, int64_t blk,
+                                               CradSmem<R> &sm, CradRowsSmem &rows, CradLists &lists) {
+    // the arguments as values: read once from the block's copy, so nothing in the loops below
+    // depends on where they are stored
+    const Eval2Args<R> a = args;
+    if (a.split || (a.skip && *a.skip)) return;
+    const CradPlace<R> w(a, blk);
+    int *list = lists.list[w.slot8], m0;
+    const int m = crad_rows(P, a, w, rows, list, m0);
+    crad_sums(P, a, w, m, m0, sm, [&](int base) { return list[base + w.lane]; });
     __syncthreads();
-    const int64_t i0 = blk * per;
-    for (int e = threadIdx.x; e < (CR_NQ + a.maskw) * per; e += blockDim.x) {
-        const int row = e / per, k = e % per;
-        if (i0 + k >= N) continue;
-        if (row < CR_NQ) {
-            const int v = row < 5 ? Q_R + row : row < 25 ? Q_EX + (row - 5) : Q_O;   // EX, DMI, ANI, SIA in turn
-            stg(a.q + v * a.qs + i0 + k, sm.q[row][k]);
-        } else {
-            stg(reinterpret_cast<int *>(a.mask) + (int64_t)(row - CR_NQ) * N + i0 + k, (int)sm.mask[row - CR_NQ][k]);
-        }
-    }
+    crad_store_masks(a, w, rows);
+    crad_store_q(a, w, sm);
+}
+
+// In two (crad_is_split): the rows, then the sums over them, which nothing before the network waits for and which
+// run beside the angular kernel, where a small system leaves both most of the GPU.  A step of 512 / 1,728 /
+// 4,096 / 8,000 / 13,824 atoms, mixed precision: 44.4 / 49.7 / 58.6 / 71.4 / 101.2 us in one kernel, 40.9 / 46.7 / 56.5 / 72.8 /
+// 104.5 in two; FP64, 512 / 1,728 / 2,744 / 4,096 atoms: 185 / 373 / 571 / 641 and 173 / 377 / 554 / 692 us.  (The line
+// lies below where the two cross.)
+template <typename R>
+__device__ __forceinline__ void crad_rows_body(const NepDev<R> &P, const Eval2Args<R> &args, int64_t blk, CradRowsSmem &sm) {
+    const Eval2Args<R> a = args;
+    if (!a.split || (a.skip && *a.skip)) return;
+    const CradPlace<R> w(a, blk);
+    int m0;
+    crad_rows(P, a, w, sm, nullptr, m0);
+    __syncthreads();
+    crad_store_masks(a, w, sm);
+}
+template <typename R>
+__device__ __forceinline__ void crad_sums_body(const NepDev<R> &P, const Eval2Args<R> &args, int64_t blk, CradSmem<R> &sm) {
+    const Eval2Args<R> a = args;
+    if (!a.split || (a.skip && *a.skip)) return;
+    const CradPlace<R> w(a, blk);
+    // pairs by species, angular rows before the others; the next round's neighbour is in flight
+    const int4 c = w.valid ? a.cnt[w.i] : make_int4(0, 0, 0, 0);   // angular of species 0, angular, others of species 0, others
+    const int m = c.y + c.w, m0 = c.x + c.z;
+    auto row = [&](int p) {
+        if (p < m0) return p < c.x ? p : a.cap_ang + p - c.x;
+        const int r = p - m0 + c.x;
+        return r < c.y ? r : a.cap_ang + c.z + (r - c.y);
+    };
+    const int2 *__restrict__ crow = a.crow + w.at;
+    int jn = w.lane < m ? crow[(int64_t)row(w.lane) * a.n].x : 0;
+    crad_sums(P, a, w, m, m0, sm, [&](int base) {
+        const int j = jn, p = base + CR_LANES + w.lane;
+        if (p < m) jn = crow[(int64_t)row(p) * a.n].x;
+        return j;
+    });
+    __syncthreads();
+    crad_store_q(a, w, sm);
 }
 
 
@@ -1597,13 +1679,29 @@ __global__ void __launch_bounds__(128, MINB) k_crad(const __grid_constant__ NepD
     __shared__ uint32_t smask[MASKW_MAX][128];   // blocks have at most 128 threads
     one_work(tab, sm, solo, [&](const Eval2Args<float> &a, int64_t blk, int64_t) { crad_body(P, a, blk, smask); });
 }
-template <typename R>
+template <typename R>   // (blocks of these three have at most 128 threads)
 __global__ void __launch_bounds__(128, sizeof(R) == 4 ? 8 : 4) k_crad_wide(const __grid_constant__ NepDev<R> P,
                                                                            const Eval2Args<R> *__restrict__ tab,
                                                                            SlotMap sm,
                                                                            const __grid_constant__ Eval2Args<R> solo) {
-    __shared__ __align__(32) CradSmem<R> scratch;   // blocks have at most 128 threads
-    one_work(tab, sm, solo, [&](const Eval2Args<R> &a, int64_t blk, int64_t) { crad_wide_body(P, a, blk, scratch); });
+    __shared__ __align__(32) CradSmem<R> scratch;
+    __shared__ CradRowsSmem rows;
+    __shared__ CradLists lists;
+    one_work(tab, sm, solo, [&](const Eval2Args<R> &a, int64_t blk, int64_t) { crad_wide_body(P, a, blk, scratch, rows, lists); });
+}
+template <typename R>
+__global__ void __launch_bounds__(128, 8) k_crad_rows(const __grid_constant__ NepDev<R> P, const Eval2Args<R> *__restrict__ tab,
+                                                      SlotMap sm, const __grid_constant__ Eval2Args<R> solo) {
+    __shared__ CradRowsSmem rows;
+    one_work(tab, sm, solo, [&](const Eval2Args<R> &a, int64_t blk, int64_t) { crad_rows_body(P, a, blk, rows); });
+}
+template <typename R>
+__global__ void __launch_bounds__(128, sizeof(R) == 4 ? 8 : 4) k_crad_sums(const __grid_constant__ NepDev<R> P,
+                                                                           const Eval2Args<R> *__restrict__ tab,
+                                                                           SlotMap sm,
+                                                                           const __grid_constant__ Eval2Args<R> solo) {
+    __shared__ __align__(32) CradSmem<R> scratch;
+    one_work(tab, sm, solo, [&](const Eval2Args<R> &a, int64_t blk, int64_t) { crad_sums_body(P, a, blk, scratch); });
 }
 template <typename R, int MINB = sizeof(R) == 4 ? 4 : 1>
 __global__ void __launch_bounds__(128, MINB) k_ang_fwd(const __grid_constant__ NepDev<R> P,
@@ -1663,6 +1761,7 @@ static Eval2Args<R> args2(Sys &s, const EvalAt &at, bool want_virial) {
         a.box = *reinterpret_cast<const BoxDev<R> *>(&s.boxf);
     }
     a.posf = at.posf ? at.posf : s.posf;
+    a.split = crad_is_split(s);
     a.skip = at.skip;
     a.nbr = s.nbr; a.seg = s.seg; a.rev = s.rev; a.capr = nbr_stride(s.cap); a.n = s.n; a.n_fe = s.n_fe;
     a.cap = s.cap; a.cap_ang = s.cap_ang;
@@ -1741,7 +1840,7 @@ void fused_put_eval(Sys &s, int r, int kind, const FusedTables &t, unsigned char
 // (L[k].block threads, 0: the default) and register budget (L[k].minb, 0: the default).
 template <typename R>
 void launch_eval_t(const FusedTables &t, const NepDev<R> &P, const Launch *L, cudaStream_t st, cudaEvent_t *ev,
-                   const Fork &fork) {
+                   const Fork &fork, const Fork &fork2) {
     // a system's own launch passes its argument block as a kernel parameter; a batch's reads
     // the table (the same for the four kernels of one launch group)
     const Eval2Args<R> *tab = L[0].solo ? nullptr : t.at<Eval2Args<R>>(t.o_eval);
@@ -1760,11 +1859,17 @@ void launch_eval_t(const FusedTables &t, const NepDev<R> &P, const Launch *L, cu
         if (L[0].grid && L[0].minb == 3) k_crad<3><<<L[0].grid, cb, 0, st>>>(P, tab, s0, so);
         else if (L[0].grid) k_crad<<<L[0].grid, cb, 0, st>>>(P, tab, s0, so);
     }
-    if (L[4].grid) k_crad_wide<R><<<L[4].grid, L[4].block ? L[4].block : 128, 0, side>>>(P, tab, L[4].slots(), so);
+    const int wb = L[4].block ? L[4].block : 128;
+    // (a batch launches both forms: a slot's blocks return at once in the one it does not take)
+    if (L[4].grid && !(L[4].solo && so.split)) k_crad_wide<R><<<L[4].grid, wb, 0, side>>>(P, tab, L[4].slots(), so);
+    const bool split = L[4].grid && !(L[4].solo && !so.split);
+    if (split) k_crad_rows<R><<<L[4].grid, wb, 0, side>>>(P, tab, L[4].slots(), so);
     fork.close(st);
+    // the sums beside the angular kernels
+    if (split) k_crad_sums<R><<<L[4].grid, wb, 0, side>>>(P, tab, L[4].slots(), so);
     bool variant = false;
     if (ev) cudaEventRecord(ev[2], st);
-    side = fork.open(st);
+    const cudaStream_t side2 = fork2.open(st);
     if constexpr (sizeof(R) == 4) {
         variant = L[1].minb == 1 && L[1].grid;
         if (variant) k_ang_fwd<R, 1><<<L[1].grid, qa, fwd_smem<R>(qa), st>>>(P, tab, s1, so);
@@ -1772,8 +1877,9 @@ void launch_eval_t(const FusedTables &t, const NepDev<R> &P, const Launch *L, cu
     if (!variant && L[1].grid) k_ang_fwd<R><<<L[1].grid, qa, fwd_smem<R>(qa), st>>>(P, tab, s1, so);
     if (L[5].grid) {
         const int b = L[5].block ? L[5].block : quad_block<R>();
-        k_ang_wide<R><<<L[5].grid, b, fwd_smem<R>(b), side>>>(P, tab, L[5].slots(), so);
+        k_ang_wide<R><<<L[5].grid, b, fwd_smem<R>(b), side2>>>(P, tab, L[5].slots(), so);
     }
+    fork2.close(st);
     fork.close(st);
     if (ev) cudaEventRecord(ev[3], st);
     if constexpr (sizeof(R) == 4) launch_net_t_tc(t, P, L[2], st);
@@ -1803,9 +1909,9 @@ void launch_eval_t(const FusedTables &t, const NepDev<R> &P, const Launch *L, cu
     if (ev) cudaEventRecord(ev[5], st);
 }
 template void launch_eval_t<float>(const FusedTables &, const NepDev<float> &, const Launch *, cudaStream_t,
-                                   cudaEvent_t *, const Fork &);
+                                   cudaEvent_t *, const Fork &, const Fork &);
 template void launch_eval_t<double>(const FusedTables &, const NepDev<double> &, const Launch *, cudaStream_t,
-                                    cudaEvent_t *, const Fork &);
+                                    cudaEvent_t *, const Fork &, const Fork &);
 
 // The system's own evaluation: at the midpoint point while s.at is set (the midpoint
 // iteration), else at the state, with the virial parts when asked for.
@@ -1816,8 +1922,10 @@ void launch_eval(Sys &s, bool want_virial, cudaEvent_t *ev, bool forward_only) {
                    solo_launch(s, FK_BWD, kind),  solo_launch(s, FK_CRADW, kind), solo_launch(s, FK_ANGW, kind),
                    solo_launch(s, FK_BWDW, kind)};
     if (forward_only) L[3].grid = L[6].grid = 0;
-    if (s.prec == 0) launch_eval_t<double>(s.solo->t, s.pd, L, s.stream, ev);
-    else launch_eval_t<float>(s.solo->t, s.pf, L, s.stream, ev);
+    // (a profiled evaluation's kernels run one after the other)
+    const Fork fork = crad_is_split(s) && !ev ? s.solo->fork : Fork();
+    if (s.prec == 0) launch_eval_t<double>(s.solo->t, s.pd, L, s.stream, ev, fork);
+    else launch_eval_t<float>(s.solo->t, s.pf, L, s.stream, ev, fork);
 }
 
 }  // namespace sl

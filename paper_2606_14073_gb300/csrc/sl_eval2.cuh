@@ -42,6 +42,7 @@ struct Eval2Args {
     v4<R> *fown, *gii;
     R *wpart;
     int want_virial;
+    int split;         // the wide radial kernel in two parts (crad_is_split)
     int *status;
     const int *skip;   // non-null and set: every evaluation kernel returns at once
 };

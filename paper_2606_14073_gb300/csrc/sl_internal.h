@@ -230,6 +230,9 @@ inline int nbr_stride(int cap) { return (cap + 31) & ~31; }   // byte rows of 32
 constexpr int64_t CRAD_WIDE_MAX = 16384;
 constexpr int CRAD_WIDE_ATOMS = 8;   // atoms per 128-thread block of k_crad_wide
 inline bool crad_is_wide(const Sys &s) { return s.prec == 0 || s.n <= CRAD_WIDE_MAX; }
+// Its form: in two kernels, rows and sums, in small systems (timed at crad_rows_body).
+constexpr int64_t CRAD_SPLIT_MAX64 = 1024, CRAD_SPLIT_MAX32 = 4096;
+inline bool crad_is_split(const Sys &s) { return s.n <= (s.prec == 0 ? CRAD_SPLIT_MAX64 : CRAD_SPLIT_MAX32); }
 // The angular and backward kernels of a system (fixed by its size likewise): a warp per atom in
 // small systems, else four lanes per atom (both timed at k_ang_wide).
 constexpr int64_t EVAL_WIDE_MAX64 = 3040, EVAL_WIDE_MAX32 = 2048;

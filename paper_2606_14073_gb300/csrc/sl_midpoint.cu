@@ -321,7 +321,8 @@ inline unsigned nblk(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 
 int midpoint_kernels_per_step(const Sys &s) {
     if (s.mid_iters <= 0) return 0;
-    return s.aa_depth > 0 ? 1 + s.mid_iters * (1 + 4 + 1 + 3) + 1 : 2 + s.mid_iters * (4 + 1) + 1;
+    const int ev = 4 + crad_is_split(s);
+    return s.aa_depth > 0 ? 1 + s.mid_iters * (1 + ev + 1 + 3) + 1 : 2 + s.mid_iters * (ev + 1) + 1;
 }
 
 size_t midpoint_scratch_doubles() { return (size_t)AA_BLOCKS * AA_VALS; }
