@@ -79,7 +79,6 @@ __device__ __forceinline__ int4 ro(const int4 *p) { return __ldg(p); }
 __device__ __forceinline__ int2 ro(const int2 *p) { return __ldg(p); }
 __device__ __forceinline__ int ro(const int *p) { return __ldg(p); }
 __device__ __forceinline__ unsigned ro(const unsigned *p) { return __ldg(p); }
-__device__ __forceinline__ unsigned short ro(const unsigned short *p) { return __ldg(p); }
 __device__ __forceinline__ float2 ro(const float2 *p) { return __ldg(p); }
 __device__ __forceinline__ double2 ro(const double2 *p) { return __ldg(p); }
 __device__ __forceinline__ float ro(const float *p) { return __ldg(p); }
@@ -93,7 +92,6 @@ __device__ __forceinline__ double4 ro(const double4 *p) {
 // memory; a store through a plain (generic) pointer might, as far as the compiler can tell,
 // land there, and every argument would be read again after it.
 __device__ __forceinline__ void stg(int *p, int v) { __stwb(p, v); }
-__device__ __forceinline__ void stg(unsigned short *p, unsigned short v) { __stwb(p, v); }
 __device__ __forceinline__ void stg(float *p, float v) { __stwb(p, v); }
 __device__ __forceinline__ void stg(double *p, double v) { __stwb(p, v); }
 __device__ __forceinline__ void stg(float4 *p, const float4 &v) { __stwb(p, v); }
@@ -106,13 +104,6 @@ __device__ __forceinline__ void stg(double4 *p, const double4 &v) {
     __stwb(reinterpret_cast<double2 *>(p) + 1, make_double2(v.z, v.w));
 }
 
-template <typename R>
-__device__ __forceinline__ R rint_(R x);
-template <>
-__device__ __forceinline__ float rint_<float>(float x) { return rintf(x); }
-template <>
-__device__ __forceinline__ double rint_<double>(double x) { return rint(x); }
-
 // Whole box lengths of a separation.  FP32: the nearest integer by adding and subtracting
 // 1.5 2^23 (one multiply-add and one add, off the conversion pipe; |x/L| < 2^22).
 __device__ __forceinline__ void minimg(const BoxDev<float> &b, float &dx, float &dy, float &dz) {
@@ -121,11 +112,10 @@ __device__ __forceinline__ void minimg(const BoxDev<float> &b, float &dx, float 
     dy = fmaf(-b.L[1], __fadd_rn(fmaf(dy, b.invL[1], big), -big), dy);
     dz = fmaf(-b.L[2], __fadd_rn(fmaf(dz, b.invL[2], big), -big), dz);
 }
-template <typename R>
-__device__ __forceinline__ void minimg(const BoxDev<R> &b, R &dx, R &dy, R &dz) {
-    dx -= b.L[0] * rint_(dx * b.invL[0]);
-    dy -= b.L[1] * rint_(dy * b.invL[1]);
-    dz -= b.L[2] * rint_(dz * b.invL[2]);
+__device__ __forceinline__ void minimg(const BoxDev<double> &b, double &dx, double &dy, double &dz) {
+    dx -= b.L[0] * rint(dx * b.invL[0]);
+    dy -= b.L[1] * rint(dy * b.invL[1]);
+    dz -= b.L[2] * rint(dz * b.invL[2]);
 }
 
 template <typename R>

@@ -68,6 +68,7 @@ constexpr uint32_t SZ_Q = DIM * TM * 4;                   // 33792, the TMA tran
 // descriptors' load issued before the weights' copy (four threads: 123 / 24.9 / 10.5).
 constexpr int RT = 2, NT = TM * RT;
 constexpr int HC = N1 / RT;                               // hidden columns of a thread
+static_assert(HC == 16, "a thread's hidden columns are one tensor-memory load");
 constexpr uint32_t OFF_E = OFF_Q + SZ_Q;                  // the row's RT partial energies
 constexpr uint32_t SMEM_BYTES = OFF_E + RT * TM * 4;
 
@@ -136,15 +137,6 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float v[16]) {
         : "r"(taddr));
 #pragma unroll
     for (int t = 0; t < 16; ++t) v[t] = __uint_as_float(r[t]);
-}
-
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float v[8]) {
-    uint32_t r[8];
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-                 : "r"(taddr));
-#pragma unroll
-    for (int t = 0; t < 8; ++t) v[t] = __uint_as_float(r[t]);
 }
 
 // One TMA tile load of the descriptor box (atoms x0 .. x0+127, all 66 rows) into shared
@@ -283,7 +275,7 @@ __device__ __forceinline__ void mlp_tc_body(const NepDev<float> &P, int64_t ntil
     int *status = nullptr;   // the status word of the last tile's system (timeouts are reported there)
 
     const float *stage = reinterpret_cast<const float *>(smem + OFF_Q);
-    [[maybe_unused]] float *energy = reinterpret_cast<float *>(smem + OFF_E);
+    float *energy = reinterpret_cast<float *>(smem + OFF_E);
     q_in_flight = blockIdx.x < ntiles;
 
     for (int64_t tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
@@ -348,12 +340,7 @@ __device__ __forceinline__ void mlp_tc_body(const NepDev<float> &P, int64_t ntil
         // epilogue 1: tanh layer, E_i, t_h into the A2 tile
         float z[HC], tt[HC];
         const int h0 = part * HC;
-        if constexpr (HC == 8) {
-            tmem_ld8(t_z + lane_off + h0, z);
-        } else {
-#pragma unroll
-            for (int c = 0; c < HC; c += 16) tmem_ld16(t_z + lane_off + h0 + c, z + c);
-        }
+        tmem_ld16(t_z + lane_off + h0, z);
         tmem_wait_ld();
         float E = part == 0 ? -P.b1 : 0.f;
 #pragma unroll
@@ -367,7 +354,7 @@ __device__ __forceinline__ void mlp_tc_body(const NepDev<float> &P, int64_t ntil
                 tt[k] = 0.f;
             }
         }
-        if constexpr (RT > 1) energy[part * TM + row] = E;
+        energy[part * TM + row] = E;
 #pragma unroll
         for (int c = 0; c < HC / 8; ++c) {
             uint4 hi, lo;
