@@ -1641,7 +1641,7 @@ static int fused_steps(sl_batch *b, const std::vector<int> &active, const int64_
     for (int64_t r = 0; r < most % g; ++r) CK(cudaGraphLaunch(f.graph_1, b->stream));
     b->graph_launches += most / g + most % g;
     b->fused_steps += most;
-    b->kernel_launches += most * sl::fused_launches_per_step(m.prec);
+    b->kernel_launches += most * f.launches_per_step();
     ++b->fused_calls;
     CK(cudaEventRecord(b->ev[0], b->stream));
     for (int i : active) CK(cudaStreamWaitEvent(b->sys[i]->s.stream, b->ev[0], 0));   // and each replica waits for it

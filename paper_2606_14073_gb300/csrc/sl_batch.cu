@@ -275,6 +275,15 @@ bool FusedBatch::find_item_nodes(cudaGraph_t graph, cudaGraphExec_t exec, int st
     return found == (int64_t)steps * 11;
 }
 
+int64_t FusedBatch::launches_per_step() const {
+    int64_t n = fused_launches_per_step(t.prec);
+    if (item_nodes.empty()) return n;
+    for (int k : {(int)FK_SECOND, (int)FK_SECONDW, (int)FK_ANG, (int)FK_ANGW, (int)FK_BWD, (int)FK_BWDW, BIT_WHOLE, BIT_SPLIT,
+                  BIT_SPLIT})   // (the split form is two kernels)
+        n -= !(taken >> k & 1u);
+    return n - (t.prec != 0 && !(taken >> FK_CRAD & 1u));
+}
+
 void FusedBatch::switch_nodes() {
     for (const ItemNode &x : item_nodes)
         if (x.bit >= 0 && cudaGraphNodeSetEnabled(x.exec, x.node, taken >> x.bit & 1u) != cudaSuccess)

@@ -220,6 +220,9 @@ private:
     static constexpr int BIT_WHOLE = FK_N, BIT_SPLIT = FK_N + 1;
     uint32_t taken = 0;
     void switch_nodes();
+public:
+    int64_t launches_per_step() const;   // of the captured graphs, the kernels switched off not counted
+private:
     cudaGraph_t tmpl[2] = {};
     int64_t atom_cap = 0;
     // block -> slot layout per atoms-per-block class (device; pinned host copy), and each

@@ -9,7 +9,8 @@
 //              neighbour species, and accumulates the radial and pairwise-magnetic basis
 //              sums over them, contracted with the coefficients once per neighbour
 //              species (q^R, q^EX, q^DMI, q^ANI, q^SIA, q^O).
-//   k_crad_wide  the same with sixteen lanes per atom (small systems, and FP64).
+//   k_crad_wide  the same with sixteen lanes per atom (small systems, and FP64); in the smallest ones as
+//              k_crad_rows (compaction) and k_crad_sums, beside the angular kernel.
 //   k_ang_fwd  four lanes per atom (k_ang_wide: a warp, in small systems).  Each lane stages one angular pair
 //              (carrier, g_n, spin weight, the 24 solid harmonics) in shared memory; then
 //              every lane accumulates B_nlm, BS_nlm for its 6 harmonics over the staged pairs.
@@ -509,7 +510,7 @@ __device__ __forceinline__ void crad_body(const NepDev<R> &P, const Eval2Args<R>
 // atom takes, but spread over a warp for every two atoms): 512 / 13,824 / 110,592 atoms 45 / 349 /
 // 2,113 us, against 511 / 525 / 2,091 us with one thread per atom.  Mixed precision: instruction
 // issue (1,270 warp instructions per atom against 570 for one thread per atom, whose chain of 110
-// candidates takes 47 us however few the atoms): 512 / 13,824 / 32,768 / 110,592 atoms 15 / 37 / 70 /
+// candidates takes 47 us however few the atoms): 512 / 13,824 / 32,768 / 110,592 atoms 15 / 35 / 70 /
 // 202 us, against 47 / 64 / 72 / 148 us.  The line lies at 16,384 atoms, below the crossing: a
 // replica keeps its kernel in a batch (its results are the same there bit for bit), where other
 // replicas fill the GPU and only the instructions count (eight replicas of 4,096 to 65,536 atoms
