@@ -30,3 +30,25 @@ def test_lists_equal_the_oracle(shape, drop):
         ref = O.neighbors(pos, box, per, cut, method=method)
         assert all(np.array_equal(a, b) for a, b in zip(lists, ref))
     assert builds >= 2
+
+
+def test_builds_on_several_streams_at_once():
+    """Systems stepped by a thread each, a build in nearly every step, so that several one-launch builds
+    want the GPU at a time: every system as when it steps alone."""
+    from concurrent.futures import ThreadPoolExecutor
+
+    def run(k):
+        s = S.system_from_workload(W.fege_cube(6 + 2 * (k % 4), T=300.0, seed=k), nep_params.load(),
+                                   precision=S.SL_PREC_MIXED, skin=0.02, seed=k)
+        s.step(40, 1.0, 300.0)
+        out = s.get_state(), s.info()["n_builds"]
+        s.destroy()
+        return out
+
+    alone = [run(k) for k in range(8)]
+    with ThreadPoolExecutor(8) as ex:
+        together = list(ex.map(run, range(8)))
+    for (a, na), (b, nb) in zip(alone, together):
+        assert na == nb and na > 20
+        for k in ("positions", "velocities", "spins", "forces", "fields"):
+            assert np.array_equal(a[k], b[k]), k
