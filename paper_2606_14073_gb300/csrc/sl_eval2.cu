@@ -1073,27 +1073,22 @@ __device__ __forceinline__ void ang_fwd_body(const NepDev<R> &P, const Eval2Args
         }
     }
     if constexpr (QUAD) {
+        // summed over the quad, lane ql ending with l = ql + 1: the pair of lanes that differ in bit 0
+        // exchange the degrees the other keeps, then those that differ in bit 1
+        const bool odd = ql & 1, high = ql & 2;
 #pragma unroll
-        for (int n = 0; n < NCH; ++n)
+        for (int n = 0; n < NCH; ++n) {
+            R v[2];
 #pragma unroll
-            for (int t = 0; t < 4; ++t) {
-                qa[n][t] += __shfl_xor_sync(0xffffffffu, qa[n][t], 1);
-                qa[n][t] += __shfl_xor_sync(0xffffffffu, qa[n][t], 2);
-                qs[n][t] += __shfl_xor_sync(0xffffffffu, qs[n][t], 1);
-                qs[n][t] += __shfl_xor_sync(0xffffffffu, qs[n][t], 2);
+            for (int c = 0; c < 2; ++c) {
+                const R *x = c == 0 ? qa[n] : qs[n];
+                const R lo = (odd ? x[1] : x[0]) + __shfl_xor_sync(0xffffffffu, odd ? x[0] : x[1], 1);
+                const R hi = (odd ? x[3] : x[2]) + __shfl_xor_sync(0xffffffffu, odd ? x[2] : x[3], 1);
+                v[c] = (high ? hi : lo) + __shfl_xor_sync(0xffffffffu, high ? lo : hi, 2);
             }
-        if (valid) {
-            // lane ql writes l = ql + 1
-#pragma unroll
-            for (int n = 0; n < NCH; ++n) {
-                R va = qa[n][0], vs = qs[n][0];
-#pragma unroll
-                for (int t = 1; t < 4; ++t) {
-                    va = ql == t ? qa[n][t] : va;
-                    vs = ql == t ? qs[n][t] : vs;
-                }
-                stg(a.q + (int64_t)(Q_A + n * 4 + ql) * a.qs + i, va);
-                stg(a.q + (int64_t)(Q_SA + n * 4 + ql) * a.qs + i, vs);
+            if (valid) {
+                stg(a.q + (int64_t)(Q_A + n * 4 + ql) * a.qs + i, v[0]);
+                stg(a.q + (int64_t)(Q_SA + n * 4 + ql) * a.qs + i, v[1]);
             }
         }
     } else {
