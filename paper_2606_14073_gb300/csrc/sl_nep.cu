@@ -251,15 +251,18 @@ __global__ void __launch_bounds__(WARPS * 32) k_eval_noalloc(const __grid_consta
     float far = 0.f;
     for (int j = tid; j < n; j += WARPS * 32) {
         const double4 p = pos[j];
-        const double x = p.x - box.L[0] * rint(p.x * box.invL[0]), y = p.y - box.L[1] * rint(p.y * box.invL[1]),
-                     z = p.z - box.L[2] * rint(p.z * box.invL[2]);
+        // (the whole box lengths in FP32: one off, should they be, only widens the band)
+        const float px = (float)p.x, py = (float)p.y, pz = (float)p.z;
+        const float x = (float)fma(-box.L[0], (double)rintf(px * (float)box.invL[0]), p.x),
+                    y = (float)fma(-box.L[1], (double)rintf(py * (float)box.invL[1]), p.y),
+                    z = (float)fma(-box.L[2], (double)rintf(pz * (float)box.invL[2]), p.z);
         const int t = species[j];
         // a species outside the model is reported and the host rejects the whole call
         if (t < 0 || t >= NS) atomicOr(status, ST_BAD_SPECIES);
-        fpos[j] = make_float4((float)x, (float)y, (float)z, __int_as_float(t & 1));
-        far = fmaxf(far, fmaxf(fmaxf((float)fabs(x), (float)fabs(y)), (float)fabs(z)));
+        fpos[j] = make_float4(x, y, z, __int_as_float(t & 1));
+        far = fmaxf(far, fmaxf(fmaxf(fabsf(x), fabsf(y)), fabsf(z)));
         // the exact test's own rounding, should a caller's coordinates span many boxes
-        far = fmaxf(far, 1e-8f * fmaxf(fmaxf((float)fabs(p.x), (float)fabs(p.y)), (float)fabs(p.z)));
+        far = fmaxf(far, 1e-8f * fmaxf(fmaxf(fabsf(px), fabsf(py)), fabsf(pz)));
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) far = fmaxf(far, __shfl_xor_sync(0xffffffffu, far, o));
