@@ -49,7 +49,8 @@ static int item_class(int k, int prec) {
     switch (k) {
         case FK_FIRST: return IC_FIRST;
         case FK_SECOND: return IC_SECOND;
-        case FK_SECONDW: return IC_GATHER;
+        case FK_SECONDW: return IC_GATHER4;
+        case FK_SECONDX: return IC_GATHER8;
         case FK_CRAD: return prec == 0 ? -1 : IC_ATOM;   // FP64: the wide kernel only
         case FK_CRADW: return IC_OCT;
         case FK_ANG: case FK_BWD: return IC_QUAD;
@@ -87,7 +88,7 @@ void FusedBatch::enqueue(cudaStream_t st) const {
     const Launch ev[7] = {L(FK_CRAD), L(FK_ANG), L(FK_NET), L(FK_BWD), L(FK_CRADW), L(FK_ANGW), L(FK_BWDW)};
     if (t.prec == 0) launch_eval_t<double>(t, pd, ev, st, nullptr, fork, fork2);
     else launch_eval_t<float>(t, pf, ev, st, nullptr, fork, fork2);
-    launch_second_half_t(t, L(FK_SECOND), L(FK_SECONDW), true, st, fork);
+    launch_second_half_t(t, L(FK_SECOND), L(FK_SECONDW), L(FK_SECONDX), true, st, fork, fork2);
 }
 
 namespace {
@@ -233,7 +234,8 @@ bool FusedBatch::same_model(const Sys &s) const {
 // network, k_mlp_tc, is persistent); -1 for the others.
 static int item_kernel_class(const char *name, int whole, int split, int &bit) {
     struct { const char *id; int cls, bit; } const k[] = {
-        {"k_first_half", IC_FIRST, -1}, {"k_second_half", IC_SECOND, FK_SECOND}, {"k_second_wide", IC_GATHER, FK_SECONDW},
+        {"k_first_half", IC_FIRST, -1}, {"k_second_half", IC_SECOND, FK_SECOND}, {"k_second_wide", IC_GATHER4, FK_SECONDW},
+        {"k_second_widest", IC_GATHER8, FK_SECONDX},
         {"k_crad", IC_ATOM, FK_CRAD}, {"k_crad_wide", IC_OCT, whole}, {"k_crad_rows", IC_OCT, split},
         {"k_crad_sums", IC_OCT, split}, {"k_mlp", IC_OCT, -1}, {"k_ang_fwd", IC_QUAD, FK_ANG}, {"k_bwd", IC_QUAD, FK_BWD},
         {"k_ang_wide", IC_WARP, FK_ANGW}, {"k_bwd_wide", IC_WARP, FK_BWDW}};
@@ -270,18 +272,19 @@ bool FusedBatch::find_item_nodes(cudaGraph_t graph, cudaGraphExec_t exec, int st
         item_nodes.push_back(ItemNode{exec, node, c, bit});
         ++found;
     }
-    // per step: the first half, four radial kernels (FP64: three, and the network), and two kernels each of
-    // the angular part, the backward and the second half
-    return found == (int64_t)steps * 11;
+    // per step: the first half, four radial kernels (FP64: three, and the network), two kernels each of the
+    // angular part and the backward, and three of the second half (FP64: two)
+    return found == (int64_t)steps * (t.prec == 0 ? 11 : 12);
 }
 
 int64_t FusedBatch::launches_per_step() const {
     int64_t n = fused_launches_per_step(t.prec);
     if (item_nodes.empty()) return n;
-    for (int k : {(int)FK_SECOND, (int)FK_SECONDW, (int)FK_ANG, (int)FK_ANGW, (int)FK_BWD, (int)FK_BWDW, BIT_WHOLE, BIT_SPLIT,
+    for (int k : {(int)FK_SECOND, (int)FK_SECONDX, (int)FK_ANG, (int)FK_ANGW, (int)FK_BWD, (int)FK_BWDW, BIT_WHOLE, BIT_SPLIT,
                   BIT_SPLIT})   // (the split form is two kernels)
         n -= !(taken >> k & 1u);
-    return n - (t.prec != 0 && !(taken >> FK_CRAD & 1u));
+    if (t.prec != 0) n -= !(taken >> FK_CRAD & 1u) + !(taken >> FK_SECONDW & 1u);
+    return n;
 }
 
 void FusedBatch::switch_nodes() {
@@ -341,7 +344,7 @@ bool FusedBatch::reserve(int64_t atoms) {
     int64_t c = 1;
     while (c < atoms) c <<= 1;
     const int q = default_quad_block(t.prec);
-    const int64_t per[IC_N] = {256, 128, q / 4, CRAD_WIDE_ATOMS, q / 32, 256, second_wide_atoms(t.prec)};
+    const int64_t per[IC_N] = {256, 128, q / 4, CRAD_WIDE_ATOMS, q / 32, 256, 64, 32};
     int64_t cap_items[IC_N], total = 0;
     for (int k = 0; k < IC_N; ++k) {
         cap_items[k] = (c + per[k] - 1) / per[k] + t.cap;   // whole blocks, one partial block per slot
@@ -413,7 +416,7 @@ cudaError_t FusedBatch::upload(const int64_t *left, cudaStream_t st) {
     if (dirty || layout_dirty) {
         // block -> slot layout of the one-item-per-block kernels: every occupied slot's blocks in
         // slot order, then no slot (-1) up to the capacity
-        const int kof[IC_N] = {FK_FIRST, FK_CRAD, FK_ANG, FK_CRADW, FK_ANGW, FK_SECOND, FK_SECONDW};
+        const int kof[IC_N] = {FK_FIRST, FK_CRAD, FK_ANG, FK_CRADW, FK_ANGW, FK_SECOND, FK_SECONDW, FK_SECONDX};
         for (int c = 0; c < IC_N; ++c) {
             int *it = h_items + item_off[c];
             int64_t o = 0;
@@ -533,14 +536,14 @@ Launch solo_launch(const Sys &s, int k, int kind) {
     if (k == FK_FIRST) {
         L.block = half_block(s.n, so.sms, 32);
         g = (s.n + L.block - 1) / L.block;
-    } else if (k == FK_SECONDW && g > 0) {
-        const int64_t lanes = 256 / second_wide_atoms(s.prec);
+    } else if ((k == FK_SECONDW || k == FK_SECONDX) && g > 0) {
+        const int64_t lanes = k == FK_SECONDW ? 4 : 8;
         L.block = half_block(s.n * lanes, so.sms, 64);
         g = (s.n * lanes + L.block - 1) / L.block;
     }
     if (k == FK_NET && s.prec != 0) g = std::min<int64_t>(g, (int64_t)so.sms * s.cfg.mlp_ctas_per_sm);   // persistent
     // the radial, angular and backward kernels and the second half: one of each kind has blocks
-    L.grid = (unsigned)(k >= FK_CRAD && k <= FK_SECONDW && k != FK_NET ? g : std::max<int64_t>(g, 1));
+    L.grid = (unsigned)(k >= FK_CRAD && k <= FK_SECONDX && k != FK_NET ? g : std::max<int64_t>(g, 1));
     // the argument block of slot `kind` as the kernel parameter (all but the rebuild group)
     const FusedTables &t = so.t;
     size_t first = 0, second = 0;
@@ -548,7 +551,7 @@ Launch solo_launch(const Sys &s, int k, int kind) {
     const unsigned char *h = so.host.data();
     switch (k) {
         case FK_FIRST: L.solo = h + t.o_first + kind * first; break;
-        case FK_SECOND: case FK_SECONDW: L.solo = h + t.o_second + kind * second; break;
+        case FK_SECOND: case FK_SECONDW: case FK_SECONDX: L.solo = h + t.o_second + kind * second; break;
         case FK_CRAD: case FK_CRADW: case FK_ANG: case FK_ANGW: case FK_BWD: case FK_BWDW: L.solo = h + t.o_eval + kind * fused_eval_size(s.prec); break;
         case FK_NET: L.solo = h + t.o_net + kind * fused_net_size(s.prec); break;
         default:   // the rebuild group: a conditional one returns at once on the system's flag

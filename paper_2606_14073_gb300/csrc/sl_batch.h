@@ -23,17 +23,19 @@ namespace sl {
 // kernels of one step, in launch order
 enum FusedKernel {
     FK_FIRST, FK_BIN, FK_SCAN, FK_SCATTER, FK_CELLSORT, FK_LISTS, FK_REV, FK_FINISH,
-    FK_CRAD, FK_CRADW, FK_ANG, FK_ANGW, FK_NET, FK_BWD, FK_BWDW, FK_SECOND, FK_SECONDW,
+    FK_CRAD, FK_CRADW, FK_ANG, FK_ANGW, FK_NET, FK_BWD, FK_BWDW, FK_SECOND, FK_SECONDW, FK_SECONDX,
     FK_N
 };
-// plan, the kernels (FP64 has the wide radial kernel only; that is three, in both its forms), the flag clear
-inline int fused_launches_per_step(int prec) { return 1 + FK_N + 2 + 1 - (prec == 0); }
+// plan, the kernels (FP64 has no one-thread radial kernel and no four-lane second half; the wide radial
+// kernel is three, in both its forms), the flag clear
+inline int fused_launches_per_step(int prec) { return 1 + FK_N + 2 + 1 - (prec == 0 ? 2 : 0); }
 constexpr int FUSED_MAX_SLOTS = 4096;
 // atoms-per-block classes of the kernels that take one work item per block: the first half (256
 // atoms), the one-thread-per-atom radial kernel (128), the angular and backward kernels (a quad
 // block's atoms), the wide radial kernel and the FP64 network (8), the wide angular and backward
-// kernels (one per warp of a quad block), the second half (256) and its wide form
-enum { IC_FIRST = 0, IC_ATOM = 1, IC_QUAD = 2, IC_OCT = 3, IC_WARP = 4, IC_SECOND = 5, IC_GATHER = 6, IC_N = 7 };
+// kernels (one per warp of a quad block), the second half (256) and its forms with four (64) and eight lanes
+// per atom (32)
+enum { IC_FIRST = 0, IC_ATOM = 1, IC_QUAD = 2, IC_OCT = 3, IC_WARP = 4, IC_SECOND = 5, IC_GATHER4 = 6, IC_GATHER8 = 7, IC_N = 8 };
 
 // what a slot's entries are set up for
 enum SlotKind {
@@ -95,7 +97,6 @@ A solo_args(const Launch &L) {
     return a;
 }
 
-int64_t second_wide_atoms(int prec);   // atoms per block of the wide second half (sl_integrate.cu)
 // sizes of the per-slot argument blocks (sl_integrate.cu, sl_eval2.cu, sl_nep.cu)
 void fused_half_sizes(int prec, size_t *first, size_t *second);
 size_t fused_eval_size(int prec);
@@ -137,8 +138,8 @@ struct Fork {
     bool make();    // false on failure (then free())
     void free();
 };
-void launch_second_half_t(const FusedTables &t, const Launch &L, const Launch &W, bool spin, cudaStream_t st,
-                          const Fork &fork = Fork());
+void launch_second_half_t(const FusedTables &t, const Launch &L, const Launch &W, const Launch &X, bool spin,
+                          cudaStream_t st, const Fork &fork = Fork(), const Fork &fork2 = Fork());
 // the rebuild group: L[0 .. 5] for the binning, scan, scatter, lists, reverse slots and finish
 // kernels; clear: then the flags of the conditional slots in L[0]'s map are cleared; loop: the
 // persistent form (a batch's), else one work item per block (a system's own launches)

@@ -288,13 +288,21 @@ __global__ void __launch_bounds__(256) k_second_half(const HalfArgs<R> *__restri
         second_half_body<R, MIXED, 1, SPIN>(h.a, h.g, blk, scratch);
     });
 }
-// the same with several lanes per atom in the gather (gather_is_wide)
+// the same with four or eight lanes per atom in the gather (gather_lanes)
 template <typename R, bool MIXED, bool SPIN>
 __global__ void __launch_bounds__(256) k_second_wide(const HalfArgs<R> *__restrict__ tab, SlotMap sm,
                                                      const __grid_constant__ HalfArgs<R> solo) {
-    __shared__ GatherSmem<R, GATHER_WIDE<R>> scratch;
+    __shared__ GatherSmem<R, 4> scratch;
     one_work(tab, sm, solo, [&](const HalfArgs<R> &h, int64_t blk, int64_t) {
-        second_half_body<R, MIXED, GATHER_WIDE<R>, SPIN>(h.a, h.g, blk, scratch);
+        second_half_body<R, MIXED, 4, SPIN>(h.a, h.g, blk, scratch);
+    });
+}
+template <typename R, bool MIXED, bool SPIN>
+__global__ void __launch_bounds__(256) k_second_widest(const HalfArgs<R> *__restrict__ tab, SlotMap sm,
+                                                       const __grid_constant__ HalfArgs<R> solo) {
+    __shared__ GatherSmem<R, 8> scratch;
+    one_work(tab, sm, solo, [&](const HalfArgs<R> &h, int64_t blk, int64_t) {
+        second_half_body<R, MIXED, 8, SPIN>(h.a, h.g, blk, scratch);
     });
 }
 
@@ -410,46 +418,52 @@ void launch_first_half_t(const FusedTables &t, const Launch &L, cudaStream_t st)
     else k_first_half<true><<<L.grid, b, 0, st>>>(tab, L.slots(), so);
 }
 
-// L, W: the launches of the one-lane and the wide form (a grid of 0: not launched)
+// L, W, X: the launches with one, four (mixed precision only) and eight lanes (a grid of 0: not launched)
 template <typename R, bool MIXED>
-static void second_half_t(const FusedTables &t, const Launch &L, const Launch &W, bool spin, cudaStream_t st,
-                          const Fork &fork) {
+static void second_half_t(const FusedTables &t, const Launch &L, const Launch &W, const Launch &X, bool spin,
+                          cudaStream_t st, const Fork &fork, const Fork &fork2) {
     const HalfArgs<R> *tab = L.solo ? nullptr : t.at<HalfArgs<R>>(t.o_second);
     const HalfArgs<R> so = solo_args<HalfArgs<R>>(L);
-    const cudaStream_t side = fork.open(st);
+    const cudaStream_t side = fork.open(st), side2 = fork2.open(st);
     if (L.grid && spin) k_second_half<R, MIXED, true><<<L.grid, 256, 0, st>>>(tab, L.slots(), so);
     else if (L.grid) k_second_half<R, MIXED, false><<<L.grid, 256, 0, st>>>(tab, L.slots(), so);
-    const int b = W.block ? W.block : 256;
-    if (W.grid && spin) k_second_wide<R, MIXED, true><<<W.grid, b, 0, side>>>(tab, W.slots(), so);
-    else if (W.grid) k_second_wide<R, MIXED, false><<<W.grid, b, 0, side>>>(tab, W.slots(), so);
+    const int b = W.block ? W.block : 256, x = X.block ? X.block : 256;
+    if constexpr (MIXED) {
+        if (W.grid && spin) k_second_wide<R, MIXED, true><<<W.grid, b, 0, side>>>(tab, W.slots(), so);
+        else if (W.grid) k_second_wide<R, MIXED, false><<<W.grid, b, 0, side>>>(tab, W.slots(), so);
+    }
+    if (X.grid && spin) k_second_widest<R, MIXED, true><<<X.grid, x, 0, side2>>>(tab, X.slots(), so);
+    else if (X.grid) k_second_widest<R, MIXED, false><<<X.grid, x, 0, side2>>>(tab, X.slots(), so);
+    fork2.close(st);
     fork.close(st);
 }
-void launch_second_half_t(const FusedTables &t, const Launch &L, const Launch &W, bool spin, cudaStream_t st,
-                          const Fork &fork) {
-    if (t.prec == 0) second_half_t<double, false>(t, L, W, spin, st, fork);
-    else second_half_t<float, true>(t, L, W, spin, st, fork);
+void launch_second_half_t(const FusedTables &t, const Launch &L, const Launch &W, const Launch &X, bool spin,
+                          cudaStream_t st, const Fork &fork, const Fork &fork2) {
+    if (t.prec == 0) second_half_t<double, false>(t, L, W, X, spin, st, fork, fork2);
+    else second_half_t<float, true>(t, L, W, X, spin, st, fork, fork2);
 }
 
 // a system's own launches, over its table
 void launch_first_half(Sys &s) { launch_first_half_t(s.solo->t, solo_launch(s, FK_FIRST, SK_STEP), s.stream); }
 void launch_second_half(Sys &s) {
-    launch_second_half_t(s.solo->t, solo_launch(s, FK_SECOND, SK_STEP), solo_launch(s, FK_SECONDW, SK_STEP), true,
-                         s.stream);
+    launch_second_half_t(s.solo->t, solo_launch(s, FK_SECOND, SK_STEP), solo_launch(s, FK_SECONDW, SK_STEP),
+                         solo_launch(s, FK_SECONDX, SK_STEP), true, s.stream);
 }
 template <typename R, bool MIXED>
 static void halves(Sys &s, unsigned long long ahead) {
-    const Launch L = solo_launch(s, FK_SECOND, SK_STEP), W = solo_launch(s, FK_SECONDW, SK_STEP);
+    const int lanes = gather_lanes(s);
+    const Launch L = solo_launch(s, lanes == 8 ? FK_SECONDX : lanes == 4 ? FK_SECONDW : FK_SECOND, SK_STEP);
     const HalfArgs<R> so = solo_args<HalfArgs<R>>(L);
-    if (L.grid) k_halves<R, MIXED, 1><<<L.grid, 256, 0, s.stream>>>(so, ahead);
-    if (W.grid) k_halves<R, MIXED, GATHER_WIDE<R>><<<W.grid, W.block, 0, s.stream>>>(so, ahead);
+    const int b = L.block ? L.block : 256;
+    with_gather_lanes<R>(s, [&](auto w) { k_halves<R, MIXED, decltype(w)::value><<<L.grid, b, 0, s.stream>>>(so, ahead); });
 }
 void launch_halves(Sys &s, int64_t ahead) {
     if (s.prec == 0) halves<double, false>(s, (unsigned long long)ahead);
     else halves<float, true>(s, (unsigned long long)ahead);
 }
 void launch_second_half_nospin(Sys &s) {
-    launch_second_half_t(s.solo->t, solo_launch(s, FK_SECOND, SK_STEP), solo_launch(s, FK_SECONDW, SK_STEP), false,
-                         s.stream);
+    launch_second_half_t(s.solo->t, solo_launch(s, FK_SECOND, SK_STEP), solo_launch(s, FK_SECONDW, SK_STEP),
+                         solo_launch(s, FK_SECONDX, SK_STEP), false, s.stream);
 }
 
 template <typename R, bool MIXED, int W>
@@ -458,9 +472,8 @@ static void sweep_rotate(Sys &s, int c) {
                                                                                  s.colour, c);
 }
 void launch_sweep_rotate(Sys &s, int c) {
-    const bool wide = gather_is_wide(s);
-    if (s.prec == 0) wide ? sweep_rotate<double, false, GATHER_WIDE<double>>(s, c) : sweep_rotate<double, false, 1>(s, c);
-    else wide ? sweep_rotate<float, true, GATHER_WIDE<float>>(s, c) : sweep_rotate<float, true, 1>(s, c);
+    if (s.prec == 0) with_gather_lanes<double>(s, [&](auto w) { sweep_rotate<double, false, decltype(w)::value>(s, c); });
+    else with_gather_lanes<float>(s, [&](auto w) { sweep_rotate<float, true, decltype(w)::value>(s, c); });
 }
 
 template <typename R, int W>
@@ -470,9 +483,8 @@ static void gather_only(Sys &s, double4 *Fo, double4 *Ho) {
 }
 void launch_gather(Sys &s, bool carried) {
     double4 *Fo = carried ? s.F : s.Fo, *Ho = carried ? s.H : s.Ho;
-    const bool wide = gather_is_wide(s);
-    if (s.prec == 0) wide ? gather_only<double, GATHER_WIDE<double>>(s, Fo, Ho) : gather_only<double, 1>(s, Fo, Ho);
-    else wide ? gather_only<float, GATHER_WIDE<float>>(s, Fo, Ho) : gather_only<float, 1>(s, Fo, Ho);
+    if (s.prec == 0) with_gather_lanes<double>(s, [&](auto w) { gather_only<double, decltype(w)::value>(s, Fo, Ho); });
+    else with_gather_lanes<float>(s, [&](auto w) { gather_only<float, decltype(w)::value>(s, Fo, Ho); });
 }
 
 // Sets *diff when the evaluation outputs (Fo, Ho) differ in any bit from ref ([n] forces,
@@ -492,7 +504,6 @@ __global__ void k_compare_bits(const double4 *__restrict__ Fo, const double4 *__
 }
 
 // ---- fused batch step (sl_batch.h)
-int64_t second_wide_atoms(int prec) { return gather_atoms(prec == 0 ? GATHER_WIDE<double> : GATHER_WIDE<float>); }
 void fused_half_sizes(int prec, size_t *first, size_t *second) {
     *first = sizeof(IntArgs);
     *second = prec == 0 ? sizeof(HalfArgs<double>) : sizeof(HalfArgs<float>);
@@ -505,8 +516,9 @@ void fused_put_half(Sys &s, int r, const FusedTables &t, unsigned char *img, int
     if (s.prec == 0) reinterpret_cast<HalfArgs<double> *>(img + t.o_second)[r] = HalfArgs<double>{a, gather_args<double>(s)};
     else reinterpret_cast<HalfArgs<float> *>(img + t.o_second)[r] = HalfArgs<float>{a, gather_args<float>(s)};
     blocks[FK_FIRST] = nblk(s.n, 256);
-    blocks[FK_SECOND] = gather_is_wide(s) ? 0 : nblk(s.n, gather_atoms(1));
-    blocks[FK_SECONDW] = gather_is_wide(s) ? nblk(s.n, second_wide_atoms(s.prec)) : 0;
+    const int lanes = gather_lanes(s);
+    blocks[FK_SECOND] = blocks[FK_SECONDW] = blocks[FK_SECONDX] = 0;
+    blocks[lanes == 8 ? FK_SECONDX : lanes == 4 ? FK_SECONDW : FK_SECOND] = nblk(s.n, gather_atoms(lanes));
 }
 
 void launch_compare_bits(Sys &s, const double4 *ref, int *diff) {

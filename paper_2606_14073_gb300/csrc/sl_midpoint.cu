@@ -336,7 +336,6 @@ int launch_midpoint(Sys &s) {
     if (s.mid_iters <= 0 || s.n == 0) return 0;
     const MidArgs a = mid_args(s);
     const unsigned nb = nblk(s.n, 256);
-    const bool wide = gather_is_wide(s);
     k_mid_start<<<1, 64, 0, s.stream>>>(s.md, s.mid_iters);
     EvalAt at;
     at.pos = s.posmid; at.spin = s.mids; at.posf = s.midposf; at.psf = s.midpsf;
@@ -346,8 +345,8 @@ int launch_midpoint(Sys &s) {
         s.at = at;
         launch_eval(s, false);
         s.at = EvalAt();
-        if (s.prec == 0) wide ? mid_update<double, false, GATHER_WIDE<double>>(s, a, m) : mid_update<double, false, 1>(s, a, m);
-        else wide ? mid_update<float, true, GATHER_WIDE<float>>(s, a, m) : mid_update<float, true, 1>(s, a, m);
+        if (s.prec == 0) with_gather_lanes<double>(s, [&](auto w) { mid_update<double, false, decltype(w)::value>(s, a, m); });
+        else with_gather_lanes<float>(s, [&](auto w) { mid_update<float, true, decltype(w)::value>(s, a, m); });
         if (s.aa_depth > 0) {
             k_aa_dots<<<AA_BLOCKS, 256, 0, s.stream>>>(a, m);
             k_aa_solve<<<1, 64, 0, s.stream>>>(a, m);

@@ -4,6 +4,8 @@
 // atomics-free force/field gather over an atom's own pair records.
 #pragma once
 
+#include <type_traits>
+
 #include "sl_common.cuh"
 #include "sl_eval2.cuh"
 #include "sl_internal.h"
@@ -74,14 +76,20 @@ __device__ __forceinline__ void rotate_delta_f(float sx, float sy, float sz, flo
 // (2.3 GB in 470 us at 884,736 atoms), and elsewhere the chain of a lane's slots, a few loads in flight
 // at a time: so eight slots' records are loaded together, without branches (FP64 at 32,768 atoms 92 instead
 // of 120 us a second half, FP32 at 110,592 83 instead of 85), and a
-// small system (gather_is_wide) takes several lanes per atom, a larger one one.  Second half, mixed
-// precision, 512 / 13,824 / 32,768 / 64,000 / 110,592 atoms: 17 / 21 / 32 / 59 / 89 us with four lanes, 27 / 31 /
-// 43 / 59 / 83 with one; FP64, 512 / 13,824 / 21,952 / 32,768 atoms: 27 / 49 / 77 / 114 us with eight, 83 / 87 /
-// 88 / 92 with one.
-template <typename R>
-constexpr int GATHER_WIDE = sizeof(R) == 4 ? 4 : 8;
+// small system (gather_lanes) takes several lanes per atom, a larger one one.  Second half, mixed
+// precision, 512 / 13,824 / 32,768 / 64,000 / 110,592 atoms: 15 / 19 / 37 us at the first three with eight lanes, 17 /
+// 21 / 32 / 59 / 89 with four, 27 / 31 / 43 / 59 / 83 with one; FP64, 512 / 13,824 / 21,952 / 32,768 atoms: 27 / 49 / 77 / 114 us with
+// eight, 83 / 87 / 88 / 92 with one.
 constexpr int gather_atoms(int W) { return 256 / W; }   // atoms per 256-thread block
-inline bool gather_is_wide(const Sys &s) { return s.n <= (s.prec == 0 ? 16384 : 65536); }
+inline int gather_lanes(const Sys &s) { return s.n <= 16384 ? 8 : s.prec != 0 && s.n <= 65536 ? 4 : 1; }
+// launch(W) with the system's W (R: its precision) as a constant
+template <typename R, typename F>
+inline void with_gather_lanes(const Sys &s, F launch) {
+    const int w = gather_lanes(s);
+    if (w == 8) launch(std::integral_constant<int, 8>());
+    else if (w == 1) launch(std::integral_constant<int, 1>());
+    else if constexpr (sizeof(R) == 4) launch(std::integral_constant<int, 4>());
+}
 
 template <typename R, int W>
 struct GatherSmem {

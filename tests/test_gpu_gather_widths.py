@@ -28,3 +28,9 @@ def test_gathered_forces(prec, n):
         assert np.abs(a - b).max() <= 10.0 * eps * 140.0
     # every pair's two contributions cancel: what is left is that rounding, over the atoms as a walk
     assert np.abs(r["F"].sum(0)).max() <= 10.0 * eps * 140.0 * np.sqrt(n) * 4.0
+
+
+@pytest.mark.parametrize("n", [7, 16384, 16385])
+def test_gathered_forces_eight_and_four_lanes(n):
+    """Mixed precision at the line between eight and four lanes: as above."""
+    test_gathered_forces(S.SL_PREC_MIXED, n)
