@@ -637,9 +637,11 @@ __device__ __forceinline__ int crad_rows(const NepDev<R> &P, const Eval2Args<R> 
         }
         const unsigned hi = (__ballot_sync(0xffffffffu, in) >> half) & 0xffffu;
         if (in) {
-            const int c = m + __popc(hi & lt);
-            if (list) list[c] = j;
-            stg(a.crow + (int64_t)(ang ? ra : a.cap_ang + (c - ra)) * N + i, make_int2(j, rrow[v]));
+            if (list) list[m + __popc(hi & lt)] = j;
+            // radial-only pairs are numbered on their own (those kept so far: m - na; of these sixteen: hi
+            // without the angular ones), so a refused angular pair leaves no gap in their rows
+            const int row = ang ? ra : a.cap_ang + (m - na) + __popc(hi & ~ha & lt);
+            stg(a.crow + (int64_t)row * N + i, make_int2(j, rrow[v]));
         }
         word = base & 16 ? word | hi << 16 : hi;
         if (lane == 0) sm.mask[base >> 5][slot8] = word;
