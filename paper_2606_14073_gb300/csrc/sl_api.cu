@@ -759,6 +759,9 @@ int sl_create_system(const double *positions, const double *spins, const double 
             (ce = cudaMemcpyAsync(s.inv, inv.data(), sizeof(int32_t) * N, cudaMemcpyHostToDevice, st)) ||
             (ce = cudaMemsetAsync(s.cells.count, 0, sizeof(int) * s.cells.ncell, st)) ||
             (ce = cudaMemsetAsync(s.cells.fill, 0, sizeof(int) * s.cells.ncell, st)) ||
+            // reverse slots are slots of a list from the start: of a pair that a cut list holds on one side only,
+            // the build may leave the entry as it was, and the evaluation addresses its record by it
+            (ce = cudaMemsetAsync(s.rev, 0, N * sl::nbr_stride(s.cap), st)) ||
             (ce = cudaMemsetAsync(s.status, 0, sizeof(int), st)) || (ce = cudaMemsetAsync(s.rebuild, 0, sizeof(int), st)) ||
             (ce = cudaMemsetAsync(s.d_step, 0, 2 * sizeof(unsigned long long), st)) ||
             (ce = cudaMemsetAsync(s.d_builds, 0, sizeof(unsigned long long), st)) ||

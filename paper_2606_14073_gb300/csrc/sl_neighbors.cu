@@ -659,8 +659,9 @@ struct RevSmem {
 // rev[i][s] = t and rev[j][t] = s (the entries with j < i are written by j's warp): one search
 // per unordered pair.  The lists are symmetric and so is each pair's segment kind (the cutoff
 // test gives the same result for (i, j) and (j, i)), so i sits in the segment of j's list for
-// (kind of slot s, species of i).  A pair found in one list only (a list cut at its capacity)
-// raises the overflow status.
+// (kind of slot s, species of i).  A pair found in one list only (a list cut at its capacity, which
+// the list build has reported) raises the overflow status, or, where it is the lower-indexed atom's list
+// that lacks it, leaves the other's entry as it was: zero or a slot of an earlier build.
 __device__ __forceinline__ void rev_body(const RevArgs &args, int64_t blk, int64_t nblk, RevSmem &sm) {
     const RevArgs a = args;   // as values: the stores below cannot make the compiler re-read them
     if (a.flag && *a.flag == 0) return;
