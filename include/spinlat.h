@@ -126,7 +126,7 @@ int sl_create_system(const double *positions, const double *spins, const double 
  *   corrector S = Rot(S, (omega(S, H + eta) + omega(S', H' + eta)) dt/2), renormalised;
  *   v += dt/2 F'/m;  (F, H) = (F', H').
  * omega(S, X) = (X + lambda S x X) / ((1 + lambda^2) hbar), eta the thermal field.
- * On SL_ENBR_OVERFLOW or SL_ENONFINITE the state is restored to that at entry. */
+ * On SL_ENBR_OVERFLOW, SL_ENONFINITE or SL_ETIMEOUT the state is restored to that at entry. */
 int sl_step(sl_system *sys, int64_t n_steps, double dt_fs, double T_K, const double B_tesla[3]);
 
 /* Evaluate the potential at the current (positions, spins) with the field of the
@@ -318,8 +318,8 @@ int sl_batch_create(sl_system *const *systems, int32_t k, sl_batch **out);
  * mode other than the occupied slots', or a system that already holds another slot. */
 int sl_batch_set(sl_batch *b, int32_t slot, sl_system *sys);
 /* n_steps[k]: steps each slot's replica takes in this call (0 = idle; must be 0 for an empty
- * slot); dt/T/B per slot.  Returns after every replica's steps are done; on a list overflow or a
- * non-finite value the failing replicas go back to their state before the call, the others
+ * slot); dt/T/B per slot.  Returns after every replica's steps are done; on a list overflow, a
+ * non-finite value or a timeout the failing replicas go back to their state before the call, the others
  * keep their steps, and the first error is returned. */
 int sl_batch_step(sl_batch *b, const int64_t *n_steps, const double *dt_fs, const double *T_K,
                   const double *B_tesla /* [k][3] */);
@@ -397,6 +397,13 @@ int sl_selftest_carrier(int32_t n_samples, double rc, double *max_rel_err_f, dou
  * outcome, the device and context stay usable), SL_OK if the wait completed, SL_EINVAL for
  * max_polls outside [1, 2^22], SL_ECUDA without a device. */
 int sl_selftest_bounded_wait(int32_t max_polls);
+
+/* Device self-test of a list build whose waits give up: a build of the system that waits no time at
+ * its first barrier, and behind it on the stream one that must not start on what the first
+ * leaves.  Returns SL_ETIMEOUT (the expected outcome; the system stays usable and makes its lists
+ * anew before it uses them), SL_EINVAL for a system whose build has no such wait (more than
+ * 131,072 atoms, or none), SL_OK if nothing gave up. */
+int sl_selftest_rebuild_wait(sl_system *sys);
 
 #ifdef __cplusplus
 }

@@ -244,16 +244,26 @@ int check_status(sl::Sys &s) {
     CK(cudaMemcpyAsync(s.h_status, s.status, sizeof(int), cudaMemcpyDeviceToHost, s.stream));
     CK(cudaStreamSynchronize(s.stream));
     const int st = *s.h_status;
+    // before the others: what a build that gave up leaves may raise those, too
+    if (st & sl::ST_TIMEOUT) {
+        CK(sl::reset_rebuild_one(s));
+        return fail(SL_ETIMEOUT, "a bounded device wait gave up (tensor-core network or list rebuild)");
+    }
     if (st & sl::ST_NBR_OVERFLOW)
         return fail(SL_ENBR_OVERFLOW, "neighbour list capacity exceeded (caps %d/%d)", s.cap, s.cap_ang);
     if (st & sl::ST_NONFINITE) return fail(SL_ENONFINITE, "non-finite force or field");
-    if (st & sl::ST_TIMEOUT) {
-        if (s.rb_count) CK(cudaMemsetAsync(s.rb_count, 0, sizeof(unsigned long long), s.stream));
-        return fail(SL_ETIMEOUT, "a bounded device wait gave up (tensor-core network or list rebuild)");
-    }
     if (st & sl::ST_MID_RANGE)
         return fail(SL_ENBR_OVERFLOW, "midpoint configuration moved beyond skin/2 of the list positions");
     return SL_OK;
+}
+
+// The lists made anew at the state's positions after a build that gave up.
+int fresh_lists(sl::Sys &s) {
+    if (!s.lists_due || s.n == 0) return SL_OK;
+    s.lists_due = false;   // (check_status sets it again if this one gives up, too)
+    CK(cudaMemsetAsync(s.status, 0, sizeof(int), s.stream));
+    sl::launch_rebuild(s, false);
+    return check_status(s);
 }
 
 // fn(lo, hi) over [0, n) in contiguous chunks on up to 8 host threads (one thread for small n);
@@ -762,6 +772,8 @@ int sl_create_system(const double *positions, const double *spins, const double 
             // reverse slots are slots of a list from the start: of a pair that a cut list holds on one side only,
             // the build may leave the entry as it was, and the evaluation addresses its record by it
             (ce = cudaMemsetAsync(s.rev, 0, N * sl::nbr_stride(s.cap), st)) ||
+            // and no atom has a candidate before the first build, should that give up
+            (ce = cudaMemsetAsync(s.seg, 0, sizeof(int4) * N, st)) ||
             (ce = cudaMemsetAsync(s.status, 0, sizeof(int), st)) || (ce = cudaMemsetAsync(s.rebuild, 0, sizeof(int), st)) ||
             (ce = cudaMemsetAsync(s.d_step, 0, 2 * sizeof(unsigned long long), st)) ||
             (ce = cudaMemsetAsync(s.d_builds, 0, sizeof(unsigned long long), st)) ||
@@ -778,7 +790,7 @@ int sl_create_system(const double *positions, const double *spins, const double 
 }
 
 // State at the start of a stepping call, kept on the device so that a call that ends in
-// a list overflow or a non-finite value leaves the system as it was before the call.
+// a list overflow, a non-finite value or a timeout leaves the system as it was before the call.
 static int snapshot_state(sl::Sys &s) {
     const size_t N = (size_t)s.n;
     CK(cudaMemcpyAsync(s.snap, s.pos, sizeof(double4) * N, cudaMemcpyDeviceToDevice, s.stream));
@@ -802,9 +814,10 @@ static int restore_state(sl::Sys &s) {
     CK(cudaMemsetAsync(s.status, 0, sizeof(int), s.stream));
     int r2;
     if ((r2 = refresh_copies(s))) return r2;
+    s.lists_due = false;
     sl::launch_rebuild(s, false);
-    CK(cudaStreamSynchronize(s.stream));
-    return SL_OK;
+    r2 = check_status(s);
+    return r2 == SL_ETIMEOUT || r2 == SL_ECUDA ? r2 : SL_OK;
 }
 
 // ------------------------------------------------------------------ coloured spin sweep
@@ -948,11 +961,11 @@ static int queue_steps(sl::Sys &s, int64_t n_steps) {
     return SL_OK;
 }
 
-// Status of the queued steps; on a list overflow or a non-finite value the state goes
+// Status of the queued steps; on a list overflow, a non-finite value or a timeout the state goes
 // back to the snapshot and the error names the step it was restored to.
 static int finish_steps(sl::Sys &s, int64_t n_steps, const char *who) {
     const int rc = check_status(s);
-    if (rc == SL_ENBR_OVERFLOW || rc == SL_ENONFINITE) {
+    if (rc == SL_ENBR_OVERFLOW || rc == SL_ENONFINITE || rc == SL_ETIMEOUT) {
         const std::string msg = g_err;
         int r2;
         if ((r2 = restore_state(s))) return r2;
@@ -977,7 +990,7 @@ int sl_step(sl_system *sys, int64_t n_steps, double dt, double T, const double B
         s.step += (uint64_t)n_steps;
         return SL_OK;
     }
-    if ((rc = snapshot_state(s))) return rc;
+    if ((rc = fresh_lists(s)) || (rc = snapshot_state(s))) return rc;
     if (s.sts) {
         for (int64_t t = 0; t < n_steps; ++t)
             if ((rc = sweep_step(s))) return rc;
@@ -998,6 +1011,7 @@ int sl_energy_forces_fields(sl_system *sys, double *energy, double *forces, doub
         return SL_OK;
     }
     int rc;
+    if ((rc = fresh_lists(s))) return rc;
     CK(cudaMemsetAsync(s.status, 0, sizeof(int), s.stream));
     if ((rc = evaluate(s, false, false, virial != nullptr))) return rc;
     if ((rc = check_status(s))) return rc;
@@ -1014,6 +1028,7 @@ int sl_get_descriptors(sl_system *sys, double *q, double *atom_energy) {
     cudaSetDevice(s.device);
     if (s.n == 0) return SL_OK;
     int rc;
+    if ((rc = fresh_lists(s))) return rc;
     sl::launch_eval(s, false, nullptr, true);   // descriptors and network only
     CK(cudaGetLastError());
     const size_t N = (size_t)s.n, bq = sizeof(double) * sl::DIM * N, be = sizeof(double) * N;
@@ -1076,6 +1091,7 @@ int sl_set_state(sl_system *sys, const double *pos, const double *vel, const dou
         // lists from the reference positions (k_finish records them as the new reference)
         if ((rc = upload_vec(s, s.pos, ref ? ref : pos, false)) || (rc = refresh_copies(s))) return rc;
         CK(cudaMemsetAsync(s.status, 0, sizeof(int), s.stream));
+        s.lists_due = false;
         sl::launch_rebuild(s, false);
         s.n_builds++;
         if (ref && ((rc = upload_vec(s, s.pos, pos, false)) || (rc = refresh_copies(s)))) return rc;
@@ -1102,6 +1118,7 @@ int sl_get_neighbors(sl_system *sys, int32_t cap, int32_t *counts_rad, int32_t *
     cudaSetDevice(s.device);
     if (s.n == 0) return SL_OK;
     CK(cudaMemsetAsync(s.status, 0, sizeof(int), s.stream));
+    s.lists_due = false;
     sl::launch_rebuild(s, false);
     s.n_builds++;
     int rc = check_status(s);
@@ -1175,6 +1192,8 @@ int sl_autotune(sl_system *sys, int32_t repeats, int32_t *chosen, double *eval_m
         if (eval_ms_after) *eval_ms_after = 0.0;
         return SL_OK;
     }
+    int rc;
+    if ((rc = fresh_lists(s))) return rc;
     // evaluation kernel groups timed by launch_eval's events: 1 radial (with compaction),
     // 2 angular forward, 3 network, 4 backward
     auto time_cfg = [&](const sl::LaunchCfg &c, double ms[5]) -> int {
@@ -1212,7 +1231,6 @@ int sl_autotune(sl_system *sys, int32_t repeats, int32_t *chosen, double *eval_m
         cand[c].bwd_minb = var ? 3 : 0;
     }
     double ms0[5], msc[4][5];
-    int rc;
     // the shapes must not change any result: the forces and fields gathered after each
     // candidate's evaluations are compared bit for bit with those of the starting shape
     double4 *ref = nullptr;
@@ -1376,6 +1394,7 @@ int sl_set_longitudinal(sl_system *sys, int32_t enable, double alpha, const doub
     int rc;
     if ((rc = upload_params(s, s.last_dt, s.last_T, s.B))) return rc;
     if (s.n == 0) return SL_OK;
+    if ((rc = fresh_lists(s))) return rc;
     CK(cudaMemsetAsync(s.status, 0, sizeof(int), s.stream));
     if (leaving) sl::launch_normalise_spins(s);
     // the carried forces and fields of the current state under the new energy
@@ -1452,6 +1471,7 @@ int sl_step_profiled(sl_system *sys, int64_t n_steps, double dt, double T, const
     if ((rc = upload_params(s, dt, T, B))) return rc;
     for (int c = 0; c < 3; ++c) s.B[c] = B[c];
     if (s.n == 0 || n_steps == 0) { s.step += (uint64_t)n_steps; return SL_OK; }
+    if ((rc = fresh_lists(s))) return rc;
     CK(cudaMemsetAsync(s.status, 0, sizeof(int), s.stream));
     // events per step: before first half, before rebuild, before each evaluation kernel (5), after the
     // last one, after second half, and after the rebuild (e[9]): in the midpoint mode the iteration
@@ -1722,7 +1742,7 @@ int sl_batch_submit(sl_batch *b, const int64_t *n_steps, const double *dt, const
         if ((rc = upload_params(s, dt[i], T[i], B + 3 * i))) return rc;
         for (int c = 0; c < 3; ++c) s.B[c] = B[3 * i + c];
         if (n_steps[i] == 0 || s.n == 0) { s.step += (uint64_t)n_steps[i]; continue; }
-        if ((rc = snapshot_state(s))) return rc;
+        if ((rc = fresh_lists(s)) || (rc = snapshot_state(s))) return rc;
         active.push_back(i);
     }
     if (active.empty()) return SL_OK;
@@ -1863,6 +1883,18 @@ int sl_selftest_bounded_wait(int32_t max_polls) {
     if (sl::selftest_bounded_wait(max_polls, &st)) return fail(SL_ECUDA, "bounded-wait self-test failed to run");
     if (st & sl::ST_TIMEOUT) return fail(SL_ETIMEOUT, "a bounded device wait gave up (self-test)");
     return SL_OK;
+}
+
+int sl_selftest_rebuild_wait(sl_system *sys) {
+    if (!sys) return fail(SL_EINVAL, "NULL system");
+    sl::Sys &s = sys->s;
+    cudaSetDevice(s.device);
+    if (!s.rb_count) return fail(SL_EINVAL, "this system's list build is no single launch and waits for nothing");
+    CK(cudaMemsetAsync(s.status, 0, sizeof(int), s.stream));
+    sl::launch_rebuild(s, false, 0);
+    sl::launch_rebuild(s, false);   // as the next step of a queue would: on what the first one leaves
+    CK(cudaGetLastError());
+    return check_status(s);
 }
 
 int sl_selftest_harmonics(int32_t n_samples, double *max_add, double *max_grad) {

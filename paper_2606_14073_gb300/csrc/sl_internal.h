@@ -139,9 +139,11 @@ struct Sys {
     void *wpart = nullptr;     // [9][n] per-atom virial parts
     double4 *Fo = nullptr, *Ho = nullptr;   // evaluation outputs (not the carried F, H)
 
-    // the one-launch rebuild (sl_neighbors.cu; null: the kernels one by one): its barrier's count, its grid
+    // the one-launch rebuild (sl_neighbors.cu; null: the kernels one by one): its barrier's count and the word
+    // that a wait has given up, its grid
     unsigned long long *rb_count = nullptr;
     int rb_grid = 0;
+    bool lists_due = false;    // a build gave up: the lists are made anew before their next use
 
     // control
     int *status = nullptr;     // device status bits
@@ -239,9 +241,11 @@ constexpr int64_t EVAL_WIDE_MAX64 = 3040, EVAL_WIDE_MAX32 = 2048;
 inline bool eval_is_wide(const Sys &s) { return s.n <= (s.prec == 0 ? EVAL_WIDE_MAX64 : EVAL_WIDE_MAX32); }
 // The largest system whose own rebuilds take one launch (both timed at k_rebuild_one).
 constexpr int64_t REBUILD_ONE_MAX = 131072;
+constexpr int REBUILD_POLLS = 1 << 22;   // of a wait at its barrier, some seconds
 int make_rebuild_one(Sys &s);
+cudaError_t reset_rebuild_one(Sys &s);   // after a build that gave up; null count: nothing to do
 void nbr_setup(Sys &s);
-void launch_rebuild(Sys &s, bool conditional);
+void launch_rebuild(Sys &s, bool conditional, int polls = REBUILD_POLLS);
 // sl_eval2.cu: the system's evaluation at the state (with the virial parts when asked for), or
 // at the midpoint point while s.at is set; ev (optional, 6 events): recorded before the
 // radial kernel, after it, after the angular kernel, the network and the backward; forward_only:

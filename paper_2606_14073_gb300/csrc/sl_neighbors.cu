@@ -807,14 +807,15 @@ constexpr int ONE_THREADS = 128;
 static_assert(ONE_THREADS == LB_WARPS * 32 && ONE_THREADS == REV_WARPS * 32, "one block shape for every phase");
 
 // Every block of the grid has arrived (thread 0 of each counts it; the count starts at a multiple
-// of the grid).  False when the wait gave up.
-__device__ __forceinline__ bool grid_barrier(unsigned long long *count, int *s_ok) {
+// of the grid).  False when the wait gave up: then no later barrier of the launch is passed by any
+// block, because a block that gave up arrives at none.
+__device__ __forceinline__ bool grid_barrier(unsigned long long *count, int polls, int *s_ok) {
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
         const unsigned long long t = atomicAdd(count, 1ull), target = (t / gridDim.x + 1ull) * gridDim.x;
         int ok = 0;
-        for (int it = 0; it < (1 << 22) && !ok; ++it) {
+        for (int it = 0; it < polls && !ok; ++it) {
             unsigned long long v;
             asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(count) : "memory");
             ok = v >= target;
@@ -826,8 +827,11 @@ __device__ __forceinline__ bool grid_barrier(unsigned long long *count, int *s_o
     return *s_ok != 0;
 }
 
+// sync: the barrier's count, and whether a wait has given up.  What such a launch leaves (a count that is no
+// multiple of the grid, cells counted or filled in part) must not be built on: until the host has put it back
+// (reset_rebuild_one) later launches of the queue report the timeout again and do nothing.
 __global__ void __launch_bounds__(ONE_THREADS, LISTS_MINB) k_rebuild_one(const __grid_constant__ RebuildArgs A,
-                                                                         unsigned long long *count) {
+                                                                         unsigned long long *sync, int polls) {
     __shared__ union {
         ListSmem lists;
         RevSmem rev;
@@ -835,10 +839,15 @@ __global__ void __launch_bounds__(ONE_THREADS, LISTS_MINB) k_rebuild_one(const _
     } sm;
     __shared__ int s_ok;
     const BinArgs &r = A.bin;
-    if (A.flag && *A.flag == 0) return;   // the flag is cleared below, after a barrier: every block has read it
+    const bool gave_up = sync[1] != 0ull, due = !A.flag || *A.flag != 0;
+    if (gave_up) {
+        if (threadIdx.x == 0) atomicOr(A.lists.status, ST_TIMEOUT);
+        return;
+    }
+    if (!due) return;   // the flag is cleared below, after a barrier: every block has read it
     const int64_t b = blockIdx.x, nb = gridDim.x;
     bool ok = true;
-    auto meet = [&]() { ok = ok && grid_barrier(count, &s_ok); };
+    auto meet = [&]() { ok = ok && grid_barrier(sync, polls, &s_ok); };
     bin_body(r, b, nb);
     meet();
     if (ok && b == 0) scan_body(r, sm.scan);
@@ -850,7 +859,10 @@ __global__ void __launch_bounds__(ONE_THREADS, LISTS_MINB) k_rebuild_one(const _
     if (ok) lists_body(A.lists, b, nb, sm.lists);
     meet();
     if (!ok) {
-        if (threadIdx.x == 0) atomicOr(A.lists.status, ST_TIMEOUT);
+        if (threadIdx.x == 0) {
+            atomicOr(A.lists.status, ST_TIMEOUT);
+            atomicExch(sync + 1, 1ull);
+        }
         return;
     }
     rev_body(A.rev, b, nb, sm.rev);
@@ -947,7 +959,7 @@ RebuildPlan rebuild_plan(Sys &s, bool conditional) {
     return pl;
 }
 
-// Whether the system's own rebuilds take the one-launch form: its barrier count (device, zero) and
+// Whether the system's own rebuilds take the one-launch form: its barrier's words (device, zero) and
 // its grid, a block for each item of the list build as far as they fit on the GPU at once.  0 on
 // success.
 int make_rebuild_one(Sys &s) {
@@ -959,18 +971,30 @@ int make_rebuild_one(Sys &s) {
         cudaGetLastError();
         return 0;
     }
-    if (cudaMalloc(&s.rb_count, sizeof(unsigned long long)) != cudaSuccess) {
+    if (cudaMalloc(&s.rb_count, 2 * sizeof(unsigned long long)) != cudaSuccess) {
         s.rb_count = nullptr;
         return -1;
     }
     const RebuildPlan pl = rebuild_plan(s, false);
     s.rb_grid = (int)std::min<int64_t>((int64_t)sms * per, std::max<int64_t>(sms, pl.blocks[RB_LISTS]));
-    return cudaMemsetAsync(s.rb_count, 0, sizeof(unsigned long long), s.stream) == cudaSuccess ? 0 : -1;
+    return cudaMemsetAsync(s.rb_count, 0, 2 * sizeof(unsigned long long), s.stream) == cudaSuccess ? 0 : -1;
+}
+
+// What a one-launch build that gave up leaves, as a finished one leaves it; the lists are then made anew
+// before their next use.
+cudaError_t reset_rebuild_one(Sys &s) {
+    if (!s.rb_count) return cudaSuccess;
+    s.lists_due = true;
+    cudaError_t e = cudaMemsetAsync(s.cells.count, 0, sizeof(int) * s.cells.ncell, s.stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(s.cells.fill, 0, sizeof(int) * s.cells.ncell, s.stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(s.rb_count, 0, 2 * sizeof(unsigned long long), s.stream);
+    return e;
 }
 
 // The system's own rebuild group: conditional (a step's, on the flag the first half raised;
-// the flag is cleared afterwards) or unconditional.
-void launch_rebuild(Sys &s, bool conditional) {
+// the flag is cleared afterwards) or unconditional; polls: the limit of a wait at the one-launch
+// form's barrier.
+void launch_rebuild(Sys &s, bool conditional, int polls) {
     const int kind = conditional ? SK_STEP : SK_FULL;
     if (s.rb_count) {
         const FusedTables &t = s.solo->t;
@@ -990,7 +1014,7 @@ void launch_rebuild(Sys &s, bool conditional) {
         c.stream = s.stream;
         c.attrs = &attr;
         c.numAttrs = 1;
-        cudaLaunchKernelEx(&c, k_rebuild_one, A, s.rb_count);
+        cudaLaunchKernelEx(&c, k_rebuild_one, A, s.rb_count, polls);
         return;
     }
     Launch L[RB_KERNELS];

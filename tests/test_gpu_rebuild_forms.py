@@ -32,6 +32,40 @@ def test_lists_equal_the_oracle(shape, drop):
     assert builds >= 2
 
 
+@pytest.mark.parametrize("cells,prec,then", [(4, S.SL_PREC_FP64, "step"), (12, S.SL_PREC_MIXED, "step"),
+                                             (4, S.SL_PREC_MIXED, "energy"), (6, S.SL_PREC_MIXED, "batch"),
+                                             (6, S.SL_PREC_FP64, "set_state")])
+def test_a_build_that_gives_up(cells, prec, then):
+    """A wait of the one-launch build runs out: SL_ETIMEOUT, the build queued behind it does not start, and the
+    system then goes on, builds included, bit for bit as one to which nothing happened."""
+    make = lambda: S.system_from_workload(W.fege_cube(cells, T=300.0, seed=cells), nep_params.load(),  # noqa: E731
+                                          precision=prec, skin=0.1)
+    a, b = make(), make()
+    builds = b.info()["n_builds"]
+    assert S.lib().sl_selftest_rebuild_wait(b.handle) == S.SL_ETIMEOUT
+    assert b.info()["n_builds"] == builds
+    for s in (a, b):
+        if then == "energy":
+            s.energy_forces_fields()
+        elif then == "set_state":
+            st = s.get_state()
+            s.set_state(st["positions"], st["velocities"], st["spins"], st["forces"], st["fields"])
+        if then == "batch":
+            batch = S.Batch([s])
+            batch.step([25], [1.0], [300.0], [(0.0, 0.0, 0.0)])
+            batch.destroy()
+        else:
+            s.step(25, 1.0, 300.0)
+    assert a.info()["n_builds"] > builds + 1
+    p, q = a.get_state(), b.get_state()
+    for k in ("positions", "velocities", "spins", "forces", "fields"):
+        assert np.array_equal(p[k], q[k]), k
+    for x, y in zip(a.get_neighbors(), b.get_neighbors()):
+        assert all(np.array_equal(u, v) for u, v in zip(x, y))
+    a.destroy()
+    b.destroy()
+
+
 def test_builds_on_several_streams_at_once():
     """Systems stepped by a thread each, a build in nearly every step, so that several one-launch builds
     want the GPU at a time: every system as when it steps alone."""
