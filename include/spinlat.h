@@ -405,6 +405,11 @@ int sl_selftest_bounded_wait(int32_t max_polls);
  * 131,072 atoms, or none), SL_OK if nothing gave up. */
 int sl_selftest_rebuild_wait(sl_system *sys);
 
+/* Self-test of a batch's captured graphs: the next `failures` attempts to switch a kernel of them on
+ * (a replica that takes another form of a kernel joined) are treated as failed, after which the
+ * batch captures its graphs again.  SL_EINVAL for a negative number. */
+int sl_selftest_batch_switch(sl_batch *b, int32_t failures);
+
 #ifdef __cplusplus
 }
 #endif

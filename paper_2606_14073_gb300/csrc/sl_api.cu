@@ -1897,6 +1897,13 @@ int sl_selftest_rebuild_wait(sl_system *sys) {
     return check_status(s);
 }
 
+int sl_selftest_batch_switch(sl_batch *b, int32_t failures) {
+    if (!b) return fail(SL_EINVAL, "NULL batch");
+    if (failures < 0) return fail(SL_EINVAL, "failures must not be negative");
+    b->fused.refuse = failures;
+    return SL_OK;
+}
+
 int sl_selftest_harmonics(int32_t n_samples, double *max_add, double *max_grad) {
     using namespace sl;
     if (n_samples < 1) return fail(SL_EINVAL, "n_samples < 1");

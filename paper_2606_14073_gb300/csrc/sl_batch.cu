@@ -287,10 +287,16 @@ int64_t FusedBatch::launches_per_step() const {
     return n;
 }
 
-void FusedBatch::switch_nodes() {
-    for (const ItemNode &x : item_nodes)
-        if (x.bit >= 0 && cudaGraphNodeSetEnabled(x.exec, x.node, taken >> x.bit & 1u) != cudaSuccess)
-            cudaGetLastError();   // (stays as it is: without blocks of its own it returns at once)
+bool FusedBatch::switch_nodes(uint32_t before) {
+    for (const ItemNode &x : item_nodes) {
+        if (x.bit < 0 || !((before ^ taken) >> x.bit & 1u)) continue;
+        const unsigned on = taken >> x.bit & 1u;
+        const cudaError_t e = on && refuse > 0 && refuse-- ? cudaErrorUnknown : cudaGraphNodeSetEnabled(x.exec, x.node, on);
+        if (e == cudaSuccess) continue;
+        cudaGetLastError();
+        if (on) return false;   // (one that stays on returns at once: it has no blocks of its own)
+    }
+    return true;
 }
 
 bool FusedBatch::resize_item_nodes() {
@@ -333,7 +339,7 @@ bool FusedBatch::graphs(int steps, const Sys &m, cudaStream_t st) {
             return graphs(steps, m, st);
         }
     }
-    switch_nodes();
+    (void)switch_nodes(~0u);   // every node is on as captured, so whatever fails here stays on
     g = steps;
     ++captures;
     return true;
@@ -410,7 +416,7 @@ cudaError_t FusedBatch::upload(const int64_t *left, cudaStream_t st) {
             if (blocks[(size_t)k * t.cap + r] > 0) now |= 1u << k;
         if (crad_is_wide(*s)) now |= 1u << (crad_is_split(*s) ? BIT_SPLIT : BIT_WHOLE);
     }
-    const bool other = now != taken;
+    const uint32_t before = taken;
     taken = now;
     if (!reserve(atoms)) return cudaErrorMemoryAllocation;
     if (dirty || layout_dirty) {
@@ -439,7 +445,8 @@ cudaError_t FusedBatch::upload(const int64_t *left, cudaStream_t st) {
             release_graphs();
         }
     }
-    if (other && graph_g) switch_nodes();
+    // a kernel that a slot needs and that cannot be switched on: the graphs are captured again likewise
+    if (now != before && graph_g && !switch_nodes(before)) release_graphs();
     std::memcpy(img + t.o_left, left, sizeof(int64_t) * t.cap);
     if (dirty) e = cudaMemcpyAsync(t.dev, img, t.upload_bytes, cudaMemcpyHostToDevice, st);
     else e = cudaMemcpyAsync(t.dev + t.o_left, img + t.o_left, sizeof(int64_t) * t.cap, cudaMemcpyHostToDevice, st);

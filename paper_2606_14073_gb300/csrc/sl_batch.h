@@ -220,8 +220,9 @@ private:
     // are switched off in the executable graphs, an empty launch less each.
     static constexpr int BIT_WHOLE = FK_N, BIT_SPLIT = FK_N + 1;
     uint32_t taken = 0;
-    void switch_nodes();
+    bool switch_nodes(uint32_t before);   // before: the bits they were set by; false: a needed one could not be switched on
 public:
+    int refuse = 0;        // self-test: switchings-on still to fail
     int64_t launches_per_step() const;   // of the captured graphs, the kernels switched off not counted
 private:
     cudaGraph_t tmpl[2] = {};

@@ -28,8 +28,8 @@ EXPORTS = ["sl_default_options", "sl_create_system", "sl_step", "sl_energy_force
            "sl_estimate_device_bytes", "sl_get_midpoint_evaluations", "sl_set_atom_fields", "sl_texture_map",
            "sl_batch_graph_launches", "sl_batch_set", "sl_batch_stats", "sl_batch_reserve", "sl_batch_submit",
            "sl_batch_wait", "sl_autotune", "sl_set_longitudinal", "sl_selftest_carrier",
-           "sl_selftest_bounded_wait", "sl_selftest_rebuild_wait", "sl_set_spin_sweep", "sl_get_sweep_colours",
-           "sl_get_launch_config"]
+           "sl_selftest_bounded_wait", "sl_selftest_rebuild_wait", "sl_selftest_batch_switch", "sl_set_spin_sweep",
+           "sl_get_sweep_colours", "sl_get_launch_config"]
 KERNEL_GROUPS = ["first_half", "rebuild", "compact", "rad_fwd", "ang_fwd", "network", "backward", "second_half"]
 
 
@@ -82,6 +82,7 @@ def lib(path: str | None = None):
             L.sl_selftest_carrier.argtypes = [I32, D, P, P]
             L.sl_selftest_bounded_wait.argtypes = [I32]
             L.sl_selftest_rebuild_wait.argtypes = [P]
+            L.sl_selftest_batch_switch.argtypes = [P, I32]
             L.sl_set_spin_sweep.argtypes = [P, I32]
             L.sl_get_sweep_colours.argtypes = [P, P, P, P]
             L.sl_batch_graph_launches.argtypes = [P, P]
@@ -115,7 +116,7 @@ def lib(path: str | None = None):
                       "sl_texture_map", "sl_batch_graph_launches", "sl_batch_set", "sl_batch_stats", "sl_batch_reserve",
                       "sl_batch_submit", "sl_batch_wait", "sl_autotune", "sl_set_longitudinal",
                       "sl_selftest_carrier", "sl_selftest_bounded_wait", "sl_selftest_rebuild_wait",
-                      "sl_set_spin_sweep", "sl_get_sweep_colours", "sl_get_launch_config"):
+                      "sl_selftest_batch_switch", "sl_set_spin_sweep", "sl_get_sweep_colours", "sl_get_launch_config"):
                 getattr(L, f).restype = C.c_int
             _lib = L
         return _lib

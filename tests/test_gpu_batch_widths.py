@@ -27,3 +27,26 @@ def test_widths_side_by_side(prec, cells, skins):
         p, q = x.get_state(), y.get_state()
         for k in ("positions", "velocities", "spins", "forces", "fields"):
             assert np.array_equal(p[k], q[k]), k
+
+
+@pytest.mark.parametrize("prec,first,joins", [(S.SL_PREC_MIXED, 4, 13), (S.SL_PREC_FP64, 9, 4)])
+def test_a_kernel_that_cannot_be_switched_on(prec, first, joins):
+    """A replica that takes other forms of the kernels joins a batch whose graphs have those switched off; the
+    switching fails, and the batch captures its graphs again: both replicas step bit for bit as alone."""
+    make = lambda: [S.system_from_workload(W.fege_cube(c, T=300.0, seed=c), nep_params.load(), precision=prec,  # noqa: E731
+                                           seed=c, steps_per_graph=3) for c in (first, joins)]
+    alone, together = make(), make()
+    b = S.Batch([together[0], None])
+    zero = [(0.0, 0.0, 0.0)] * 2
+    for s, n in zip(alone, (10, 5)):
+        s.step(n, 1.0, 300.0)
+    b.step([5, 0], [1.0] * 2, [300.0] * 2, zero)
+    captures = b.stats()["fused_captures"]
+    b.set(1, together[1])
+    assert S.lib().sl_selftest_batch_switch(b.handle, 1) == S.SL_OK
+    b.step([5, 5], [1.0] * 2, [300.0] * 2, zero)
+    assert b.stats()["fused_captures"] == captures + 1
+    for x, y in zip(alone, together):
+        p, q = x.get_state(), y.get_state()
+        for k in ("positions", "velocities", "spins", "forces", "fields"):
+            assert np.array_equal(p[k], q[k]), k

@@ -110,6 +110,7 @@ def test_bounded_wait_selftest_argument_checks():
     assert S.lib().sl_selftest_bounded_wait(0) == S.SL_EINVAL
     assert S.lib().sl_selftest_bounded_wait(1 << 23) == S.SL_EINVAL
     assert S.lib().sl_selftest_rebuild_wait(None) == S.SL_EINVAL
+    assert S.lib().sl_selftest_batch_switch(None, 1) == S.SL_EINVAL
 
 
 def test_spin_sweep_entry_points_need_a_system():
