@@ -936,7 +936,7 @@ static int sweep_step(sl::Sys &s) {
     sl::launch_second_half_nospin(s);
     CK(cudaGetLastError());
     s.sweep_evaluations += 2 * C + 1;
-    s.n_launches += step_kernels(s) + (int64_t)2 * C * 5;
+    s.n_launches += step_kernels(s) + (int64_t)2 * C * (5 + sl::crad_is_split(s));   // an evaluation and the rotation
     return SL_OK;
 }
 

@@ -257,8 +257,9 @@ int make_coeff_table(Sys &s);                    // s.ctab from the model; 0 on 
 int make_q_tensor_map(Sys &s);                   // sl_mlp_tc.cu: the TMA map of s.q; 0 on success
 int make_net_table(Sys &s);                      // sl_nep.cu: the FP64 network's weights; 0 on success
 int make_mlp_image(Sys &s);                      // sl_mlp_tc.cu: s.mlp_img from s.pf; 0 on success
-// first half, rebuild group (7), compaction with radial forward, angular forward, network, backward,
-// second half
+// first half, rebuild group (7) and the clearing of its flag, compaction with radial forward, angular forward,
+// network, backward, second half; less or more in the one-launch rebuild's and the split radial kernel's
+// systems (step_kernels)
 constexpr int KERNELS_PER_STEP = 1 + 8 + 2 + 1 + 1 + 1;
 // sl_integrate.cu
 void launch_first_half(Sys &s);

@@ -84,3 +84,16 @@ def test_sweep_is_refused_where_it_does_not_apply_and_can_be_left(params):
         assert np.array_equal(ga[k], gr[k]), k
     a.destroy()
     ref.destroy()
+
+
+@pytest.mark.parametrize("cells,prec,radial", [(4, S.SL_PREC_FP64, 2), (6, S.SL_PREC_MIXED, 2), (9, S.SL_PREC_MIXED, 1)])
+def test_launches_of_a_sweep_are_counted(cells, prec, radial, params):
+    """Per step two halves and a rebuild of one launch; per evaluation the radial part (in two kernels in the
+    smallest systems), angular part, network and backward; a rotation after every evaluation but a step's last."""
+    s = S.system_from_workload(W.fege_cube(cells, seed=3), params, precision=prec)
+    s.set_spin_sweep(True)
+    before, steps = s.info()["n_launches"], 2
+    s.step(steps, 1.0, 300.0)
+    evaluations = s.sweep_colours()[2]
+    assert s.info()["n_launches"] - before == 3 * steps + evaluations * (radial + 3) + (evaluations - steps)
+    s.destroy()
