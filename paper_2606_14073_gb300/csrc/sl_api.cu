@@ -1639,7 +1639,7 @@ static int fused_steps(sl_batch *b, const std::vector<int> &active, const int64_
     const int k = (int)b->sys.size();
     const sl::Sys &m = b->sys[active[0]]->s;
     sl::FusedBatch &f = b->fused;
-    if (!f.ready(m.prec, k, m.device) && !f.setup(m.prec, k, m.device))
+    if (!f.ready(m.prec, k, m.device) && !f.setup(m.prec, k, m.device, b->stream))
         return fail(SL_ENOMEM, "fused batch tables (%d slots)", k);
     for (int i = 0; i < k; ++i) f.assign(i, b->sys[i] ? &b->sys[i]->s : nullptr);
     f.reserve(b->reserve_atoms);

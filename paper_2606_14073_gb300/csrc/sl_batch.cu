@@ -178,7 +178,7 @@ void FusedBatch::release() {
     for (int64_t &x : grid_items) x = 0;
 }
 
-bool FusedBatch::setup(int prec, int cap, int device) {
+bool FusedBatch::setup(int prec, int cap, int device, cudaStream_t st) {
     release();
     if (cap < 1 || cap > FUSED_MAX_SLOTS) return false;
     fused_layout(t, prec, cap);
@@ -194,7 +194,8 @@ bool FusedBatch::setup(int prec, int cap, int device) {
         return false;
     }
     std::memset(img, 0, t.upload_bytes);
-    if (cudaMemset(t.dev, 0, t.bytes) != cudaSuccess) {
+    // on the batch's stream, which is not ordered against the default stream's work
+    if (cudaMemsetAsync(t.dev, 0, t.bytes, st) != cudaSuccess) {
         release();
         return false;
     }

@@ -163,7 +163,7 @@ public:
     ~FusedBatch();
 
     // tables for `cap` slots in precision `prec` on the current device; false on failure
-    bool setup(int prec, int cap, int device);
+    bool setup(int prec, int cap, int device, cudaStream_t st);
     bool ready(int prec, int cap, int device) const {
         return t.dev && t.prec == prec && t.cap == cap && dev_ == device;
     }

@@ -50,3 +50,23 @@ def test_a_kernel_that_cannot_be_switched_on(prec, first, joins):
         p, q = x.get_state(), y.get_state()
         for k in ("positions", "velocities", "spins", "forces", "fields"):
             assert np.array_equal(p[k], q[k]), k
+
+
+def test_default_stream_busy_while_a_batch_is_set_up():
+    """Work that the caller has queued on the default stream does not delay the clearing of a new batch's tables
+    past their use."""
+    import torch
+    make = lambda: [S.system_from_workload(W.fege_cube(c, T=300.0, seed=c), nep_params.load(),  # noqa: E731
+                                           precision=S.SL_PREC_MIXED, seed=c) for c in (4, 6)]
+    alone, together = make(), make()
+    for s in alone:
+        s.step(6, 1.0, 300.0)
+    b = S.Batch(together)
+    torch.cuda._sleep(200_000_000)   # some 0.1 s
+    for _ in range(2):
+        b.step([3, 3], [1.0] * 2, [300.0] * 2, [(0.0, 0.0, 0.0)] * 2)
+        torch.cuda.synchronize()
+    for x, y in zip(alone, together):
+        p, q = x.get_state(), y.get_state()
+        for k in ("positions", "velocities", "spins", "forces", "fields"):
+            assert np.array_equal(p[k], q[k]), k
