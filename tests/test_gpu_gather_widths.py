@@ -1,6 +1,7 @@
 """The gather on both sides of the sizes where one lane per atom takes over from several (16,384 atoms
-in FP64, 65,536 in mixed precision): forces sum to zero and the forces and fields carried
-by a step agree with those of the full evaluation at the same state."""
+in FP64, 65,536 in mixed precision, where up to 16,384 take eight and the others four): forces sum to
+zero, and the forces and fields that a system carries from its creation agree with those of the full
+evaluation at the same state."""
 import numpy as np
 import pytest
 

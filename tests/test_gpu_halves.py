@@ -13,7 +13,7 @@ pytestmark = pytest.mark.gpu
     (S.SL_PREC_FP64, 5, (1, 1, 1), None), (S.SL_PREC_FP64, 517, (1, 0, 0), "field"),
     (S.SL_PREC_FP64, 16385, (1, 1, 1), None), (S.SL_PREC_MIXED, 33, (1, 1, 1), "longitudinal"),
     (S.SL_PREC_MIXED, 4095, (1, 1, 0), "field"), (S.SL_PREC_FP64, 260, (1, 1, 1), "longitudinal"),
-    (S.SL_PREC_MIXED, 65537, (1, 1, 1), None)])
+    (S.SL_PREC_MIXED, 16385, (1, 1, 1), "field"), (S.SL_PREC_MIXED, 65537, (1, 1, 1), None)])
 def test_one_call_equals_single_steps(prec, n, per, extra):
     rng = np.random.default_rng(n)
     cells = max(3, int(np.ceil((n / 8.0) ** (1.0 / 3.0))))

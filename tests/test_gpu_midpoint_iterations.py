@@ -10,7 +10,8 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("prec,n,depth", [(S.SL_PREC_FP64, 5, 0), (S.SL_PREC_FP64, 16385, 0), (S.SL_PREC_MIXED, 33, 2),
-                                          (S.SL_PREC_MIXED, 4095, 0), (S.SL_PREC_MIXED, 65537, 0)])
+                                          (S.SL_PREC_MIXED, 4095, 0), (S.SL_PREC_MIXED, 16385, 0),
+                                          (S.SL_PREC_MIXED, 65537, 0)])
 def test_evaluations_per_step(prec, n, depth):
     rng = np.random.default_rng(n)
     cells = max(3, int(np.ceil((n / 8.0) ** (1.0 / 3.0))))
