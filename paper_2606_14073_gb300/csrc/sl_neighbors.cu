@@ -839,12 +839,12 @@ __global__ void __launch_bounds__(ONE_THREADS, LISTS_MINB) k_rebuild_one(const _
     } sm;
     __shared__ int s_ok;
     const BinArgs &r = A.bin;
-    const bool gave_up = sync[1] != 0ull, due = !A.flag || *A.flag != 0;
-    if (gave_up) {
-        if (threadIdx.x == 0) atomicOr(A.lists.status, ST_TIMEOUT);
+    // (one branch on both words, so that their loads are in flight together)
+    const int gave_up = sync[1] != 0ull, idle = A.flag ? *A.flag == 0 : 0;
+    if (gave_up | idle) {   // the flag is cleared below, after a barrier: every block has read it
+        if (gave_up && threadIdx.x == 0) atomicOr(A.lists.status, ST_TIMEOUT);
         return;
     }
-    if (!due) return;   // the flag is cleared below, after a barrier: every block has read it
     const int64_t b = blockIdx.x, nb = gridDim.x;
     bool ok = true;
     auto meet = [&]() { ok = ok && grid_barrier(sync, polls, &s_ok); };
