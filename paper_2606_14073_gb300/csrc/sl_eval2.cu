@@ -269,8 +269,9 @@ __device__ __forceinline__ R kappa_of_lm(int lm) {
 // angular and backward kernels and the gather.  The sums are
 // contracted with the coefficients once per neighbour species (q^R, q^EX, q^DMI, q^ANI,
 // q^SIA); q^O = |S|^2.
-// What bounds it: latency, at 16 warps per SM (the sums take 45 of 128 registers): 53% of issue slots, no
-// unit above 66%.  So the loads are kept in flight: the next candidate's coordinates in A, the next
+// What bounds it: latency, at 16 warps per SM (the sums take 45 of 128 registers): 50% of issue slots, no
+// unit above 56% (0.78 ms at 884,736 atoms on a crystal, 1.00 ms after 600 steps at 300 K, when a warp's atoms
+// have uneven lists).  So the loads are kept in flight: the next candidate's coordinates in A, the next
 // four's in B, the next row's in C, and the first species' 25 values all at once before the second's
 // are stored (each load behind the store before it cost 25 trips to the L2 cache): 921 to 881 us at
 // 884,736 atoms, 161 to 147 us at 110,592 (two candidates ahead in A: 898 and 147 us; A as four at a
@@ -866,9 +867,9 @@ struct AngLanes {
     // Atom grp's stages in its warp's.  With four lanes per atom (FP32) the eight atoms start in different
     // groups of four banks, 16 banks apart within a pair of atoms and 8 between pairs, so that eight
     // lanes writing their stages, a quad reading one together and the lanes reading their own
-    // harmonics meet no bank twice.  What bounds the kernel is the shared-memory and L1 data path (74%
-    // busy); with the quads 4 words apart a third of the shared-memory wavefronts were bank
-    // conflicts: 519 to 493 us at 884,736 atoms, 79 to 75 us at 110,592.
+    // harmonics meet no bank twice.  What bounds the kernel is the shared-memory and L1 data path (59%
+    // busy, issue 56%); with the quads 4 words apart (74% busy) a third of the shared-memory wavefronts were
+    // bank conflicts: 519 to 493 us at 884,736 atoms, 79 to 75 us at 110,592.
     static __device__ int stage_at(int grp) {
         return LPA == 32 ? 0 : grp * (4 * FSTAGE) + 8 * ((grp >> 1) & 1) + 12 * (grp >> 2);
     }
@@ -1572,8 +1573,8 @@ __device__ __forceinline__ void bwd_body(const NepDev<R> &P, const Eval2Args<R> 
             *reinterpret_cast<v2<R> *>(d + 8) = x2;
             __syncwarp(quad);
         }
-        // angular adjoints of this lane's harmonics lm = ql + LPA m from their records (three
-        // 16-byte loads each)
+        // angular adjoints of this lane's harmonics (lm_of) from their records of ten entries: two neighbouring
+        // harmonics' in five loads of four values, with a warp per atom one's in five of two
 #pragma unroll
         for (int m = 0; m < (NLM + LPA - 1) / LPA; ++m) {
             const int lm = lm_of<LPA>(ql, m);
@@ -1723,7 +1724,9 @@ __global__ void __launch_bounds__(128, MINB) k_bwd(const __grid_constant__ NepDe
 // us, backward 75 / 198 / 321 instead of 380 / 387 / 398 us (its 21 angular pairs fill two thirds of a
 // round of 32 lanes, so in larger systems four lanes need fewer FP64 instructions).  Mixed precision
 // at 512 / 1,728 / 2,744 / 4,096 atoms: angular 10 / 10 / 14.5 / 16 instead of 12 / 12 / 12 / 12 us,
-// backward 12 / 15 / 20 / 27 instead of 23 / 24 / 24 / 25 us.
+// backward 12 / 15 / 20 / 27 instead of 23 / 24 / 24 / 25 us.  One line serves both kernels: in mixed precision, at
+// 2,048 atoms, below where their sum crosses (2,744 atoms: 34.5 against 36 us); in FP64, at 3,040, little
+// above the largest size timed, where both still gain.
 template <typename R>
 __global__ void __launch_bounds__(128, sizeof(R) == 4 ? 4 : 1) k_ang_wide(const __grid_constant__ NepDev<R> P,
                                                                           const Eval2Args<R> *__restrict__ tab,

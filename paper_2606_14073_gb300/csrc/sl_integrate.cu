@@ -51,7 +51,7 @@ __device__ __forceinline__ void add_landau(const StepDev &P, int t, const double
 
 
 // Whether the high word (under mask) of a component times 1/L reaches `from`.
-// (The first half is bound by FP64 instructions, 74% of its pipe; with floor and rint left out where they
+// (The first half is bound by FP64 instructions, 73% of its pipe; with floor and rint left out where they
 // are 0 it takes 121 instead of 131 us at 884,736 atoms, mixed precision.)
 __device__ __forceinline__ bool outside(double x, double y, double z, const BoxDev<double> &b, unsigned mask,
                                         unsigned from) {

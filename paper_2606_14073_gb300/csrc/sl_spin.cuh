@@ -74,12 +74,14 @@ __device__ __forceinline__ void rotate_delta_f(float sx, float sy, float sz, flo
 // that neighbouring atoms read at one slot are neighbours in memory (slot-major layout); the
 // lanes' sums are added in a fixed order.  What bounds it: the records' DRAM traffic in large FP32 systems
 // (2.3 GB in 470 us at 884,736 atoms), and elsewhere the chain of a lane's slots, a few loads in flight
-// at a time: so eight slots' records are loaded together, without branches (FP64 at 32,768 atoms 92 instead
-// of 120 us a second half, FP32 at 110,592 83 instead of 85), and a
+// at a time: so several slots' records are loaded together, without branches, eight with one or four lanes per
+// atom and four with eight, which have no more of a mask word (FP64 at 32,768 atoms 92 instead of 120 us a
+// second half, FP32 at 110,592 83 instead of 85), and a
 // small system (gather_lanes) takes several lanes per atom, a larger one one.  Second half, mixed
 // precision, 512 / 13,824 / 32,768 / 64,000 / 110,592 atoms: 15 / 19 / 37 us at the first three with eight lanes, 17 /
 // 21 / 32 / 59 / 89 with four, 27 / 31 / 43 / 59 / 83 with one; FP64, 512 / 13,824 / 21,952 / 32,768 atoms: 27 / 49 / 77 / 114 us with
-// eight, 83 / 87 / 88 / 92 with one.
+// eight, 83 / 87 / 88 / 92 with one.  The eight lanes' line is one for both precisions, near where mixed
+// precision's four lanes catch up; FP64's own crossing lies between 21,952 and 32,768 atoms.
 constexpr int gather_atoms(int W) { return 256 / W; }   // atoms per 256-thread block
 inline int gather_lanes(const Sys &s) { return s.n <= 16384 ? 8 : s.prec != 0 && s.n <= 65536 ? 4 : 1; }
 // launch(W) with the system's W (R: its precision) as a constant
@@ -128,7 +130,7 @@ __device__ __forceinline__ void gather_lane(const GatherArgs<R> &g, int64_t k, i
 #pragma unroll 1
     for (int w = 0; w < g.maskw; ++w) {
         const uint32_t word = ro(g.mask + (int64_t)w * N + k);
-constexpr int U = 4 * W <= 16 ? 8 : 4;   // slots at a time
+        constexpr int U = 4 * W <= 16 ? 8 : 4;   // slots at a time
 #pragma unroll 1
         for (int b = q; b < 32; b += U * W) {
             if ((word >> b) == 0u) break;
